@@ -79,8 +79,8 @@ typedef struct {
                         /* flattens out, Sec. "A new computational philosophy")           */
   int reduce_slices;    /* 0: the products with an n x n operand (the reduction to standard */
                         /* form, W = C Q, X = L^-H Q, A X, B X) run on the FP64 pipe. 1..8: */
-                        /* they are emulated on the tensor cores with that many 7-bit digits */
-                        /* per entry (Ozaki scheme, exact digit products; 8 digits keep     */
+                        /* they are emulated on the tensor cores with entries of that many 7-bit */
+                        /* digits (exact integer products by residues; 8 digits keep        */
                         /* FP64-class accuracy), see gevp_zgemm_emulated; the batched form  */
                         /* emulates them one k-point at a time. Requires n <= 30720.        */
 } gevp_opts;
@@ -339,16 +339,20 @@ gevp_status gevp_assign_min_cost(int ko, int kn, const double* cost, int64_t* pe
  * A is M x K (opA 0, lda >= K) or K x M (opA 1, lda >= M), B is K x N (opB 0, ldb >= N) or
  * N x K (opB 1, ldb >= K); device row-major complex128. Each row of op(A) and each column
  * of op(B) is scaled by a power of two so its
- * largest real or imaginary part lies in [1/4, 1/2), rounded to `slices` signed 7-bit
- * digits (1..8) and the digit planes are multiplied exactly in BF16 with FP32
- * accumulation (units of at most 2048 complex terms); pairs of digits whose weights sum
- * past the last digit are left out; the exact integer sums are combined in FP64.
- *   Error of entry (i, j): at most about 2K (slices + 3) 2^(-7 slices + 2) max_k|op(A)_ik|
+ * largest real or imaginary part lies in [1/4, 1/2) and rounded to a whole number of
+ * 2^(-7 slices) (1..8: `slices` 7-bit digits). The product of the whole numbers is formed
+ * exactly, modulo enough coprime numbers below 256 (16 for 8 digits and K up to about 7900,
+ * at most 17), whose residues are multiplied in BF16 with FP32 accumulation (at most 1024
+ * real terms at a time); it is recovered by the Chinese remainder theorem in integer
+ * arithmetic and rounded to FP64 once.
+ *   Error of entry (i, j): at most about 2K 2^(-7 slices + 4) max_k|op(A)_ik|
  *   max_k|op(B)_kj| (FP64's own bound is K u sum_k |op(A)_ik||op(B)_kj|, u = 2^-53); with
  *   8 digits the two are of the same order.
  *   K <= 30720 (else GEVP_ERR_UNSUPPORTED); GEVP_ERR_INVALID_VALUE on NaN or Inf in A or B.
- *   Device scratch of slices * (4 M_pad + 6 N_pad) * K_pad bytes (M_pad, N_pad: M, N
- *   rounded up to 128; K_pad: K rounded up to 64) is kept by the handle. Needs an sm_103 device (GEVP_ERR_UNSUPPORTED otherwise).
+ *   Device scratch of up to 68 (M + N) K + 34 M N bytes at 8 digits (the latter at most 1 GiB
+ * or 256 rows of the result) is kept by the handle; where the operands' part would take more
+ * than a third of the device's memory or cannot be had, a quarter of it. Needs an sm_103
+ * device (GEVP_ERR_UNSUPPORTED otherwise).
  *   Returns after the work is complete. */
 gevp_status gevp_zgemm_emulated(gevp_handle h, int opA, int opB, int M, int N, int K, const void* A, int64_t lda,
                                 const void* B, int64_t ldb, void* D, int64_t ldd, int slices);
@@ -406,8 +410,8 @@ gevp_status gevp_kernel_timing(int enable);
 /* out (host, 12 doubles): for class 0 (FP64 complex GEMM), class 1 (emulated product) and
  * class 2 (tall-skinny Gram kernel), four values each: launches, total milliseconds,
  * algorithmic flop (8 per complex multiply-add over the K ranges the tiles process, at
- * 64-, 128- resp. 16-row block granularity) and executed flop (class 1: the digit pairs'
- * BF16 real products, 36x the algorithmic at 8 digits). Waits for the recorded events. */
+ * 64-, 256- resp. 16-row block granularity) and executed flop (class 1: the residues' BF16
+ * real products, 16x the algorithmic at 8 digits). Waits for the recorded events. */
 gevp_status gevp_kernel_timing_read(double* out);
 
 /* Number of kernels the library launched since it was loaded, process-wide: every handle,

@@ -119,31 +119,29 @@ struct BatchPlan {
   float t_step = 0.f, t_rest = 0.f;   // ms per filter step (whole batch), ms per round besides the filter
   std::vector<int> bucket;
   int cap_bucket[kBuckets];
-  // emulated reduction: digit forms of every k-point's L^-1 (left operand) and L^-H (right
-  // operand), made once per call, plus one k-point's worth of scratch for tril(A) and T
+  // emulated products: residues of every k-point's L^-1 (rows; conjugated, the columns of
+  // L^-H), made once per call, plus one k-point's worth of scratch for tril(A) and T
   int oz_S = 0;
+  int oz_group = 0;   // moduli per group the operands are kept in (0: all of them)
   int oz_key = 0;   // reduce_slices the plan (and its captured round) was built for
   char* oz_mem = nullptr;
-  size_t oz_bytes = 0;
   std::vector<OzOperand> ozLA, ozLB;
   OzOperand ozAB, ozTA;
   char* oz_scratch = nullptr;
-  // W = C Q of every round: the digits of each k-point's C (made once per step) and one
+  // W = C Q of every round: the residues of each k-point's C (made once per step) and one
   // k-point's block (made per round, inside the captured round)
   std::vector<OzOperand> ozC;
   OzOperand ozQ;
   char* oz_cq = nullptr;
-  size_t oz_cq_bytes = 0;
-  char* oz_qs = nullptr;   // the block's digits (inside oz_cq)
-  // the final check's X = L^-H Q, A X, B X: digits of every k-point's L^-H (rows) and B
+  char* oz_qs = nullptr;   // the block's residues (inside oz_cq)
+  // the final check's X = L^-H Q, A X, B X: residues of every k-point's L^-H (rows) and B
   // (rows), made once per call, and one k-point's A (per check)
   std::vector<OzOperand> ozLH, ozBd;
   OzOperand ozAd;
   char* oz_fin = nullptr;
-  size_t oz_fin_bytes = 0;
-  char* oz_ad = nullptr;   // A's digits (inside oz_fin)
-  double* oz_ws = nullptr;  // split-K partials of one k-point's thin product
-  size_t oz_ws_doubles = 0;
+  char* oz_ad = nullptr;   // A's residues (inside oz_fin)
+  char* oz_ws = nullptr;  // residues of one k-point's product
+  size_t oz_ws_bytes = 0;
   int* oz_flags = nullptr;   // device: [0] kernel error code, [1] non-finite entry
   std::vector<cudaEvent_t> ev;
 };
@@ -521,8 +519,8 @@ void enqueue_rr(BatchPlan* P, cudaStream_t s, bool tune) {
     // W = C Q emulated per k-point; a converged k-point's launches do nothing
     for (int k = 0; k < np; ++k) {
       const BDesc& d = P->hD[k];
-      oz_split(P->ozQ, P->oz_qs, d.m, d.n, d.Q, d.m, 0, 0, P->oz_S, 3, P->oz_flags + 1, s, true, d.flags);
-      oz_gemm(P->ozC[k], P->ozQ, 0, 0, d.Wt, d.m, P->oz_flags, s, d.flags, P->oz_ws, P->oz_ws_doubles);
+      oz_split(P->ozQ, P->oz_qs, d.m, d.n, d.Q, d.m, 0, 0, P->oz_S, P->oz_flags + 1, s, true, d.flags, P->oz_group);
+      oz_gemm(P->ozC[k], P->ozQ, 0, 0, d.Wt, d.m, P->oz_flags, s, d.flags, P->oz_ws, P->oz_ws_bytes);
     }
   } else {
     launch(P, P->c_wt, s, tune);
@@ -743,26 +741,47 @@ extern "C" gevp_status gevp_solve_batched(gevp_handle h, int nk, int nsteps, con
   enum { EV_T0 = 2, EV_CHOL, EV_RED, EV_BND, EV_RND0, EV_RND1, EV_FIN0, EV_FIN1, EV_F0, EV_F1, EV_END };
   BCK(cudaEventRecord(evt(P, EV_T0), s));
 
-  // digit memory of the emulated products (o.reduce_slices digits per entry): the L^-1
-  // operands of every k-point and a scratch pair; the factorisations below use the front
-  // of it before the L^-1 operands are split there
+  // memory of the emulated products (o.reduce_slices digits per entry): the L^-1 operands of
+  // every k-point and a scratch pair (the factorisations below use the front of it before the
+  // L^-1 operands are written there); the C operands and one block; the final check's; the
+  // residues of a product. All moduli at once, or groups of four when that cannot be had.
   P->oz_S = P->nmax <= 30720 ? P->oz_key : 0;
-  if (P->oz_S > 0) {
+  if (P->oz_S > 0 && !P->oz_mem) {
+    // (kept while the plan is: the captured round holds these addresses)
     const int S = P->oz_S;
-    size_t need = 256, scratch = 0;
-    for (int k = 0; k < np; ++k) {
-      const int nk_ = (int)n[k];
-      need += oz_operand_bytes(nk_, nk_, S, 2) + oz_operand_bytes(nk_, nk_, S, 3);
-      scratch = std::max(scratch, oz_operand_bytes(nk_, nk_, S, 2) + oz_operand_bytes(nk_, nk_, S, 3));
+    for (int group : {0, 4}) {
+      size_t mem = 256, scratch = 0, cq = 256, qs = 0, fb = 256, ab = 0, ws = 0;
+      for (int k = 0; k < np; ++k) {
+        const int nk_ = (int)n[k];
+        const size_t b = oz_operand_bytes(nk_, nk_, S, group);
+        mem += b;
+        scratch = std::max(scratch, 2 * b);
+        cq += b;
+        qs = std::max(qs, oz_operand_bytes(m[k], nk_, S, group));
+        fb += 2 * b;
+        ab = std::max(ab, b);
+        ws = std::max(ws, std::max(oz_work_bytes(256, nk_, nk_, S),
+                                   std::min<size_t>(oz_work_bytes(nk_, nk_, nk_, S), (size_t)1 << 30)));
+      }
+      cudaError_t e = cudaMalloc(&P->oz_mem, mem + scratch);
+      if (e == cudaSuccess) e = cudaMalloc(&P->oz_cq, cq + qs);
+      if (e == cudaSuccess) e = cudaMalloc(&P->oz_fin, fb + ab);
+      if (e == cudaSuccess) e = cudaMalloc(&P->oz_ws, ws);
+      if (e == cudaSuccess) {
+        P->oz_group = group;
+        P->oz_qs = P->oz_cq + cq;
+        P->oz_ws_bytes = ws;
+        break;
+      }
+      for (char** q : {&P->oz_mem, &P->oz_cq, &P->oz_fin, &P->oz_ws}) {
+        if (*q) cudaFree(*q);
+        *q = nullptr;
+      }
+      cudaGetLastError();
+      if (group != 0 || e != cudaErrorMemoryAllocation) return fail(e, "operands of the emulated products");
     }
-    need += scratch;
-    if (need > P->oz_bytes) {
-      if (P->oz_mem) cudaFree(P->oz_mem);
-      P->oz_mem = nullptr;
-      P->oz_bytes = 0;
-      BCK(cudaMalloc(&P->oz_mem, need));
-      P->oz_bytes = need;
-    }
+  }
+  if (P->oz_S > 0) {
     P->oz_flags = (int*)P->oz_mem;
     BCK(cudaMemsetAsync(P->oz_flags, 0, 2 * sizeof(int), s));
   }
@@ -777,11 +796,12 @@ extern "C" gevp_status gevp_solve_batched(gevp_handle h, int nk, int nsteps, con
     if (P->oz_S > 0) {
       CholRes r{};
       r.memA = P->oz_mem + 256;
-      r.memB = r.memA + oz_operand_bytes((int)n[k], (int)n[k], P->oz_S, 2);
+      r.memB = r.memA + oz_operand_bytes((int)n[k], (int)n[k], P->oz_S, P->oz_group);
       r.T = d.T;
       r.ldt = n[k];
       r.ws = P->oz_ws;
-      r.ws_doubles = P->oz_ws_doubles;
+      r.ws_bytes = P->oz_ws_bytes;
+      r.group = P->oz_group;
       r.flags = P->oz_flags;
       r.info = P->dInfo + k;
       r.S = P->oz_S;
@@ -812,42 +832,13 @@ extern "C" gevp_status gevp_solve_batched(gevp_handle h, int nk, int nsteps, con
     for (int k = 0; k < np; ++k) {
       const BDesc& d = P->hD[k];
       const int nk_ = (int)n[k];
-      BCK(oz_split(P->ozLA[k], q, nk_, nk_, d.Linv, n[k], 0, 2, S, 2, P->oz_flags + 1, s));
-      q += oz_operand_bytes(nk_, nk_, S, 2);
-      BCK(oz_split(P->ozLB[k], q, nk_, nk_, d.Linv, n[k], 1, 2, S, 3, P->oz_flags + 1, s));
-      q += oz_operand_bytes(nk_, nk_, S, 3);
+      BCK(oz_split(P->ozLA[k], q, nk_, nk_, d.Linv, n[k], 0, 2, S, P->oz_flags + 1, s, false, nullptr, P->oz_group));
+      P->ozLB[k] = P->ozLA[k];
+      P->ozLB[k].conj = 1;
+      q += oz_operand_bytes(nk_, nk_, S, P->oz_group);
     }
     P->oz_scratch = q;
-    // digits of C (one per k-point) and of one block (the largest)
-    size_t cq = 256, qs = 0;
-    for (int k = 0; k < np; ++k) {
-      cq += oz_operand_bytes((int)n[k], (int)n[k], S, 2);
-      qs = std::max(qs, oz_operand_bytes(P->hD[k].m, (int)n[k], S, 3));
-    }
-    cq += qs;
-    if (cq > P->oz_cq_bytes) {
-      if (P->oz_cq) cudaFree(P->oz_cq);
-      P->oz_cq = nullptr;
-      P->oz_cq_bytes = 0;
-      BCK(cudaMalloc(&P->oz_cq, cq));
-      P->oz_cq_bytes = cq;
-    }
-    P->oz_qs = P->oz_cq + (cq - qs);
     P->ozC.assign(np, OzOperand{});
-    // L^-H and B digits for the final check, and room for one A
-    size_t fb = 256, ab = 0;
-    for (int k = 0; k < np; ++k) {
-      fb += 2 * oz_operand_bytes((int)n[k], (int)n[k], S, 2);
-      ab = std::max(ab, oz_operand_bytes((int)n[k], (int)n[k], S, 2));
-    }
-    fb += ab;
-    if (fb > P->oz_fin_bytes) {
-      if (P->oz_fin) cudaFree(P->oz_fin);
-      P->oz_fin = nullptr;
-      P->oz_fin_bytes = 0;
-      BCK(cudaMalloc(&P->oz_fin, fb));
-      P->oz_fin_bytes = fb;
-    }
     P->ozLH.assign(np, OzOperand{});
     P->ozBd.assign(np, OzOperand{});
     char* f = P->oz_fin;
@@ -855,21 +846,13 @@ extern "C" gevp_status gevp_solve_batched(gevp_handle h, int nk, int nsteps, con
       const BDesc& d = P->hD[k];
       const int nk_ = (int)n[k];
       // rows of L^-H (upper) = conjugated columns of L^-1
-      BCK(oz_split(P->ozLH[k], f, nk_, nk_, d.Linv, n[k], 1, 3, S, 2, P->oz_flags + 1, s, true));
-      f += oz_operand_bytes(nk_, nk_, S, 2);
-      BCK(oz_split(P->ozBd[k], f, nk_, nk_, (const double2*)B[k], ldb[k], 0, 0, S, 2, P->oz_flags + 1, s));
-      f += oz_operand_bytes(nk_, nk_, S, 2);
+      BCK(oz_split(P->ozLH[k], f, nk_, nk_, d.Linv, n[k], 1, 3, S, P->oz_flags + 1, s, true, nullptr, P->oz_group));
+      f += oz_operand_bytes(nk_, nk_, S, P->oz_group);
+      BCK(oz_split(P->ozBd[k], f, nk_, nk_, (const double2*)B[k], ldb[k], 0, 0, S, P->oz_flags + 1, s, false, nullptr,
+                   P->oz_group));
+      f += oz_operand_bytes(nk_, nk_, S, P->oz_group);
     }
     P->oz_ad = f;
-    size_t wd = 0;
-    for (int k = 0; k < np; ++k) wd = std::max(wd, oz_split_k_doubles((int)n[k], P->hD[k].m));
-    if (wd > P->oz_ws_doubles) {
-      if (P->oz_ws) cudaFree(P->oz_ws);
-      P->oz_ws = nullptr;
-      P->oz_ws_doubles = 0;
-      BCK(cudaMalloc(&P->oz_ws, wd * sizeof(double)));
-      P->oz_ws_doubles = wd;
-    }
   }
   float ms = 0.f;
   cudaEventElapsedTime(&ms, evt(P, EV_T0), evt(P, EV_CHOL));
@@ -934,11 +917,11 @@ extern "C" gevp_status gevp_solve_batched(gevp_handle h, int nk, int nsteps, con
         const BDesc& d = P->hD[k];
         const int nk_ = (int)n[k], S = P->oz_S;
         char* base = P->oz_scratch;
-        BCK(oz_split(P->ozAB, base, nk_, nk_, d.A, d.lda, 1, 1, S, 3, P->oz_flags + 1, s));
-        BCK(oz_gemm(P->ozLA[k], P->ozAB, 1, 1, d.T, n[k], P->oz_flags, s));
-        BCK(oz_split(P->ozTA, base + oz_operand_bytes(nk_, nk_, S, 3), nk_, nk_, d.T, n[k], 0, 2, S, 2,
-                     P->oz_flags + 1, s));
-        BCK(oz_gemm(P->ozTA, P->ozLB[k], 1, 2, d.C, n[k], P->oz_flags, s));
+        BCK(oz_split(P->ozAB, base, nk_, nk_, d.A, d.lda, 1, 1, S, P->oz_flags + 1, s, false, nullptr, P->oz_group));
+        BCK(oz_gemm(P->ozLA[k], P->ozAB, 1, 1, d.T, n[k], P->oz_flags, s, nullptr, P->oz_ws, P->oz_ws_bytes));
+        BCK(oz_split(P->ozTA, base + oz_operand_bytes(nk_, nk_, S, P->oz_group), nk_, nk_, d.T, n[k], 0, 2, S,
+                     P->oz_flags + 1, s, false, nullptr, P->oz_group));
+        BCK(oz_gemm(P->ozTA, P->ozLB[k], 1, 2, d.C, n[k], P->oz_flags, s, nullptr, P->oz_ws, P->oz_ws_bytes));
       }
     } else {
       launch(P, P->c_red1, s, tune);
@@ -946,12 +929,13 @@ extern "C" gevp_status gevp_solve_batched(gevp_handle h, int nk, int nsteps, con
     }
     bk_herm_sum(P->dD, np, P->nmax, s);
     if (P->oz_S > 0) {
-      // the digits of every C for the rounds' W = C Q
+      // the residues of every C for the rounds' W = C Q
       char* q = P->oz_cq;
       for (int k = 0; k < np; ++k) {
         const BDesc& d = P->hD[k];
-        BCK(oz_split(P->ozC[k], q, (int)n[k], (int)n[k], d.C, n[k], 0, 0, P->oz_S, 2, P->oz_flags + 1, s));
-        q += oz_operand_bytes((int)n[k], (int)n[k], P->oz_S, 2);
+        BCK(oz_split(P->ozC[k], q, (int)n[k], (int)n[k], d.C, n[k], 0, 0, P->oz_S, P->oz_flags + 1, s, false, nullptr,
+                     P->oz_group));
+        q += oz_operand_bytes((int)n[k], (int)n[k], P->oz_S, P->oz_group);
       }
     }
     BCK(cudaEventRecord(evt(P, EV_RED), s));
@@ -1008,12 +992,14 @@ extern "C" gevp_status gevp_solve_batched(gevp_handle h, int nk, int nsteps, con
           for (int k = 0; k < np; ++k) {
             const BDesc& d = P->hD[k];
             const int* fin = d.flags + 12;
-            BCK(oz_split(P->ozQ, P->oz_qs, d.nev, d.n, d.Q, d.m, 0, 0, S, 3, P->oz_flags + 1, s, true, fin));
-            BCK(oz_gemm(P->ozLH[k], P->ozQ, 2, 0, d.Xf, d.m, P->oz_flags, s, fin, P->oz_ws, P->oz_ws_doubles));
-            BCK(oz_split(P->ozAd, P->oz_ad, d.n, d.n, d.A, d.lda, 0, 0, S, 2, P->oz_flags + 1, s, false, fin));
-            BCK(oz_split(P->ozQ, P->oz_qs, d.nev, d.n, d.Xf, d.m, 0, 0, S, 3, P->oz_flags + 1, s, true, fin));
-            BCK(oz_gemm(P->ozAd, P->ozQ, 0, 0, d.Y1, d.m, P->oz_flags, s, fin, P->oz_ws, P->oz_ws_doubles));
-            BCK(oz_gemm(P->ozBd[k], P->ozQ, 0, 0, d.Y2, d.m, P->oz_flags, s, fin, P->oz_ws, P->oz_ws_doubles));
+            BCK(oz_split(P->ozQ, P->oz_qs, d.nev, d.n, d.Q, d.m, 0, 0, S, P->oz_flags + 1, s, true, fin, P->oz_group));
+            BCK(oz_gemm(P->ozLH[k], P->ozQ, 2, 0, d.Xf, d.m, P->oz_flags, s, fin, P->oz_ws, P->oz_ws_bytes));
+            BCK(oz_split(P->ozAd, P->oz_ad, d.n, d.n, d.A, d.lda, 0, 0, S, P->oz_flags + 1, s, false, fin,
+                         P->oz_group));
+            BCK(oz_split(P->ozQ, P->oz_qs, d.nev, d.n, d.Xf, d.m, 0, 0, S, P->oz_flags + 1, s, true, fin,
+                         P->oz_group));
+            BCK(oz_gemm(P->ozAd, P->ozQ, 0, 0, d.Y1, d.m, P->oz_flags, s, fin, P->oz_ws, P->oz_ws_bytes));
+            BCK(oz_gemm(P->ozBd[k], P->ozQ, 0, 0, d.Y2, d.m, P->oz_flags, s, fin, P->oz_ws, P->oz_ws_bytes));
           }
         } else {
           launch(P, P->c_xf, s, tune);

@@ -354,14 +354,13 @@ struct CholRec {
   cudaError_t err = cudaSuccess;
 
   bool product(OzOperand& a, OzOperand& b, int triA, int triB, double2* D, int64_t ldd) {
-    const bool ws = r.ws && oz_split_k_doubles(a.rows, b.rows) <= r.ws_doubles;
-    err = oz_gemm(a, b, triA, triB, D, ldd, r.flags, r.s, nullptr, ws ? r.ws : nullptr, ws ? r.ws_doubles : 0);
+    err = oz_gemm(a, b, triA, triB, D, ldd, r.flags, r.s, nullptr, r.ws, r.ws_bytes);
     return err == cudaSuccess;
   }
   bool split(OzOperand& op, bool roleA, int rows, int K, const double2* X, int64_t ldx, int conj, int mask,
              bool cols) {
-    err = oz_split(op, roleA ? r.memA : r.memB, rows, K, X, ldx, conj, mask, r.S, roleA ? 2 : 3, r.flags + 1, r.s,
-                   cols);
+    err = oz_split(op, roleA ? r.memA : r.memB, rows, K, X, ldx, conj, mask, r.S, r.flags + 1, r.s, cols, nullptr,
+                   r.group);
     return err == cudaSuccess;
   }
   // false with err == cudaSuccess: a leaf could not be launched (nothing enqueued if k0 == 0)

@@ -61,11 +61,16 @@ struct gevp_ctx {
   size_t vd2_bytes = 0;
   char* dvbuf = nullptr;                    // deviation-angle scratch (grown on demand)
   size_t dvbuf_bytes = 0;
-  // emulated FP64 products of the reduction (digit form of L^-1 for both roles, and per
-  // stream the digit forms of tril(A) and of T = L^-1 tril(A)); grown on demand
+  // emulated FP64 products (residue form of L^-1, and per stream those of tril(A) and of
+  // T = L^-1 tril(A)); grown on demand
   int oz_slices = 0;                        // 0: FP64 pipe; 1..8: emulated with that many digits
   char* ozmem[2] = {nullptr, nullptr};      // [0] L^-1 operands + main-stream scratch, [1] side stream
   size_t ozmem_bytes[2] = {0, 0};
+  int oz_regions = 6;                       // operand regions of ozmem[0] that the entry point uses
+  int oz_group[2] = {0, 0};                 // moduli per group the operands are kept in (0: all of them)
+  int64_t oz_n[2] = {0, 0};                 // order the scratch was last prepared for
+  int oz_S[2] = {0, 0};
+  int64_t oz_full_max = INT64_MAX;          // order from which on only a group's planes are kept
   gevp::OzOperand ozLA, ozLB, ozAB[2], ozTA[2];
   // solver products on the main stream: C (rows, per problem), A (rows, per final check),
   // B (rows, kept while the factorisation is), the block (columns, per product)
@@ -79,10 +84,8 @@ struct gevp_ctx {
   int64_t* jidx = nullptr;                  // device copy of the changed rows
   size_t jidx_cap = 0;
   int64_t ozLH_gen = -1;                    // chol_gen the L^-H rows (ozLH) were split from
-  double* ozws = nullptr;                   // split-K partials of the thin emulated products
-  size_t ozws_doubles = 0;
-  const void* ozC_src = nullptr;            // the C whose digits ozC holds (null: none)
-  const void* ozB_src = nullptr;            // the B whose digits ozB holds, for chol_gen ozB_gen
+  const void* ozC_src = nullptr;            // the C whose residues ozC holds (null: none)
+  const void* ozB_src = nullptr;            // the B whose residues ozB holds, for chol_gen ozB_gen
   int64_t ozB_gen = -1;
   int64_t oz_l_gen = -1;                    // chol_gen the L^-1 operands were split from
   int oz_l_S = 0;
@@ -373,9 +376,9 @@ void reduce_into_ws(int64_t n, const double2* Linv, const double2* A, int64_t ld
 }
 
 // The same reduction with the n^3 products emulated on the tensor cores (slices digits
-// per entry): T = L^-1 tril_half(A) and M = T L^-H as digit-form products, then C = M + M^H.
+// per entry): T = L^-1 tril_half(A) and M = T L^-H as products of residues, then C = M + M^H.
 // side 0 runs on the main stream, side 1 on the pipeline's side stream (own scratch). The
-// digit forms of L^-1 are made once per factorisation of B, on the main stream.
+// residues of L^-1 are made once per factorisation of B, on the main stream.
 // the device status words of the emulated products ([0] error code, [1] non-finite entry)
 gevp_status oz_flags_ready(gevp_ctx* h) {
   if (h->ozflags) return GEVP_OK;
@@ -386,56 +389,93 @@ gevp_status oz_flags_ready(gevp_ctx* h) {
   return GEVP_OK;
 }
 
-// device scratch of the emulated products: ozmem[side] of at least `need` bytes
-gevp_status oz_reserve(gevp_ctx* h, int side, size_t need) {
+// Device scratch of the emulated products of order n on a stream (side 0: main, 1: the
+// pipeline's side stream): [residues of a result | operand regions]. Main stream: 0 L^-1 rows,
+// 1 tril(A) / the block, 2 T / C, 3 L^-H rows (the back-transform's left operand), 4 A, 5 B, the
+// last three only for the solver (the solver's C takes the region of T and the block that of
+// tril(A): the reduction of a problem is finished before its solve starts, on the same
+// stream); side stream: 0 tril(A), 1 T.
+// A region holds the residues of all moduli (64 bytes per entry at 8 digits), unless that
+// would take more than a third of the device's memory or cannot be had: then those of a group
+// of four (16 bytes per entry), rewritten from the matrix for every product.
+size_t oz_result_bytes(int64_t n, int S) {
+  const size_t panel = gevp::oz_work_bytes(256, (int)n, (int)n, S);
+  return al(std::max(panel, std::min<size_t>(gevp::oz_work_bytes((int)n, (int)n, (int)n, S), (size_t)1 << 30)));
+}
+size_t oz_region_bytes(const gevp_ctx* h, int side, int64_t n) {
+  return al(gevp::oz_operand_bytes((int)n, (int)n, h->oz_slices, h->oz_group[side]));
+}
+gevp_status oz_prepare(gevp_ctx* h, int side, int64_t n) {
   TRY(oz_flags_ready(h));
-  if (need <= h->ozmem_bytes[side]) return GEVP_OK;
-  // the other stream may still read this side's (or, for side 0, the shared) operands
-  cudaDeviceSynchronize();
-  if (h->ozmem[side]) cudaFree(h->ozmem[side]);
-  h->ozmem[side] = nullptr;
-  h->ozmem_bytes[side] = 0;
-  if (side == 0) {
-    h->oz_l_gen = -1;
-    h->ozC_src = nullptr;
-    h->ozB_src = nullptr;
-    h->ozLH_gen = -1;
+  const int S = h->oz_slices, regions = side == 0 ? h->oz_regions : 2;
+  if (n < h->oz_full_max) {
+    size_t freeb = 0, total = 0;
+    CK(cudaMemGetInfo(&freeb, &total));
+    const size_t full = regions * al(gevp::oz_operand_bytes((int)n, (int)n, S, 0));
+    if (full > total / 3) h->oz_full_max = n;
   }
-  void* p = nullptr;
-  CK(cudaMalloc(&p, need));
-  h->ozmem[side] = (char*)p;
-  h->ozmem_bytes[side] = need;
-  return GEVP_OK;
+  for (int pass = 0; pass < 2; ++pass) {
+    const int group = (pass == 0 && n < h->oz_full_max) ? 0 : 4;
+    const size_t need = oz_result_bytes(n, S) + regions * al(gevp::oz_operand_bytes((int)n, (int)n, S, group));
+    if (need > h->ozmem_bytes[side]) {
+      // the other stream may still read this side's (or, for side 0, the shared) operands
+      cudaDeviceSynchronize();
+      if (h->ozmem[side]) cudaFree(h->ozmem[side]);
+      h->ozmem[side] = nullptr;
+      h->ozmem_bytes[side] = 0;
+      h->oz_n[side] = 0;
+      void* p = nullptr;
+      const cudaError_t e = cudaMalloc(&p, need);
+      if (e == cudaErrorMemoryAllocation && group == 0) {
+        cudaGetLastError();
+        h->oz_full_max = n;
+        continue;
+      }
+      CK(e);
+      h->ozmem[side] = (char*)p;
+      h->ozmem_bytes[side] = need;
+    }
+    if (h->oz_n[side] != n || h->oz_S[side] != S || h->oz_group[side] != group) {
+      if (side == 0) {
+        h->oz_l_gen = -1;
+        h->ozC_src = nullptr;
+        h->ozB_src = nullptr;
+        h->ozLH_gen = -1;
+      }
+      h->oz_n[side] = n;
+      h->oz_S[side] = S;
+      h->oz_group[side] = group;
+    }
+    return GEVP_OK;
+  }
+  return GEVP_ERR_OOM;
 }
-
-// Main-stream digit scratch: [L^-1 rows | L^-H columns | reduction: tril(A) | T | A | B |
-// L^-H rows (the back-transform's left operand)]
-// (the solver's C digits reuse the T region and the block's digits the tril(A) region:
-// the reduction of a problem is finished before its solve starts, on the same stream)
-size_t oz_main_bytes(int64_t n, int S) {
-  const size_t bA = gevp::oz_operand_bytes((int)n, (int)n, S, 2), bB = gevp::oz_operand_bytes((int)n, (int)n, S, 3);
-  return 5 * bA + 2 * bB;
+char* oz_region(gevp_ctx* h, int64_t n, int which, int side = 0) {
+  return h->ozmem[side] + oz_result_bytes(n, h->oz_slices) + which * oz_region_bytes(h, side, n);
 }
-// 0 L^-1, 1 L^-H columns, 2 tril(A)/block, 3 T/C, 4 A, 5 B, 6 L^-H rows
-char* oz_region(gevp_ctx* h, int64_t n, int which) {
-  const int S = h->oz_slices;
-  const size_t bA = gevp::oz_operand_bytes((int)n, (int)n, S, 2), bB = gevp::oz_operand_bytes((int)n, (int)n, S, 3);
-  const size_t off[7] = {0, bA, bA + bB, bA + 2 * bB, 2 * bA + 2 * bB, 3 * bA + 2 * bB, 4 * bA + 2 * bB};
-  return h->ozmem[0] + off[which];
+// D = A B of two operands of order n's scratch
+cudaError_t oz_product(gevp_ctx* h, int side, int64_t n, const gevp::OzOperand& A, const gevp::OzOperand& B, int triA,
+                       int triB, double2* D, int64_t ldd, cudaStream_t s) {
+  return gevp::oz_gemm(A, B, triA, triB, D, ldd, h->ozflags, s, nullptr, h->ozmem[side],
+                       oz_result_bytes(n, h->oz_slices));
+}
+cudaError_t oz_operand(gevp_ctx* h, int side, gevp::OzOperand& op, char* mem, int rows, int K, const double2* X,
+                       int64_t ldx, int conj, int mask, cudaStream_t s, bool cols = false) {
+  return gevp::oz_split(op, mem, rows, K, X, ldx, conj, mask, h->oz_slices, h->ozflags + 1, s, cols, nullptr,
+                        h->oz_group[side]);
 }
 
 // D (n x ncols, ld ldd) = M X with M one of the cached square operands (ozC, ozA, ozB) and
 // X the n x ncols block (ld ldx), emulated on the main stream
 gevp_status oz_times_block(gevp_ctx* h, const gevp::OzOperand& M, int64_t n, int ncols, const double2* X,
                            int64_t ldx, double2* D, int64_t ldd) {
-  CK(gevp::oz_split(h->ozQ, oz_region(h, n, 2), ncols, (int)n, X, ldx, 0, 0, h->oz_slices, 3, h->ozflags + 1,
-                    h->stream, true));
-  CK(gevp::oz_gemm(M, h->ozQ, 0, 0, D, ldd, h->ozflags, h->stream, nullptr, h->ozws, h->ozws_doubles));
+  CK(oz_operand(h, 0, h->ozQ, oz_region(h, n, 1), ncols, (int)n, X, ldx, 0, 0, h->stream, true));
+  CK(oz_product(h, 0, n, M, h->ozQ, 0, 0, D, ldd, h->stream));
   return GEVP_OK;
 }
 
-// h->L (holding B) -> L, h->Linv -> L^-1 by chol_recursive (cholqr.cu), its digit operands
-// in the first two regions of the main-stream scratch (the L^-1 digits, remade after it).
+// h->L (holding B) -> L, h->Linv -> L^-1 by chol_recursive (cholqr.cu), its operands in the
+// block's and C's regions of the main-stream scratch (both free between solves).
 // false: not done (order above the emulated products' limit, or the cluster leaves not
 // launchable: nothing was enqueued; *st set on a failure after work was enqueued).
 bool factor_emulated(gevp_ctx* h, int64_t n, gevp_status* st) {
@@ -444,30 +484,15 @@ bool factor_emulated(gevp_ctx* h, int64_t n, gevp_status* st) {
   const int S = h->oz_slices;
   gevp::CholRes r{};
   if (n > gevp::kCholLeaf) {
-    if ((*st = oz_reserve(h, 0, oz_main_bytes(n, S))) != GEVP_OK) return false;
-    // split-K partials for the products near the leaves (up to 512 x 512 at 4 slices)
-    const size_t wd = gevp::oz_split_k_doubles(512, 512) / 2;
-    if (h->ozws_doubles < wd) {
-      if (h->ozws) {
-        cudaStreamSynchronize(h->stream);
-        cudaFree(h->ozws);
-      }
-      h->ozws = nullptr;
-      h->ozws_doubles = 0;
-      void* p = nullptr;
-      if (cudaMalloc(&p, wd * sizeof(double)) != cudaSuccess) {
-        *st = GEVP_ERR_OOM;
-        return false;
-      }
-      h->ozws = (double*)p;
-      h->ozws_doubles = wd;
-    }
-    r.memA = oz_region(h, n, 0);
-    r.memB = oz_region(h, n, 1);
+    if ((*st = oz_prepare(h, 0, n)) != GEVP_OK) return false;
+    h->ozC_src = nullptr;
+    r.memA = oz_region(h, n, 1);
+    r.memB = oz_region(h, n, 2);
     r.T = h->T;
     r.ldt = n;
-    r.ws = h->ozws;
-    r.ws_doubles = h->ozws_doubles;
+    r.ws = h->ozmem[0];
+    r.ws_bytes = oz_result_bytes(n, S);
+    r.group = h->oz_group[0];
   }
   r.flags = h->ozflags;
   r.info = h->info;
@@ -486,22 +511,21 @@ gevp_status reduce_emulated(gevp_ctx* h, int side, int64_t n, const double2* A, 
                             int64_t ldc, double2* T, cudaStream_t s) {
   const int S = h->oz_slices;
   const int nn = (int)n;
-  const size_t bA = gevp::oz_operand_bytes(nn, nn, S, 2), bB = gevp::oz_operand_bytes(nn, nn, S, 3);
-  TRY(oz_reserve(h, side, side == 0 ? oz_main_bytes(n, S) : bA + bB));
-  char* mem = h->ozmem[side];
+  TRY(oz_prepare(h, side, n));
   if (side == 0 && (h->oz_l_gen != h->chol_gen || h->oz_l_S != S)) {
-    // L^-1 as the left operand (rows, lower) and L^-H as the right one (rows of L^-1, conjugated)
-    CK(gevp::oz_split(h->ozLA, mem, nn, nn, h->Linv, n, 0, 2, S, 2, h->ozflags + 1, h->stream));
-    CK(gevp::oz_split(h->ozLB, mem + bA, nn, nn, h->Linv, n, 1, 2, S, 3, h->ozflags + 1, h->stream));
+    // L^-1 as the left operand (rows, lower); as the right one, L^-H's columns are the same rows
+    // conjugated
+    CK(oz_operand(h, 0, h->ozLA, oz_region(h, n, 0), nn, nn, h->Linv, n, 0, 2, h->stream));
+    h->ozLB = h->ozLA;
+    h->ozLB.conj = 1;
     h->oz_l_gen = h->chol_gen;
     h->oz_l_S = S;
   }
-  if (side == 0) mem += bA + bB;
   // columns of tril_half(A) are the conjugated rows of the Hermitian A from the diagonal on
-  CK(gevp::oz_split(h->ozAB[side], mem, nn, nn, A, lda, 1, 1, S, 3, h->ozflags + 1, s));
-  CK(gevp::oz_gemm(h->ozLA, h->ozAB[side], 1, 1, T, n, h->ozflags, s));
-  CK(gevp::oz_split(h->ozTA[side], mem + bB, nn, nn, T, n, 0, 2, S, 2, h->ozflags + 1, s));
-  CK(gevp::oz_gemm(h->ozTA[side], h->ozLB, 1, 2, Cout, ldc, h->ozflags, s));
+  CK(oz_operand(h, side, h->ozAB[side], oz_region(h, n, side == 0 ? 1 : 0, side), nn, nn, A, lda, 1, 1, s));
+  CK(oz_product(h, side, n, h->ozLA, h->ozAB[side], 1, 1, T, n, s));
+  CK(oz_operand(h, side, h->ozTA[side], oz_region(h, n, side == 0 ? 2 : 1, side), nn, nn, T, n, 0, 2, s));
+  CK(oz_product(h, side, n, h->ozTA[side], h->ozLB, 1, 2, Cout, ldc, s));
   herm_sum_inplace(n, Cout, ldc, s);
   return GEVP_OK;
 }
@@ -585,7 +609,7 @@ gevp_status ensure_pipeline(gevp_ctx* h) {
 // Li = L^-1 D with D W D + sh I = L L^H (one cluster launch, *info set on a non-positive
 // pivot), dst = src Li^H = src D L^-H. False if the cluster factorisation is not available
 // for this order (nothing enqueued after the Gram matrix then).
-// The product runs emulated on the tensor cores when the solve's products are (its digit
+// The product runs emulated on the tensor cores when the solve's products are (its
 // operands in the block region of the main-stream scratch, free between the filter and the
 // Rayleigh-Ritz rotation), else on the FP64 pipe.
 bool cholqr_pass(gevp_ctx* h, int64_t n, int ma, const double2* src, int64_t lds, double2* dst, int64_t ldd, double sh,
@@ -594,16 +618,14 @@ bool cholqr_pass(gevp_ctx* h, int64_t n, int ma, const double2* src, int64_t lds
   zgram(n, ma, ma, src, lds, src, lds, h->Gw, ma, 1, h->split, h->split_elems, h->gcnt, h->stream);
   if (!cholinv_small(ma, h->Gw, ma, sh, h->Gwi, ma, nullptr, 0, info, h->stream)) return false;
   const int S = h->oz_slices;
-  if (S > 0 && h->ozmem[0] && h->ozmem_bytes[0] >= oz_main_bytes(n, S) &&
-      gevp::oz_operand_bytes((int)n, ma, S, 2) + gevp::oz_operand_bytes(ma, ma, S, 3) <=
-          gevp::oz_operand_bytes((int)n, (int)n, S, 3)) {
+  const size_t yb = S > 0 ? al(gevp::oz_operand_bytes((int)n, ma, S, h->oz_group[0])) : 0;
+  if (S > 0 && h->ozmem[0] && h->oz_n[0] == n && h->oz_S[0] == S &&
+      yb + gevp::oz_operand_bytes(ma, ma, S, h->oz_group[0]) <= oz_region_bytes(h, 0, n)) {
     // dst = Y (L^-1 D)^H: the columns of (L^-1 D)^H are the conjugated rows of the lower L^-1 D
-    char* mem = oz_region(h, n, 2);
-    if (gevp::oz_split(h->ozY, mem, (int)n, ma, src, lds, 0, 0, S, 2, h->ozflags + 1, h->stream) == cudaSuccess &&
-        gevp::oz_split(h->ozLiH, mem + gevp::oz_operand_bytes((int)n, ma, S, 2), ma, ma, h->Gwi, ma, 1, 2, S, 3,
-                       h->ozflags + 1, h->stream) == cudaSuccess &&
-        gevp::oz_gemm(h->ozY, h->ozLiH, 0, 2, dst, ldd, h->ozflags, h->stream, nullptr, h->ozws, h->ozws_doubles) ==
-            cudaSuccess)
+    char* mem = oz_region(h, n, 1);
+    if (oz_operand(h, 0, h->ozY, mem, (int)n, ma, src, lds, 0, 0, h->stream) == cudaSuccess &&
+        oz_operand(h, 0, h->ozLiH, mem + yb, ma, ma, h->Gwi, ma, 1, 2, h->stream) == cudaSuccess &&
+        oz_product(h, 0, n, h->ozY, h->ozLiH, 0, 2, dst, ldd, h->stream) == cudaSuccess)
       return true;
     cudaGetLastError();
   }
@@ -714,7 +736,7 @@ gevp_status orthonormalize(gevp_ctx* h, int64_t n, int nlock, double2* Y, int64_
   return GEVP_ERR_NOT_HPD;
 }
 
-// Out = C Qa (n x ma, ld of the block), emulated when C's digits are held
+// Out = C Qa (n x ma, ld of the block), emulated when C's residues are held
 gevp_status times_C(gevp_ctx* h, int64_t n, int ma, const double2* C, int64_t ldc, const double2* Qa, double2* Out) {
   const int64_t ld = h->cap_m;
   if (h->oz_slices > 0 && h->ozC_src == (const void*)C) {
@@ -740,18 +762,16 @@ gevp_status rayleigh_ritz(gevp_ctx* h, int64_t n, int nlock, int ma, const doubl
   // FP64 launch (a batch of two products sharing Z). Q's result goes through T or Xf (free
   // until the final check), so that the filtered block in Y1/Y2 stays intact.
   const int S = h->oz_slices;
-  const size_t qw_bytes = S > 0 ? gevp::oz_operand_bytes(2 * (int)n, ma, S, 2) + gevp::oz_operand_bytes(ma, ma, S, 3)
-                                : 0;
-  // (the emulated operands' memory is reserved for this n while C's digits are held)
+  const size_t qw = S > 0 ? al(gevp::oz_operand_bytes(2 * (int)n, ma, S, h->oz_group[0])) : 0;
+  // (the emulated operands' memory is prepared for this n while C's residues are held)
   if (S > 0 && h->ozC_src == (const void*)C && 2 * n * (int64_t)ma <= n * n &&
-      qw_bytes <= gevp::oz_operand_bytes((int)n, (int)n, S, 3)) {
+      qw + gevp::oz_operand_bytes(ma, ma, S, h->oz_group[0]) <= oz_region_bytes(h, 0, n)) {
     zcopy2d(n, ma, Qa, ld, h->T, ma, h->stream);
     zcopy2d(n, ma, h->Wt, ld, h->T + n * ma, ma, h->stream);
-    char* mem = oz_region(h, n, 2);
-    CK(gevp::oz_split(h->ozQW, mem, 2 * (int)n, ma, h->T, ma, 0, 0, S, 2, h->ozflags + 1, h->stream));
-    CK(gevp::oz_split(h->ozZ, mem + gevp::oz_operand_bytes(2 * (int)n, ma, S, 2), ma, ma, h->Zs, ma, 0, 0, S, 3,
-                      h->ozflags + 1, h->stream, true));
-    CK(gevp::oz_gemm(h->ozQW, h->ozZ, 0, 0, h->T, ma, h->ozflags, h->stream, nullptr, h->ozws, h->ozws_doubles));
+    char* mem = oz_region(h, n, 1);
+    CK(oz_operand(h, 0, h->ozQW, mem, 2 * (int)n, ma, h->T, ma, 0, 0, h->stream));
+    CK(oz_operand(h, 0, h->ozZ, mem + qw, ma, ma, h->Zs, ma, 0, 0, h->stream, true));
+    CK(oz_product(h, 0, n, h->ozQW, h->ozZ, 0, 0, h->T, ma, h->stream));
     zcopy2d(n, ma, h->T, ma, Qa, ld, h->stream);
     zcopy2d(n, ma, h->T + n * ma, ma, h->W + nlock, ld, h->stream);
   } else {
@@ -882,28 +902,13 @@ gevp_status solve_one(gevp_ctx* h, int64_t n, const double2* A, int64_t lda, con
     CK(filter_tc_reserve(&h->tc, n, m, h->stream));
     CK(filter_tc_set_matrix(h->tc, n, h->C, n, nsplit, h->stream));
   }
-  // emulated products: the digits of C for every W = C Q of this problem
+  // emulated products: the residues of C for every W = C Q of this problem
   const bool oz = h->oz_slices > 0;
   bool oz_a_ready = false;
   if (oz) {
-    TRY(oz_reserve(h, 0, oz_main_bytes(n, h->oz_slices)));
-    CK(gevp::oz_split(h->ozC, oz_region(h, n, 3), (int)n, (int)n, h->C, n, 0, 0, h->oz_slices, 2, h->ozflags + 1,
-                      h->stream));
+    TRY(oz_prepare(h, 0, n));
+    CK(oz_operand(h, 0, h->ozC, oz_region(h, n, 2), (int)n, (int)n, h->C, n, 0, 0, h->stream));
     h->ozC_src = h->C;
-    // split-K partials of the n x m products (W = C Q, the back-transform, A X, B X)
-    const size_t wd = gevp::oz_split_k_doubles((int)n, m);
-    if (wd > h->ozws_doubles) {
-      if (h->ozws) {
-        cudaStreamSynchronize(h->stream);
-        cudaFree(h->ozws);
-      }
-      h->ozws = nullptr;
-      h->ozws_doubles = 0;
-      void* p = nullptr;
-      CK(cudaMalloc(&p, wd * sizeof(double)));
-      h->ozws = (double*)p;
-      h->ozws_doubles = wd;
-    }
   }
   tm.mark(PH_BOUNDS);
   if (!warm) {
@@ -937,35 +942,30 @@ gevp_status solve_one(gevp_ctx* h, int64_t n, const double2* A, int64_t lda, con
         // X = L^-H Q: the rows of L^-H (upper) are the conjugated columns of L^-1, made
         // once per factorisation
         if (h->ozLH_gen != h->chol_gen || h->ozLH.S != h->oz_slices) {
-          CK(gevp::oz_split(h->ozLH, oz_region(h, n, 6), (int)n, (int)n, h->Linv, n, 1, 3, h->oz_slices, 2,
-                            h->ozflags + 1, h->stream, true));
+          CK(oz_operand(h, 0, h->ozLH, oz_region(h, n, 3), (int)n, (int)n, h->Linv, n, 1, 3, h->stream, true));
           h->ozLH_gen = h->chol_gen;
         }
-        CK(gevp::oz_split(h->ozQ, oz_region(h, n, 2), nev, (int)n, h->Q, ld, 0, 0, h->oz_slices, 3, h->ozflags + 1,
-                          h->stream, true));
-        CK(gevp::oz_gemm(h->ozLH, h->ozQ, 2, 0, h->Xf, ld, h->ozflags, h->stream, nullptr, h->ozws, h->ozws_doubles));
+        CK(oz_operand(h, 0, h->ozQ, oz_region(h, n, 1), nev, (int)n, h->Q, ld, 0, 0, h->stream, true));
+        CK(oz_product(h, 0, n, h->ozLH, h->ozQ, 2, 0, h->Xf, ld, h->stream));
       } else {
         ZgemmArgs x = zg((int)n, nev, (int)n, h->Linv, n, 1, h->Q, ld, 0, h->Xf, ld);
         x.triA = 2;
         zgemm(x, h->split, h->split_elems, h->stream);
       }
       if (oz) {
-        // A X and B X emulated: A's digits once per problem, B's while it stays factorised
+        // A X and B X emulated: A's residues once per problem, B's while it stays factorised
         if (!oz_a_ready) {
-          CK(gevp::oz_split(h->ozA, oz_region(h, n, 4), (int)n, (int)n, A, lda, 0, 0, h->oz_slices, 2,
-                            h->ozflags + 1, h->stream));
+          CK(oz_operand(h, 0, h->ozA, oz_region(h, n, 4), (int)n, (int)n, A, lda, 0, 0, h->stream));
           oz_a_ready = true;
         }
         if (h->ozB_src != (const void*)B || h->ozB_gen != h->chol_gen) {
-          CK(gevp::oz_split(h->ozB, oz_region(h, n, 5), (int)n, (int)n, B, ldb, 0, 0, h->oz_slices, 2,
-                            h->ozflags + 1, h->stream));
+          CK(oz_operand(h, 0, h->ozB, oz_region(h, n, 5), (int)n, (int)n, B, ldb, 0, 0, h->stream));
           h->ozB_src = B;
           h->ozB_gen = h->chol_gen;
         }
-        CK(gevp::oz_split(h->ozQ, oz_region(h, n, 2), nev, (int)n, h->Xf, ld, 0, 0, h->oz_slices, 3, h->ozflags + 1,
-                          h->stream, true));
-        CK(gevp::oz_gemm(h->ozA, h->ozQ, 0, 0, h->Y1, ld, h->ozflags, h->stream, nullptr, h->ozws, h->ozws_doubles));
-        CK(gevp::oz_gemm(h->ozB, h->ozQ, 0, 0, h->Y2, ld, h->ozflags, h->stream, nullptr, h->ozws, h->ozws_doubles));
+        CK(oz_operand(h, 0, h->ozQ, oz_region(h, n, 1), nev, (int)n, h->Xf, ld, 0, 0, h->stream, true));
+        CK(oz_product(h, 0, n, h->ozA, h->ozQ, 0, 0, h->Y1, ld, h->stream));
+        CK(oz_product(h, 0, n, h->ozB, h->ozQ, 0, 0, h->Y2, ld, h->stream));
       } else {
         ZgemmArgs ax = zg((int)n, nev, (int)n, A, lda, 0, h->Xf, ld, 0, h->Y1, ld);
         zgemm(ax, h->split, h->split_elems, h->stream);
@@ -1096,7 +1096,7 @@ gevp_status solve_one(gevp_ctx* h, int64_t n, const double2* A, int64_t lda, con
   CK(cudaMemcpyAsync(res_out, h->resf, nev * sizeof(double), cudaMemcpyDeviceToDevice, h->stream));
   if (X_out) zcopy2d(n, nev, h->Xf, ld, X_out, ldx, h->stream);
   if (st) st->converged = converged ? 1 : 0;
-  h->ozC_src = nullptr;   // C's digits are this problem's only
+  h->ozC_src = nullptr;   // C's residues are this problem's only
   return converged ? GEVP_OK : GEVP_ERR_NO_CONVERGENCE;
 }
 
@@ -1176,7 +1176,7 @@ void gevp_default_opts(gevp_opts* o) {
   o->lanczos_steps = 32;
   o->refine_iters = 3;
   o->keep_all_X = 0;
-  // the reduction's n^3 products emulated with 8 digits: FP64-class accuracy, about 17x
+  // the reduction's n^3 products emulated with 8 digits: FP64-class accuracy, about 50x
   // the FP64 pipe's rate at n = 2048
   o->reduce_slices = 8;
 }
@@ -1223,7 +1223,6 @@ gevp_status gevp_destroy(gevp_handle h) {
   for (int i = 0; i < 2; ++i)
     if (h->ozmem[i]) cudaFree(h->ozmem[i]);
   if (h->ozflags) cudaFree(h->ozflags);
-  if (h->ozws) cudaFree(h->ozws);
   if (h->jidx) cudaFree(h->jidx);
   if (h->hb2) cudaFreeHost(h->hb2);
   for (cudaEvent_t e : {h->ev_main, h->ev_side, h->ev_user})
@@ -1327,22 +1326,19 @@ gevp_status gevp_reduce_update(gevp_handle h, int64_t n, const void* B, int64_t 
   gevp_status st = GEVP_OK;
   if (slices > 0) {
     // W = L^-1 R^H (L^-1 rows, lower; columns of R^H = conjugated rows of R), emulated
-    const int S = slices;
     const int nn = (int)n;
-    const size_t bA = gevp::oz_operand_bytes(nn, nn, S, 2);
-    st = oz_reserve(h, 0, oz_main_bytes(n, S));
-    if (st == GEVP_OK && (h->oz_l_gen != h->chol_gen || h->oz_l_S != S)) {
-      char* mem = h->ozmem[0];
-      if (gevp::oz_split(h->ozLA, mem, nn, nn, h->Linv, n, 0, 2, S, 2, h->ozflags + 1, s) != cudaSuccess ||
-          gevp::oz_split(h->ozLB, mem + bA, nn, nn, h->Linv, n, 1, 2, S, 3, h->ozflags + 1, s) != cudaSuccess)
+    h->oz_regions = 3;
+    st = oz_prepare(h, 0, n);
+    if (st == GEVP_OK && (h->oz_l_gen != h->chol_gen || h->oz_l_S != slices)) {
+      if (oz_operand(h, 0, h->ozLA, oz_region(h, n, 0), nn, nn, h->Linv, n, 0, 2, s) != cudaSuccess)
         st = cuda_fail(h, cudaGetLastError(), "oz_split");
+      h->ozLB = h->ozLA;
+      h->ozLB.conj = 1;
       h->oz_l_gen = h->chol_gen;
-      h->oz_l_S = S;
+      h->oz_l_S = slices;
     }
-    if (st == GEVP_OK &&
-        (gevp::oz_split(h->ozR, oz_region(h, n, 2), k, nn, R, n, 1, 0, S, 3, h->ozflags + 1, s) != cudaSuccess ||
-         gevp::oz_gemm(h->ozLA, h->ozR, 1, 0, UV + k, k2, h->ozflags, s, nullptr, h->ozws, h->ozws_doubles) !=
-             cudaSuccess))
+    if (st == GEVP_OK && (oz_operand(h, 0, h->ozR, oz_region(h, n, 1), k, nn, R, n, 1, 0, s) != cudaSuccess ||
+                          oz_product(h, 0, n, h->ozLA, h->ozR, 1, 0, UV + k, k2, s) != cudaSuccess))
       st = cuda_fail(h, cudaGetLastError(), "oz_gemm");
   } else {
     ZgemmArgs w = zg((int)n, k, (int)n, h->Linv, n, 0, R, n, 1, UV + k, k2);
@@ -1359,16 +1355,10 @@ gevp_status gevp_reduce_update(gevp_handle h, int64_t n, const void* B, int64_t 
     // C += [U V] [V U]^H = U V^H + V U^H, lower triangle, then its Hermitian completion
     if (slices > 0) {
       const int nn = (int)n;
-      // [U V] rows in the T/C region, the conjugated rows of [V U] from the A region on
-      // (up to three regions' room: the cached digits of B and of L^-H are invalidated)
-      h->ozB_src = nullptr;
-      h->ozB_gen = -1;
-      h->ozLH_gen = -1;
-      if (gevp::oz_split(h->ozUV, oz_region(h, n, 3), nn, (int)k2, UV, k2, 0, 0, slices, 2, h->ozflags + 1, s) !=
-              cudaSuccess ||
-          gevp::oz_split(h->ozVU, oz_region(h, n, 4), nn, (int)k2, VU, k2, 1, 0, slices, 3, h->ozflags + 1, s) !=
-              cudaSuccess ||
-          gevp::oz_gemm(h->ozUV, h->ozVU, 0, 0, h->C, n, h->ozflags, s) != cudaSuccess)
+      // [U V] rows in the C region, the conjugated rows of [V U] in the block's
+      if (oz_operand(h, 0, h->ozUV, oz_region(h, n, 2), nn, (int)k2, UV, k2, 0, 0, s) != cudaSuccess ||
+          oz_operand(h, 0, h->ozVU, oz_region(h, n, 1), nn, (int)k2, VU, k2, 1, 0, s) != cudaSuccess ||
+          oz_product(h, 0, n, h->ozUV, h->ozVU, 0, 0, h->C, n, s) != cudaSuccess)
         st = cuda_fail(h, cudaGetLastError(), "oz_gemm");
       if (st == GEVP_OK) add_lower_herm(n, (double2*)C, ldc, h->C, n, s);
     } else {
@@ -1380,6 +1370,7 @@ gevp_status gevp_reduce_update(gevp_handle h, int64_t n, const void* B, int64_t 
     }
   }
   h->oz_slices = keep;
+  h->oz_regions = 6;
   if (st != GEVP_OK) return st;
   CK(cudaStreamSynchronize(s));
   CK(cudaGetLastError());
@@ -1936,16 +1927,42 @@ gevp_status gevp_zgemm_emulated(gevp_handle h, int opA, int opB, int M, int N, i
     CK(cudaStreamSynchronize(h->stream));
     return GEVP_OK;
   }
-  const size_t bA = gevp::oz_operand_bytes(M, K, slices, 2), bB = gevp::oz_operand_bytes(N, K, slices, 3);
-  TRY(oz_reserve(h, 1, bA + bB));
+  // all moduli's residues of both operands, or groups of four where that would take more than a
+  // third of the device's memory
+  size_t freeb = 0, total = 0;
+  CK(cudaMemGetInfo(&freeb, &total));
+  const auto opb = [&](int rows, int group) { return al(gevp::oz_operand_bytes(rows, K, slices, group)); };
+  const size_t panel = gevp::oz_work_bytes(256, N, K, slices);
+  const size_t work = al(std::max(panel, std::min<size_t>(gevp::oz_work_bytes(M, N, K, slices), (size_t)1 << 30)));
+  int group = opb(M, 0) + opb(N, 0) > total / 3 ? 4 : 0;
+  TRY(oz_flags_ready(h));
+  for (; work + opb(M, group) + opb(N, group) > h->ozmem_bytes[1]; group = 4) {
+    const size_t need = work + opb(M, group) + opb(N, group);
+    cudaDeviceSynchronize();
+    if (h->ozmem[1]) cudaFree(h->ozmem[1]);
+    h->ozmem[1] = nullptr;
+    h->ozmem_bytes[1] = 0;
+    h->oz_n[1] = 0;
+    void* p = nullptr;
+    const cudaError_t e = cudaMalloc(&p, need);
+    if (e == cudaErrorMemoryAllocation && group == 0) {
+      cudaGetLastError();
+      continue;
+    }
+    CK(e);
+    h->ozmem[1] = (char*)p;
+    h->ozmem_bytes[1] = need;
+    break;
+  }
+  char* mem = h->ozmem[1] + work;
   gevp::OzOperand a, b;
   // rows of op(A): rows of A, or conjugated columns; columns of op(B): columns of B, or
   // conjugated rows
-  CK(gevp::oz_split(a, h->ozmem[1], M, K, (const double2*)A, lda, opA, 0, slices, 2, h->ozflags + 1, h->stream,
-                    opA == 1));
-  CK(gevp::oz_split(b, h->ozmem[1] + bA, N, K, (const double2*)B, ldb, opB, 0, slices, 3, h->ozflags + 1,
-                    h->stream, opB == 0));
-  CK(gevp::oz_gemm(a, b, 0, 0, (double2*)D, ldd, h->ozflags, h->stream));
+  CK(gevp::oz_split(a, mem, M, K, (const double2*)A, lda, opA, 0, slices, h->ozflags + 1, h->stream, opA == 1, nullptr,
+                    group));
+  CK(gevp::oz_split(b, mem + opb(M, group), N, K, (const double2*)B, ldb, opB, 0, slices, h->ozflags + 1, h->stream,
+                    opB == 0, nullptr, group));
+  CK(gevp::oz_gemm(a, b, 0, 0, (double2*)D, ldd, h->ozflags, h->stream, nullptr, h->ozmem[1], work));
   return oz_check(h);
 }
 
@@ -1963,7 +1980,9 @@ gevp_status gevp_reduce_emulated(gevp_handle h, int64_t n, const void* A, int64_
   }
   const int keep = h->oz_slices;
   h->oz_slices = slices;
+  h->oz_regions = 3;
   gevp_status st = gevp_reduce(h, n, A, lda, B, ldb, L, ldl, C, ldc, info);
+  h->oz_regions = 6;
   if (st == GEVP_OK) st = oz_check(h);
   h->oz_slices = keep;
   return st;

@@ -187,9 +187,9 @@ bool cholinv_small(int m, const double2* W, int64_t ldw, double shift, double2* 
 // order n > kCholLeaf splits as n1 + n2 (n1 a multiple of 128 near n / 2) with
 // L21 = A21 L11^-H, L22 L22^H = A22 - L21 L21^H, (L^-1)21 = -L22^-1 L21 L11^-1 as emulated
 // products; leaves of order <= kCholLeaf are factored and inverted by cholinv_small.
-// Resources (CholRes): digit memory for one operand of up to n x n in the A role (memA,
-// oz_operand_bytes(n, n, S, 2)) and one in the B role (memB, npl 3), an n x n scratch T
-// (ld ldt), optional split-K partials, the products' status words (flags[0] error code,
+// Resources (CholRes): memory for two operands of up to n x n (memA, memB:
+// oz_operand_bytes(n, n, S, group)), an n x n scratch T (ld ldt), the products' residues (ws, as
+// for oz_gemm with N = n), the products' status words (flags[0] error code,
 // flags[1] non-finite entry), the pivot word and the stream (memA, memB, T unused for
 // n <= kCholLeaf). Returns cudaSuccess when enqueued; cudaErrorNotSupported when nothing
 // was enqueued (no cluster launch possible); another error after work was enqueued. A
@@ -202,8 +202,9 @@ struct CholRes {
   char* memB;
   double2* T;
   int64_t ldt;
-  double* ws;
-  size_t ws_doubles;
+  void* ws;
+  size_t ws_bytes;
+  int group;
   int* flags;
   int* info;
   int S;
@@ -326,30 +327,39 @@ void matrix_variation(int64_t n, const double2* A, int64_t lda, const double2* B
                       cudaStream_t s);
 
 // ---------------------------------------------------------------- emulated FP64 GEMM
-// An operand of the emulated product in digit form: `rows` rows of op(A) (npl = 2: planes
-// re, im) or columns of op(B) (npl = 3: re, im, -im), each K entries split into S base-128
-// digits, planes [npl][S][rows_pad][k_pad] BF16, followed by one exponent per row.
+// An operand of the emulated product in residue form: `rows` rows of op(A) or columns of
+// op(B), each K entries rounded to 7 S bits; BF16 residue planes [part][modulus][rows][k_pad],
+// followed by one exponent per row. conj: the operand's imaginary part changes sign (the
+// planes do not). nmod below the number of moduli that K and S need: room for one group of
+// moduli only; the product then writes each group's residues from X before it uses them (X
+// has to stay as it was until then).
 constexpr int kOzSlicesMax = 8;
 struct OzOperand {
   __nv_bfloat16* planes = nullptr;
   int* ex = nullptr;
-  int rows = 0, K = 0, rows_pad = 0, k_pad = 0, S = 0, npl = 0;
+  int rows = 0, K = 0, k_pad = 0, S = 0, nmod = 0;
+  const double2* X = nullptr;
+  int64_t ldx = 0;
+  int conj = 0, mask = 0;
+  bool cols = false;
+  int* bad = nullptr;
 };
-size_t oz_operand_bytes(int rows, int K, int S, int npl);
+// group 0: all moduli at once
+size_t oz_operand_bytes(int rows, int K, int S, int group = 0);
 bool oz_supported();
 // rows of X (cols = false; X is rows x K) or its columns (cols = true; X is K x rows) as
 // operand rows, conjugated if conj, mask 1: k >= r with the diagonal halved, 2: k <= r,
-// 3: k >= r; into digit form in `mem` (oz_operand_bytes); *bad = 1 on a non-finite entry
+// 3: k >= r; into residue form in `mem` (oz_operand_bytes); *bad = 1 on a non-finite entry
 // active: nullable device flag, 0 = the launch does nothing (a converged batch problem)
 cudaError_t oz_split(OzOperand& op, void* mem, int rows, int K, const double2* X, int64_t ldx, int conj, int mask,
-                     int S, int npl, int* bad, cudaStream_t s, bool cols = false, const int* active = nullptr);
-// D (A.rows x B.rows) = op(A) op(B); triA 1: op(A) lower; triB 1: op(B) lower, 2: upper
-// ws (nullable, ws_doubles >= oz_split_k_doubles(M, N)): when the grid would leave SMs
-// idle, K is cut into up to kOzSplitKMax slices whose FP64 partials are summed in slice order
-constexpr int kOzSplitKMax = 8;
-size_t oz_split_k_doubles(int M, int N);
+                     int S, int* bad, cudaStream_t s, bool cols = false, const int* active = nullptr, int group = 0);
+// D (A.rows x B.rows) = op(A) op(B); triA 1: op(A) lower, 2: upper; triB 1: op(B) lower, 2:
+// upper. ws: room for the result's residues; oz_work_bytes(M, N, K, S) holds the whole
+// result, less makes the product run in panels of rows (at least one of min(M, 256) rows).
+// D may be the memory of A's source (a row of D depends on that row of A alone).
+size_t oz_work_bytes(int M, int N, int K, int S);
 cudaError_t oz_gemm(const OzOperand& A, const OzOperand& B, int triA, int triB, double2* D, int64_t ldd, int* err,
-                    cudaStream_t s, const int* active = nullptr, double* ws = nullptr, size_t ws_doubles = 0);
+                    cudaStream_t s, const int* active, void* ws, size_t ws_bytes);
 
 // ---------------------------------------------------------------- deviation angles
 // slices of the column-norm reduction (part needs slices * k doubles)
