@@ -238,11 +238,7 @@ gevp_status build_plan(gevp_ctx* h, BatchPlan* P, std::string& err) {
       d.hscal = (double*)take(16 * 8);
       d.V = (float2*)take((size_t)65 * n * 8);
       d.lvec = (float2*)take((size_t)n * 8);
-      d.T32 = (float2*)take(64 * 64 * 8);
-      d.LZ32 = (float2*)take(64 * 64 * 8);
       d.ab = (float*)take(140 * 4);
-      d.lw32 = (float*)take(64 * 4);
-      d.lperm = (int*)take(64 * 4);
       d.theta = (double*)take((size_t)m * 8);
       d.res = (double*)take((size_t)m * 8);
       d.lamf = (double*)take((size_t)m * 8);

@@ -344,52 +344,6 @@ __global__ void __launch_bounds__(1024) b_lanczos_update(const BDesc* D, int j) 
   for (int64_t i = threadIdx.x; i < n; i += blockDim.x) { float2 b = w[i]; vn[i] = make_float2(b.x * inv, b.y * inv); }
 }
 
-// the k x k tridiagonal, padded far above the spectrum after a breakdown
-__global__ void b_build_T(const BDesc* D, int k) {
-  const BDesc& d = D[blockIdx.x];
-  if (!live(d)) return;
-  int* kf = (int*)(d.ab + 2 * KMAX);
-  const int ke = kf[0];
-  int kk = ke < 0 ? -ke : (ke > k ? k : ke);
-  if (kk < 1) kk = 1;
-  __syncthreads();
-  if (threadIdx.x == 0) kf[1] = kk;
-  for (int e = threadIdx.x; e < k * k; e += blockDim.x) {
-    int i = e / k, j = e % k;
-    float v = 0.f;
-    if (i >= kk || j >= kk) v = (i == j) ? 1e30f : 0.f;
-    else if (i == j) v = d.ab[2 * i];
-    else if (j == i + 1) v = d.ab[2 * i + 1];
-    else if (i == j + 1) v = d.ab[2 * j + 1];
-    d.T32[e] = make_float2(v, 0.f);
-  }
-}
-
-__global__ void b_lanczos_finish(const BDesc* D, int k, int use_count, int out_off) {
-  const BDesc& d = D[blockIdx.x];
-  if (!live(d) || threadIdx.x != 0) return;
-  const int* kf = (const int*)(d.ab + 2 * KMAX);
-  const int ke = kf[0], kk = kf[1];
-  const double tmin = d.lw32[0], tmax = d.lw32[kk - 1];
-  const double beta = (ke < 0) ? 0.0 : fabs((double)d.ab[2 * (kk - 1) + 1]);
-  const double span = fmax(fabs(tmin), fabs(tmax));
-  double* out = d.bounds + out_off;
-  out[0] = tmin;
-  out[1] = tmax;
-  out[2] = tmax + beta + 1e-5 * span;
-  out[4] = beta;
-  double aest = tmax;
-  if (use_count) {
-    double cum = 0.0;
-    for (int r = 0; r < kk; ++r) {
-      float2 z0 = d.LZ32[d.lperm[r]];   // first row of the eigenvector matrix
-      cum += ((double)z0.x * z0.x + (double)z0.y * z0.y) * (double)d.n;
-      if (cum >= (double)d.m) { aest = d.lw32[r]; break; }
-    }
-  }
-  out[3] = aest;
-}
-
 // start of a problem of the sequence: every problem iterates again
 __global__ void b_step_reset(const BDesc* D, int np, double tol, int filter64) {
   int p = blockIdx.x * blockDim.x + threadIdx.x;
@@ -951,19 +905,18 @@ void bk_lanczos(const BDesc* D, int np, int64_t nmax, int k, int use_count, int 
     b_lanczos_update<<<np, 1024, 0, s>>>(D, j);
     LAUNCH_NOTE(2);
   }
-  b_build_T<<<np, 256, 0, s>>>(D, k);
-  LAUNCH_NOTE(1);
-  jacobi32_batched(D, np, 1, k, k, 30, s);
-  b_lanczos_finish<<<np, 32, 0, s>>>(D, k, use_count, out_off);
-  LAUNCH_NOTE(1);
+  lanczos_tail_batched(D, np, k, use_count, KMAX, out_off, s);
 }
 void bk_heev_prep(const BDesc* D, int np, int mmax, cudaStream_t s) {
   b_g_to_c<<<g2((int64_t)mmax * mmax, np), 256, 0, s>>>(D);
   LAUNCH_NOTE(1);
-  jacobi32_batched(D, np, 0, 0, mmax, 40, s);
-  b_gather_z<<<g2((int64_t)mmax * mmax, np), 256, 0, s>>>(D);
+  if (!heev32_batched(D, np, mmax, s)) {
+    jacobi32_batched(D, np, mmax, 40, s);
+    b_gather_z<<<g2((int64_t)mmax * mmax, np), 256, 0, s>>>(D);
+    LAUNCH_NOTE(1);
+  }
   b_frob<<<np, 1024, 0, s>>>(D);
-  LAUNCH_NOTE(2);
+  LAUNCH_NOTE(1);
 }
 void bk_oa_scalars(const BDesc* D, int np, cudaStream_t s) {
   b_oa_scalars<<<np, 1024, 0, s>>>(D);

@@ -207,11 +207,6 @@ size_t layout(gevp_ctx* h, char* base, int64_t n, int m) {
   h->lw.V = (float2*)take((size_t)65 * n * 8);
   h->lw.ab = (float*)take(140 * 4);
   h->lw.w = (float2*)take((size_t)n * 8);
-  h->lw.T32 = (float2*)take(64 * 64 * 8);
-  h->lw.Z32 = (float2*)take(64 * 64 * 8);
-  h->lw.w32 = (float*)take(64 * 4);
-  h->lw.perm = (int*)take(64 * 4);
-  h->lw.out = nullptr;
   h->theta = (double*)take(m * 8 + 64);
   h->res = (double*)take(m * 8 + 64);
   h->lam = (double*)take(m * 8 + 64);
@@ -580,11 +575,6 @@ gevp_status ensure_pipeline(gevp_ctx* h) {
     h->lw2.V = (float2*)take((size_t)65 * n * 8);
     h->lw2.ab = (float*)take(140 * 4);
     h->lw2.w = (float2*)take((size_t)n * 8);
-    h->lw2.T32 = (float2*)take(64 * 64 * 8);
-    h->lw2.Z32 = (float2*)take(64 * 64 * 8);
-    h->lw2.w32 = (float*)take(64 * 4);
-    h->lw2.perm = (int*)take(64 * 4);
-    h->lw2.out = nullptr;
     h->bounds2 = (double*)take(24 * 8);
     return off;
   };

@@ -141,12 +141,19 @@ struct HeevWork {
 size_t heev_ws_bytes(int m, size_t split_elems);
 void heev_small(int m, const double2* G, int64_t ldg, double* theta, double2* Z, int64_t ldz,
                 const HeevWork& w, int refine_iters, cudaStream_t s);
-// FP32 Jacobi on a (possibly real) Hermitian matrix in FP32 (single CTA); sorted output.
-void jacobi32(int m, float2* G, float2* Z, float* w, int* perm, int max_sweeps, cudaStream_t s);
+// FP32 eigenvectors of G (m x m FP32 Hermitian; not modified) in ascending order into the columns
+// of Z (FP64, ld ldz), by tridiagonalisation and QL (tridiag32.cu). Scratch: w (m floats), ctl (4
+// ints), tau (m), sV, sR, sS, sZ (m x m each). may_skip: a nearly diagonal G may give the unit
+// vectors in the order of its diagonal. false: not launchable (m > 600), nothing was enqueued.
+bool heev32(int m, const float2* G, double2* Z, int64_t ldz, float* w, int* ctl, float2* tau, double2* sV, double2* sR,
+            double2* sS, double2* sZ, int may_skip, cudaStream_t s);
+// The end of a Lanczos run: out[0..4] of lanczos_bounds from its alpha and beta (ab; the steps
+// made at ab[2 k_max])
+void lanczos_tail(int k, int64_t n, int count, const float* ab, int k_max, double* out, cudaStream_t s);
 
 // ---------------------------------------------------------------- Lanczos bounds (FP32)
 struct LanczosOut { double lam_min, lam_max, upper, a_est, beta_last; };
-struct LanczosWork { float2* V; float* ab; float2* w; float2* T32; float2* Z32; float* w32; int* perm; double* out; };
+struct LanczosWork { float2* V; float* ab; float2* w; };
 size_t lanczos_ws_bytes(int64_t n, int k);
 // k-step Lanczos with full re-orthogonalisation on the FP32 copy of a Hermitian matrix.
 // Writes to dev_out[0..4] = {theta_min, theta_max, upper bound, estimate of the count-th
@@ -255,7 +262,7 @@ struct BDesc {
   double2 *hZ, *hR, *hS, *hT, *hE;      // m x m
   double *hlam, *hscal;
   // Lanczos
-  float2 *V, *lvec, *T32, *LZ32; float *ab, *lw32; int* lperm;
+  float2 *V, *lvec; float* ab;
   // per-column and per-problem scalars
   double *theta, *res, *lamf, *resf, *dscale, *partial;
   double* bounds;             // see bkernels.cu for the slot map
@@ -303,8 +310,11 @@ void bk_force_final(const BDesc* D, int np, cudaStream_t s);
 struct BOut { double* lam; double* res; double2* X; int64_t ldx; };
 void bk_write_out(const BDesc* D, const BOut* O, int np, int64_t nm_max, cudaStream_t s);
 size_t bk_partial_elems(int m);
-// batched FP32 Jacobi: which = 0 -> G32 (m x m) into Z32/w32/perm; 1 -> T32 (k x k) into LZ32/lw32/lperm
-void jacobi32_batched(const BDesc* D, int np, int which, int k, int mmax, int max_sweeps, cudaStream_t s);
+// batched forms: FP32 eigenvectors of every G32 into hZ (scratch hR, hS, hT, hE, Z32, w32, perm);
+// where that cannot be launched (mmax > 600), Jacobi into Z32 / w32 / perm; the Lanczos ends
+bool heev32_batched(const BDesc* D, int np, int mmax, cudaStream_t s);
+void jacobi32_batched(const BDesc* D, int np, int mmax, int max_sweeps, cudaStream_t s);
+void lanczos_tail_batched(const BDesc* D, int np, int k, int use_count, int k_max, int out_off, cudaStream_t s);
 void cluster_jacobi_batched(const BDesc* D, int np, int zsel, double rel, int max_sweeps, cudaStream_t s);
 
 // grouped tensor-core filter (residual-corrected recurrence) over the problems of a batch

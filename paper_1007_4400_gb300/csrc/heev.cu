@@ -2,12 +2,9 @@
 //
 // One SM executes FP64 at about 1.7 FMA per clock on this part, so an FP64 Jacobi in one
 // CTA would take milliseconds. Instead:
-//   1. parallel-ordered two-sided Jacobi in FP32 (FP32 runs at 128 FMA per clock per SM),
-//      giving eigenvectors accurate to about 1e-6: one CTA below m = 32, the eight CTAs
-//      of a thread-block cluster sharing G through distributed shared memory up to
-//      m = 256, all SMs (cooperative launch) above. The cluster form runs no sweep when
-//      G is already nearly diagonal (the projection of an almost converged block: the
-//      refinement starts from Z = I, see jacobi32_cluster_kernel);
+//   1. FP32 eigenvectors accurate to about 1e-6 (FP32 runs at 128 FMA per clock per SM):
+//      Householder tridiagonalisation and QL in a thread-block cluster (tridiag32.cu); orders
+//      above its limit by parallel-ordered two-sided Jacobi on all SMs (cooperative launch);
 //   2. Ogita & Aishima's iterative refinement for symmetric/Hermitian eigenvector
 //      matrices (Japan J. Ind. Appl. Math. 35, 2018), which converges quadratically and
 //      consists of four FP64 GEMMs per step spread over all SMs. Pairs closer than the
@@ -29,10 +26,6 @@ namespace gevp {
 namespace {
 
 constexpr int JT = 1024;   // threads of the Jacobi CTA
-
-// split cluster barrier: arrive (release) and, later, wait (acquire) for the phase
-__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release;" ::: "memory"); }
-__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire;" ::: "memory"); }
 
 __device__ __forceinline__ void block_pair(int step, int k, int np, int* p, int* q) {
   // circle method: position 0 fixed, the other np-1 players rotate by one per round
@@ -69,9 +62,8 @@ __device__ __forceinline__ float2 ld2(const float2* p) {
 }
 
 // Element access to G for the Jacobi rounds: a plain matrix (shared or global memory, the
-// one-CTA forms), a global matrix read through L2 (the cooperative form: other CTAs wrote
-// it and L1 is not coherent across SMs), or row bands held in the shared memory of the CTAs
-// of a thread-block cluster (the cluster form; rows [c mb, (c + 1) mb) in CTA c).
+// one-CTA forms), or a global matrix read through L2 (the cooperative form: other CTAs wrote
+// it and L1 is not coherent across SMs).
 struct GPlain {
   float2* g;
   int m;
@@ -84,14 +76,6 @@ struct GL2 {
   __device__ __forceinline__ float2 ld(int i, int j) const { return __ldcg(g + i * m + j); }
   __device__ __forceinline__ void st(int i, int j, float2 v) const { g[i * m + j] = v; }
 };
-struct GBand {
-  float2* const* band;   // per cluster rank: the generic address of that CTA's band
-  int m, mb;
-  __device__ __forceinline__ float2* at(int i, int j) const { return band[i / mb] + (i % mb) * m + j; }
-  __device__ __forceinline__ float2 ld(int i, int j) const { return *at(i, j); }
-  __device__ __forceinline__ void st(int i, int j, float2 v) const { *at(i, j) = v; }
-};
-
 // Rotation of pair k of round `step`: U = [[c, s], [-s conj(ph), c conj(ph)]] acting on
 // columns (p, q), stored as (c, s, Re ph, Im ph); identity for the dummy index q = m of
 // odd orders and for couplings below FP32 significance relative to the diagonal.
@@ -322,170 +306,19 @@ __global__ void __launch_bounds__(JT) jacobi32_coop_kernel(int m, float2* G, flo
   }
 }
 
-// Cluster form for mid-size orders: the rounds of jacobi32_body spread over the kJC CTAs
-// of one thread-block cluster. G lives in the CTAs' shared memory as row bands (two
-// buffers: a round reads one and writes the other, so CTAs still computing the round's
-// rotations never see rotated entries), read and written through distributed shared
-// memory; one cluster barrier per round instead of one CTA doing every 2 x 2 block. Z is
-// held as row bands too: the update Z <- Z U mixes two columns within each row, so every
-// CTA rotates its own rows in its own shared memory (two thirds of a round's tasks, which
-// no longer go through L2), and writes its band to Z at the end. The round's barrier is
-// split around that work: a CTA arrives once its share of G is written and waits only
-// after rotating its rows of Z (the rotations are double-buffered by round parity). The
-// arithmetic of every element is that of jacobi32_body, so the results are identical. Gin
-// (m x m) is read, not modified.
-constexpr int kJC = 8;
-constexpr int kJClusterMax = 256;
-
-__global__ void __launch_bounds__(JT, 1) jacobi32_cluster_kernel(int m, const float2* Gin, float2* Z, float* w,
-                                                                 int* perm, int max_sweeps, int may_skip) {
-  namespace cg = cooperative_groups;
-  cg::cluster_group cl = cg::this_cluster();
-  extern __shared__ float2 jband[];   // [2][mb][m] G bands, then [mb][m] the Z band
-  // rotations of round k in buffer k & 1: a thread may compute round k + 1's while another
-  // still rotates its rows of Z with round k's
-  __shared__ float4 U2[2][512];
-  __shared__ int PQ2[2][512][2];
-  __shared__ float red[32];
-  __shared__ float part[64];          // this CTA's partial sums: [0] ||G||_F^2, [1 + sweep] off-norm
-  __shared__ float dg[kJClusterMax];  // the diagonal of G
-  __shared__ int coupled;             // this CTA's rows hold a coupling the refinement cannot start from
-  __shared__ float2* bandp[2][kJC];   // generic addresses of every CTA's two bands
-  const int tid = threadIdx.x;
-  const int rank = (int)cl.block_rank();
-  const int mb = (m + kJC - 1) / kJC;
-  if (tid < kJC) {
-    bandp[0][tid] = cl.map_shared_rank(jband, tid);
-    bandp[1][tid] = cl.map_shared_rank(jband + mb * m, tid);
-  }
-  // own band of G into buffer 0 (rows past m are never addressed)
-  const int r0 = rank * mb;
-  for (int e = tid; e < mb * m; e += JT) {
-    const int r = r0 + e / m;
-    jband[e] = r < m ? Gin[r * m + (e % m)] : make_float2(0.f, 0.f);
-  }
-  const int gtid = rank * JT + tid, gsz = kJC * JT;
-  const int rows = max(0, min(mb, m - r0));
-  float2* zband = jband + 2 * mb * m;   // own rows r0 .. r0 + rows - 1 of Z
-  for (int e = tid; e < rows * m; e += JT) zband[e] = make_float2((r0 + e / m) == (e % m) ? 1.f : 0.f, 0.f);
-  const int np = (m % 2) ? m + 1 : m;
-  const int npairs = np / 2;
-  float f = 0.f;
-  for (int e = tid; e < rows * m; e += JT) { float2 g = jband[e]; f += g.x * g.x + g.y * g.y; }
-  for (int j = tid; j < m; j += JT) dg[j] = Gin[j * m + j].x;
-  if (tid == 0) coupled = 0;
-  f = block_sum(f, red);
-  if (tid == 0) part[0] = f;
-  cl.sync();
-  // every CTA sums the partials in the same order: the same decisions everywhere
-  auto cluster_sum = [&](int slot) {
-    float t = 0.f;
-    for (int c = 0; c < kJC; ++c) t += *cl.map_shared_rank(&part[slot], c);
-    return t;
-  };
-  const float fro2 = cluster_sum(0);
-  const float tol2 = 1e-16f * fro2;
-  float off_prev = 3.0e38f;
-  int cur = 0;
-  if (max_sweeps > 62) max_sweeps = 62;
-  for (int sweep = 0; sweep < max_sweeps && m > 1; ++sweep) {
-    float off = 0.f;
-    const float2* Gc = jband + cur * mb * m;
-    for (int e = tid; e < rows * m; e += JT) {
-      const int i = r0 + e / m, j = e % m;
-      if (i != j) { float2 g = Gc[e]; off += g.x * g.x + g.y * g.y; }
-    }
-    off = block_sum(off, red);
-    if (tid == 0) part[1 + sweep] = off;
-    cl.sync();
-    off = cluster_sum(1 + sweep);
-    if (off <= tol2 || (off > 0.9f * off_prev && off <= 1e-12f * fro2)) break;
-    if (sweep == 0 && may_skip) {
-      // Nearly diagonal already (the projection of a block that has almost converged):
-      // every coupling at most 1e-3 of its diagonal gap (gaps below eta0 = 1e-6 ||G||_F
-      // counted as eta0: clusters, which FP32 sweeps cannot resolve either), and at most
-      // 1e-5 of it for gaps between eta0 and delta = 2 ||offdiag(G)||_F. The FP64
-      // refinement started from Z = I has the clustering threshold delta in its first step:
-      // it corrects the pairs farther apart than delta there (to about 1e-6), those between
-      // eta0 and delta in its second step (to about 1e-10), and, converging quadratically,
-      // reaches FP64 accuracy in its last step as it would from the sweeps' result; the
-      // clusters go to the exact rotations after it. No sweep is run.
-      const float eta0 = 1e-6f * sqrtf(fro2), delta = 2.f * sqrtf(off);
-      bool c = false;
-      for (int e = tid; e < rows * m; e += JT) {
-        const int i = r0 + e / m, j = e % m;
-        if (i == j) continue;
-        const float2 g = Gc[e];
-        const float gap = fabsf(dg[i] - dg[j]);
-        const float a = hypotf(g.x, g.y);
-        c |= a > 1e-3f * fmaxf(gap, eta0) || (gap > eta0 && gap <= delta && a > 1e-5f * gap);
-      }
-      if (__any_sync(0xffffffffu, c) && (tid & 31) == 0) coupled = 1;
-      cl.sync();
-      int any = 0;
-      for (int r = 0; r < kJC; ++r) any |= *cl.map_shared_rank(&coupled, r);
-      if (!any) break;
-    }
-    off_prev = off;
-    for (int step = 0; step < np - 1; ++step) {
-      const GBand Ac{bandp[cur], m, mb}, An{bandp[cur ^ 1], m, mb};
-      float4* U = U2[step & 1];
-      int(*PQ)[2] = PQ2[step & 1];
-      for (int k = tid; k < npairs; k += JT) jacobi_pair_params(Ac, m, np, step, k, U, PQ);
-      __syncthreads();
-      for (int e = gtid; e < npairs * npairs; e += gsz) jacobi_apply<GBand, true>(Ac, An, Z, m, npairs, e, U, PQ);
-      // the round's G is written: arrive, and rotate the own rows of Z (columns r, s of each
-      // pair, this CTA's shared memory only) while the other CTAs finish theirs
-      cluster_arrive();
-      for (int t = tid; t < rows * npairs; t += JT) {
-        const int il = t / npairs, b = t % npairs;
-        const int r = PQ[b][0], sc = PQ[b][1];
-        if (sc >= m) continue;
-        const float4 u = U[b];
-        const float c = u.x, sn = u.y;
-        const float2 phc = make_float2(u.z, -u.w);
-        float2* zrow = zband + il * m;
-        const float2 zr = zrow[r], zs = cmulf(zrow[sc], phc);
-        zrow[r] = make_float2(c * zr.x - sn * zs.x, c * zr.y - sn * zs.y);
-        zrow[sc] = make_float2(sn * zr.x + c * zs.x, sn * zr.y + c * zs.y);
-      }
-      cluster_wait();
-      cur ^= 1;
-    }
-  }
-  if (rank == 0) {
-    const GBand Ac{bandp[cur], m, mb};
-    for (int i = tid; i < m; i += JT) {
-      const float wi = Ac.ld(i, i).x;
-      int r = 0;
-      for (int j = 0; j < m; ++j) {
-        const float wj = Ac.ld(j, j).x;
-        r += (wj < wi) || (wj == wi && j < i);
-      }
-      perm[r] = i;
-      w[r] = wi;
-    }
-  }
-  for (int e = tid; e < rows * m; e += JT) Z[(int64_t)r0 * m + e] = zband[e];
-  // no CTA leaves while rank 0 may still read its shared memory
-  cl.sync();
-}
-
 __global__ void __launch_bounds__(JT) jacobi32_kernel(int m, float2* G, float2* Z, float* w, int* perm,
                                                       int max_sweeps) {
   extern __shared__ float2 jsm[];
   jacobi32_body(m, G, Z, w, perm, max_sweeps, m <= kJacobiSmemMax ? jsm : nullptr);
 }
 
-// one CTA per problem of a batch: which = 0 -> the Rayleigh-Ritz matrix, 1 -> Lanczos T;
-// smem_m: the launch provided shared-memory room for matrices up to smem_m x smem_m
-__global__ void __launch_bounds__(JT) jacobi32_batched_kernel(const BDesc* D, int which, int k, int max_sweeps,
-                                                              int smem_m) {
+// one CTA per problem of a batch; smem_m: the launch provided shared-memory room for matrices up
+// to smem_m x smem_m
+__global__ void __launch_bounds__(JT) jacobi32_batched_kernel(const BDesc* D, int max_sweeps, int smem_m) {
   extern __shared__ float2 jsm[];
   const BDesc& d = D[blockIdx.x];
   if (d.active && *d.active == 0) return;
-  if (which == 0) jacobi32_body(d.m, d.G32, d.Z32, d.w32, d.perm, max_sweeps, d.m <= smem_m ? jsm : nullptr);
-  else jacobi32_body(k, d.T32, d.LZ32, d.lw32, d.lperm, max_sweeps, k <= smem_m ? jsm : nullptr);
+  jacobi32_body(d.m, d.G32, d.Z32, d.w32, d.perm, max_sweeps, d.m <= smem_m ? jsm : nullptr);
 }
 
 // dynamic shared memory of a Jacobi launch on matrices up to m x m (0: global memory)
@@ -661,10 +494,10 @@ __global__ void __launch_bounds__(256) zupd32_kernel(int m, const double2* Z, co
 __device__ void cluster_jacobi_body(int m, double2* S, double2* Z, double* lam, const double* fro, double rel,
                                     int max_sweeps) {
   const double tol = rel * fro[0];
-  // FP32 Jacobi leaves eigenvalue errors of order 1e-4 ||G|| at m ~ 300 (accumulated
-  // rounding of many rotations), so dense clusters can leave several hundred couplings
-  constexpr int kMaxPairs = 1024;
-  __shared__ int PI[kMaxPairs], PJ[kMaxPairs];
+  // the FP32 stage leaves every coupling inside a cluster that FP32 cannot resolve: a cluster of c
+  // values c (c - 1) / 2 of them (60 values within 1e-5 ||G||: 1770)
+  constexpr int kMaxPairs = 4096;
+  __shared__ short PI[kMaxPairs], PJ[kMaxPairs];
   __shared__ int npairs;
   __shared__ double2 ucs[3];   // c, s (real), ph
   for (int sweep = 0; sweep < max_sweeps; ++sweep) {
@@ -676,7 +509,7 @@ __device__ void cluster_jacobi_body(int m, double2* S, double2* Z, double* lam, 
       double2 v = S[e];
       if (hypot(v.x, v.y) > tol) {
         int k = atomicAdd(&npairs, 1);
-        if (k < kMaxPairs) { PI[k] = i; PJ[k] = j; }
+        if (k < kMaxPairs) { PI[k] = (short)i; PJ[k] = (short)j; }
       }
     }
     __syncthreads();
@@ -799,54 +632,12 @@ bool jacobi32_coop(int m, float2* G, float2* Gb, float2* Z, float* w, int* perm,
   return true;
 }
 
-// Cluster Jacobi for 32 <= m <= kJClusterMax; false if it cannot be launched (then the
-// caller runs the one-CTA kernel).
-bool jacobi32_cluster(int m, const float2* G, float2* Z, float* w, int* perm, int max_sweeps, int may_skip,
-                      cudaStream_t s) {
-  if (m < 32 || m > kJClusterMax) return false;
-  const int mb = (m + kJC - 1) / kJC;
-  const size_t smem = (size_t)3 * mb * m * sizeof(float2);
-  static bool attr = false;
-  if (!attr) {
-    if (cudaFuncSetAttribute(jacobi32_cluster_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)(3 * ((kJClusterMax + kJC - 1) / kJC) * kJClusterMax * sizeof(float2))) !=
-        cudaSuccess) {
-      cudaGetLastError();
-      return false;
-    }
-    attr = true;
-  }
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(kJC, 1, 1);
-  cfg.blockDim = dim3(JT, 1, 1);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = s;
-  cudaLaunchAttribute at[1];
-  at[0].id = cudaLaunchAttributeClusterDimension;
-  at[0].val.clusterDim.x = kJC;
-  at[0].val.clusterDim.y = 1;
-  at[0].val.clusterDim.z = 1;
-  cfg.attrs = at;
-  cfg.numAttrs = 1;
-  if (cudaLaunchKernelEx(&cfg, jacobi32_cluster_kernel, m, G, Z, w, perm, max_sweeps, may_skip) != cudaSuccess) {
-    cudaGetLastError();
-    return false;
-  }
-  LAUNCH_NOTE(1);
-  return true;
-}
-
-void jacobi32(int m, float2* G, float2* Z, float* w, int* perm, int max_sweeps, cudaStream_t s) {
-  jacobi32_kernel<<<1, JT, jacobi_smem(m), s>>>(m, G, Z, w, perm, max_sweeps);
-  LAUNCH_NOTE(1);
-}
-
-// mmax: the largest matrix order among the problems (k for the Lanczos matrices)
-void jacobi32_batched(const BDesc* D, int np, int which, int k, int mmax, int max_sweeps, cudaStream_t s) {
+// mmax: the largest matrix order among the problems
+void jacobi32_batched(const BDesc* D, int np, int mmax, int max_sweeps, cudaStream_t s) {
   // problems with m <= 160 keep G on chip even when the batch's largest m is above that
-  const int cap = std::min(which == 0 ? mmax : k, kJacobiSmemMax);
+  const int cap = std::min(mmax, kJacobiSmemMax);
   const size_t sm = jacobi_smem(cap);
-  jacobi32_batched_kernel<<<np, JT, sm, s>>>(D, which, k, max_sweeps, sm > 0 ? cap : 0);
+  jacobi32_batched_kernel<<<np, JT, sm, s>>>(D, max_sweeps, sm > 0 ? cap : 0);
   LAUNCH_NOTE(1);
 }
 
@@ -862,22 +653,21 @@ void heev_small(int m, const double2* G, int64_t ldg, double* theta, double2* Zo
   int blocks = (int)std::min<int64_t>((mm + 255) / 256, 152 * 4);
   g_to_c_kernel<<<blocks, 256, 0, s>>>(m, G, ldg, w.G32);
   LAUNCH_NOTE(1);
-  // large orders on all SMs (cooperative launch); otherwise, or if that launch is not
-  // possible, one CTA
-  // 32 <= m <= 256 on the eight CTAs of a cluster; larger orders on all SMs (cooperative
-  // launch; the FP64 scratch E, unused until the refinement, holds its second FP32 buffer);
-  // small ones, or when neither launch is possible, in one CTA
-  // (the sweeps may be skipped for a nearly diagonal G when the refinement has the three
-  // steps that its start from Z = I needs)
-  bool done = jacobi32_cluster(m, w.G32, w.Z32, w.w32, w.perm, 40, refine_iters >= 3 ? 1 : 0, s);
-  if (!done && m > kJacobiSmemMax)
-    done = jacobi32_coop(m, w.G32, (float2*)w.E, w.Z32, w.w32, w.perm, 40, (float*)(w.scal + 16), s);
-  if (!done) {
-    jacobi32_kernel<<<1, JT, jacobi_smem(m), s>>>(m, w.G32, w.Z32, w.w32, w.perm, 40);
+  // FP32 eigenvectors by tridiagonalisation (a nearly diagonal G may start from Z = I when the
+  // refinement has the three steps that needs; the FP64 scratch is free until then). Orders above
+  // its limit: Jacobi on all SMs (cooperative launch; E holds its second FP32 buffer), or, when
+  // that cannot be launched, in one CTA.
+  if (!heev32(m, w.G32, w.Z, m, w.w32, (int*)(w.scal + 16), w.Z32, w.T, w.R, w.S, w.E, refine_iters >= 3 ? 1 : 0, s)) {
+    bool done = false;
+    if (m > kJacobiSmemMax)
+      done = jacobi32_coop(m, w.G32, (float2*)w.E, w.Z32, w.w32, w.perm, 40, (float*)(w.scal + 16), s);
+    if (!done) {
+      jacobi32_kernel<<<1, JT, jacobi_smem(m), s>>>(m, w.G32, w.Z32, w.w32, w.perm, 40);
+      LAUNCH_NOTE(1);
+    }
+    gather_z_kernel<<<blocks, 256, 0, s>>>(m, w.Z32, w.perm, w.Z, m);
     LAUNCH_NOTE(1);
   }
-  gather_z_kernel<<<blocks, 256, 0, s>>>(m, w.Z32, w.perm, w.Z, m);
-  LAUNCH_NOTE(1);
   // partial sums in E (free until the refinement's first product writes it)
   const int nblk = (int)std::min<int64_t>(64, std::max<int64_t>(1, ((int64_t)m * m + 255) / 256));
   double* part = (double*)w.E;
@@ -923,7 +713,7 @@ void heev_small(int m, const double2* G, int64_t ldg, double* theta, double2* Zo
   ZgemmArgs b2 = zg(m, m, m, G, ldg, 0, Z, m, 0, w.E, m);
   zgemm(b2, w.split_ws, w.split_ws_elems, s);
   zgram(m, m, m, Z, m, w.E, m, w.S, m, 1, w.split_ws, w.split_ws_elems, w.gcnt, s);
-  cluster_jacobi_kernel<<<1, 1024, 0, s>>>(m, w.S, Z, w.lam, w.scal + 1, 1e-15, 12);
+  cluster_jacobi_kernel<<<1, 1024, 0, s>>>(m, w.S, Z, w.lam, w.scal + 1, 1e-15, 20);
   LAUNCH_NOTE(1);
   sort_pairs_kernel<<<1, 1024, 0, s>>>(m, w.lam, Z, theta, Zout, ldz);
   LAUNCH_NOTE(1);

@@ -128,49 +128,6 @@ __global__ void __launch_bounds__(1024) lanczos_update_kernel(int64_t n, int j, 
   for (int64_t i = threadIdx.x; i < n; i += blockDim.x) { float2 b = w[i]; vn[i] = make_float2(b.x * inv, b.y * inv); }
 }
 
-// T (k x k, stride k): the tridiagonal of the first kk steps, padded with a diagonal far
-// above the spectrum for indices >= kk (kk < k only after a breakdown).
-__global__ void build_T_kernel(int k, const float* ab, float2* T, int* kout, float big) {
-  const int* keff = (const int*)(ab + 2 * KMAX);
-  int ke = *keff;
-  int kk = ke < 0 ? -ke : (ke > k ? k : ke);
-  if (kk < 1) kk = 1;
-  if (threadIdx.x == 0) *kout = kk;
-  for (int e = threadIdx.x; e < k * k; e += blockDim.x) {
-    int i = e / k, j = e % k;
-    float v = 0.f;
-    if (i >= kk || j >= kk) v = (i == j) ? big : 0.f;
-    else if (i == j) v = ab[2 * i];
-    else if (j == i + 1) v = ab[2 * i + 1];
-    else if (i == j + 1) v = ab[2 * j + 1];
-    T[e] = make_float2(v, 0.f);
-  }
-}
-
-__global__ void lanczos_finish_kernel(int k, int64_t n, int count, const float* ab, const int* kout, const float* w,
-                                      const int* perm, const float2* Z, double* out) {
-  if (threadIdx.x != 0) return;
-  int kk = *kout;
-  double tmin = w[0], tmax = w[kk - 1];
-  int ke = ((const int*)(ab + 2 * KMAX))[0];
-  double beta = (ke < 0) ? 0.0 : fabs((double)ab[2 * (kk - 1) + 1]);
-  double span = fmax(fabs(tmin), fabs(tmax));
-  out[0] = tmin;
-  out[1] = tmax;
-  out[2] = tmax + beta + 1e-5 * span;
-  out[4] = beta;
-  double aest = tmax;
-  if (count > 0) {
-    double cum = 0.0;
-    for (int r = 0; r < kk; ++r) {
-      float2 z0 = Z[0 * k + perm[r]];
-      cum += (double)(z0.x * z0.x + z0.y * z0.y) * (double)n;
-      if (cum >= (double)count) { aest = w[r]; break; }
-    }
-  }
-  out[3] = aest;
-}
-
 }  // namespace
 
 size_t lanczos_ws_bytes(int64_t n, int k) {
@@ -178,8 +135,7 @@ size_t lanczos_ws_bytes(int64_t n, int k) {
   b += (size_t)(KMAX + 1) * n * sizeof(float2);   // V
   b += (2 * KMAX + 4) * sizeof(float);           // ab
   b += n * sizeof(float2);                        // w
-  b += 2 * (size_t)KMAX * KMAX * sizeof(float2);  // T32, Z32
-  b += KMAX * sizeof(float) + KMAX * sizeof(int) + 8 * sizeof(double) + 16 * 256;
+  b += 16 * 256;
   return b;
 }
 
@@ -196,12 +152,7 @@ void lanczos_bounds(int64_t n, const float2* M32, int64_t ldm, int k, int count,
     lanczos_update_kernel<<<1, 1024, 0, s>>>(n, j, w.V, w.w, w.ab);
     LAUNCH_NOTE(1);
   }
-  int* kout = (int*)(w.ab + 2 * KMAX) + 1;
-  build_T_kernel<<<1, 256, 0, s>>>(k, w.ab, w.T32, kout, 1e30f);
-  LAUNCH_NOTE(1);
-  jacobi32(k, w.T32, w.Z32, w.w32, w.perm, 30, s);
-  lanczos_finish_kernel<<<1, 32, 0, s>>>(k, n, count, w.ab, kout, w.w32, w.perm, w.Z32, dev_out);
-  LAUNCH_NOTE(1);
+  lanczos_tail(k, n, count, w.ab, KMAX, dev_out, s);
 }
 
 }  // namespace gevp
