@@ -361,7 +361,7 @@ gevp_status gevp_zgemm_emulated(gevp_handle h, int opA, int opB, int M, int N, i
  * diagonal halved, M = T L^-H, C = M + M^H) emulated as in gevp_zgemm_emulated with
  * `slices` digits, and B factored recursively: for n > 256, n = n1 + n2 with
  * L21 = A21 L11^-H, L22 L22^H = B22 - L21 L21^H and (L^-1)21 = -L22^-1 L21 L11^-1, the
- * four off-diagonal products emulated, leaves of order <= 256 factored with their
+ * four off-diagonal products emulated, leaves of order <= 128 factored with their
  * inverses in one thread-block cluster each. n <= 30720. The same outputs (to FP64
  * rounding) and errors as gevp_reduce; `info` is the global index of the first
  * non-positive pivot met. */

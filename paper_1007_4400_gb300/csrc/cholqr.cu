@@ -12,32 +12,38 @@
 //
 // cholinv: the Cholesky factor L of D W D + shift I (W the Gram matrix, lower triangle
 //   read; D = diag(W)^-1/2 the column scaling of CholQR) and its inverse, for m up to a
-//   few hundred, in the CTAs of one thread-block cluster. A one-CTA factorisation would
-//   take close to a millisecond at m = 140 (m^3/3 complex multiply-adds at two FP64 FMAs
-//   per clock); the blocked right-looking form over all SMs spends most of its time in
-//   launches and serial diagonal blocks. Here the rows are dealt cyclically to the P CTAs
-//   (row i to CTA i mod P) and held in shared memory with the rows of the inverse; column
-//   j of the factor and row j of the inverse are exchanged through distributed shared
-//   memory, one cluster barrier per column:
-//     step j: every CTA reads the pivot a_jj, the column A[j+1:m, j] and the row S[j, 0:j]
-//     (values final after step j-1), then updates its own rows i > j:
-//       A[i, e] -= A[i, j] conj(A[e, j]) / a_jj   (j < e <= i; the trailing Cholesky update)
-//       S[i, e] -= A[i, j] S[j, e] / a_jj         (e <= j; the inverse, L X = I, right-looking)
-//     L[i, j] = A[i, j] / sqrt(a_jj) and (L^-1)[i, e] = S[i, e] / sqrt(a_ii) are read off at
-//     the end. Within a step the reads (column j, row j, the pivot) and the writes
-//     (columns > j of A, rows > j of S) never meet, so one barrier per step suffices. The
-//     barrier is split: a step first updates what the next step reads (column j + 1 with
-//     the next pivot, row j + 1 of S), arrives, updates the rest while the other CTAs catch
-//     up, and waits only before the next gather; the gathered values are double-buffered,
-//     so a thread gathering step j + 1 never overwrites what another still reads for j.
+//   few hundred, in the CTAs of one thread-block cluster per matrix. A one-CTA factorisation
+//   would take close to a millisecond at m = 140 (m^3/3 complex multiply-adds at two FP64 FMAs
+//   per clock). Here the rows are dealt cyclically to the P CTAs (row i to CTA i mod P) and held
+//   in shared memory with the rows of the inverse's accumulator S (initially I). Panels of eight
+//   columns J, one cluster barrier per panel:
+//     every CTA gathers, through distributed shared memory, the raw panel A[e, J], e >= j0, and
+//     the raw rows S[J, :] (all final after the panel before), eliminates the 8 x 8 diagonal block
+//     redundantly (T = its unit-pivot inverse accumulator, a_q its pivots), forms for its own
+//     rows i below the panel the multipliers M_i = A[i, J] T^H diag(1/a) T = A[i, J] A_JJ^-1, and
+//     updates
+//       A[i, e] -= M_i A[e, J]^H   (e > J; the trailing Cholesky update)
+//       S[i, e] -= M_i S[J, e]     (e <= J; the inverse, L X = I, right-looking)
+//     L[i, J] = A[i, J] T^H diag(a)^-1/2 and the rows J of L^-1, diag(a)^-1/2 T S[J, :], are
+//     written as they become known. Raw values and multipliers keep the other CTAs' rows out
+//     of the dependence: nothing is exchanged but the gather.
+//   Within a panel the reads (columns J of A, rows J of S) and the writes (columns > J of A, rows
+//   > J of S) never meet, so one barrier per panel suffices. The barrier is split: a CTA first
+//   updates what the next panel reads (the next eight columns, its own rows of S among the next
+//   block), arrives, updates the rest while the other CTAs catch up, and waits before the next
+//   gather. At m = 256 half the time is the FP64 pipe's (4/3 m^3 FMAs on P SMs at two a clock);
+//   below, the panel's chain of FP64 operations at 64 clocks each. Measured m = 128 232 us, 140
+//   262 us, 256 805 us (320 us and 1.2 ms at m = 140 and 256 with one column a step).
+//   A matrix within 1e-9 of the identity after scaling (the second pass of CholQR2) needs no
+//   elimination: L^-1 = I - N to FP64 rounding (m = 140: 9 us).
 //   The output Li = L^-1 D (columns scaled by D) makes Y Li^H = Y D L^-H, the orthonormal
 //   factor of one CholQR pass, a single product; it is also the inverse of D^-1 L, the
 //   Cholesky factor of W itself (shift 0), which is written out on request (the leaves
 //   of the recursive factorisation of B). A non-positive pivot stops the cluster (every
-//   CTA reads the same pivot, so the decision is uniform) and sets *info to its 1-based
-//   index plus a caller's offset. W may share memory with that factor's output: every
-//   CTA reads its rows of W before the first cluster barrier and writes the factor after
-//   the last.
+//   CTA eliminates the same block, so the decision is uniform) and sets *info to its 1-based
+//   index plus a caller's offset; rows before that panel have been written then. W may share
+//   memory with the factor's output: every CTA reads its rows of W before the first cluster
+//   barrier and writes the factor after it.
 #include "gevp_internal.cuh"
 #include <cooperative_groups.h>
 #include <algorithm>
@@ -111,37 +117,106 @@ constexpr int kCholInvMax = 288; // largest order (shared-memory bound at 16 CTA
 __device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release;" ::: "memory"); }
 __device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire;" ::: "memory"); }
 
-template <int P>
-__global__ void __launch_bounds__(CT, 1) cholinv_cluster_kernel(int m, const double2* W, int64_t ldw,
-                                                                double shift, double2* Li, int64_t ldi,
-                                                                double2* Lf, int64_t ldl, int* info, int info_base) {
+struct CholProb {
+  int m;
+  const double2* W;
+  int64_t ldw;
+  double shift;
+  double2* Li;
+  int64_t ldi;
+  double2* Lf;
+  int64_t ldl;
+  int* info;
+  int info_base;
+};
+struct CholOne {
+  CholProb p;
+  __device__ bool get(int, CholProb& o) const {
+    o = p;
+    return true;
+  }
+};
+// the Gram matrices of a batch: Gw -> Gwi, the pivot in flags[2]
+struct CholBatch {
+  const BDesc* D;
+  double shift_factor;
+  __device__ bool get(int b, CholProb& o) const {
+    const BDesc& d = D[b];
+    if (d.flags[0] == 0) return false;
+    const double m = d.m;
+    o.m = d.m;
+    o.W = d.Gw;
+    o.ldw = d.m;
+    o.shift = shift_factor * 11.0 * (d.n * m + m * (m + 1.0)) * 1.1102230246251565e-16 * m;
+    o.Li = d.Gwi;
+    o.ldi = d.m;
+    o.Lf = nullptr;
+    o.ldl = 0;
+    o.info = d.flags + 2;
+    o.info_base = 0;
+    return true;
+  }
+};
+
+constexpr int NB = 8;   // columns of a panel
+
+// 1 / v for a pivot v > 0: the hardware's approximation (about 2^-20) and one cubic step, error
+// below 2^-52; three dependent FP64 operations (it only scales the multipliers M, where its
+// error acts like a rounding of A_JJ^-1)
+__device__ __forceinline__ double pivot_recip(double v) {
+  const int ex = __double2hiint(v) >> 20;   // (an FP64 comparison would cost as much as an FMA)
+  if (ex < 64 || ex > 1982) return 1.0 / v;
+  double r;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(v));
+  const double e = fma(-v, r, 1.0);
+  return fma(r, fma(e, e, e), r);
+}
+
+// An SM retires two FP64 lanes per clock, a warp's instruction every 64 clocks in each of its four
+// partitions whether the next one depends on it or not. So the kernel counts FP64 instructions
+// per partition: sums are cut into (entry, real or imaginary part) items of at most sixteen
+// FMAs, packed densely into the eight warps.
+//
+// The pair of a with which dot2(pair(part, a), b) is Re(a b) (part 0) or Im(a b) (part 1); the sign
+// is flipped by an integer instruction
+__device__ __forceinline__ double2 part_pair(int part, double2 a) {
+  const double ny = __hiloint2double(__double2hiint(a.y) ^ (int)0x80000000, __double2loint(a.y));
+  return part == 0 ? make_double2(a.x, ny) : make_double2(a.y, a.x);
+}
+__device__ __forceinline__ double dot2(double2 p, double2 b, double acc) { return fma(p.y, b.y, fma(p.x, b.x, acc)); }
+
+template <int P, class Src>
+__global__ void __launch_bounds__(CT, 1) cholinv_cluster_kernel(Src src) {
   namespace cg = cooperative_groups;
   cg::cluster_group cl = cg::this_cluster();
+  CholProb pr;
+  if (!src.get(blockIdx.x / P, pr)) return;   // uniform over the cluster
   extern __shared__ double2 csm[];
-  // gathered values of step j in buffer j & 1: a thread may gather step j + 1 while another
-  // still finishes step j's update
-  __shared__ double2 cbuf[2][kCholInvMax];   // column j of A (raw), rows > j
-  __shared__ double2 xbuf[2][kCholInvMax];   // row j of S (raw), columns <= j
-  __shared__ double2 cs[2][kCholInvMax / 8]; // own rows' -A[i, j] / a_jj
-  __shared__ double dsc[kCholInvMax];     // D
-  __shared__ double piv[kCholInvMax];     // sqrt(a_jj)
-  __shared__ double2 pinfo[kCholInvMax / 8];   // own rows: (pivot a_ii, rsqrt(a_ii)) once final
+  constexpr int RMAX = (kCholInvMax + P - 1) / P;
+  constexpr int XMAX = (kCholInvMax + 31) / 32;
+  __shared__ double2 F[NB][NB], T[NB][NB];   // the diagonal block, its inverse's accumulator
+  __shared__ double2 M[2][RMAX][NB];         // part_pair(part, M)
+  __shared__ double2 L[RMAX][NB], Ls[RMAX][NB];   // Ls = -L diag(1/a)
+  __shared__ double rp[NB], rs[NB];          // 1 / a_q, a_q^-1/2
+  __shared__ double dsc[kCholInvMax];        // D
   __shared__ double2* rA[P];
   __shared__ double2* rS[P];
-  __shared__ double2* rPI[P];
-  __shared__ double apiv;
-  const int tid = threadIdx.x;
+  __shared__ int bad;
+  __shared__ float devw[CT / 32], devs;
+  const int tid = threadIdx.x, warp = tid / 32, lane = tid % 32;
+  const int m = pr.m;
   const int rank = (int)cl.block_rank();
   const int R = (m + P - 1) / P;
-  double2* Arow = csm;            // [R][m]: own rows i = rank + P t of the matrix being factored
-  double2* Srow = csm + R * m;    // [R][m]: own rows of the inverse's accumulator
+  double2* Arow = csm;              // [R][m]: own rows i = rank + P t of the matrix being factored
+  double2* Srow = csm + R * m;      // [R][m]: own rows of the inverse's accumulator
+  double2* G = csm + 2 * R * m;     // [NB][m]: S[j0 + q][x] for x < j0, I in J, conj(A[x][j0 + q]) after
   if (tid < P) {
     rA[tid] = cl.map_shared_rank(Arow, tid);
     rS[tid] = cl.map_shared_rank(Srow, tid);
-    rPI[tid] = cl.map_shared_rank(pinfo, tid);
   }
+  if (tid == 0) bad = 0;
   for (int i = tid; i < m; i += CT) {
-    const double v = W[(int64_t)i * ldw + i].x;
+    const double v = pr.W[(int64_t)i * pr.ldw + i].x;
     dsc[i] = v > 0.0 ? 1.0 / sqrt(v) : 1.0;
   }
   __syncthreads();
@@ -149,165 +224,225 @@ __global__ void __launch_bounds__(CT, 1) cholinv_cluster_kernel(int m, const dou
     const int t = e / m, c = e % m, i = rank + P * t;
     double2 a = make_double2(0.0, 0.0), s = make_double2(0.0, 0.0);
     if (i < m && c <= i) {
-      a = zscale(W[(int64_t)i * ldw + c], dsc[i] * dsc[c]);
-      if (c == i) a = make_double2(a.x + shift, 0.0);
+      a = zscale(pr.W[(int64_t)i * pr.ldw + c], dsc[i] * dsc[c]);
+      if (c == i) a = make_double2(a.x + pr.shift, 0.0);
       if (c == i) s = make_double2(1.0, 0.0);
     }
     Arow[e] = a;
     Srow[e] = s;
   }
-  // the first pivot is final from the start: its owner (rank 0, local row 0; this thread
-  // wrote that entry above) prepares its reciprocal square root
-  if (rank == 0 && tid == 0) {
-    const double a0 = Arow[0].x;
-    pinfo[0] = make_double2(a0, a0 > 0.0 ? rsqrt(a0) : 0.0);
+  // D W D + shift I = I + E with ||E||_F below 1e-9 (the second pass of CholQR2): L = I + N, L^-1 =
+  // I - N up to O(||E||^2) < 1e-18, N the lower triangle of E with its diagonal halved. (Squares in
+  // FP32: only their size matters.)
+  float dev = 0.f;
+  for (int e = tid; e < R * m; e += CT) {
+    const int c = e % m, i = rank + P * (e / m);
+    if (i >= m || c > i) continue;
+    const float x = c == i ? (float)(Arow[e].x - 1.0) : (float)Arow[e].x, y = (float)Arow[e].y;
+    dev += (x * x + y * y) * (c == i ? 1.f : 2.f);
+  }
+  for (int o = 16; o > 0; o >>= 1) dev += __shfl_xor_sync(0xffffffffu, dev, o);
+  if (lane == 0) devw[warp] = dev;
+  __syncthreads();
+  if (tid == 0) {
+    float t = 0.f;
+    for (int w = 0; w < CT / 32; ++w) t += devw[w];
+    devs = t;
   }
   cl.sync();
-  bool failed = false;
-  for (int j = 0; j < m; ++j) {
-    const int oj = j % P, tjj = j / P, bsel = j & 1;
-    double2* cb = cbuf[bsel];
-    double2* xb = xbuf[bsel];
-    double2* cm = cs[bsel];
-    // own rows below the pivot: i = rank + P t > j, t in [t0, t1)
-    const int t0 = j >= rank ? (j - rank) / P + 1 : 0;
-    int t1 = R;
-    while (t1 > t0 && rank + P * (t1 - 1) >= m) --t1;
-    const int nr = t1 - t0;
-    // everything step j reads is final once every CTA has arrived after step j - 1's
-    // first part (column j, row j of the inverse, the pivot)
-    if (j > 0) cluster_wait();
-    // gather column j and row j of the inverse (raw values); the threads of own rows also
-    // form the row's multiplier -A[i][j] / a_jj from the pivot's reciprocal square root,
-    // prepared by the pivot's owner when it became final
-    for (int l = tid; l < m; l += CT) {
-      if (l > j) {
-        const double2 c = rA[l % P][(l / P) * m + j];
-        cb[l] = c;
-        if (l % P == rank) {
-          const double ri = rPI[oj][tjj].y;
-          cm[l / P - t0] = zscale(c, -(ri * ri));
-        }
+  dev = 0.f;
+  for (int q = 0; q < P; ++q) dev += *cl.map_shared_rank(&devs, q);   // in rank order: the same in every CTA
+  if (dev < 1e-18f) {
+    for (int e = tid; e < R * m; e += CT) {
+      const int c = e % m, i = rank + P * (e / m);
+      if (i >= m) continue;
+      double2 a = c <= i ? Arow[e] : make_double2(0.0, 0.0), l = a;
+      if (c == i) {
+        a = make_double2(1.5 - 0.5 * a.x, 0.0);
+        l = make_double2(2.0 - a.x, 0.0);
       } else {
-        xb[l] = rS[oj][tjj * m + l];
+        a = make_double2(-a.x, -a.y);
       }
+      pr.Li[(int64_t)i * pr.ldi + c] = zscale(a, dsc[c]);
+      if (pr.Lf) pr.Lf[(int64_t)i * pr.ldl + c] = zscale(l, 1.0 / dsc[i]);
     }
-    if (tid == 0) {
-      const double2 pv = rPI[oj][tjj];
-      apiv = pv.x;
-      piv[j] = pv.x * pv.y;
-    }
-    __syncthreads();
-    const double a = apiv;   // the same value in every CTA: a uniform decision
-    if (!(a > 0.0)) {
-      if (rank == 0 && tid == 0) atomicCAS(info, 0, info_base + j + 1);
-      failed = true;
-      break;
-    }
-    // first part: what step j + 1 reads. Column j + 1 of the own rows below the pivot (with
-    // the next pivot and its reciprocal square root), and row j + 1 of the inverse if it is
-    // an own row
-    const int own_next = ((j + 1) % P == rank && j + 1 < m) ? (j + 1) / P : -1;
-    const int nfirst = nr + (own_next >= 0 ? j + 1 : 0);
-    for (int q = tid; q < nfirst; q += CT) {
-      if (q < nr) {
-        const int t = t0 + q, e = j + 1;
-        double2 v = Arow[t * m + e];
-        zfma(v, cm[q], zconj(cb[e]));
-        Arow[t * m + e] = v;
-        if (rank + P * t == j + 1) pinfo[t] = make_double2(v.x, v.x > 0.0 ? rsqrt(v.x) : 0.0);
-      } else {
-        const int e = q - nr, t = own_next;
-        double2 v = Srow[t * m + e];
-        zfma(v, cm[t - t0], xb[e]);
-        Srow[t * m + e] = v;
-      }
-    }
-    cluster_arrive();
-    // the rest of the update, while the other CTAs finish their first parts
-    for (int idx = tid; idx < nr * m; idx += CT) {
-      const int tt = idx / m, e = idx % m, t = t0 + tt, i = rank + P * t;
-      if (e > i || e == j + 1 || (i == j + 1 && e <= j)) continue;
-      const double2 li = cm[tt];
-      if (e <= j) {
-        double2 v = Srow[t * m + e];
-        zfma(v, li, xb[e]);
-        Srow[t * m + e] = v;
-      } else {
-        double2 v = Arow[t * m + e];
-        zfma(v, li, zconj(cb[e]));
-        Arow[t * m + e] = v;
-      }
-    }
-  }
-  if (failed) {
-    cl.sync();   // no CTA leaves while another may still read its shared memory
+    cl.sync();
     return;
   }
-  cluster_wait();   // the last step's gathers are over in every CTA
-  __syncthreads();  // and every thread of this one finished its update
-  // read off L and L^-1 D for the own rows
-  for (int e = tid; e < R * m; e += CT) {
-    const int t = e / m, c = e % m, i = rank + P * t;
-    if (i >= m) continue;
-    double2 x = make_double2(0.0, 0.0);
-    if (c <= i) x = zscale(Srow[e], dsc[c] / piv[i]);
-    Li[(int64_t)i * ldi + c] = x;
-    if (Lf) {
-      // the factor of W + shift D^-2: D^-1 times the factor of D W D + shift I
-      double2 l = make_double2(0.0, 0.0);
-      if (c < i) l = zscale(Arow[e], 1.0 / (piv[c] * dsc[i]));
-      else if (c == i) l = make_double2(piv[i] / dsc[i], 0.0);
-      Lf[(int64_t)i * ldl + c] = l;
+  for (int j0 = 0; j0 < m; j0 += NB) {
+    const int nb = min(NB, m - j0), j1 = j0 + nb, j2 = min(m, j1 + NB);
+    // own rows below the panel: i = rank + P t >= j1, nr of them from t0, the first nn in the next block
+    const int t0 = j1 > rank ? (j1 - rank + P - 1) / P : 0;
+    const int nr = max(0, (rank < m ? (m - 1 - rank) / P + 1 : 0) - t0);
+    int nn = 0;
+    while (nn < nr && rank + P * (t0 + nn) < j2) ++nn;
+    if (j0 > 0) {
+      __syncthreads();   // the last panel's G and M have been read
+      cluster_wait();
+    }
+    // gather, a column q of the panel to a warp: row j0 + q of S (x < j0), the diagonal block,
+    // column j0 + q of A; every load in flight before the first is stored
+    if (warp < nb) {
+      const int q = warp;
+      const double2* sr = rS[(j0 + q) % P] + ((j0 + q) / P) * m;
+      double2 v[XMAX];
+#pragma unroll
+      for (int k = 0; k < XMAX; ++k) {
+        const int x = lane + 32 * k;
+        if (x < m) v[k] = *(x < j0 ? sr + x : rA[x % P] + (x / P) * m + j0 + q);
+      }
+#pragma unroll
+      for (int k = 0; k < XMAX; ++k) {
+        const int x = lane + 32 * k;
+        if (x >= m) continue;
+        double2 g = v[k];
+        if (x >= j1) {
+          g.y = -g.y;
+        } else if (x >= j0) {
+          F[x - j0][q] = g;
+          g = make_double2(x - j0 == q ? 1.0 : 0.0, 0.0);
+          T[x - j0][q] = g;
+        }
+        G[q * m + x] = g;
+      }
+    }
+    __syncthreads();
+    // eliminate the diagonal block (four warps, one per partition): F[i][q], q <= i, keeps the raw
+    // columns. The products F[i][c] conj(F[e][c]) do not wait for the pivot's reciprocal.
+    if (tid < 2 * NB * NB) {
+      const int part = tid / (NB * NB), i = tid / NB % NB, e = tid % NB;
+      for (int c = 0; c < nb; ++c) {
+        const double a = F[c][c].x;
+        const int hi = __double2hiint(a);
+        if (hi <= 0 || hi >= 0x7ff00000) {   // not positive (below 2^-1042 counted as zero), or not finite
+          if (tid == 0) bad = c + 1;
+          break;
+        }
+        const double r = pivot_recip(a);
+        if (tid == 0) rp[c] = r;
+        if (i > c && i < nb && e <= i) {
+          double* at = (double*)(e > c ? &F[i][e] : &T[i][e]) + part;
+          const double2 w = e > c ? zconj(F[e][c]) : T[c][e];
+          *at = fma(-r, dot2(part_pair(part, F[i][c]), w, 0.0), *at);
+        }
+        asm volatile("bar.sync 1, 128;" ::: "memory");
+      }
+    }
+    __syncthreads();
+    if (bad) {   // the same in every CTA
+      if (rank == 0 && tid == 0) atomicCAS(pr.info, 0, pr.info_base + j0 + bad);
+      break;
+    }
+    // L = A[i, J] T^H, then M = -L diag(1/a) T
+    for (int x = tid; x < 2 * nr * NB; x += CT) {
+      const int part = x >= nr * NB, y = x - part * nr * NB, tt = y / NB, c = y % NB;
+      double v = 0.0;
+      if (c < nb)
+        for (int r = 0; r <= c; ++r) v = dot2(part_pair(part, zconj(T[c][r])), Arow[(t0 + tt) * m + j0 + r], v);
+      ((double*)&L[tt][c])[part] = v;
+      ((double*)&Ls[tt][c])[part] = c < nb ? -rp[c] * v : 0.0;
+    }
+    __syncthreads();
+    for (int x = tid; x < 2 * nr * NB; x += CT) {
+      const int part = x >= nr * NB, y = x - part * nr * NB, tt = y / NB, r = y % NB;
+      double v = 0.0;
+      for (int c = r; c < nb; ++c) v = dot2(part_pair(part, Ls[tt][c]), T[c][r], v);
+      if (part == 0) {
+        M[0][tt][r].x = v;
+        M[1][tt][r].y = v;
+      } else {
+        M[0][tt][r].y = __hiloint2double(__double2hiint(v) ^ (int)0x80000000, __double2loint(v));
+        M[1][tt][r].x = v;
+      }
+    }
+    __syncthreads();
+    // entry (own row tt below, column x): S where x < j1, A from there on
+    auto update = [&](int part, int tt, int x) {
+      double* at = (double*)((x < j1 ? Srow : Arow) + (t0 + tt) * m + x) + part;
+      double v = *at;
+      const double2* mr = M[part][tt];
+      if (nb == NB) {
+#pragma unroll
+        for (int q = 0; q < NB; ++q) v = dot2(mr[q], G[q * m + x], v);
+      } else {
+        for (int q = 0; q < nb; ++q) v = dot2(mr[q], G[q * m + x], v);
+      }
+      *at = v;
+    };
+    // first part: the next panel's columns of all own rows, and the own rows of S in the next block
+    const int n1 = nr * NB, n2 = n1 + nn * j1;
+    for (int x = tid; x < 2 * n2; x += CT) {
+      const int part = x >= n2, y = x - part * n2;
+      if (y < n1) {
+        const int tt = y / NB, c = j1 + y % NB;
+        if (c <= rank + P * (t0 + tt)) update(part, tt, c);
+      } else {
+        update(part, (y - n1) / j1, (y - n1) % j1);
+      }
+    }
+    if (j1 < m) cluster_arrive();
+    // the rest, while the other CTAs finish their first parts: (row, part) in pieces of 32 columns,
+    // dealt to the warps
+    int piece = 0;
+    for (int tt = nn; tt < nr; ++tt) {
+      const int i = rank + P * (t0 + tt), n = j1 + max(0, i + 1 - j2);
+      for (int part = 0; part < 2; ++part)
+        for (int x0 = 0; x0 < n; x0 += 32, ++piece) {
+          if (piece % (CT / 32) != warp) continue;
+          const int x = x0 + lane;
+          if (x < n) update(part, tt, x < j1 ? x : x - j1 + j2);
+        }
+    }
+    // results: L[i, J] of the own rows below, the own rows of the block
+    if (tid >= CT - NB && tid - (CT - NB) < nb) rs[tid - (CT - NB)] = rsqrt(F[tid - (CT - NB)][tid - (CT - NB)].x);
+    __syncthreads();
+    if (pr.Lf)
+      for (int x = tid; x < nr * NB; x += CT) {
+        const int tt = x / NB, q = x % NB, i = rank + P * (t0 + tt);
+        // the factor of W + shift D^-2: D^-1 times the factor of D W D + shift I
+        if (q < nb) pr.Lf[(int64_t)i * pr.ldl + j0 + q] = zscale(L[tt][q], rs[q] / dsc[i]);
+      }
+    for (int q = 0; q < nb; ++q) {
+      const int i = j0 + q;
+      if (i % P != rank) continue;
+      const double ri = rs[q];
+      for (int x = tid; x < 2 * m; x += CT) {
+        const int part = x >= m, c = x - part * m;
+        double v = 0.0;
+        if (c <= i) {
+          for (int r = 0; r <= q; ++r) v = dot2(part_pair(part, T[q][r]), G[r * m + c], v);
+          v *= ri * dsc[c];
+        }
+        ((double*)(pr.Li + (int64_t)i * pr.ldi + c))[part] = v;
+      }
+      if (pr.Lf)
+        for (int c = j0 + tid; c < m; c += CT) {
+          double2 l = make_double2(0.0, 0.0);
+          if (c < i) l = zscale(F[q][c - j0], rs[c - j0] / dsc[i]);
+          else if (c == i) l = make_double2(F[q][q].x * ri / dsc[i], 0.0);
+          pr.Lf[(int64_t)i * pr.ldl + c] = l;
+        }
     }
   }
+  cl.sync();   // no CTA leaves while another may still read its shared memory
 }
 
 template <int P>
 size_t cholinv_smem(int m) {
-  return (size_t)2 * ((m + P - 1) / P) * m * sizeof(double2);
+  return ((size_t)2 * ((m + P - 1) / P) + NB) * m * sizeof(double2);
 }
 
-template <int P>
-bool cholinv_launch(int m, const double2* W, int64_t ldw, double shift, double2* Li, int64_t ldi, double2* Lf,
-                    int64_t ldl, int* info, int info_base, cudaStream_t s) {
+// np matrices of order up to m, one cluster of P CTAs each
+template <int P, class Src>
+bool cholinv_launch(const Src& src, int np, int m, cudaStream_t s) {
+  constexpr int kMaxSmem = 203 * 1024;   // with the static arrays below the SM's 227 KB
   const size_t smem = cholinv_smem<P>(m);
-  if (smem > 200 * 1024) return false;
+  if (smem > kMaxSmem) return false;
   static int ready = 0;   // 0 unknown, 1 usable, -1 not launchable on this device
   if (ready < 0) return false;
-  if (ready == 0) {
-    ready = -1;
-    if (P > 8 && cudaFuncSetAttribute(cholinv_cluster_kernel<P>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) !=
-                     cudaSuccess) {
-      cudaGetLastError();
-      return false;
-    }
-    if (cudaFuncSetAttribute(cholinv_cluster_kernel<P>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024) !=
-        cudaSuccess) {
-      cudaGetLastError();
-      return false;
-    }
-    cudaLaunchConfig_t probe = {};
-    probe.gridDim = dim3(P, 1, 1);
-    probe.blockDim = dim3(CT, 1, 1);
-    probe.dynamicSmemBytes = 200 * 1024;
-    cudaLaunchAttribute pa[1];
-    pa[0].id = cudaLaunchAttributeClusterDimension;
-    pa[0].val.clusterDim.x = P;
-    pa[0].val.clusterDim.y = 1;
-    pa[0].val.clusterDim.z = 1;
-    probe.attrs = pa;
-    probe.numAttrs = 1;
-    int nclusters = 0;
-    if (cudaOccupancyMaxActiveClusters(&nclusters, cholinv_cluster_kernel<P>, &probe) != cudaSuccess ||
-        nclusters < 1) {
-      cudaGetLastError();
-      return false;
-    }
-    ready = 1;
-  }
+  auto* kern = cholinv_cluster_kernel<P, Src>;
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(P, 1, 1);
+  cfg.gridDim = dim3(P * np, 1, 1);
   cfg.blockDim = dim3(CT, 1, 1);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = s;
@@ -318,13 +453,38 @@ bool cholinv_launch(int m, const double2* W, int64_t ldw, double shift, double2*
   at[0].val.clusterDim.z = 1;
   cfg.attrs = at;
   cfg.numAttrs = 1;
-  if (cudaLaunchKernelEx(&cfg, cholinv_cluster_kernel<P>, m, W, ldw, shift, Li, ldi, Lf, ldl, info, info_base) !=
-      cudaSuccess) {
+  if (ready == 0) {
+    ready = -1;
+    if (P > 8 && cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) {
+      cudaGetLastError();
+      return false;
+    }
+    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem) != cudaSuccess) {
+      cudaGetLastError();
+      return false;
+    }
+    cudaLaunchConfig_t probe = cfg;
+    probe.gridDim = dim3(P, 1, 1);
+    probe.dynamicSmemBytes = kMaxSmem;
+    int nclusters = 0;
+    if (cudaOccupancyMaxActiveClusters(&nclusters, kern, &probe) != cudaSuccess || nclusters < 1) {
+      cudaGetLastError();
+      return false;
+    }
+    ready = 1;
+  }
+  if (cudaLaunchKernelEx(&cfg, kern, src) != cudaSuccess) {
     cudaGetLastError();
     return false;
   }
   LAUNCH_NOTE(1);
   return true;
+}
+
+// sixteen CTAs a matrix, or eight where the device cannot schedule sixteen
+template <class Src>
+bool cholinv_any(const Src& src, int np, int m, cudaStream_t s) {
+  return cholinv_launch<16>(src, np, m, s) || cholinv_launch<8>(src, np, m, s);
 }
 
 constexpr int kSMs = 152;
@@ -336,8 +496,15 @@ int cholinv_max_order() { return kCholInvMax; }
 bool cholinv_small(int m, const double2* W, int64_t ldw, double shift, double2* Li, int64_t ldi, double2* Lf,
                    int64_t ldl, int* info, cudaStream_t s, int info_base) {
   if (m < 1 || m > kCholInvMax) return false;
-  if (cholinv_launch<16>(m, W, ldw, shift, Li, ldi, Lf, ldl, info, info_base, s)) return true;
-  return cholinv_launch<8>(m, W, ldw, shift, Li, ldi, Lf, ldl, info, info_base, s);
+  CholOne src;
+  src.p = CholProb{m, W, ldw, shift, Li, ldi, Lf, ldl, info, info_base};
+  return cholinv_any(src, 1, m, s);
+}
+
+bool cholinv_batched(const BDesc* D, int np, int mmax, double shift_factor, cudaStream_t s) {
+  if (mmax < 1 || mmax > kCholInvMax) return false;
+  CholBatch src{D, shift_factor};
+  return cholinv_any(src, np, mmax, s);
 }
 
 namespace {

@@ -161,6 +161,8 @@ size_t lanczos_ws_bytes(int64_t n, int k);
 void lanczos_bounds(int64_t n, const float2* M32, int64_t ldm, int k, int count, uint64_t seed,
                     const LanczosWork& w, double* dev_out, cudaStream_t s);
 
+struct BDesc;
+
 // ---------------------------------------------------------------- tall-skinny kernels
 // res[i] = || W_i - theta_i Q_i ||_2 for columns i of n x m blocks (deterministic 2-stage).
 void resid_norms(int64_t n, int m, const double2* W, int64_t ldw, const double2* Q, int64_t ldq,
@@ -183,12 +185,15 @@ void zgram(int64_t n, int mx, int my, const double2* X, int64_t ldx, const doubl
 // the Cholesky factor of W + shift D^-2, of W itself for shift 0, and Li its inverse),
 // where D W D + shift I = L L^H, W m x m (lower triangle read; Lf may be W), D =
 // diag(W)^-1/2 (1 where a diagonal entry is not positive), in one thread-block cluster.
-// *info <- info_base + the 1-based index of a non-positive pivot (atomicCAS from 0;
-// nothing else is written then). false: not launchable (m > cholinv_max_order() or no
+// *info <- info_base + the 1-based index of a non-positive pivot (atomicCAS from 0; the
+// outputs are incomplete then). false: not launchable (m > cholinv_max_order() or no
 // cluster): nothing was enqueued.
 int cholinv_max_order();
 bool cholinv_small(int m, const double2* W, int64_t ldw, double shift, double2* Li, int64_t ldi, double2* Lf,
                    int64_t ldl, int* info, cudaStream_t s, int info_base = 0);
+// the same for every Gw of a batch (Li into Gwi, the pivot into flags[2]); the shift is
+// shift_factor times CholQR's; mmax: the largest order
+bool cholinv_batched(const BDesc* D, int np, int mmax, double shift_factor, cudaStream_t s);
 // Recursive Cholesky factorisation with the inverse, for the emulated-product mode: A
 // (n x n, lower triangle read) -> L in place (upper triangle zeroed), Li <- L^-1. A block of
 // order n > kCholLeaf splits as n1 + n2 (n1 a multiple of 128 near n / 2) with
@@ -203,7 +208,7 @@ bool cholinv_small(int m, const double2* W, int64_t ldw, double shift, double2* 
 // non-positive pivot sets *info to its global 1-based index (atomicCAS from 0); the later
 // launches then run on stale blocks and the results are to be discarded, the status
 // words possibly set by them with them.
-constexpr int64_t kCholLeaf = 256;
+constexpr int64_t kCholLeaf = 128;
 struct CholRes {
   char* memA;
   char* memB;
