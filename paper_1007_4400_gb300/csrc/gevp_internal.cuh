@@ -227,6 +227,8 @@ cudaError_t chol_recursive(int64_t n, double2* A, int64_t lda, double2* Li, int6
 // ---------------------------------------------------------------- backward
 // GA = gE X X^H, GB = -gE X diag(lam) X^H (lower tiles by GEMM, then Hermitian completion
 // scaled by the device scalar *gE). XL: n x nev scratch.
+// XL <- X diag(lam)
+void scale_by_lam(int64_t n, int nev, const double2* X, int64_t ldx, const double* lam, double2* XL, cudaStream_t s);
 void energy_backward_ws(int64_t n, int nev, const double2* X, int64_t ldx, const double* lam, const double* gE,
                         double2* GA, double2* GB, int64_t ldg, double2* XL, double2* split, size_t split_elems,
                         cudaStream_t s);
@@ -358,6 +360,8 @@ struct OzOperand {
   int conj = 0, mask = 0;
   bool cols = false;
   int* bad = nullptr;
+  const int* ks = nullptr;   // rows only: entry k scaled by 2^(ks_sign ks[k]) (exponents of another operand)
+  int ks_sign = 0;
 };
 // group 0: all moduli at once
 size_t oz_operand_bytes(int rows, int K, int S, int group = 0);
@@ -367,14 +371,17 @@ bool oz_supported();
 // 3: k >= r; into residue form in `mem` (oz_operand_bytes); *bad = 1 on a non-finite entry
 // active: nullable device flag, 0 = the launch does nothing (a converged batch problem)
 cudaError_t oz_split(OzOperand& op, void* mem, int rows, int K, const double2* X, int64_t ldx, int conj, int mask,
-                     int S, int* bad, cudaStream_t s, bool cols = false, const int* active = nullptr, int group = 0);
+                     int S, int* bad, cudaStream_t s, bool cols = false, const int* active = nullptr, int group = 0,
+                     const int* ks = nullptr, int ks_sign = 0);
 // D (A.rows x B.rows) = op(A) op(B); triA 1: op(A) lower, 2: upper; triB 1: op(B) lower, 2:
 // upper. ws: room for the result's residues; oz_work_bytes(M, N, K, S) holds the whole
 // result, less makes the product run in panels of rows (at least one of min(M, 256) rows).
-// D may be the memory of A's source (a row of D depends on that row of A alone).
+// D may be the memory of A's source (a row of D depends on that row of A alone). triD 1: the
+// lower triangle of D is written (and what of the upper one shares its 256-row tiles may be).
+// An entry that a non-finite row or column enters is NaN.
 size_t oz_work_bytes(int M, int N, int K, int S);
 cudaError_t oz_gemm(const OzOperand& A, const OzOperand& B, int triA, int triB, double2* D, int64_t ldd, int* err,
-                    cudaStream_t s, const int* active, void* ws, size_t ws_bytes);
+                    cudaStream_t s, const int* active, void* ws, size_t ws_bytes, int triD = 0);
 
 // ---------------------------------------------------------------- deviation angles
 // slices of the column-norm reduction (part needs slices * k doubles)

@@ -63,6 +63,11 @@ __device__ __forceinline__ float oz_mod(float x, float p, float ip) {
   return __fmaf_rn(-p, q, x);
 }
 
+// exponents of an all-zero row stay at the memset pattern of the column splitter; a row with a
+// non-finite entry is marked, and every result that it enters is NaN
+constexpr int kExpNone = (int)0x80808080;
+constexpr int kExpBad = 0x7f000000;
+
 struct OzModTab {
   float p[OZ_NMOD], ip[OZ_NMOD];
   float c1[OZ_NMOD], c2[OZ_NMOD], c3[OZ_NMOD];   // 2^14, 2^28, 2^42 modulo p, centred
@@ -187,6 +192,7 @@ struct OzParams {
   int kblocks;         // 64-blocks of K
   int triA;            // 1: op(A)[i][k] = 0 for k > i;  2: op(A)[i][k] = 0 for k < i
   int triB;            // 1: op(B)[k][j] = 0 for k < j;  2: op(B)[k][j] = 0 for k > j
+  int triD;            // 1: tiles above the diagonal are left out
   int mod0, nmod;      // moduli of this launch
   int za, zb;          // tensor-map plane of modulus mod0's real part in A, B
   int pa, pb;          // planes from a real to an imaginary part
@@ -255,6 +261,7 @@ __device__ __forceinline__ void oz_commit(uint64_t* bar) {
 
 struct OzUnit {
   int slice, mod, m0, n0, klo, khi;   // klo, khi in 64-blocks
+  bool skip;
 };
 
 // Unit u of a launch: slice-major, then modulus, then tiles in bands of eight column tiles (the
@@ -280,6 +287,8 @@ __device__ __forceinline__ OzUnit oz_unit(const OzParams& p, int u) {
     t.klo = max(t.klo, t.slice * p.kspan);
     t.khi = min(t.khi, (t.slice + 1) * p.kspan);
   }
+  t.skip = p.triD && t.n0 > t.m0 + 255;
+  if (t.skip) t.khi = t.klo;
   return t;
 }
 
@@ -420,7 +429,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) __cluster_dims__(2, 1, 1)
       int8_t* out = p.R + ((int64_t)(t.slice * 2) * p.nm + t.mod) * p.plane + (int64_t)row * p.ldr + t.n0;
       const int64_t opart = (int64_t)p.nm * p.plane;
       if (t.klo >= t.khi) {
-        if (row < p.M)
+        if (row < p.M && !t.skip)
           for (int g = warp >> 2; g < ng; g += 4) {
             *(uint4*)(out + 16 * g) = make_uint4(0, 0, 0, 0);
             *(uint4*)(out + opart + 16 * g) = make_uint4(0, 0, 0, 0);
@@ -474,9 +483,6 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) __cluster_dims__(2, 1, 1)
 }
 
 // ---------------------------------------------------------------- reconstruction
-// exponents of an all-zero row stay at the memset pattern of the column splitter
-constexpr int kExpNone = (int)0x80808080;
-
 // x = P frac, frac the 160-bit two's complement fraction w (little-endian), rounded to the
 // nearest double (integers below 2^53 exactly) and scaled by 2^ex
 __device__ __forceinline__ double oz_crt_value(uint32_t w0, uint32_t w1, uint32_t w2, uint32_t w3, uint32_t w4,
@@ -543,19 +549,22 @@ __device__ __forceinline__ double oz_crt_value(uint32_t w0, uint32_t w1, uint32_
 __global__ void __launch_bounds__(256) oz_crt_kernel(int M, int N, const int8_t* R, int ldr, int64_t plane, int nm,
                                                      int ksplit, const __grid_constant__ OzCrtTab tab, const int* ea,
                                                      const int* eb, int e0, double2* D, int64_t ldd,
-                                                     const int* active) {
+                                                     int row0, int triD, const int* active) {
   if (active && *active == 0) return;
   const int nq = (N + 3) / 4;
   const int64_t total = (int64_t)M * nq;
   for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < total; e += (int64_t)gridDim.x * blockDim.x) {
     const int row = (int)(e / nq), c0 = (int)(e % nq) * 4;
+    if (triD && c0 > row0 + row) continue;
     double v[2][4];
     const int er = ea[row] == kExpNone ? 0 : ea[row];
     int ex[4];
+    bool bad[4];
 #pragma unroll
     for (int c = 0; c < 4; ++c) {
       const int f = c0 + c < N ? eb[c0 + c] : 0;
       ex[c] = er + (f == kExpNone ? 0 : f) + e0;
+      bad[c] = er == kExpBad || f == kExpBad;
     }
 #pragma unroll
     for (int part = 0; part < 2; ++part) {
@@ -596,7 +605,10 @@ __global__ void __launch_bounds__(256) oz_crt_kernel(int M, int N, const int8_t*
     }
 #pragma unroll
     for (int c = 0; c < 4; ++c)
-      if (c0 + c < N) D[(int64_t)row * ldd + c0 + c] = make_double2(v[0][c], v[1][c]);
+      if (c0 + c < N) {
+        const double nan = __longlong_as_double(0x7ff8000000000000ll);
+        D[(int64_t)row * ldd + c0 + c] = bad[c] ? make_double2(nan, nan) : make_double2(v[0][c], v[1][c]);
+      }
   }
 }
 
@@ -615,10 +627,24 @@ __device__ __forceinline__ double2 oz_masked(double2 v, int r, int k, int mask) 
   return v;
 }
 
-__device__ __forceinline__ double2 oz_entry(const double2* X, int64_t ldx, int r, int k, int K,
-                                              int mask) {
+// x 2^s on the exponent field (0 for a value that is, or becomes, subnormal; Inf and NaN stay)
+__device__ __forceinline__ double oz_shift2(double x, int s) {
+  const int hi = __double2hiint(x), e = (hi >> 20) & 0x7FF;
+  if (e == 0x7FF) return x;
+  if (e == 0 || e + s <= 0) return 0.0;
+  return __hiloint2double(hi + (min(s, 2046 - e) << 20), __double2loint(x));
+}
+
+// ks (nullable), sg: entry k is scaled by 2^(sg ks[k]) first
+__device__ __forceinline__ double2 oz_entry(const double2* X, int64_t ldx, int r, int k, int K, int mask,
+                                            const int* ks, int sg) {
   if (k >= K) return make_double2(0.0, 0.0);
-  return oz_masked(X[(int64_t)r * ldx + k], r, k, mask);
+  double2 v = oz_masked(X[(int64_t)r * ldx + k], r, k, mask);
+  if (ks) {
+    const int q = ks[k];
+    if (q != kExpNone && q != kExpBad) v = make_double2(oz_shift2(v.x, sg * q), oz_shift2(v.y, sg * q));
+  }
+  return v;
 }
 
 // The splitting works on the IEEE-754 fields with integer instructions only: one SM
@@ -707,8 +733,9 @@ __device__ __forceinline__ void oz_write_pair(double2 v0, double2 v1, int shift,
 // warp writes 128 contiguous bytes of each plane). Bound by the planes' bytes: 16 read, 64
 // written per entry at 16 moduli. need_ex: find (and write) the exponent; else read it.
 __global__ void __launch_bounds__(256) oz_split_rows_kernel(int rows, int K, const double2* X, int64_t ldx, int mask,
-                                                            int S, int mod0, int cnt, int nmod, int k_pad,
-                                                            __nv_bfloat16* planes, int* ex, int need_ex, int* bad,
+                                                            const int* ks, int sg, int S, int mod0, int cnt, int nmod,
+                                                            int k_pad, __nv_bfloat16* planes, int* ex, int need_ex,
+                                                            int* bad,
                                                             const __grid_constant__ OzModTab tab, const int* active) {
   if (active && *active == 0) return;
   __shared__ unsigned long long red[8];
@@ -718,12 +745,13 @@ __global__ void __launch_bounds__(256) oz_split_rows_kernel(int rows, int K, con
     unsigned long long mx = 0;   // largest magnitude key of the finite entries
     bool nonfinite = false;
     for (int k = threadIdx.x; k < K; k += 256) {
-      const double2 v = oz_entry(X, ldx, r, k, K, mask);
+      const double2 v = oz_entry(X, ldx, r, k, K, mask, ks, sg);
       const unsigned long long kx = oz_abs_key(v.x), ky = oz_abs_key(v.y);
       if (!oz_key_finite(kx) || !oz_key_finite(ky)) nonfinite = true;
       else mx = max(mx, max(kx, ky));
     }
-    if (__any_sync(0xffffffffu, nonfinite) && (threadIdx.x & 31) == 0) atomicExch(bad, 1);
+    if (nonfinite) atomicExch(bad, 1);
+    nonfinite = __syncthreads_or(nonfinite) != 0;
     for (int o = 16; o > 0; o >>= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
     if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = mx;
     __syncthreads();
@@ -731,14 +759,14 @@ __global__ void __launch_bounds__(256) oz_split_rows_kernel(int rows, int K, con
     for (int w = 1; w < 8; ++w) mx = max(mx, red[w]);
     // 2^e > 2 max|entry|: the scaled row lies below 1/2
     e = mx > 0 ? oz_key_ilogb(mx) + 2 : 0;
-    if (threadIdx.x == 0) ex[r] = e;
+    if (threadIdx.x == 0) ex[r] = nonfinite ? kExpBad : e;
   } else {
-    e = ex[r];
+    e = ex[r] == kExpBad ? 0 : ex[r];
   }
   if (cnt == 0) return;
   const size_t plane = (size_t)rows * k_pad;
   for (int k = 2 * threadIdx.x; k < k_pad; k += 512)
-    oz_write_pair(oz_entry(X, ldx, r, k, K, mask), oz_entry(X, ldx, r, k + 1, K, mask), 7 * S - e, tab, mod0, cnt,
+    oz_write_pair(oz_entry(X, ldx, r, k, K, mask, ks, sg), oz_entry(X, ldx, r, k + 1, K, mask, ks, sg), 7 * S - e, tab, mod0, cnt,
                   (size_t)nmod * plane, plane, planes + (size_t)r * k_pad + k);
 }
 
@@ -769,7 +797,10 @@ __global__ void __launch_bounds__(256) oz_cols_exp_kernel(int R, int K, const do
       if (!oz_key_finite(kx) || !oz_key_finite(ky)) nonfinite = true;
       else mx = max(mx, max(kx, ky));
     }
-  if (nonfinite) atomicExch(bad, 1);
+  if (nonfinite) {
+    atomicExch(bad, 1);
+    atomicMax(&ex[j], kExpBad);
+  }
   red[threadIdx.y][threadIdx.x] = mx;
   __syncthreads();
   if (threadIdx.y == 0 && j < R) {
@@ -796,7 +827,7 @@ __global__ void __launch_bounds__(256) oz_split_cols_kernel(int R, int K, const 
   for (int jj = threadIdx.y; jj < OZ_CT; jj += 8) {
     const int j = j0 + jj;
     if (j >= R) break;
-    const int e = ex[j];
+    const int e = ex[j] == kExpBad ? 0 : ex[j];
     oz_write_pair(tile[kk][jj], tile[kk + 1][jj], 7 * S - (e == kExpNone ? 0 : e), tab, mod0, cnt,
                   (size_t)nmod * plane, plane,                  planes + (size_t)j * k_pad + k);
   }
@@ -843,8 +874,8 @@ cudaError_t oz_split_group(const OzOperand& op, int mod0, int cnt, bool need_ex,
   if (op.rows == 0) return cudaSuccess;
   const OzModTab& tab = oz_mod_tab();
   if (!op.cols) {
-    oz_split_rows_kernel<<<op.rows, 256, 0, s>>>(op.rows, op.K, op.X, op.ldx, op.mask, op.S, mod0, cnt, op.nmod, op.k_pad,
-                                                 op.planes, op.ex, need_ex ? 1 : 0, bad, tab, active);
+    oz_split_rows_kernel<<<op.rows, 256, 0, s>>>(op.rows, op.K, op.X, op.ldx, op.mask, op.ks, op.ks_sign, op.S, mod0,
+                                                 cnt, op.nmod, op.k_pad, op.planes, op.ex, need_ex ? 1 : 0, bad, tab, active);
     LAUNCH_NOTE(1);
     return cudaGetLastError();
   }
@@ -885,7 +916,8 @@ bool oz_supported() {
 }
 
 cudaError_t oz_split(OzOperand& op, void* mem, int rows, int K, const double2* X, int64_t ldx, int conj, int mask,
-                     int S, int* bad, cudaStream_t s, bool cols, const int* active, int group) {
+                     int S, int* bad, cudaStream_t s, bool cols, const int* active, int group, const int* ks,
+                     int ks_sign) {
   const int nm = oz_moduli(K, S);
   if (S < 1 || S > kOzSlicesMax || nm > OZ_NMOD) return cudaErrorInvalidValue;
   op.rows = rows;
@@ -901,12 +933,14 @@ cudaError_t oz_split(OzOperand& op, void* mem, int rows, int K, const double2* X
   op.mask = mask;
   op.cols = cols;
   op.bad = bad;
+  op.ks = cols ? nullptr : ks;
+  op.ks_sign = ks_sign;
   // in groups: the exponents only (oz_gemm writes each group's residues before it uses them)
   return oz_split_group(op, 0, op.nmod == nm ? nm : 0, true, bad, s, active);
 }
 
 cudaError_t oz_gemm(const OzOperand& A, const OzOperand& B, int triA, int triB, double2* D, int64_t ldd, int* err,
-                    cudaStream_t s, const int* active, void* ws, size_t ws_bytes) {
+                    cudaStream_t s, const int* active, void* ws, size_t ws_bytes, int triD) {
   if (A.K != B.K || A.S != B.S || A.k_pad != B.k_pad || !ws) return cudaErrorInvalidValue;
   if (A.rows == 0 || B.rows == 0) return cudaSuccess;
   const int nm = oz_moduli(A.K, A.S);
@@ -927,6 +961,7 @@ cudaError_t oz_gemm(const OzOperand& A, const OzOperand& B, int triA, int triB, 
   p.kblocks = (A.K + OZ_TK - 1) / OZ_TK;
   p.triA = triA;
   p.triB = triB;
+  p.triD = triD;
   p.nm = nm;
   p.err = err;
   p.active = active;
@@ -1012,6 +1047,7 @@ cudaError_t oz_gemm(const OzOperand& A, const OzOperand& B, int triA, int triB, 
             if (triB == 1) klo = std::max(klo, n0 / OZ_TK);
             if (triB == 2) khi = std::min(khi, (n0 + p.tn + OZ_TK - 1) / OZ_TK);
             const int rows = std::min(256, row0 + p.M - m0), cols = std::min(p.tn, p.N - n0);
+            if (triD && n0 > m0 + 255) continue;
             if (khi > klo && rows > 0 && cols > 0) alg += 8.0 * rows * cols * (double)(khi - klo) * OZ_TK;
           }
         kt_end(kt0, 1, alg * p.nmod / nm, alg * p.nmod, s);
@@ -1020,7 +1056,7 @@ cudaError_t oz_gemm(const OzOperand& A, const OzOperand& B, int triA, int triB, 
     const int64_t quads = (int64_t)p.M * ((p.N + 3) / 4);
     const int blocks = (int)std::min<int64_t>((quads + 255) / 256, 152 * 16);
     oz_crt_kernel<<<blocks, 256, 0, s>>>(p.M, p.N, p.R, p.ldr, p.plane, nm, p.ksplit, oz_crt_tab(nm), A.ex + row0, B.ex,
-                                         -14 * A.S, D + (int64_t)row0 * ldd, ldd, active);
+                                         -14 * A.S, D + (int64_t)row0 * ldd, ldd, row0, triD, active);
     LAUNCH_NOTE(1);
   }
   return cudaGetLastError();

@@ -199,6 +199,13 @@ void gram_scale(int m, double2* W, int64_t ldw, double* dscale, cudaStream_t s) 
   LAUNCH_NOTE(1);
 }
 
+void scale_by_lam(int64_t n, int nev, const double2* X, int64_t ldx, const double* lam, double2* XL, cudaStream_t s) {
+  const int64_t total = n * nev;
+  const int blocks = (int)std::min<int64_t>((total + 255) / 256, 152 * 8);
+  scale_rows_by_lam_kernel<<<blocks, 256, 0, s>>>(n, nev, X, ldx, lam, XL);
+  LAUNCH_NOTE(1);
+}
+
 void energy_backward_ws(int64_t n, int nev, const double2* X, int64_t ldx, const double* lam, const double* gE,
                         double2* GA, double2* GB, int64_t ldg, double2* XL, double2* split, size_t split_elems,
                         cudaStream_t s) {
@@ -208,10 +215,7 @@ void energy_backward_ws(int64_t n, int nev, const double2* X, int64_t ldx, const
   a.triD = 1;
   zgemm(a, split, split_elems, s);
   hermitize_scale_lower(n, GA, ldg, gE, 1.0, s);
-  int64_t total = n * nev;
-  int blocks = (int)std::min<int64_t>((total + 255) / 256, 152 * 8);
-  scale_rows_by_lam_kernel<<<blocks, 256, 0, s>>>(n, nev, X, ldx, lam, XL);
-  LAUNCH_NOTE(1);
+  scale_by_lam(n, nev, X, ldx, lam, XL, s);
   ZgemmArgs b = zg((int)n, (int)n, nev, XL, nev, 0, X, ldx, 1, GB, ldg);
   b.triD = 1;
   zgemm(b, split, split_elems, s);
