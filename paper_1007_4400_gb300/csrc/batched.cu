@@ -295,7 +295,6 @@ gevp_status build_plan(gevp_ctx* h, BatchPlan* P, std::string& err) {
       d.mtiles = n_pad[p] / 128;
       d.ks = ks[p];
       d.kbps = kbps[p];
-      d.nseg = tcg_nseg(P->nsplit);
       unsigned tcols = 32;
       while (tcols < 3u * (unsigned)nchunk[p]) tcols *= 2;
       d.tmem_cols = tcols;

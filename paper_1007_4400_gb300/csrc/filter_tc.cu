@@ -7,9 +7,11 @@
 //
 // Precision. Each real operand x is stored as nsplit BF16 pieces x = x0 + x1 + x2 + ...
 // (x0 = bf16(x), x1 = bf16(x - x0), ...). nsplit = 1 is the BF16 filter. nsplit = 3 keeps
-// the six products x_a y_b with a + b <= 2 (about 24 significant bits, FP32 class); the
-// products are extra segments of the K loop accumulating into the same TMEM accumulators,
-// so the kernel is unchanged apart from which tensor map each segment loads.
+// the six products x_a y_b with a + b <= 2 (about 24 significant bits, FP32 class), accumulated in
+// the same TMEM accumulators. A pipeline stage then holds the three pieces of one part (re, im or
+// re + im) of C and of Y for one K block, which serve all six products of that part: half the
+// bytes through L2 and shared memory of a stage per product pair (n = 2048, m = 140, six
+// products: 27.8 us a step; 31.5 with the operands of one piece pair a stage).
 //
 // Layout (all K-major, as the MMA wants both operands): the planes of C are n_pad x n_pad
 // row-major BF16 (row i = output row, contiguous k); the block Y is stored transposed,
@@ -47,7 +49,6 @@ constexpr int MAXSEG = 6;
 // segments (a piece, b piece) with a + b <= nsplit - 1
 __constant__ int kSegA[MAXSEG] = {0, 0, 1, 0, 1, 2};
 __constant__ int kSegB[MAXSEG] = {0, 1, 0, 2, 1, 0};
-inline int nseg_for(int nsplit) { return nsplit == 1 ? 1 : (nsplit == 2 ? 3 : 6); }
 
 struct TcMaps {
   CUtensorMap a[MAXSPLIT * 3];   // C planes: [piece][re, im, re+im]
@@ -59,7 +60,7 @@ struct TcParams {
   int nchunk;
   int kb_per_split;
   int ncols_pad;      // rows of the Y^T planes (multiple of nchunk)
-  int nseg;
+  int nsplit;         // pieces per operand
   uint32_t tmem_cols; // power of two >= 3 * nchunk
   float2* ws;         // [ksplit][ncols_pad][n_pad]
   int* err;
@@ -79,9 +80,10 @@ __device__ __forceinline__ void tc_tile(const CUtensorMap* amaps, const CUtensor
   const int kb0 = z * p.kb_per_split;
   const int kb1 = min(kb0 + p.kb_per_split, nkb_total);
   const int nkb = max(0, kb1 - kb0);
-  // K-block-major: all segments of one K block back to back, so the C piece a segment
-  // reloads (piece 0 serves three segments, piece 1 two) is still in L2
-  const int niter = nkb * p.nseg;
+  // a stage: one K block, either the three parts of a single piece, or the pieces of one part
+  const bool by_part = p.nsplit > 1;
+  const int group = by_part ? 3 : 1, boxes = by_part ? p.nsplit : 3;
+  const int niter = nkb * group;
   const uint32_t a_bytes = TM * TK * 2;
   const uint32_t b_bytes = (uint32_t)p.nchunk * TK * 2;
   const uint32_t stage_bytes = 3 * a_bytes + 3 * b_bytes;
@@ -114,17 +116,14 @@ __device__ __forceinline__ void tc_tile(const CUtensorMap* amaps, const CUtensor
       int s = i % STAGES;
       uint32_t ph = (uint32_t)(i / STAGES) & 1u;
       if (i >= STAGES && !mbar_wait(&empty[s], ph ^ 1u, p.err, 1)) break;
-      mbar_expect_tx(&full[s], stage_bytes);
-      const int seg = i % p.nseg;
-      const int kx = (kb0 + i / p.nseg) * TK;
-      const CUtensorMap* A = amaps + 3 * kSegA[seg];
-      const CUtensorMap* B = bmaps + 3 * kSegB[seg];
-      tma_load_2d(tile(s, 0), A + 0, kx, m0, &full[s]);
-      tma_load_2d(tile(s, 1), A + 1, kx, m0, &full[s]);
-      tma_load_2d(tile(s, 2), A + 2, kx, m0, &full[s]);
-      tma_load_2d(tile(s, 3), B + 0, kx, c0, &full[s]);
-      tma_load_2d(tile(s, 4), B + 1, kx, c0, &full[s]);
-      tma_load_2d(tile(s, 5), B + 2, kx, c0, &full[s]);
+      mbar_expect_tx(&full[s], (uint32_t)boxes * (a_bytes + b_bytes));
+      const int part = i % group;
+      const int kx = (kb0 + i / group) * TK;
+      for (int w = 0; w < boxes; ++w) {
+        const int map = by_part ? 3 * w + part : w;
+        tma_load_2d(tile(s, w), amaps + map, kx, m0, &full[s]);
+        tma_load_2d(tile(s, 3 + w), bmaps + map, kx, c0, &full[s]);
+      }
     }
     // every copy issued has landed before the CTA leaves (bounded; immediate unless a wait
     // elsewhere gave up)
@@ -137,15 +136,30 @@ __device__ __forceinline__ void tc_tile(const CUtensorMap* amaps, const CUtensor
       uint32_t ph = (uint32_t)(i / STAGES) & 1u;
       if (!mbar_wait(&full[s], ph, p.err, 2)) break;
       fence_after();
-      const uint64_t dr = sdesc(su32(tile(s, 0))), di = sdesc(su32(tile(s, 1))), ds = sdesc(su32(tile(s, 2)));
-      const uint64_t er = sdesc(su32(tile(s, 3))), ei = sdesc(su32(tile(s, 4))), es = sdesc(su32(tile(s, 5)));
+      const uint64_t d0 = sdesc(su32(tile(s, 0))), d1 = sdesc(su32(tile(s, 1))), d2 = sdesc(su32(tile(s, 2)));
+      const uint64_t e0 = sdesc(su32(tile(s, 3))), e1 = sdesc(su32(tile(s, 4))), e2 = sdesc(su32(tile(s, 5)));
+      if (!by_part) {
 #pragma unroll
-      for (int kk = 0; kk < TK / 16; ++kk) {
-        uint32_t acc = (i > 0 || kk > 0) ? 1u : 0u;
-        uint64_t off = (uint64_t)(kk * 32) >> 4;   // 16 bf16 = 32 B along K inside the swizzle row
-        umma(tmem, dr + off, er + off, idesc, acc);
-        umma(tmem + (uint32_t)p.nchunk, di + off, ei + off, idesc, acc);
-        umma(tmem + 2u * (uint32_t)p.nchunk, ds + off, es + off, idesc, acc);
+        for (int kk = 0; kk < TK / 16; ++kk) {
+          const uint32_t acc = (i > 0 || kk > 0) ? 1u : 0u;
+          const uint64_t off = (uint64_t)(kk * 32) >> 4;   // 16 bf16 = 32 B along K inside the swizzle row
+          umma(tmem, d0 + off, e0 + off, idesc, acc);
+          umma(tmem + (uint32_t)p.nchunk, d1 + off, e1 + off, idesc, acc);
+          umma(tmem + 2u * (uint32_t)p.nchunk, d2 + off, e2 + off, idesc, acc);
+        }
+      } else {
+        const uint32_t dt = tmem + (uint32_t)((i % group) * p.nchunk);
+        const uint32_t acc0 = i >= group ? 1u : 0u;
+        const int nseg = p.nsplit == 2 ? 3 : 6;
+        for (int seg = 0; seg < nseg; ++seg) {
+          const int pa = kSegA[seg], pb = kSegB[seg];
+          const uint64_t a = pa == 0 ? d0 : (pa == 1 ? d1 : d2), b = pb == 0 ? e0 : (pb == 1 ? e1 : e2);
+#pragma unroll
+          for (int kk = 0; kk < TK / 16; ++kk) {
+            const uint64_t off = (uint64_t)(kk * 32) >> 4;
+            umma(dt, a + off, b + off, idesc, (seg > 0 || kk > 0) ? 1u : acc0);
+          }
+        }
       }
       umma_commit(&empty[s]);
     }
@@ -186,26 +200,59 @@ __global__ void __launch_bounds__(128, 1) cheb_tc_kernel(const __grid_constant__
   tc_tile(maps.a, maps.b, p, blockIdx.x * TM, blockIdx.y * p.nchunk, blockIdx.z);
 }
 
-// Split v into nsplit BF16 pieces written at stride `ps` (piece p at base + p * ps).
-__device__ __forceinline__ void split_store(double v, int nsplit, __nv_bfloat16* base, size_t ps, int64_t e) {
-  double r = v;
-  for (int p = 0; p < nsplit; ++p) {
-    __nv_bfloat16 h = __double2bfloat16(r);
-    base[(size_t)p * ps + e] = h;
-    r -= (double)__bfloat162float(h);
+// v = hi + lo to about 2^-48, hi the leading 24 bits of v (truncated), from the IEEE-754 fields: an
+// FP64 conversion or addition takes 64 times an FP32 one here, and the pieces of a matrix need
+// ten of them per value.
+struct FPair {
+  float hi, lo;
+};
+__device__ __forceinline__ FPair fsplit(double v) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(v);
+  const int ef = (int)((b >> 52) & 0x7FF) - 896;   // the FP32 exponent field
+  FPair r;
+  if (ef <= 52 || ef >= 255) {   // 0, tiny (the low part would be subnormal), too large, Inf or NaN
+    r.hi = (float)v;
+    r.lo = 0.f;
+    return r;
   }
+  const uint32_t sign = (uint32_t)(b >> 32) & 0x80000000u;
+  r.hi = __uint_as_float(sign | (uint32_t)ef << 23 | ((uint32_t)(b >> 29) & 0x7FFFFFu));
+  const uint32_t m = (uint32_t)b & 0x1FFFFFFFu;   // 29 bits, unit 2^(ef - 179)
+  r.lo = (float)(int)m * __uint_as_float(sign | (uint32_t)(ef - 52) << 23);
+  return r;
+}
+// the sum of two such values (exact first sum, rounded low part)
+__device__ __forceinline__ FPair fsum(FPair a, FPair b) {
+  FPair r;
+  const float s = a.hi + b.hi, t = s - a.hi;
+  const float lo = ((a.hi - (s - t)) + (b.hi - t)) + (a.lo + b.lo);
+  r.hi = s + lo;   // (after a cancellation the low part is not below half a unit of s)
+  r.lo = lo - (r.hi - s);
+  return r;
 }
 
-// The same pieces for a value that is already FP32, in FP32 arithmetic: each piece is the
-// nearest BF16 of the remainder, and the remainder minus its nearest BF16 is exact in FP32
-// (the two are within a factor of two: Sterbenz), so the pieces equal split_store's
-// bit for bit without FP64 instructions (the FP64 pipe is 1/64 of the FP32 rate here).
-__device__ __forceinline__ void split_store_f32(float v, int nsplit, __nv_bfloat16* base, size_t ps, int64_t e) {
-  float r = v;
-  for (int p = 0; p < nsplit; ++p) {
-    __nv_bfloat16 h = __float2bfloat16_rn(r);
-    base[(size_t)p * ps + e] = h;
-    r -= __bfloat162float(h);
+// nsplit BF16 pieces of two neighbouring values, one 4-byte store per piece (piece p at base + p ps):
+// each piece is the nearest BF16 of the remainder, and the remainder minus it is exact in FP32
+// (Sterbenz); the low part, below half a unit of hi, decides where hi alone is a tie and joins
+// after the first piece
+__device__ __forceinline__ void store_pieces(const FPair& a, const FPair& b, int nsplit, __nv_bfloat16* at, size_t ps) {
+  auto first = [](const FPair& v) {
+    uint32_t b = __float_as_uint(v.hi);
+    if ((b & 0xFFFFu) == 0x8000u && v.lo != 0.f) b += (__float_as_uint(v.lo) ^ b) >> 31 ? ~0u : 1u;
+    return __float2bfloat16_rn(__uint_as_float(b));
+  };
+  __nv_bfloat16 ha = first(a), hb = first(b);
+  float ra = (a.hi - __bfloat162float(ha)) + a.lo, rb = (b.hi - __bfloat162float(hb)) + b.lo;
+  for (int p = 0;; ++p) {
+    __nv_bfloat162 v;
+    v.x = ha;
+    v.y = hb;
+    *(__nv_bfloat162*)(at + (size_t)p * ps) = v;
+    if (p + 1 >= nsplit) break;
+    ha = __float2bfloat16_rn(ra);
+    hb = __float2bfloat16_rn(rb);
+    ra -= __bfloat162float(ha);
+    rb -= __bfloat162float(hb);
   }
 }
 
@@ -213,11 +260,12 @@ struct YPlanes {
   __nv_bfloat16* base;   // [piece][part re, im, re+im][ncols_pad][n_pad]
   size_t plane;          // ncols_pad * n_pad
   int nsplit;
-  __device__ __forceinline__ void store(int64_t e, float2 y) const {
-    split_store_f32(y.x, nsplit, base, 3 * plane, e);
-    split_store_f32(y.y, nsplit, base + plane, 3 * plane, e);
-    // the exact sum of two FP32 values needs up to 25 significant bits: split in FP64
-    split_store((double)y.x + (double)y.y, nsplit, base + 2 * plane, 3 * plane, e);
+  // entries e and e + 1 (e even)
+  __device__ __forceinline__ void store2(int64_t e, float2 y0, float2 y1) const {
+    const FPair x0{y0.x, 0.f}, x1{y1.x, 0.f}, z0{y0.y, 0.f}, z1{y1.y, 0.f};
+    store_pieces(x0, x1, nsplit, base + e, 3 * plane);
+    store_pieces(z0, z1, nsplit, base + plane + e, 3 * plane);
+    store_pieces(fsum(x0, z0), fsum(x1, z1), nsplit, base + 2 * plane + e, 3 * plane);
   }
 };
 
@@ -230,39 +278,38 @@ __device__ __forceinline__ void tc_epilogue_body(int n, int ncols, int n_pad, in
                                                  const float2* ws, const float2* cur, const float2* prev, float2* outp,
                                                  const YPlanes& yp, float alpha, float beta, float gamma,
                                                  const float2* R, const float* pc) {
-  int64_t total = (int64_t)ncols_pad * n_pad;
-  int64_t plane = total;
-  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < total; e += (int64_t)gridDim.x * blockDim.x) {
-    int col = (int)(e / n_pad), row = (int)(e % n_pad);
-    float2 y = make_float2(0.f, 0.f);
+  // two neighbouring rows (n_pad is even) of a column a thread
+  const int64_t plane = (int64_t)ncols_pad * n_pad;
+  const uint32_t half = (uint32_t)n_pad / 2, total = (uint32_t)ncols_pad * half;
+  for (uint32_t q = blockIdx.x * blockDim.x + threadIdx.x; q < total; q += gridDim.x * blockDim.x) {
+    const int col = (int)(q / half), row = 2 * (int)(q % half);
+    const int64_t e = (int64_t)col * n_pad + row;
+    float4 y = make_float4(0.f, 0.f, 0.f, 0.f);
     if (col < ncols && row < n) {
-      float2 acc = make_float2(0.f, 0.f);
+      float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 4
       for (int z = 0; z < ksplit; ++z) {
-        float2 v = ws[(int64_t)z * plane + e];
+        const float4 v = *(const float4*)(ws + (int64_t)z * plane + e);
         acc.x += v.x;
         acc.y += v.y;
+        acc.z += v.z;
+        acc.w += v.w;
       }
-      y.x = alpha * acc.x;
-      y.y = alpha * acc.y;
-      if (cur) {
-        float2 c = cur[e];
-        y.x += beta * c.x;
-        y.y += beta * c.y;
-      }
-      if (prev) {
-        float2 q = prev[e];
-        y.x += gamma * q.x;
-        y.y += gamma * q.y;
-      }
-      if (R) {
-        float2 r = R[e];
-        float w = pc[col];
-        y.x += w * r.x;
-        y.y += w * r.y;
-      }
+      y = make_float4(alpha * acc.x, alpha * acc.y, alpha * acc.z, alpha * acc.w);
+      auto axpy = [&](float f, const float2* p) {
+        const float4 v = *(const float4*)(p + e);
+        y.x += f * v.x;
+        y.y += f * v.y;
+        y.z += f * v.z;
+        y.w += f * v.w;
+      };
+      if (cur) axpy(beta, cur);
+      if (prev) axpy(gamma, prev);
+      if (R) axpy(pc[col], R);
+      if (row + 1 >= n) y.z = y.w = 0.f;
     }
-    outp[e] = y;
-    yp.store(e, y);
+    *(float4*)(outp + e) = y;
+    yp.store2(e, make_float2(y.x, y.y), make_float2(y.z, y.w));
   }
 }
 
@@ -327,16 +374,29 @@ __global__ void defect_to_y(int n, int m, int n_pad, const float2* Dt, const dou
   defect_to_y_body(n, m, n_pad, Dt, Q, ldq, pd, Y, ldy, blockIdx.x * 32, blockIdx.y * 32);
 }
 
-// C (FP64, n x n) -> BF16 pieces [piece][re, im, re+im][n_pad][n_pad] (zero padding).
-__global__ void c_to_planes(int64_t n, int n_pad, const double2* C, int64_t ldc, __nv_bfloat16* planes, int nsplit) {
-  int64_t total = (int64_t)n_pad * n_pad;
-  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < total; e += (int64_t)gridDim.x * blockDim.x) {
-    int64_t i = e / n_pad, j = e % n_pad;
-    double2 v = (i < n && j < n) ? C[i * ldc + j] : make_double2(0.0, 0.0);
-    split_store(v.x, nsplit, planes, 3 * (size_t)total, e);
-    split_store(v.y, nsplit, planes + total, 3 * (size_t)total, e);
-    split_store(v.x + v.y, nsplit, planes + 2 * total, 3 * (size_t)total, e);
+// C (FP64, n x n) -> BF16 pieces [piece][re, im, re+im][n_pad][n_pad] (zero padding), two
+// neighbouring entries a thread. Bound by its integer and FP32 instructions and the planes' bytes
+// (n = 2048, three pieces: 28 us; 205 with FP64 conversions).
+__device__ __forceinline__ void c_to_planes_body(int64_t n, int n_pad, const double2* C, int64_t ldc,
+                                                 __nv_bfloat16* planes, int nsplit) {
+  const size_t total = (size_t)n_pad * n_pad;
+  const uint32_t half = (uint32_t)n_pad / 2;
+  for (uint64_t q = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; q < total / 2;
+       q += (uint64_t)gridDim.x * blockDim.x) {
+    const int64_t i = (int64_t)(q / half), j = 2 * (int64_t)(q % half);
+    const double2 zero = make_double2(0.0, 0.0);
+    const double2 u = (i < n && j < n) ? C[i * ldc + j] : zero, v = (i < n && j + 1 < n) ? C[i * ldc + j + 1] : zero;
+    const FPair ux = fsplit(u.x), uy = fsplit(u.y), vx = fsplit(v.x), vy = fsplit(v.y);
+    __nv_bfloat16* at = planes + (size_t)i * n_pad + j;
+    store_pieces(ux, vx, nsplit, at, 3 * total);
+    store_pieces(uy, vy, nsplit, at + total, 3 * total);
+    store_pieces(fsum(ux, uy), fsum(vx, vy), nsplit, at + 2 * total, 3 * total);
   }
+}
+
+__global__ void __launch_bounds__(256) c_to_planes(int64_t n, int n_pad, const double2* C, int64_t ldc,
+                                                   __nv_bfloat16* planes, int nsplit) {
+  c_to_planes_body(n, n_pad, C, ldc, planes, nsplit);
 }
 
 // Y (FP64 row-major n x m, ld) -> transposed FP32 state + BF16 pieces (ncols_pad x n_pad),
@@ -352,13 +412,13 @@ __global__ void y_to_state(int n, int m, int n_pad, int ncols_pad, const double2
     t[k][tx] = make_float2((float)v.x, (float)v.y);
   }
   __syncthreads();
-  for (int k = ty; k < 32; k += 8) {
-    int c = c0 + k, r = r0 + tx;
+  for (int k = threadIdx.x / 16; k < 32; k += 16) {
+    const int c = c0 + k, r = r0 + 2 * (threadIdx.x % 16);
     if (c < ncols_pad && r < n_pad) {
-      float2 v = t[tx][k];
-      int64_t e = (int64_t)c * n_pad + r;
-      st[e] = v;
-      yp.store(e, v);
+      const float2 u = t[r - r0][k], v = t[r - r0 + 1][k];
+      const int64_t e = (int64_t)c * n_pad + r;
+      *(float4*)(st + e) = make_float4(u.x, u.y, v.x, v.y);
+      yp.store2(e, u, v);
     }
   }
 }
@@ -425,7 +485,8 @@ void chunking(int m, int* nchunks, int* nchunk) {
 }  // namespace
 
 struct FilterTC {
-  int n_pad = 0, ncols_pad = 0;
+  int n_pad = 0;                    // of the problem it was last reserved for
+  int cap_n = 0, cap_cols = 0;      // what the arena holds
   int c_nsplit = 0;                 // pieces of C currently stored
   __nv_bfloat16* Cp = nullptr;      // [MAXSPLIT][3][n_pad][n_pad]
   __nv_bfloat16* Yp = nullptr;      // [MAXSPLIT][3][ncols_pad][n_pad]
@@ -456,10 +517,12 @@ cudaError_t filter_tc_reserve(FilterTC** pf, int64_t n, int m, cudaStream_t s) {
   int n_pad = pad_to((int)n, TM);
   int nchunks, nchunk;
   chunking(m, &nchunks, &nchunk);
-  int ncols_pad = nchunks * nchunk;
-  if (n_pad <= f->n_pad && ncols_pad <= f->ncols_pad && f->arena) return cudaSuccess;
-  n_pad = std::max(n_pad, f->n_pad);
-  ncols_pad = std::max(ncols_pad, f->ncols_pad);
+  int ncols_pad = nchunks * pad_to(nchunk, 32);   // also as twice as many tiles of half the width
+  // the padding and the launch follow the problem, not the largest one so far
+  f->n_pad = n_pad;
+  if (n_pad <= f->cap_n && ncols_pad <= f->cap_cols && f->arena) return cudaSuccess;
+  n_pad = std::max(n_pad, f->cap_n);
+  ncols_pad = std::max(ncols_pad, f->cap_cols);
   if (f->arena) cudaFree(f->arena);
   f->arena = nullptr;
   f->c_nsplit = 0;
@@ -469,7 +532,7 @@ cudaError_t filter_tc_reserve(FilterTC** pf, int64_t n, int m, cudaStream_t s) {
                  al((size_t)kKsplitMax * nc * 8) + al((size_t)kDegMax * ncols_pad * 4) + al((size_t)ncols_pad * 8) +
                  1024;
   cudaError_t e = cudaMalloc(&f->arena, bytes);
-  if (e != cudaSuccess) { f->arena = nullptr; f->n_pad = f->ncols_pad = 0; return e; }
+  if (e != cudaSuccess) { f->arena = nullptr; f->cap_n = f->cap_cols = 0; return e; }
   e = cudaMemsetAsync(f->arena, 0, bytes, s);
   if (e != cudaSuccess) return e;
   char* p = (char*)f->arena;
@@ -489,8 +552,8 @@ cudaError_t filter_tc_reserve(FilterTC** pf, int64_t n, int m, cudaStream_t s) {
   cudaMallocHost(&f->h_pcoef, (size_t)kDegMax * ncols_pad * 4);
   cudaMallocHost(&f->h_pfinal, (size_t)ncols_pad * 8);
   f->err = (int*)p;
-  f->n_pad = n_pad;
-  f->ncols_pad = ncols_pad;
+  f->cap_n = n_pad;
+  f->cap_cols = ncols_pad;
   f->bytes = bytes;
   return cudaSuccess;
 }
@@ -505,7 +568,7 @@ void filter_tc_release(FilterTC* f) {
 
 // Convert C (FP64) into its BF16 pieces; once per problem.
 cudaError_t filter_tc_set_matrix(FilterTC* f, int64_t n, const double2* C, int64_t ldc, int nsplit, cudaStream_t s) {
-  int64_t total = (int64_t)f->n_pad * f->n_pad;
+  int64_t total = (int64_t)f->n_pad * f->n_pad / 2;
   int blocks = (int)std::min<int64_t>((total + 255) / 256, 152 * 16);
   c_to_planes<<<blocks, 256, 0, s>>>(n, f->n_pad, C, ldc, f->Cp, nsplit);
   LAUNCH_NOTE(1);
@@ -524,7 +587,21 @@ cudaError_t run_filter(FilterTC* f, int64_t n, int m, const double2* Y, int64_t 
   int nchunks, nchunk;
   chunking(m, &nchunks, &nchunk);
   const int n_pad = f->n_pad;
-  const int ncols_pad = f->ncols_pad;
+  const int mtiles = n_pad / TM;
+  const int nkb = n_pad / TK;
+  // K slices: those of the arena's order (the largest served so far), which keeps the
+  // order of the FP32 sums, and with it the result, what it is with the block padded to that order
+  const int cap_kb = f->cap_n / TK;
+  const int want = std::max(1, std::min(std::min(kKsplitMax, cap_kb / 2), 152 / std::max(f->cap_n / TM * nchunks, 1)));
+  const int kbps = (cap_kb + want - 1) / want;
+  const int ks = (nkb + kbps - 1) / kbps;
+  // where that leaves SMs idle, narrower column tiles: they share no sums, so they change nothing else
+  // (n = 2048, m = 140 in an arena of order 4224: 58.6 us a step, 62.3 with 144-wide tiles)
+  if (nchunk > 64 && 2 * mtiles * nchunks * ks <= 152) {
+    nchunk = pad_to((m + 2 * nchunks - 1) / (2 * nchunks), 16);
+    nchunks = (m + nchunk - 1) / nchunk;
+  }
+  const int ncols_pad = nchunks * nchunk;   // of the active columns, at most what was reserved
   const size_t cplane = (size_t)n_pad * n_pad, yplane = (size_t)ncols_pad * n_pad;
   TcMaps maps;
   std::memset(&maps, 0, sizeof(maps));
@@ -535,18 +612,12 @@ cudaError_t run_filter(FilterTC* f, int64_t n, int m, const double2* Y, int64_t 
         return cudaErrorNotSupported;
     }
   YPlanes yp{f->Yp, yplane, nsplit};
-  const int mtiles = n_pad / TM;
-  const int nkb = n_pad / TK;
-  int base = mtiles * nchunks;
-  int ks = std::max(1, std::min(std::min(kKsplitMax, nkb / 2), 152 / std::max(base, 1)));
-  int kbps = (nkb + ks - 1) / ks;
-  ks = (nkb + kbps - 1) / kbps;
   TcParams p;
   p.n_pad = n_pad;
   p.nchunk = nchunk;
   p.kb_per_split = kbps;
   p.ncols_pad = ncols_pad;
-  p.nseg = nseg_for(nsplit);
+  p.nsplit = nsplit;
   p.ws = f->ws;
   p.err = f->err;
   p.tmem_cols = 32;
@@ -573,7 +644,7 @@ cudaError_t run_filter(FilterTC* f, int64_t n, int m, const double2* Y, int64_t 
     }
   }
   dim3 tg((n_pad + 31) / 32, (ncols_pad + 31) / 32);
-  int64_t total = (int64_t)ncols_pad * n_pad;
+  int64_t total = (int64_t)ncols_pad * n_pad / 2;
   int eblocks = (int)std::min<int64_t>((total + 255) / 256, 152 * 16);
   dim3 grid(mtiles, nchunks, ks);
   float2* prev = nullptr;
@@ -689,7 +760,7 @@ __global__ void __launch_bounds__(128, 1) cheb_tcg_kernel(const BDesc* D, int np
   p.nchunk = d.nchunk;
   p.kb_per_split = d.kbps;
   p.ncols_pad = d.ncols_pad;
-  p.nseg = d.nseg;
+  p.nsplit = d.nsplit;
   p.tmem_cols = d.tmem_cols;
   p.ws = d.tws;
   p.err = err;
@@ -736,14 +807,7 @@ __global__ void tcg_defect_to_y(const BDesc* D) {
 __global__ void tcg_c_to_planes(const BDesc* D) {
   const BDesc& d = D[blockIdx.y];
   if (d.flags[0] == 0) return;
-  const int64_t n = d.n, n_pad = d.n_pad, total = n_pad * n_pad;
-  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < total; e += (int64_t)gridDim.x * blockDim.x) {
-    int64_t i = e / n_pad, k = e % n_pad;
-    double2 v = (i < n && k < n) ? d.C[i * n + k] : make_double2(0.0, 0.0);
-    split_store(v.x, d.nsplit, d.Cp, 3 * (size_t)total, e);
-    split_store(v.y, d.nsplit, d.Cp + total, 3 * (size_t)total, e);
-    split_store(v.x + v.y, d.nsplit, d.Cp + 2 * total, 3 * (size_t)total, e);
-  }
+  c_to_planes_body(d.n, d.n_pad, d.C, d.n, d.Cp, d.nsplit);
 }
 
 }  // namespace
@@ -753,8 +817,6 @@ void tcg_geometry(int64_t n, int m, int* n_pad, int* ncols_pad, int* nchunk, int
   chunking(m, nchunks, nchunk);
   *ncols_pad = *nchunks * *nchunk;
 }
-
-int tcg_nseg(int nsplit) { return nseg_for(nsplit); }
 
 size_t tcg_smem_bytes(int nchunk_max) {
   return (size_t)STAGES * (3 * TM * TK * 2 + 3 * (size_t)nchunk_max * TK * 2) + 1024;
@@ -777,7 +839,7 @@ bool tcg_encode_maps(const BDesc& d, void* maps_host) {
 }
 
 void tcg_set_matrix(const BDesc* D, int np, int64_t npad2_max, cudaStream_t s) {
-  int blocks = (int)std::max<int64_t>(1, std::min<int64_t>((npad2_max + 255) / 256, 256));
+  int blocks = (int)std::max<int64_t>(1, std::min<int64_t>((npad2_max / 2 + 255) / 256, 512));
   tcg_c_to_planes<<<dim3(blocks, np), 256, 0, s>>>(D);
   LAUNCH_NOTE(1);
 }
@@ -792,7 +854,7 @@ cudaError_t tcg_prepare(int nchunk_max) {
 cudaError_t tcg_filter(const BDesc* D, const TcgShape& g, int* err, cudaStream_t s) {
   const size_t smem = tcg_smem_bytes(g.nchunk_max);
   dim3 tg((g.n_pad_max + 31) / 32, (g.ncols_pad_max + 31) / 32, g.np);
-  int eb = (int)std::max<int64_t>(1, std::min<int64_t>((g.nc_max + 255) / 256, 64));
+  int eb = (int)std::max<int64_t>(1, std::min<int64_t>((g.nc_max / 2 + 255) / 256, 128));
   tcg_resid_to_state<<<tg, 256, 0, s>>>(D);
   tcg_epilogue<<<dim3(eb, g.np), 256, 0, s>>>(D, 0);
   LAUNCH_NOTE(2);

@@ -279,7 +279,7 @@ struct BDesc {
   int* stepact;               // [kBDegMax] FP64 filter: step j runs for this problem
   const int* active;          // = flags
   // tensor-core filter state
-  int n_pad, ncols_pad, nchunk, nchunks, mtiles, ks, kbps, nseg;
+  int n_pad, ncols_pad, nchunk, nchunks, mtiles, ks, kbps;
   unsigned tmem_cols; int unit_start;
   const void* maps;           // 18 CUtensorMap (C pieces, then block pieces), 64-byte aligned
   __nv_bfloat16 *Cp, *Yp;
@@ -326,7 +326,6 @@ void cluster_jacobi_batched(const BDesc* D, int np, int zsel, double rel, int ma
 
 // grouped tensor-core filter (residual-corrected recurrence) over the problems of a batch
 void tcg_geometry(int64_t n, int m, int* n_pad, int* ncols_pad, int* nchunk, int* nchunks);
-int tcg_nseg(int nsplit);
 size_t tcg_smem_bytes(int nchunk_max);
 size_t tcg_map_bytes();                                  // bytes of one problem's tensor maps
 bool tcg_encode_maps(const BDesc& d, void* maps_host);   // host copy of d's maps (Cp, Yp set)
