@@ -45,6 +45,7 @@ inline size_t al256(size_t b) { return (b + 255) & ~(size_t)255; }
 
 constexpr int kNB = 24;        // doubles of per-problem bounds
 constexpr int kNF = 16;        // ints of per-problem flags
+constexpr int kLanes = 4;      // streams the k-points' emulated products are spread over
 constexpr int kBuckets = 8;    // size buckets of the degree autotuner (n / 512)
 
 enum CallClass { CC_REDUCE, CC_CQ, CC_GRAM, CC_TALL, CC_SMALL, CC_FINAL, CC_FILTER, CC_N };
@@ -120,28 +121,33 @@ struct BatchPlan {
   std::vector<int> bucket;
   int cap_bucket[kBuckets];
   // emulated products: residues of every k-point's L^-1 (rows; conjugated, the columns of
-  // L^-H), made once per call, plus one k-point's worth of scratch for tril(A) and T
+  // L^-H), made once per call
   int oz_S = 0;
   int oz_group = 0;   // moduli per group the operands are kept in (0: all of them)
   int oz_key = 0;   // reduce_slices the plan (and its captured round) was built for
   char* oz_mem = nullptr;
   std::vector<OzOperand> ozLA, ozLB;
-  OzOperand ozAB, ozTA;
-  char* oz_scratch = nullptr;
-  // W = C Q of every round: the residues of each k-point's C (made once per step) and one
-  // k-point's block (made per round, inside the captured round)
-  std::vector<OzOperand> ozC;
-  OzOperand ozQ;
+  // W = C Q of every round: the residues of each k-point's C (made once per step) and of its
+  // block (made per round, inside the captured round)
+  std::vector<OzOperand> ozC, ozQ;
   char* oz_cq = nullptr;
-  char* oz_qs = nullptr;   // the block's residues (inside oz_cq)
+  std::vector<char*> oz_qs;   // each block's residues (inside oz_cq)
+  // the round's other large products (Gram matrices, the triangular products, G = Q^H W, Q Z, W Z)
+  // emulated too: oz_round_worth
+  bool oz_round = false;
   // the final check's X = L^-H Q, A X, B X: residues of every k-point's L^-H (rows) and B
   // (rows), made once per call, and one k-point's A (per check)
   std::vector<OzOperand> ozLH, ozBd;
-  OzOperand ozAd;
   char* oz_fin = nullptr;
-  char* oz_ad = nullptr;   // A's residues (inside oz_fin)
-  char* oz_ws = nullptr;  // residues of one k-point's product
-  size_t oz_ws_bytes = 0;
+  // Lanes: the emulated products of one k-point leave most SMs idle where the block is narrow or the
+  // order small, and every one ends in a reconstruction and a launch gap, so the k-points take
+  // `lanes` streams in turn (lane 0 is the caller's), each with its own scratch: two n x n operands,
+  // two narrow ones and a product's residues.
+  int lanes = 1;
+  cudaStream_t lane_s[kLanes] = {};
+  cudaEvent_t lane_fork = nullptr, lane_done[kLanes] = {};
+  char* oz_lane = nullptr;
+  size_t lane_bytes = 0, lane_big = 0, lane_tall = 0, oz_ws_bytes = 0;
   int* oz_flags = nullptr;   // device: [0] kernel error code, [1] non-finite entry
   std::vector<cudaEvent_t> ev;
 };
@@ -154,7 +160,15 @@ void batch_release(BatchPlan* P) {
   if (P->oz_mem) cudaFree(P->oz_mem);
   if (P->oz_cq) cudaFree(P->oz_cq);
   if (P->oz_fin) cudaFree(P->oz_fin);
-  if (P->oz_ws) cudaFree(P->oz_ws);
+  for (int i = 0; i < kLanes; ++i) {
+    if (P->lane_s[i]) {
+      cudaStreamSynchronize(P->lane_s[i]);
+      cudaStreamDestroy(P->lane_s[i]);
+    }
+    if (P->lane_done[i]) cudaEventDestroy(P->lane_done[i]);
+  }
+  if (P->lane_fork) cudaEventDestroy(P->lane_fork);
+  if (P->oz_lane) cudaFree(P->oz_lane);
   if (P->hD) cudaFreeHost(P->hD);
   for (auto e : P->ev) cudaEventDestroy(e);
   delete P;
@@ -490,13 +504,86 @@ void launch(BatchPlan* P, int ci, cudaStream_t s, bool tune) {
   zgemm_grouped(P->pool + c.off, ni, c.total, c.tile, c.f, s);
 }
 
+// ---------------------------------------------------------------- lanes
+struct Lane {
+  cudaStream_t s;
+  char *big, *big2, *tall, *small, *ws;
+};
+Lane lane_of(BatchPlan* P, int k, cudaStream_t s) {
+  const int i = k % P->lanes;
+  char* p = P->oz_lane + (size_t)i * P->lane_bytes;
+  Lane l;
+  l.s = i == 0 ? s : P->lane_s[i];
+  l.big = p;
+  l.big2 = p + P->lane_big;
+  l.tall = l.big2 + P->lane_big;
+  l.small = l.tall + P->lane_tall;
+  l.ws = p + P->lane_bytes - P->oz_ws_bytes;
+  return l;
+}
+// f(k, lane) for every k-point, the lanes' streams forked from s and joined to it again (also when
+// f fails, so that nothing runs on behind the caller, and inside a capture)
+template <class F>
+cudaError_t over_lanes(BatchPlan* P, cudaStream_t s, F f) {
+  cudaError_t e = cudaSuccess;
+  auto also = [&](cudaError_t r) {
+    if (e == cudaSuccess) e = r;
+  };
+  if (P->lanes > 1) {
+    also(cudaEventRecord(P->lane_fork, s));
+    for (int i = 1; i < P->lanes; ++i) also(cudaStreamWaitEvent(P->lane_s[i], P->lane_fork, 0));
+  }
+  for (int k = 0; k < P->np && e == cudaSuccess; ++k) also(f(k, lane_of(P, k, s)));
+  if (P->lanes > 1)
+    for (int i = 1; i < P->lanes; ++i) {
+      also(cudaEventRecord(P->lane_done[i], P->lane_s[i]));
+      also(cudaStreamWaitEvent(s, P->lane_done[i], 0));
+    }
+  return e;
+}
+cudaError_t lane_split(BatchPlan* P, const Lane& l, OzOperand& op, char* mem, int rows, int K, const double2* X,
+                       int64_t ldx, int conj, int mask, bool cols, const int* active, const int* ks = nullptr,
+                       int sign = 0) {
+  return oz_split(op, mem, rows, K, X, ldx, conj, mask, P->oz_S, P->oz_flags + 1, l.s, cols, active, P->oz_group, ks,
+                  sign);
+}
+cudaError_t lane_gemm(BatchPlan* P, const Lane& l, const OzOperand& a, const OzOperand& b, int triA, int triB,
+                      double2* D, int64_t ldd, const int* active) {
+  return oz_gemm(a, b, triA, triB, D, ldd, P->oz_flags, l.s, active, l.ws, P->oz_ws_bytes);
+}
+// The round's products of all k-points, emulated or on the FP64 pipe. A grouped FP64 Gram matrix
+// takes 1.07 us a row of the largest order (one chain of K steps a tile) or its share of the pipe, the
+// emulated one four launches a k-point: 250 us for 8 k-points, n = 800 to 1900, m = 68 to 160, where
+// FP64 takes 2030 (the triangular product 230 and 1093 us). Whole calls of three steps, FP64 and
+// emulated: 8 k-points of 30-60: 33.8 and 37.3 ms, 80-120: 37.4 and 36.8, 200-300: 60.7 and 48.2; 16
+// of 100-200: 59.1 and 62.2; 32 of 150-250 (two steps): 57.1 and 69.8.
+bool oz_round_worth(const BatchPlan* P) {
+  double macs = 0.0;
+  for (int k = 0; k < P->np; ++k) macs += 0.5 * (double)P->n[k] * P->m[k] * P->m[k];
+  const double fp64 = std::max(1.07e-6 * (double)P->nmax, 8.0 * macs / 1.05e12);
+  return P->oz_S == 8 && fp64 > 60e-6 * ((P->np + P->lanes - 1) / P->lanes);
+}
+
 // ---------------------------------------------------------------- phases
-void enqueue_orth(BatchPlan* P, cudaStream_t s, bool tune) {
+cudaError_t enqueue_orth(BatchPlan* P, cudaStream_t s, bool tune) {
   const int np = P->np;
   const int64_t nm = P->nmax * P->mmax;
   const int src_idx[3] = {0, 1, 0};   // nm blocks: 0 Y1, 1 Y2, 2 Q
   for (int k = 0; k < 3; ++k) {
-    launch(P, P->c_gram[k], s, tune);
+    if (P->oz_round) {
+      cudaError_t e = over_lanes(P, s, [&](int j, const Lane& l) {
+        const BDesc& d = P->hD[j];
+        OzOperand& y = P->ozQ[j];
+        cudaError_t r = lane_split(P, l, y, P->oz_qs[j], d.m, d.n, k == 1 ? d.Y2 : d.Y1, d.m, 1, 0, true, d.flags);
+        if (r != cudaSuccess) return r;
+        OzOperand b = y;
+        b.conj = 0;
+        return lane_gemm(P, l, y, b, 0, 0, d.Gw, d.m, d.flags);
+      });
+      if (e != cudaSuccess) return e;
+    } else {
+      launch(P, P->c_gram[k], s, tune);
+    }
     // the first pass is shifted CholQR (always positive definite for cond(Y) up to about
     // 1/u), the two plain ones that follow restore orthonormality to FP64 rounding. The factor's
     // inverse with the column scaling in a cluster per problem (8 problems of m = 68..160: 0.36 ms a
@@ -509,23 +596,48 @@ void enqueue_orth(BatchPlan* P, cudaStream_t s, bool tune) {
       bk_trtri_small(P->dD, np, s);
       bk_col_scale(P->dD, np, nm, src_idx[k], s);
     }
-    launch(P, P->c_apply[k], s, tune);
+    if (P->oz_round) {
+      // Y Li^H; the columns' exponents move from Y, whose columns may differ much in length (the rows
+      // are scaled as a whole), to Li, whose rows then have theirs taken out again
+      cudaError_t e = over_lanes(P, s, [&](int j, const Lane& l) {
+        const BDesc& d = P->hD[j];
+        const double2* src = k == 1 ? d.Y2 : d.Y1;
+        double2* dst = k == 0 ? d.Y2 : (k == 1 ? d.Y1 : d.Q);
+        const int* ex = P->ozQ[j].ex;
+        OzOperand y, li;
+        cudaError_t r = lane_split(P, l, y, l.tall, d.n, d.m, src, d.m, 0, 0, false, d.flags, ex, -1);
+        if (r == cudaSuccess) r = lane_split(P, l, li, l.small, d.m, d.m, d.Gwi, d.m, 1, 2, false, d.flags, ex, 1);
+        return r == cudaSuccess ? lane_gemm(P, l, y, li, 0, 2, dst, d.m, d.flags) : r;
+      });
+      if (e != cudaSuccess) return e;
+    } else {
+      launch(P, P->c_apply[k], s, tune);
+    }
   }
+  return cudaGetLastError();
 }
 
-void enqueue_rr(BatchPlan* P, cudaStream_t s, bool tune) {
+cudaError_t enqueue_rr(BatchPlan* P, cudaStream_t s, bool tune) {
   const int np = P->np, mmax = P->mmax;
   if (P->oz_S > 0 && (int)P->ozC.size() == np) {
-    // W = C Q emulated per k-point; a converged k-point's launches do nothing
-    for (int k = 0; k < np; ++k) {
+    // W = C Q emulated per k-point (a converged k-point's launches do nothing), and G = Q^H W with
+    // the block's residues again
+    cudaError_t e = over_lanes(P, s, [&](int k, const Lane& l) {
       const BDesc& d = P->hD[k];
-      oz_split(P->ozQ, P->oz_qs, d.m, d.n, d.Q, d.m, 0, 0, P->oz_S, P->oz_flags + 1, s, true, d.flags, P->oz_group);
-      oz_gemm(P->ozC[k], P->ozQ, 0, 0, d.Wt, d.m, P->oz_flags, s, d.flags, P->oz_ws, P->oz_ws_bytes);
-    }
+      OzOperand& q = P->ozQ[k];
+      cudaError_t r = lane_split(P, l, q, P->oz_qs[k], d.m, d.n, d.Q, d.m, 0, 0, true, d.flags);
+      if (r == cudaSuccess) r = lane_gemm(P, l, P->ozC[k], q, 0, 0, d.Wt, d.m, d.flags);
+      if (!P->oz_round || r != cudaSuccess) return r;
+      OzOperand qh = q, w;
+      qh.conj = 1;
+      r = lane_split(P, l, w, l.tall, d.m, d.n, d.Wt, d.m, 0, 0, true, d.flags);
+      return r == cudaSuccess ? lane_gemm(P, l, qh, w, 0, 0, d.G, d.m, d.flags) : r;
+    });
+    if (e != cudaSuccess) return e;
   } else {
     launch(P, P->c_wt, s, tune);
   }
-  launch(P, P->c_g, s, tune);
+  if (!P->oz_round) launch(P, P->c_g, s, tune);
   bk_heev_prep(P->dD, np, mmax, s);
   for (int it = 0; it <= P->refine; ++it) {
     const int par = it & 1;
@@ -542,10 +654,26 @@ void enqueue_rr(BatchPlan* P, cudaStream_t s, bool tune) {
   bk_hermitize_avg_S(P->dD, np, mmax, s);
   cluster_jacobi_batched(P->dD, np, zsel, 1e-15, 12, s);
   bk_sort_pairs(P->dD, np, zsel, s);
-  launch(P, P->c_qz, s, tune);
-  bk_copy_nm(P->dD, np, P->nmax * mmax, 0, 2, s);   // Q <- Y1
-  launch(P, P->c_wz, s, tune);
+  if (P->oz_round) {
+    // Q <- Q Z, W = W' Z
+    cudaError_t e = over_lanes(P, s, [&](int k, const Lane& l) {
+      const BDesc& d = P->hD[k];
+      OzOperand x, z;
+      cudaError_t r = lane_split(P, l, z, l.small, d.m, d.m, d.Zs, d.m, 0, 0, true, d.flags);
+      if (r == cudaSuccess) r = lane_split(P, l, x, l.tall, d.n, d.m, d.Wt, d.m, 0, 0, false, d.flags);
+      if (r == cudaSuccess) r = lane_gemm(P, l, x, z, 0, 0, d.W, d.m, d.flags);
+      if (r == cudaSuccess) r = lane_split(P, l, x, l.tall, d.n, d.m, d.Q, d.m, 0, 0, false, d.flags);
+      return r == cudaSuccess ? lane_gemm(P, l, x, z, 0, 0, d.Y1, d.m, d.flags) : r;
+    });
+    if (e != cudaSuccess) return e;
+    bk_copy_nm(P->dD, np, P->nmax * mmax, 0, 2, s);   // Q <- Y1
+  } else {
+    launch(P, P->c_qz, s, tune);
+    bk_copy_nm(P->dD, np, P->nmax * mmax, 0, 2, s);   // Q <- Y1
+    launch(P, P->c_wz, s, tune);
+  }
   bk_resid(P->dD, np, mmax, s);
+  return cudaGetLastError();
 }
 
 cudaError_t enqueue_filter(BatchPlan* P, cudaStream_t s, bool tune, int deg_min) {
@@ -742,43 +870,72 @@ extern "C" gevp_status gevp_solve_batched(gevp_handle h, int nk, int nsteps, con
   BCK(cudaEventRecord(evt(P, EV_T0), s));
 
   // memory of the emulated products (o.reduce_slices digits per entry): the L^-1 operands of
-  // every k-point and a scratch pair (the factorisations below use the front of it before the
-  // L^-1 operands are written there); the C operands and one block; the final check's; the
-  // residues of a product. All moduli at once, or groups of four when that cannot be had.
+  // every k-point; the C operands and the blocks; the final check's (the factorisations below use
+  // a k-point's part of those before they are written); the lanes' scratch. All moduli at once, or
+  // groups of four when that cannot be had.
   P->oz_S = P->nmax <= 30720 ? P->oz_key : 0;
   if (P->oz_S > 0 && !P->oz_mem) {
     // (kept while the plan is: the captured round holds these addresses)
     const int S = P->oz_S;
-    for (int group : {0, 4}) {
-      size_t mem = 256, scratch = 0, cq = 256, qs = 0, fb = 256, ab = 0, ws = 0;
+    cudaError_t e = cudaSuccess;
+    for (int form = 0; form < 3; ++form) {
+      // all moduli at once, with lanes and without; then groups of four
+      const int group = form < 2 ? 0 : 4, lanes = form == 0 ? std::min(kLanes, np) : 1;
+      if (form == 1 && np == 1) continue;
+      size_t mem = 256, cq = 256, fb = 256, big = 0, tall = 0, small = 0, ws = 0;
       for (int k = 0; k < np; ++k) {
         const int nk_ = (int)n[k];
-        const size_t b = oz_operand_bytes(nk_, nk_, S, group);
+        const size_t b = al256(oz_operand_bytes(nk_, nk_, S, group));
         mem += b;
-        scratch = std::max(scratch, 2 * b);
-        cq += b;
-        qs = std::max(qs, oz_operand_bytes(m[k], nk_, S, group));
+        cq += b + al256(oz_operand_bytes(m[k], nk_, S, group));
         fb += 2 * b;
-        ab = std::max(ab, b);
+        big = std::max(big, b);
+        tall = std::max(tall, al256(std::max(oz_operand_bytes(m[k], nk_, S, group),
+                                             oz_operand_bytes(nk_, m[k], S, group))));
+        small = std::max(small, al256(oz_operand_bytes(m[k], m[k], S, group)));
         ws = std::max(ws, std::max(oz_work_bytes(256, nk_, nk_, S),
                                    std::min<size_t>(oz_work_bytes(nk_, nk_, nk_, S), (size_t)1 << 30)));
       }
-      cudaError_t e = cudaMalloc(&P->oz_mem, mem + scratch);
-      if (e == cudaSuccess) e = cudaMalloc(&P->oz_cq, cq + qs);
-      if (e == cudaSuccess) e = cudaMalloc(&P->oz_fin, fb + ab);
-      if (e == cudaSuccess) e = cudaMalloc(&P->oz_ws, ws);
+      ws = al256(ws);
+      const size_t lane = 2 * big + tall + small + ws;
+      e = cudaMalloc(&P->oz_mem, mem);
+      if (e == cudaSuccess) e = cudaMalloc(&P->oz_cq, cq);
+      if (e == cudaSuccess) e = cudaMalloc(&P->oz_fin, fb);
+      if (e == cudaSuccess) e = cudaMalloc(&P->oz_lane, lanes * lane);
       if (e == cudaSuccess) {
         P->oz_group = group;
-        P->oz_qs = P->oz_cq + cq;
+        P->lanes = lanes;
+        P->lane_bytes = lane;
+        P->lane_big = big;
+        P->lane_tall = tall;
         P->oz_ws_bytes = ws;
         break;
       }
-      for (char** q : {&P->oz_mem, &P->oz_cq, &P->oz_fin, &P->oz_ws}) {
+      for (char** q : {&P->oz_mem, &P->oz_cq, &P->oz_fin, &P->oz_lane}) {
         if (*q) cudaFree(*q);
         *q = nullptr;
       }
       cudaGetLastError();
-      if (group != 0 || e != cudaErrorMemoryAllocation) return fail(e, "operands of the emulated products");
+      if (e != cudaErrorMemoryAllocation) break;
+    }
+    if (e != cudaSuccess) return fail(e, "operands of the emulated products");
+    // a lane whose stream cannot be had is left out
+    int prio = 0;
+    if (cudaStreamGetPriority(s, &prio) != cudaSuccess) prio = 0;
+    if (P->lanes > 1 && cudaEventCreateWithFlags(&P->lane_fork, cudaEventDisableTiming) != cudaSuccess) P->lanes = 1;
+    for (int i = 1; i < P->lanes; ++i)
+      if (cudaStreamCreateWithPriority(&P->lane_s[i], cudaStreamNonBlocking, prio) != cudaSuccess ||
+          cudaEventCreateWithFlags(&P->lane_done[i], cudaEventDisableTiming) != cudaSuccess)
+        P->lanes = i;
+    cudaGetLastError();
+    P->oz_round = oz_round_worth(P);
+    P->ozQ.assign(np, OzOperand{});
+    P->oz_qs.assign(np, nullptr);
+    char* q = P->oz_cq;
+    for (int k = 0; k < np; ++k) q += al256(oz_operand_bytes((int)n[k], (int)n[k], S, P->oz_group));
+    for (int k = 0; k < np; ++k) {
+      P->oz_qs[k] = q;
+      q += al256(oz_operand_bytes(m[k], (int)n[k], S, P->oz_group));
     }
   }
   if (P->oz_S > 0) {
@@ -789,30 +946,42 @@ extern "C" gevp_status gevp_solve_batched(gevp_handle h, int nk, int nsteps, con
   // ---- Cholesky of every B_k (sequence-invariant): recursive with emulated off-diagonal
   // products when the products are emulated, else blocked on the FP64 pipe
   BCK(cudaMemsetAsync(P->dInfo, 0, np * sizeof(int), s));
-  for (int k = 0; k < np; ++k) {
-    BDesc& d = P->hD[k];
-    zcopy2d(n[k], n[k], (const double2*)B[k], ldb[k], d.L, n[k], s);
-    cudaError_t ce = cudaErrorNotSupported;
-    if (P->oz_S > 0) {
+  std::vector<char> factored(np, 0);
+  if (P->oz_S > 0) {
+    // the chain of leaves of one matrix leaves most SMs idle: 8 orders of 800 to 1900 take 17 ms
+    // over four lanes, 42 one after another
+    std::vector<char*> at(np);
+    char* f = P->oz_fin;
+    for (int k = 0; k < np; ++k) {
+      at[k] = f;
+      f += 2 * al256(oz_operand_bytes((int)n[k], (int)n[k], P->oz_S, P->oz_group));
+    }
+    BCK(over_lanes(P, s, [&](int k, const Lane& l) {
+      const BDesc& d = P->hD[k];
+      zcopy2d(n[k], n[k], (const double2*)B[k], ldb[k], d.L, n[k], l.s);
       CholRes r{};
-      r.memA = P->oz_mem + 256;
-      r.memB = r.memA + oz_operand_bytes((int)n[k], (int)n[k], P->oz_S, P->oz_group);
+      r.memA = at[k];
+      r.memB = r.memA + al256(oz_operand_bytes((int)n[k], (int)n[k], P->oz_S, P->oz_group));
       r.T = d.T;
       r.ldt = n[k];
-      r.ws = P->oz_ws;
+      r.ws = l.ws;
       r.ws_bytes = P->oz_ws_bytes;
       r.group = P->oz_group;
       r.flags = P->oz_flags;
       r.info = P->dInfo + k;
       r.S = P->oz_S;
-      r.s = s;
-      ce = chol_recursive(n[k], d.L, n[k], d.Linv, n[k], r);
-      if (ce != cudaSuccess && ce != cudaErrorNotSupported) return fail(ce, "chol_recursive");
-    }
-    if (ce == cudaErrorNotSupported) {
-      potrf_lower(n[k], d.L, n[k], P->dInfo + k, d.Linv, n[k], s);
-      trtri_lower(n[k], d.L, n[k], d.Linv, n[k], P->trtri_ws, P->trtri_elems, s, true);
-    }
+      r.s = l.s;
+      const cudaError_t ce = chol_recursive(n[k], d.L, n[k], d.Linv, n[k], r);
+      factored[k] = ce == cudaSuccess;
+      return ce == cudaErrorNotSupported ? cudaSuccess : ce;
+    }));
+  }
+  for (int k = 0; k < np; ++k) {
+    if (factored[k]) continue;
+    const BDesc& d = P->hD[k];
+    zcopy2d(n[k], n[k], (const double2*)B[k], ldb[k], d.L, n[k], s);
+    potrf_lower(n[k], d.L, n[k], P->dInfo + k, d.Linv, n[k], s);
+    trtri_lower(n[k], d.L, n[k], d.Linv, n[k], P->trtri_ws, P->trtri_elems, s, true);
   }
   BCK(cudaMemcpyAsync(P->hInfo, P->dInfo, np * sizeof(int), cudaMemcpyDeviceToHost, s));
   BCK(cudaEventRecord(evt(P, EV_CHOL), s));
@@ -835,9 +1004,8 @@ extern "C" gevp_status gevp_solve_batched(gevp_handle h, int nk, int nsteps, con
       BCK(oz_split(P->ozLA[k], q, nk_, nk_, d.Linv, n[k], 0, 2, S, P->oz_flags + 1, s, false, nullptr, P->oz_group));
       P->ozLB[k] = P->ozLA[k];
       P->ozLB[k].conj = 1;
-      q += oz_operand_bytes(nk_, nk_, S, P->oz_group);
+      q += al256(oz_operand_bytes(nk_, nk_, S, P->oz_group));
     }
-    P->oz_scratch = q;
     P->ozC.assign(np, OzOperand{});
     P->ozLH.assign(np, OzOperand{});
     P->ozBd.assign(np, OzOperand{});
@@ -847,12 +1015,11 @@ extern "C" gevp_status gevp_solve_batched(gevp_handle h, int nk, int nsteps, con
       const int nk_ = (int)n[k];
       // rows of L^-H (upper) = conjugated columns of L^-1
       BCK(oz_split(P->ozLH[k], f, nk_, nk_, d.Linv, n[k], 1, 3, S, P->oz_flags + 1, s, true, nullptr, P->oz_group));
-      f += oz_operand_bytes(nk_, nk_, S, P->oz_group);
+      f += al256(oz_operand_bytes(nk_, nk_, S, P->oz_group));
       BCK(oz_split(P->ozBd[k], f, nk_, nk_, (const double2*)B[k], ldb[k], 0, 0, S, P->oz_flags + 1, s, false, nullptr,
                    P->oz_group));
-      f += oz_operand_bytes(nk_, nk_, S, P->oz_group);
+      f += al256(oz_operand_bytes(nk_, nk_, S, P->oz_group));
     }
-    P->oz_ad = f;
   }
   float ms = 0.f;
   cudaEventElapsedTime(&ms, evt(P, EV_T0), evt(P, EV_CHOL));
@@ -913,16 +1080,15 @@ extern "C" gevp_status gevp_solve_batched(gevp_handle h, int nk, int nsteps, con
     // ---- reduction C = L^-1 A L^-H for every k-point
     if (P->oz_S > 0) {
       // emulated: T = L^-1 tril_half(A), M = T L^-H per k-point (each product fills the GPU)
-      for (int k = 0; k < np; ++k) {
+      BCK(over_lanes(P, s, [&](int k, const Lane& l) {
         const BDesc& d = P->hD[k];
-        const int nk_ = (int)n[k], S = P->oz_S;
-        char* base = P->oz_scratch;
-        BCK(oz_split(P->ozAB, base, nk_, nk_, d.A, d.lda, 1, 1, S, P->oz_flags + 1, s, false, nullptr, P->oz_group));
-        BCK(oz_gemm(P->ozLA[k], P->ozAB, 1, 1, d.T, n[k], P->oz_flags, s, nullptr, P->oz_ws, P->oz_ws_bytes));
-        BCK(oz_split(P->ozTA, base + oz_operand_bytes(nk_, nk_, S, P->oz_group), nk_, nk_, d.T, n[k], 0, 2, S,
-                     P->oz_flags + 1, s, false, nullptr, P->oz_group));
-        BCK(oz_gemm(P->ozTA, P->ozLB[k], 1, 2, d.C, n[k], P->oz_flags, s, nullptr, P->oz_ws, P->oz_ws_bytes));
-      }
+        const int nk_ = (int)n[k];
+        OzOperand ab, ta;
+        cudaError_t r = lane_split(P, l, ab, l.big, nk_, nk_, d.A, d.lda, 1, 1, false, nullptr);
+        if (r == cudaSuccess) r = lane_gemm(P, l, P->ozLA[k], ab, 1, 1, d.T, n[k], nullptr);
+        if (r == cudaSuccess) r = lane_split(P, l, ta, l.big2, nk_, nk_, d.T, n[k], 0, 2, false, nullptr);
+        return r == cudaSuccess ? lane_gemm(P, l, ta, P->ozLB[k], 1, 2, d.C, n[k], nullptr) : r;
+      }));
     } else {
       launch(P, P->c_red1, s, tune);
       launch(P, P->c_red2, s, tune);
@@ -935,7 +1101,7 @@ extern "C" gevp_status gevp_solve_batched(gevp_handle h, int nk, int nsteps, con
         const BDesc& d = P->hD[k];
         BCK(oz_split(P->ozC[k], q, (int)n[k], (int)n[k], d.C, n[k], 0, 0, P->oz_S, P->oz_flags + 1, s, false, nullptr,
                      P->oz_group));
-        q += oz_operand_bytes((int)n[k], (int)n[k], P->oz_S, P->oz_group);
+        q += al256(oz_operand_bytes((int)n[k], (int)n[k], P->oz_S, P->oz_group));
       }
     }
     BCK(cudaEventRecord(evt(P, EV_RED), s));
@@ -951,9 +1117,9 @@ extern "C" gevp_status gevp_solve_batched(gevp_handle h, int nk, int nsteps, con
       bk_randn(P->dD, np, nm_max, o.seed * 1000003ull + (uint64_t)l, nullptr, s);
       if (l == 0 && !xcall.items.empty())
         zgemm_grouped(P->pool + xcall.off, (int)xcall.items.size(), xcall.total, xcall.tile, xcall.f, s);
-      enqueue_orth(P, s, tune);
+      BCK(enqueue_orth(P, s, tune));
     }
-    enqueue_rr(P, s, tune);
+    BCK(enqueue_rr(P, s, tune));
     enqueue_status(P, s);
     BCK(cudaEventRecord(evt(P, EV_BND), s));
     BCK(cudaGetLastError());
@@ -975,8 +1141,8 @@ extern "C" gevp_status gevp_solve_batched(gevp_handle h, int nk, int nsteps, con
         // blocks (the others only repeat an orthonormalisation of orthonormal columns)
         BCK(cudaMemcpyAsync(P->dMask, P->hMask, np * sizeof(int), cudaMemcpyHostToDevice, s));
         bk_randn(P->dD, np, nm_max, o.seed * 7777ull + 131ull * rounds + l, P->dMask, s);
-        enqueue_orth(P, s, false);
-        enqueue_rr(P, s, false);
+        BCK(enqueue_orth(P, s, false));
+        BCK(enqueue_rr(P, s, false));
         enqueue_status(P, s);
         BCK(cudaStreamSynchronize(s));
         bs->orth_fallbacks++;
@@ -988,19 +1154,17 @@ extern "C" gevp_status gevp_solve_batched(gevp_handle h, int nk, int nsteps, con
         BCK(cudaEventRecord(evt(P, EV_FIN0), s));
         if (P->oz_S > 0 && (int)P->ozLH.size() == np) {
           // emulated per k-point; launches of k-points without a pending check do nothing
-          const int S = P->oz_S;
-          for (int k = 0; k < np; ++k) {
+          BCK(over_lanes(P, s, [&](int k, const Lane& l) {
             const BDesc& d = P->hD[k];
             const int* fin = d.flags + 12;
-            BCK(oz_split(P->ozQ, P->oz_qs, d.nev, d.n, d.Q, d.m, 0, 0, S, P->oz_flags + 1, s, true, fin, P->oz_group));
-            BCK(oz_gemm(P->ozLH[k], P->ozQ, 2, 0, d.Xf, d.m, P->oz_flags, s, fin, P->oz_ws, P->oz_ws_bytes));
-            BCK(oz_split(P->ozAd, P->oz_ad, d.n, d.n, d.A, d.lda, 0, 0, S, P->oz_flags + 1, s, false, fin,
-                         P->oz_group));
-            BCK(oz_split(P->ozQ, P->oz_qs, d.nev, d.n, d.Xf, d.m, 0, 0, S, P->oz_flags + 1, s, true, fin,
-                         P->oz_group));
-            BCK(oz_gemm(P->ozAd, P->ozQ, 0, 0, d.Y1, d.m, P->oz_flags, s, fin, P->oz_ws, P->oz_ws_bytes));
-            BCK(oz_gemm(P->ozBd[k], P->ozQ, 0, 0, d.Y2, d.m, P->oz_flags, s, fin, P->oz_ws, P->oz_ws_bytes));
-          }
+            OzOperand q, a;
+            cudaError_t r = lane_split(P, l, q, l.tall, d.nev, d.n, d.Q, d.m, 0, 0, true, fin);
+            if (r == cudaSuccess) r = lane_gemm(P, l, P->ozLH[k], q, 2, 0, d.Xf, d.m, fin);
+            if (r == cudaSuccess) r = lane_split(P, l, a, l.big, d.n, d.n, d.A, d.lda, 0, 0, false, fin);
+            if (r == cudaSuccess) r = lane_split(P, l, q, l.tall, d.nev, d.n, d.Xf, d.m, 0, 0, true, fin);
+            if (r == cudaSuccess) r = lane_gemm(P, l, a, q, 0, 0, d.Y1, d.m, fin);
+            return r == cudaSuccess ? lane_gemm(P, l, P->ozBd[k], q, 0, 0, d.Y2, d.m, fin) : r;
+          }));
         } else {
           launch(P, P->c_xf, s, tune);
           launch(P, P->c_ax, s, tune);
@@ -1041,8 +1205,8 @@ extern "C" gevp_status gevp_solve_batched(gevp_handle h, int nk, int nsteps, con
         cudaError_t fe = enqueue_filter(P, s, tr_tune, o.deg_min);
         if (fe != cudaSuccess) return fail(fe, "batched filter launch");
         BCK(cudaEventRecord(evt(P, EV_F1), s));
-        enqueue_orth(P, s, tr_tune);
-        enqueue_rr(P, s, tr_tune);
+        BCK(enqueue_orth(P, s, tr_tune));
+        BCK(enqueue_rr(P, s, tr_tune));
         enqueue_status(P, s);
         BCK(cudaEventRecord(evt(P, EV_END), s));
         BCK(cudaStreamSynchronize(s));
@@ -1065,8 +1229,8 @@ extern "C" gevp_status gevp_solve_batched(gevp_handle h, int nk, int nsteps, con
         cudaError_t ce = cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal);
         if (ce == cudaSuccess) {
           cudaError_t fe = enqueue_filter(P, cs, false, o.deg_min);
-          enqueue_orth(P, cs, false);
-          enqueue_rr(P, cs, false);
+          if (fe == cudaSuccess) fe = enqueue_orth(P, cs, false);
+          if (fe == cudaSuccess) fe = enqueue_rr(P, cs, false);
           enqueue_status(P, cs);
           ce = cudaStreamEndCapture(cs, &P->graph);
           if (fe != cudaSuccess) ce = fe;
