@@ -772,7 +772,14 @@ __global__ void b_round_status(const BDesc* D, int* out) {
     d.flags[4] += 1;
     d.bounds[18] = mx;
     if (info) d.flags[8] += 1;
-    if (!info && mx <= d.bounds[6]) {
+    // no finite bound of C (a NaN or Inf in A): neither rounds nor restarts help
+    const bool lost = !(d.bounds[7] < 1e300);
+    if (lost) {
+      d.flags[0] = 0;
+      d.flags[3] = 1;
+      d.flags[12] = 1;
+      d.flags[11] = max(d.flags[11], 2);
+    } else if (!info && mx <= d.bounds[6]) {
       d.flags[3] = 1;
       d.flags[0] = 0;
       d.flags[12] = 1;
@@ -790,7 +797,7 @@ __global__ void b_round_status(const BDesc* D, int* out) {
       }
     }
     d.bounds[8] = mx;
-    out[p] = d.flags[0] | (info ? 2 : 0);
+    out[p] = d.flags[0] | (info && !lost ? 2 : 0);
   }
 }
 
@@ -811,6 +818,7 @@ __global__ void b_randn(const BDesc* D, uint64_t seed, const int* mask) {
   const int p = blockIdx.y;
   const BDesc& d = D[p];
   if (mask ? mask[p] == 0 : !live(d)) return;
+  if (mask && blockIdx.x == 0 && threadIdx.x == 0) d.flags[2] = 0;   // the restart's factorisation decides anew
   const int64_t total = (int64_t)d.n * d.m;
   const uint64_t sd = seed ^ (0xD1B54A32D192ED03ull * (uint64_t)(p + 1));
   for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < total; e += (int64_t)gridDim.x * blockDim.x) {
