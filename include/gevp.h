@@ -188,7 +188,8 @@ typedef struct {
   int orth_fallbacks;   /* CholQR breakdowns repaired by a random restart              */
   int final_passes;     /* original-space checks, summed over problems and steps        */
   int converged;        /* 1 if every residual of every problem <= tol                 */
-  int tile[8];          /* autotuner: grouped FP64 GEMM tile chosen per call class      */
+  int tile[8];          /* autotuner: grouped FP64 GEMM tile chosen per call class (0:  */
+                        /* 4 x 8, or no such call)                                      */
   int deg_cap[8];       /* autotuner: filter degree cap per size bucket (last step)     */
   double max_resid;
   double flops_fp64, flops_lowp;   /* executed-flop model                              */

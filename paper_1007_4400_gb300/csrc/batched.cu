@@ -20,8 +20,8 @@
 // final residuals in the original space (re-opening a problem with a tighter tolerance
 // and the FP64 filter if they miss tol).
 //
-// Autotuner: (1) every grouped GEMM call of a new batch shape is timed with 32 x 32 and
-// 64 x 64 tiles on its first execution and keeps the faster; (2) after each step the
+// Autotuner: (1) every grouped GEMM call of a new batch shape is timed with 4 x 8,
+// 32 x 32 and 64 x 64 tiles on its first execution and keeps the fastest; (2) after each step the
 // filter degree cap of every size bucket is set by minimising the modelled time of the
 // next step, R (T_rest + sum_b d_b T_step share_b), over the number of rounds R, where
 // d_b(R) is the degree at which the Chebyshev factor rho_b of the bucket's slowest wanted
@@ -476,7 +476,7 @@ cudaEvent_t evt(BatchPlan* P, size_t i) {
   return P->ev[i];
 }
 
-// one grouped GEMM call; on its first run for a new shape both tiles are timed
+// one grouped GEMM call; on its first run for a new shape the tiles are timed
 void launch(BatchPlan* P, int ci, cudaStream_t s, bool tune) {
   GCall& c = P->calls[ci];
   const int ni = (int)c.items.size();
@@ -484,7 +484,7 @@ void launch(BatchPlan* P, int ci, cudaStream_t s, bool tune) {
   if (tune && !c.tuned) {
     float best = 1e30f;
     int best_tile = c.tile;
-    for (int t : {32, 64}) {
+    for (int t : {0, 32, 64}) {
       std::vector<ZgemmItem> tmp = c.items;
       int tot = zgemm_group_layout(tmp.data(), ni, t);
       cudaMemcpyAsync(P->tune_pool, tmp.data(), ni * sizeof(ZgemmItem), cudaMemcpyHostToDevice, s);

@@ -45,6 +45,7 @@
 //   memory with the factor's output: every CTA reads its rows of W before the first cluster
 //   barrier and writes the factor after it.
 #include "gevp_internal.cuh"
+#include "zsmall.cuh"
 #include <cooperative_groups.h>
 #include <algorithm>
 
@@ -108,6 +109,21 @@ __global__ void __launch_bounds__(256) zgram_kernel(int64_t n, int mx, int my, c
     G[(int64_t)i * ldg + j] = acc;
     G[(int64_t)j * ldg + i] = zconj(acc);
   }
+}
+
+// the same for short columns, on 4 x 8 tiles (zsmall.cuh)
+__global__ void __launch_bounds__(ZS_THREADS) zgram_small_kernel(int n, int mx, int my, const double2* __restrict__ X,
+                                                                 int64_t ldx, const double2* __restrict__ Y,
+                                                                 int64_t ldy, double2* G, int64_t ldg, int herm) {
+  __shared__ double part[ZS_WARPS][64];
+  const int m0 = blockIdx.y * ZS_M, n0 = blockIdx.x * ZS_N;
+  if (herm && n0 > m0 + ZS_M - 1) return;
+  const double v = zsmall_tile<1, 0>(mx, my, X, ldx, Y, ldy, 0, m0, n0, 0, n, part);
+  const int lane = threadIdx.x % 32, comp = threadIdx.x / 32;
+  const int i = m0 + lane / ZS_N, j = n0 + lane % ZS_N;
+  if (comp > 1 || i >= mx || j >= my || (herm && j > i)) return;
+  ((double*)(G + (int64_t)i * ldg + j))[comp] = herm && i == j && comp ? 0.0 : v;
+  if (herm && j < i) ((double*)(G + (int64_t)j * ldg + i))[comp] = comp ? -v : v;
 }
 
 constexpr int CT = 256;          // threads per cholinv CTA
@@ -596,7 +612,16 @@ void zgram(int64_t n, int mx, int my, const double2* X, int64_t ldx, const doubl
   slices = n > 0 ? (n + per - 1) / per : 1;
   dim3 grid((unsigned)tiles, (unsigned)slices);
   void* kt0 = kt_enabled() ? kt_begin(s) : nullptr;
-  zgram_kernel<<<grid, GT * GT, 0, s>>>(n, mx, my, X, ldx, Y, ldy, G, ldg, herm, ntj, (int)slices, per, part, cnt);
+  // 4 x 8 tiles where the busiest SM's share of them is the smaller (slices: a second pass over the
+  // partials)
+  const int64_t tm = (mx + ZS_M - 1) / ZS_M, tn = (my + ZS_N - 1) / ZS_N;
+  const double small = std::ceil((double)(herm ? tm * tn / 2 + std::min(tm, tn) : tm * tn) / kSMs) *
+                       (ZS_M * ZS_N * (double)n + kZsOverhead);
+  const double large = std::ceil((double)(active * slices) / kSMs) * (GT * GT * (double)per) +
+                       (slices > 1 ? 2.0 * kZsOverhead : 0.0);
+  if (n > 0 && small < large && tm <= 65535)
+    zgram_small_kernel<<<dim3((unsigned)tn, (unsigned)tm), ZS_THREADS, 0, s>>>((int)n, mx, my, X, ldx, Y, ldy, G, ldg, herm);
+  else zgram_kernel<<<grid, GT * GT, 0, s>>>(n, mx, my, X, ldx, Y, ldy, G, ldg, herm, ntj, (int)slices, per, part, cnt);
   LAUNCH_NOTE(1);
   if (kt0) {
     // work: 8 flop per complex multiply-add of the tiles formed (16 x 16 granularity)

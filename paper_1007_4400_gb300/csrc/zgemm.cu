@@ -4,6 +4,7 @@
 // every one of the 152 SMs is busy, which the host-side tiling choice below arranges
 // (tile size and split-K picked so that the grid covers the SMs in full waves).
 #include "gevp_internal.cuh"
+#include "zsmall.cuh"
 #include <algorithm>
 #include <cmath>
 
@@ -137,6 +138,27 @@ zgemm_kernel(ZgemmArgs p, double2* ws) {
   }
 }
 
+// the same on 4 x 8 tiles (zsmall.cuh), without split-K
+__global__ void __launch_bounds__(ZS_THREADS) zgemm_small_kernel(ZgemmArgs p) {
+  __shared__ double part[ZS_WARPS][64];
+  const int m0 = blockIdx.y * ZS_M, n0 = blockIdx.x * ZS_N, b = blockIdx.z;
+  if (p.triD == 1 && n0 > m0 + ZS_M - 1) return;
+  int kb = 0, ke = p.K;
+  if (p.triA == 1) ke = min(ke, m0 + ZS_M);
+  if (p.triA == 2) kb = max(kb, m0);
+  if (p.triB == 1 || p.maskB) kb = max(kb, n0);
+  if (p.triB == 2) ke = min(ke, n0 + ZS_N);
+  double v = zsmall_tile(p.opA, p.opB, p.M, p.N, p.A + (int64_t)b * p.sA, p.lda, p.B + (int64_t)b * p.sB, p.ldb,
+                         p.maskB, m0, n0, kb, ke, part);
+  const int lane = threadIdx.x % 32, comp = threadIdx.x / 32;
+  const int gm = m0 + lane / ZS_N, gn = n0 + lane % ZS_N;
+  if (comp > 1 || gm >= p.M || gn >= p.N) return;
+  v *= p.alpha;
+  if (p.Cin) v = fma(p.beta, ((const double*)(p.Cin + (int64_t)b * p.sC + (int64_t)gm * p.ldc + gn))[comp], v);
+  if (p.Ein) v = fma(p.gamma, ((const double*)(p.Ein + (int64_t)b * p.sE + (int64_t)gm * p.lde + gn))[comp], v);
+  ((double*)(p.D + (int64_t)b * p.sD + (int64_t)gm * p.ldd + gn))[comp] = v;
+}
+
 // Sum the k-slices in a fixed order (deterministic) and apply the epilogue.
 __global__ void zgemm_reduce_kernel(ZgemmArgs p, const double2* ws, int BM, int BN) {
   int64_t total = (int64_t)p.M * p.N;
@@ -191,7 +213,8 @@ void zgemm(const ZgemmArgs& in, double2* split_ws, size_t split_ws_elems, cudaSt
   // Every SM has the same (slow) FP64 pipe, so time ~ the busiest SM's share of FMAs.
   // For each tile size (64, 32, 16) and split-K factor, estimate
   //   waves = ceil(active_tiles * ksplit / SMs),  cost = waves * bm * bn * (K / ksplit)
-  // and take the cheapest (ties to larger tiles, which cost fewer shared-memory reads).
+  // and take the cheapest (ties to larger tiles, which cost fewer shared-memory reads); the 4 x 8
+  // tiles, whose K is split inside the CTA, where their share is smaller still.
   auto active_tiles = [&](int bm, int bn) {
     int64_t tm = (p.M + bm - 1) / bm, tn = (p.N + bn - 1) / bn;
     int64_t t = tm * tn;
@@ -226,11 +249,21 @@ void zgemm(const ZgemmArgs& in, double2* split_ws, size_t split_ws_elems, cudaSt
       if (p.ksplit > 1) break;
     }
   }
-  p.ksplit = best_ks;
+  if (p.ksplit <= 1) {
+    const int64_t tm = (p.M + ZS_M - 1) / ZS_M, tn = (p.N + ZS_N - 1) / ZS_N;
+    const int64_t t = (p.triD == 1 ? tm * tn / 2 + std::min(tm, tn) : tm * tn) * p.batch;
+    if (std::ceil((double)t / kSMs) * (ZS_M * ZS_N * (double)std::max(p.K, 1) + kZsOverhead) < best_cost &&
+        tm <= 65535 && p.batch <= 65535)
+      best_b = 0;
+  }
+  p.ksplit = best_b == 0 ? 1 : best_ks;
   int bm = best_b, bn = best_b;
-  dim3 grid((p.N + bn - 1) / bn, (p.M + bm - 1) / bm, p.batch * p.ksplit);
+  dim3 grid;
+  if (bm > 0) grid = dim3((p.N + bn - 1) / bn, (p.M + bm - 1) / bm, p.batch * p.ksplit);
   void* kt0 = kt_enabled() ? kt_begin(s) : nullptr;
-  if (bm == 64) zgemm_kernel<64, 64, 8, 4, 4><<<grid, 256, 0, s>>>(p, split_ws);
+  if (bm == 0)
+    zgemm_small_kernel<<<dim3((p.N + ZS_N - 1) / ZS_N, (p.M + ZS_M - 1) / ZS_M, p.batch), ZS_THREADS, 0, s>>>(p);
+  else if (bm == 64) zgemm_kernel<64, 64, 8, 4, 4><<<grid, 256, 0, s>>>(p, split_ws);
   else if (bm == 32) zgemm_kernel<32, 32, 8, 2, 2><<<grid, 256, 0, s>>>(p, split_ws);
   else zgemm_kernel<16, 16, 16, 1, 1><<<grid, 256, 0, s>>>(p, split_ws);
   LAUNCH_NOTE(1);

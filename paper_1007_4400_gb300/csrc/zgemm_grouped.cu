@@ -7,6 +7,7 @@
 // keeps the launch shape fixed from one round to the next. The scalars may come from
 // device memory (coef), so a launch sequence can be captured once and replayed.
 #include "gevp_internal.cuh"
+#include "zsmall.cuh"
 #include <algorithm>
 
 namespace gevp {
@@ -119,6 +120,41 @@ zgemm_group_kernel(const ZgemmItem* __restrict__ items, int nitems, int total_ti
   }
 }
 
+// the same list in 4 x 8 tiles (zsmall.cuh; layout tile 0)
+__global__ void __launch_bounds__(ZS_THREADS)
+zgemm_group_small_kernel(const ZgemmItem* __restrict__ items, int nitems, int total_tiles, ZgemmGroupFlags f) {
+  __shared__ double part[2][ZS_WARPS][64];   // two in turn: one barrier a tile
+  int turn = 0;
+  for (int t = blockIdx.x; t < total_tiles; t += gridDim.x) {
+    int lo = 0, hi = nitems - 1;
+    while (lo < hi) {
+      int mid = (lo + hi + 1) / 2;
+      if (items[mid].tile_start <= t) lo = mid; else hi = mid - 1;
+    }
+    const ZgemmItem& it = items[lo];
+    if (it.active && *it.active == 0) continue;
+    const int local = t - it.tile_start;
+    const int m0 = (local / it.tiles_n) * ZS_M, n0 = (local % it.tiles_n) * ZS_N;
+    if (f.triD == 1 && n0 > m0 + ZS_M - 1) continue;
+    int kb = 0, ke = it.K;
+    if (f.triA == 1) ke = min(ke, m0 + ZS_M);
+    if (f.triA == 2) kb = max(kb, m0);
+    if (f.triB == 1 || f.maskB) kb = max(kb, n0);
+    if (f.triB == 2) ke = min(ke, n0 + ZS_N);
+    double v = zsmall_tile(f.opA, f.opB, it.M, it.N, it.A, it.lda, it.B, it.ldb, f.maskB, m0, n0, kb, ke, part[turn]);
+    turn ^= 1;
+    const int lane = threadIdx.x % 32, comp = threadIdx.x / 32;
+    const int gm = m0 + lane / ZS_N, gn = n0 + lane % ZS_N;
+    if (comp > 1 || gm >= it.M || gn >= it.N) continue;
+    v *= it.coef ? it.coef[0] : it.alpha;
+    if (it.Cin)
+      v = fma(it.coef ? it.coef[1] : it.beta, ((const double*)(it.Cin + (int64_t)gm * it.ldc + gn))[comp], v);
+    if (it.Ein)
+      v = fma(it.coef ? it.coef[2] : it.gamma, ((const double*)(it.Ein + (int64_t)gm * it.lde + gn))[comp], v);
+    ((double*)(it.D + (int64_t)gm * it.ldd + gn))[comp] = v;
+  }
+}
+
 }  // namespace
 
 int zgemm_group_tile(const ZgemmItem* items_host, int nitems) {
@@ -133,8 +169,8 @@ int zgemm_group_layout(ZgemmItem* items_host, int nitems, int tile) {
   int total = 0;
   for (int i = 0; i < nitems; ++i) {
     ZgemmItem& it = items_host[i];
-    it.tiles_n = (it.N + tile - 1) / tile;
-    int tm = (it.M + tile - 1) / tile;
+    it.tiles_n = tile ? (it.N + tile - 1) / tile : (it.N + ZS_N - 1) / ZS_N;
+    int tm = tile ? (it.M + tile - 1) / tile : (it.M + ZS_M - 1) / ZS_M;
     it.tile_start = total;
     total += (it.M > 0 && it.N > 0) ? tm * it.tiles_n : 0;
   }
@@ -145,7 +181,8 @@ void zgemm_grouped(const ZgemmItem* items_dev, int nitems, int total_tiles, int 
                    cudaStream_t s) {
   if (total_tiles <= 0 || nitems <= 0) return;
   int grid = std::min(total_tiles, 152 * 4);
-  if (tile == 64) zgemm_group_kernel<64, 64, 8, 4, 4><<<grid, 256, 0, s>>>(items_dev, nitems, total_tiles, f);
+  if (tile == 0) zgemm_group_small_kernel<<<grid, ZS_THREADS, 0, s>>>(items_dev, nitems, total_tiles, f);
+  else if (tile == 64) zgemm_group_kernel<64, 64, 8, 4, 4><<<grid, 256, 0, s>>>(items_dev, nitems, total_tiles, f);
   else zgemm_group_kernel<32, 32, 8, 2, 2><<<grid, 256, 0, s>>>(items_dev, nitems, total_tiles, f);
   LAUNCH_NOTE(1);
 }
