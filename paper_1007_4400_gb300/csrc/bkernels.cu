@@ -278,72 +278,6 @@ __global__ void b_matvec32(const BDesc* D, int j) {
   }
 }
 
-// two passes of classical Gram-Schmidt against V[0..j], then normalise into V[j+1]
-__global__ void __launch_bounds__(1024) b_lanczos_update(const BDesc* D, int j) {
-  const BDesc& d = D[blockIdx.x];
-  if (!live(d)) return;
-  __shared__ float2 red[32][KMAX + 1];
-  __shared__ float2 h[KMAX + 1];
-  __shared__ float nrm;
-  const int lane = threadIdx.x % 32, wp = threadIdx.x / 32, nw = blockDim.x / 32;
-  int* keff = (int*)(d.ab + 2 * KMAX);
-  if (*keff < j) return;
-  const int64_t n = d.n;
-  float2* w = d.lvec;
-  for (int pass = 0; pass < 2; ++pass) {
-    for (int c = 0; c <= j; ++c) {
-      const float2* vc = d.V + (int64_t)c * n;
-      float2 p = make_float2(0.f, 0.f);
-      for (int64_t i = threadIdx.x; i < n; i += blockDim.x) {
-        float2 a = vc[i], b = w[i];
-        p.x += a.x * b.x + a.y * b.y;
-        p.y += a.x * b.y - a.y * b.x;
-      }
-      for (int o = 16; o > 0; o >>= 1) {
-        p.x += __shfl_xor_sync(0xffffffffu, p.x, o);
-        p.y += __shfl_xor_sync(0xffffffffu, p.y, o);
-      }
-      if (lane == 0) red[wp][c] = p;
-    }
-    __syncthreads();
-    for (int c = threadIdx.x; c <= j; c += blockDim.x) {
-      float2 t = make_float2(0.f, 0.f);
-      for (int q = 0; q < nw; ++q) { t.x += red[q][c].x; t.y += red[q][c].y; }
-      h[c] = t;
-      if (pass == 0 && c == j) d.ab[2 * j] = t.x;
-    }
-    __syncthreads();
-    for (int64_t i = threadIdx.x; i < n; i += blockDim.x) {
-      float2 b = w[i];
-      for (int c = 0; c <= j; ++c) {
-        float2 a = d.V[(int64_t)c * n + i], hc = h[c];
-        b.x -= a.x * hc.x - a.y * hc.y;
-        b.y -= a.x * hc.y + a.y * hc.x;
-      }
-      w[i] = b;
-    }
-    __syncthreads();
-  }
-  float s = 0.f;
-  for (int64_t i = threadIdx.x; i < n; i += blockDim.x) { float2 b = w[i]; s += b.x * b.x + b.y * b.y; }
-  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-  if (lane == 0) red[wp][0].x = s;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    float t = 0.f;
-    for (int q = 0; q < nw; ++q) t += red[q][0].x;
-    nrm = sqrtf(t);
-    d.ab[2 * j + 1] = nrm;
-    float scale = fabsf(d.ab[2 * j]) + (j > 0 ? d.ab[2 * j - 1] : 0.f);
-    *keff = (nrm > 1e-6f * scale && nrm > 0.f) ? j + 1 : -(j + 1);
-  }
-  __syncthreads();
-  if (*keff < 0) return;
-  const float inv = 1.f / nrm;
-  float2* vn = d.V + (int64_t)(j + 1) * n;
-  for (int64_t i = threadIdx.x; i < n; i += blockDim.x) { float2 b = w[i]; vn[i] = make_float2(b.x * inv, b.y * inv); }
-}
-
 // start of a problem of the sequence: every problem iterates again
 __global__ void b_step_reset(const BDesc* D, int np, double tol, int filter64) {
   int p = blockIdx.x * blockDim.x + threadIdx.x;
@@ -908,11 +842,12 @@ void bk_lanczos(const BDesc* D, int np, int64_t nmax, int k, int use_count, int 
   LAUNCH_NOTE(1);
   const int rows_per_block = 8;
   const int blocks = (int)std::max<int64_t>(1, std::min<int64_t>((nmax + rows_per_block - 1) / rows_per_block, 256));
-  for (int j = 0; j < k; ++j) {
-    b_matvec32<<<dim3(blocks, np), 32 * rows_per_block, 0, s>>>(D, j);
-    b_lanczos_update<<<np, 1024, 0, s>>>(D, j);
-    LAUNCH_NOTE(2);
-  }
+  if (!lanczos_batched(D, np, nmax, 0, k, 1, s))
+    for (int j = 0; j < k; ++j) {
+      b_matvec32<<<dim3(blocks, np), 32 * rows_per_block, 0, s>>>(D, j);
+      LAUNCH_NOTE(1);
+      lanczos_batched(D, np, nmax, j, j + 1, 0, s);
+    }
   lanczos_tail_batched(D, np, k, use_count, KMAX, out_off, s);
 }
 void bk_heev_prep(const BDesc* D, int np, int mmax, cudaStream_t s) {

@@ -321,6 +321,7 @@ size_t bk_partial_elems(int m);
 // where that cannot be launched (mmax > 600), Jacobi into Z32 / w32 / perm; the Lanczos ends
 bool heev32_batched(const BDesc* D, int np, int mmax, cudaStream_t s);
 void jacobi32_batched(const BDesc* D, int np, int mmax, int max_sweeps, cudaStream_t s);
+bool lanczos_batched(const BDesc* D, int np, int64_t nmax, int j0, int k, int full, cudaStream_t s);
 void lanczos_tail_batched(const BDesc* D, int np, int k, int use_count, int k_max, int out_off, cudaStream_t s);
 void cluster_jacobi_batched(const BDesc* D, int np, int zsel, double rel, int max_sweeps, cudaStream_t s);
 
