@@ -313,7 +313,7 @@ gevp_status build_plan(gevp_ctx* h, BatchPlan* P, std::string& err) {
       while (tcols < 3u * (unsigned)nchunk[p]) tcols *= 2;
       d.tmem_cols = tcols;
       d.unit_start = unit;
-      unit += d.mtiles * d.nchunks * d.ks;
+      unit += (d.mtiles + 1) / 2 * d.nchunks * d.ks;
     } else {
       d.pcoef = nullptr;
       d.pfinal = nullptr;
@@ -330,7 +330,7 @@ gevp_status build_plan(gevp_ctx* h, BatchPlan* P, std::string& err) {
     int64_t ncm = 0;
     for (int p = 0; p < np; ++p) ncm = std::max<int64_t>(ncm, (int64_t)ncols_pad[p] * n_pad[p]);
     P->tg.nc_max = ncm;
-    e = tcg_prepare(P->tg.nchunk_max);
+    e = tcg_prepare();
     if (e != cudaSuccess) { err = "tensor-core filter: shared memory attribute refused"; return GEVP_ERR_CUDA; }
     const size_t mb = tcg_map_bytes();
     std::vector<char> maps(mb * np);

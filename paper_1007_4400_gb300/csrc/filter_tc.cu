@@ -11,20 +11,24 @@
 // the same TMEM accumulators. A pipeline stage then holds the three pieces of one part (re, im or
 // re + im) of C and of Y for one K block, which serve all six products of that part: half the
 // bytes through L2 and shared memory of a stage per product pair (n = 2048, m = 140, six
-// products: 27.8 us a step; 31.5 with the operands of one piece pair a stage).
+// products: 27.8 us a step; 31.5 with the operands of one piece pair a stage). With the pairs and the
+// unrolled issue by three threads: 26.7 us, n = 4096, m = 250: 118 to 95.5 us (67 clocks an MMA at the
+// tensor cores' rate, 78 here, 96 before).
 //
 // Layout (all K-major, as the MMA wants both operands): the planes of C are n_pad x n_pad
 // row-major BF16 (row i = output row, contiguous k); the block Y is stored transposed,
 // Y^T planes ncols x n_pad (row c = column c of Y, contiguous k), and so is the FP32 state.
 // Padding rows/columns are zero, so the padded K contributes nothing.
 //
-// One CTA: 128 rows of C (UMMA M = 128) x one chunk of up to 160 columns of Y (N), over a
-// slice of K (split-K across grid.z, so that n = 2048 still fills the 152 SMs). Warp 0
-// lane 0 issues TMA loads (128B-swizzled boxes, 2-stage mbarrier pipeline), warp 1 lane 0
-// issues the MMAs (3 per 16-wide K step into three TMEM accumulators of N columns each),
-// then all four warps read TMEM back (warp w owns lanes 32w..32w+31) and write the FP32
-// partial product transposed (coalesced along rows). A second kernel sums the split-K
-// partials in a fixed order (deterministic) and applies the recurrence.
+// A pair of CTAs (cta_group::2): 256 rows of C (UMMA M = 256) x one chunk of up to 160 columns of Y
+// (N), over a slice of K (split-K across grid.z, so that n = 2048 still fills the 152 SMs). Each CTA
+// holds its 128 rows of C and half of the columns, so Y is loaded once a pair: n = 4100, m = 211 in
+// BF16, bound by the loads of 90 KB for 12 MMAs, 43.3 to 32.1 us a step. Warp 0 lane 0 of each CTA
+// issues its TMA loads (128B-swizzled boxes, a pipeline of two or three stages), one lane of warps 1
+// to 3 of the leader the MMAs of both CTAs, a warp for each of the three TMEM accumulators of N
+// columns; then all four warps read TMEM back (warp w owns lanes 32w..32w+31) and write the FP32
+// partial product transposed (coalesced along rows). A second kernel sums the split-K partials in a
+// fixed order (deterministic) and applies the recurrence.
 //
 // Every mbarrier wait is bounded; on expiry the kernel records an error code, skips the
 // rest of its work, frees its TMEM and returns.
@@ -41,14 +45,12 @@ namespace {
 
 constexpr int TM = 128;
 constexpr int TK = 64;
-constexpr int STAGES = 2;
+constexpr int STAGES = 3;          // at most; two for the widest tiles
+constexpr int NFULL = 6;           // barriers of arrived stages: a multiple of 3 and of the stages
+constexpr size_t TC_SMEM = 231424;  // dynamic shared memory: one CTA an SM
 constexpr int NMAX = 160;
 constexpr int MAXSPLIT = 3;
 constexpr int MAXSEG = 6;
-
-// segments (a piece, b piece) with a + b <= nsplit - 1
-__constant__ int kSegA[MAXSEG] = {0, 0, 1, 0, 1, 2};
-__constant__ int kSegB[MAXSEG] = {0, 1, 0, 2, 1, 0};
 
 struct TcMaps {
   CUtensorMap a[MAXSPLIT * 3];   // C planes: [piece][re, im, re+im]
@@ -62,17 +64,18 @@ struct TcParams {
   int ncols_pad;      // rows of the Y^T planes (multiple of nchunk)
   int nsplit;         // pieces per operand
   uint32_t tmem_cols; // power of two >= 3 * nchunk
+  int nst;            // pipeline stages (tc_stages)
   float2* ws;         // [ksplit][ncols_pad][n_pad]
   int* err;
 };
 
-// One output tile: rows m0..m0+127 of C times columns c0..c0+nchunk-1 of the block over
-// K slice z. amaps/bmaps: the tensor maps of the pieces of C and of the block (kernel
-// parameter space or global memory).
+// One output tile of a pair of CTAs: rows m0..m0+255 of C times columns c0..c0+nchunk-1 of the block
+// over K slice z, this CTA's (rank of the pair) the 128 rows from m0 + 128 rank. amaps/bmaps: the
+// tensor maps of the pieces of C and of the block (kernel parameter space or global memory).
 __device__ __forceinline__ void tc_tile(const CUtensorMap* amaps, const CUtensorMap* bmaps, const TcParams& p,
-                                        int m0, int c0, int z) {
+                                        int m0, int c0, int z, int rank) {
   extern __shared__ uint8_t smem_raw[];
-  __shared__ __align__(8) uint64_t full[STAGES], empty[STAGES], done;
+  __shared__ __align__(8) uint64_t full[NFULL], empty[STAGES], done;
   __shared__ uint32_t tmem_sh;
   uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
   const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
@@ -85,90 +88,94 @@ __device__ __forceinline__ void tc_tile(const CUtensorMap* amaps, const CUtensor
   const int group = by_part ? 3 : 1, boxes = by_part ? p.nsplit : 3;
   const int niter = nkb * group;
   const uint32_t a_bytes = TM * TK * 2;
-  const uint32_t b_bytes = (uint32_t)p.nchunk * TK * 2;
+  const uint32_t b_bytes = (uint32_t)(p.nchunk / 2) * TK * 2;   // half of the columns in each CTA
   const uint32_t stage_bytes = 3 * a_bytes + 3 * b_bytes;
   auto tile = [&](int s, int which) -> uint8_t* {
     uint8_t* base = smem + (size_t)s * stage_bytes;
     return which < 3 ? base + which * a_bytes : base + 3 * a_bytes + (which - 3) * b_bytes;
   };
   if (threadIdx.x == 0) {
-    for (int s = 0; s < STAGES; ++s) {
-      mbar_init(&full[s], 1);
-      mbar_init(&empty[s], 1);
-    }
-    mbar_init(&done, 1);
+    for (int s = 0; s < NFULL; ++s) mbar_init(&full[s], 1);
+    for (int s = 0; s < STAGES; ++s) mbar_init(&empty[s], by_part ? 1 : 3);   // a commit of each issuing warp
+    mbar_init(&done, 3);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == 0) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(su32(&tmem_sh)),
+    asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(su32(&tmem_sh)),
                  "r"(p.tmem_cols)
                  : "memory");
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
   }
   fence_before();
   __syncthreads();
+  pair_sync();   // both CTAs' barriers are initialised before any remote arrival
   fence_after();
   const uint32_t tmem = tmem_sh;
+  const int row0 = m0 + TM * rank;
 
   if (warp == 0 && lane == 0) {
     int issued = 0;
     for (int i = 0; i < niter; ++i, issued = i) {
-      int s = i % STAGES;
-      uint32_t ph = (uint32_t)(i / STAGES) & 1u;
-      if (i >= STAGES && !mbar_wait(&empty[s], ph ^ 1u, p.err, 1)) break;
-      mbar_expect_tx(&full[s], (uint32_t)boxes * (a_bytes + b_bytes));
+      const int s = i % p.nst;
+      if (i >= p.nst && !pair_wait(&empty[s], ((uint32_t)(i / p.nst) & 1u) ^ 1u, p.err, 1)) break;
+      if (rank == 0) mbar_expect_tx(&full[i % NFULL], 2u * (uint32_t)boxes * (a_bytes + b_bytes));
+      const uint32_t bar = pair_mapa(su32(&full[i % NFULL]), 0);
       const int part = i % group;
       const int kx = (kb0 + i / group) * TK;
       for (int w = 0; w < boxes; ++w) {
         const int map = by_part ? 3 * w + part : w;
-        tma_load_2d(tile(s, w), amaps + map, kx, m0, &full[s]);
-        tma_load_2d(tile(s, 3 + w), bmaps + map, kx, c0, &full[s]);
+        pair_tma_2d(tile(s, w), amaps + map, kx, row0, bar);
+        pair_tma_2d(tile(s, 3 + w), bmaps + map, kx, c0 + rank * (p.nchunk / 2), bar);
       }
     }
-    // every copy issued has landed before the CTA leaves (bounded; immediate unless a wait
+    // every copy issued has landed before the CTAs leave (bounded; immediate unless a wait
     // elsewhere gave up)
-    for (int i = max(0, issued - STAGES); i < issued; ++i)
-      mbar_wait(&full[i % STAGES], (uint32_t)(i / STAGES) & 1u, p.err, 4);
-  } else if (warp == 1 && lane == 0) {
-    const uint32_t idesc = idesc_bf16(TM, p.nchunk);
-    for (int i = 0; i < niter; ++i) {
-      int s = i % STAGES;
-      uint32_t ph = (uint32_t)(i / STAGES) & 1u;
-      if (!mbar_wait(&full[s], ph, p.err, 2)) break;
+    if (rank == 0)
+      for (int i = max(0, issued - p.nst); i < issued; ++i)
+        mbar_wait(&full[i % NFULL], (uint32_t)(i / NFULL) & 1u, p.err, 4);
+  } else if (warp > 0 && lane == 0 && rank == 0) {
+    // Warp 1 + part issues that part's MMAs, so that three threads share the issue: one alone takes
+    // 80 clocks an MMA, more than the 72 of a 144-wide tile. The order within an accumulator is one
+    // thread's. Iteration i signals full[i % 6]: by parts, that barrier is always the same warp's (6 is
+    // a multiple of 3), so the warp sees each of its phases, and none is waited for a phase early.
+    const uint32_t idesc = idesc_bf16(2 * TM, p.nchunk);
+    const int part = warp - 1;
+    const uint32_t dt = tmem + (uint32_t)(part * p.nchunk);
+    for (int i = by_part ? part : 0; i < niter; i += group) {
+      const int s = i % p.nst;
+      if (!mbar_wait(&full[i % NFULL], (uint32_t)(i / NFULL) & 1u, p.err, 2)) break;
       fence_after();
-      const uint64_t d0 = sdesc(su32(tile(s, 0))), d1 = sdesc(su32(tile(s, 1))), d2 = sdesc(su32(tile(s, 2)));
-      const uint64_t e0 = sdesc(su32(tile(s, 3))), e1 = sdesc(su32(tile(s, 4))), e2 = sdesc(su32(tile(s, 5)));
+      const uint32_t acc0 = i >= group ? 1u : 0u;
       if (!by_part) {
+        const uint64_t a = sdesc(su32(tile(s, part))), b = sdesc(su32(tile(s, 3 + part)));
 #pragma unroll
         for (int kk = 0; kk < TK / 16; ++kk) {
-          const uint32_t acc = (i > 0 || kk > 0) ? 1u : 0u;
           const uint64_t off = (uint64_t)(kk * 32) >> 4;   // 16 bf16 = 32 B along K inside the swizzle row
-          umma(tmem, d0 + off, e0 + off, idesc, acc);
-          umma(tmem + (uint32_t)p.nchunk, d1 + off, e1 + off, idesc, acc);
-          umma(tmem + 2u * (uint32_t)p.nchunk, d2 + off, e2 + off, idesc, acc);
+          pair_umma(dt, a + off, b + off, idesc, kk > 0 ? 1u : acc0);
         }
       } else {
-        const uint32_t dt = tmem + (uint32_t)((i % group) * p.nchunk);
-        const uint32_t acc0 = i >= group ? 1u : 0u;
-        const int nseg = p.nsplit == 2 ? 3 : 6;
-        for (int seg = 0; seg < nseg; ++seg) {
-          const int pa = kSegA[seg], pb = kSegB[seg];
-          const uint64_t a = pa == 0 ? d0 : (pa == 1 ? d1 : d2), b = pb == 0 ? e0 : (pb == 1 ? e1 : e2);
+        const uint64_t d[3] = {sdesc(su32(tile(s, 0))), sdesc(su32(tile(s, 1))), sdesc(su32(tile(s, 2)))};
+        const uint64_t e[3] = {sdesc(su32(tile(s, 3))), sdesc(su32(tile(s, 4))), sdesc(su32(tile(s, 5)))};
+#pragma unroll
+        for (int seg = 0; seg < MAXSEG; ++seg) {
+          // (a piece, b piece) with a + b <= nsplit - 1
+          constexpr int kA[MAXSEG] = {0, 0, 1, 0, 1, 2}, kB[MAXSEG] = {0, 1, 0, 2, 1, 0};
+          if (seg >= 3 && p.nsplit < 3) break;
 #pragma unroll
           for (int kk = 0; kk < TK / 16; ++kk) {
             const uint64_t off = (uint64_t)(kk * 32) >> 4;
-            umma(dt, a + off, b + off, idesc, (seg > 0 || kk > 0) ? 1u : acc0);
+            pair_umma(dt, d[kA[seg]] + off, e[kB[seg]] + off, idesc, (seg > 0 || kk > 0) ? 1u : acc0);
           }
         }
       }
-      umma_commit(&empty[s]);
+      pair_commit(&empty[s]);
     }
-    umma_commit(&done);
+    pair_commit(&done);
   }
   __syncwarp();
-  const bool have = __all_sync(0xffffffffu, mbar_wait(&done, 0, p.err, 3) ? 1 : 0) != 0;
+  const bool have = __all_sync(0xffffffffu, pair_wait(&done, 0, p.err, 3) ? 1 : 0) != 0;
   fence_after();
-  const int row = m0 + warp * 32 + lane;
+  const int row = row0 + warp * 32 + lane;
   float2* out = p.ws + (size_t)z * p.ncols_pad * p.n_pad;
   const uint32_t lane_base = (uint32_t)(warp * 32) << 16;
   for (int cc = 0; cc < p.nchunk; cc += 16) {
@@ -191,13 +198,16 @@ __device__ __forceinline__ void tc_tile(const CUtensorMap* amaps, const CUtensor
   }
   fence_before();
   __syncthreads();
-  if (warp == 0) {
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(p.tmem_cols) : "memory");
-  }
+  pair_sync();   // neither CTA leaves while the other's MMAs or copies may touch it
+  fence_after();
+  if (warp == 0)
+    asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(p.tmem_cols) : "memory");
+  pair_sync();
 }
 
-__global__ void __launch_bounds__(128, 1) cheb_tc_kernel(const __grid_constant__ TcMaps maps, TcParams p) {
-  tc_tile(maps.a, maps.b, p, blockIdx.x * TM, blockIdx.y * p.nchunk, blockIdx.z);
+__global__ void __launch_bounds__(128, 1) __cluster_dims__(2, 1, 1)
+    cheb_tc_kernel(const __grid_constant__ TcMaps maps, const __grid_constant__ TcParams p) {
+  tc_tile(maps.a, maps.b, p, (int)(blockIdx.x >> 1) * 2 * TM, blockIdx.y * p.nchunk, blockIdx.z, blockIdx.x & 1);
 }
 
 // v = hi + lo to about 2^-48, hi the leading 24 bits of v (truncated), from the IEEE-754 fields: an
@@ -473,6 +483,9 @@ bool encode_2d(CUtensorMap* map, void* base, uint64_t inner, uint64_t outer, uin
 constexpr int kKsplitMax = 16;
 constexpr int kDegMax = 64;
 
+int tc_stages(int nchunk) {
+  return (int)std::min<size_t>(STAGES, (TC_SMEM - 1024) / (3 * TM * TK * 2 + 3 * (size_t)(nchunk / 2) * TK * 2));
+}
 int pad_to(int x, int a) { return (x + a - 1) / a * a; }
 
 void chunking(int m, int* nchunks, int* nchunk) {
@@ -596,7 +609,7 @@ cudaError_t run_filter(FilterTC* f, int64_t n, int m, const double2* Y, int64_t 
   const int kbps = (cap_kb + want - 1) / want;
   const int ks = (nkb + kbps - 1) / kbps;
   // where that leaves SMs idle, narrower column tiles: they share no sums, so they change nothing else
-  // (n = 2048, m = 140 in an arena of order 4224: 58.6 us a step, 62.3 with 144-wide tiles)
+  // (n = 2048, m = 140 in an arena of order 4096: 41.6 us a step, 52.8 with 144-wide tiles)
   if (nchunk > 64 && 2 * mtiles * nchunks * ks <= 152) {
     nchunk = pad_to((m + 2 * nchunks - 1) / (2 * nchunks), 16);
     nchunks = (m + nchunk - 1) / nchunk;
@@ -608,7 +621,7 @@ cudaError_t run_filter(FilterTC* f, int64_t n, int m, const double2* Y, int64_t 
   for (int pc = 0; pc < nsplit; ++pc)
     for (int part = 0; part < 3; ++part) {
       if (!encode_2d(&maps.a[3 * pc + part], f->Cp + (3 * pc + part) * cplane, n_pad, n_pad, TK, TM) ||
-          !encode_2d(&maps.b[3 * pc + part], f->Yp + (3 * pc + part) * yplane, n_pad, ncols_pad, TK, nchunk))
+          !encode_2d(&maps.b[3 * pc + part], f->Yp + (3 * pc + part) * yplane, n_pad, ncols_pad, TK, nchunk / 2))
         return cudaErrorNotSupported;
     }
   YPlanes yp{f->Yp, yplane, nsplit};
@@ -622,9 +635,8 @@ cudaError_t run_filter(FilterTC* f, int64_t n, int m, const double2* Y, int64_t 
   p.err = f->err;
   p.tmem_cols = 32;
   while (p.tmem_cols < 3u * (uint32_t)nchunk) p.tmem_cols *= 2;
-  const uint32_t stage_bytes = 3 * TM * TK * 2 + 3 * (uint32_t)nchunk * TK * 2;
-  const size_t smem = (size_t)STAGES * stage_bytes + 1024;
-  cudaFuncSetAttribute(cheb_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  p.nst = tc_stages(nchunk);
+  cudaFuncSetAttribute(cheb_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TC_SMEM);
   cudaMemsetAsync(f->err, 0, sizeof(int), s);
   // recurrence coefficients (the same for the block and for the scalars p_j(theta))
   double e = 0.5 * (hi - lo), c = 0.5 * (hi + lo);
@@ -646,7 +658,7 @@ cudaError_t run_filter(FilterTC* f, int64_t n, int m, const double2* Y, int64_t 
   dim3 tg((n_pad + 31) / 32, (ncols_pad + 31) / 32);
   int64_t total = (int64_t)ncols_pad * n_pad / 2;
   int eblocks = (int)std::min<int64_t>((total + 255) / 256, 152 * 16);
-  dim3 grid(mtiles, nchunks, ks);
+  dim3 grid((mtiles + 1) / 2 * 2, nchunks, ks);
   float2* prev = nullptr;
   float2* cur = f->S0;
   float2* nxt = f->S1;
@@ -679,7 +691,7 @@ cudaError_t run_filter(FilterTC* f, int64_t n, int m, const double2* Y, int64_t 
     LAUNCH_NOTE(1);
   }
   for (int j = j0; j < deg; ++j) {
-    cheb_tc_kernel<<<grid, 128, smem, s>>>(maps, p);
+    cheb_tc_kernel<<<grid, 128, TC_SMEM, s>>>(maps, p);
     LAUNCH_NOTE(1);
     const float2* Rj = corrected ? f->S3 : nullptr;
     const float* pcj = corrected ? f->pcoef + (size_t)j * ncols_pad : nullptr;
@@ -742,8 +754,9 @@ namespace {
 
 __device__ __forceinline__ bool tcg_runs(const BDesc& d, int j) { return d.flags[6] != 0 && j < d.flags[1]; }
 
-__global__ void __launch_bounds__(128, 1) cheb_tcg_kernel(const BDesc* D, int np, int j, int* err) {
-  const int u = blockIdx.x;
+__global__ void __launch_bounds__(128, 1) __cluster_dims__(2, 1, 1)
+    cheb_tcg_kernel(const BDesc* D, int np, int j, int nst, int* err) {
+  const int u = blockIdx.x >> 1;   // a pair of CTAs a unit
   int lo = 0, hi = np - 1;
   while (lo < hi) {
     const int mid = (lo + hi + 1) / 2;
@@ -752,7 +765,7 @@ __global__ void __launch_bounds__(128, 1) cheb_tcg_kernel(const BDesc* D, int np
   const BDesc& d = D[lo];
   if (!tcg_runs(d, j)) return;
   const int local = u - d.unit_start;
-  const int per_z = d.mtiles * d.nchunks;
+  const int per_z = (d.mtiles + 1) / 2 * d.nchunks;
   const int z = local / per_z, r = local % per_z;
   if (z >= d.ks) return;
   TcParams p;
@@ -762,10 +775,11 @@ __global__ void __launch_bounds__(128, 1) cheb_tcg_kernel(const BDesc* D, int np
   p.ncols_pad = d.ncols_pad;
   p.nsplit = d.nsplit;
   p.tmem_cols = d.tmem_cols;
+  p.nst = nst;
   p.ws = d.tws;
   p.err = err;
   const CUtensorMap* maps = (const CUtensorMap*)d.maps;
-  tc_tile(maps, maps + MAXSPLIT * 3, p, (r / d.nchunks) * TM, (r % d.nchunks) * d.nchunk, z);
+  tc_tile(maps, maps + MAXSPLIT * 3, p, (r / d.nchunks) * 2 * TM, (r % d.nchunks) * d.nchunk, z, blockIdx.x & 1);
 }
 
 // j = 0: D_1 = alpha_0 R; j >= 1: D_{j+1} from the split-K partials of C D_j. D_k is kept
@@ -818,10 +832,6 @@ void tcg_geometry(int64_t n, int m, int* n_pad, int* ncols_pad, int* nchunk, int
   *ncols_pad = *nchunks * *nchunk;
 }
 
-size_t tcg_smem_bytes(int nchunk_max) {
-  return (size_t)STAGES * (3 * TM * TK * 2 + 3 * (size_t)nchunk_max * TK * 2) + 1024;
-}
-
 size_t tcg_map_bytes() { return sizeof(CUtensorMap) * MAXSPLIT * 3 * 2; }
 
 bool tcg_encode_maps(const BDesc& d, void* maps_host) {
@@ -832,7 +842,7 @@ bool tcg_encode_maps(const BDesc& d, void* maps_host) {
   for (int pc = 0; pc < d.nsplit; ++pc)
     for (int part = 0; part < 3; ++part) {
       if (!encode_2d(&a[3 * pc + part], d.Cp + (3 * pc + part) * cplane, d.n_pad, d.n_pad, TK, TM) ||
-          !encode_2d(&b[3 * pc + part], d.Yp + (3 * pc + part) * yplane, d.n_pad, d.ncols_pad, TK, d.nchunk))
+          !encode_2d(&b[3 * pc + part], d.Yp + (3 * pc + part) * yplane, d.n_pad, d.ncols_pad, TK, d.nchunk / 2))
         return false;
     }
   return true;
@@ -844,22 +854,21 @@ void tcg_set_matrix(const BDesc* D, int np, int64_t npad2_max, cudaStream_t s) {
   LAUNCH_NOTE(1);
 }
 
-cudaError_t tcg_prepare(int nchunk_max) {
-  return cudaFuncSetAttribute(cheb_tcg_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              (int)tcg_smem_bytes(nchunk_max));
+cudaError_t tcg_prepare() {
+  return cudaFuncSetAttribute(cheb_tcg_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TC_SMEM);
 }
 
 // The launch sequence of one filter application (no host synchronisation, capturable);
-// tcg_prepare must have been called for this nchunk_max first.
+// tcg_prepare must have been called first.
 cudaError_t tcg_filter(const BDesc* D, const TcgShape& g, int* err, cudaStream_t s) {
-  const size_t smem = tcg_smem_bytes(g.nchunk_max);
+  const int nst = tc_stages(g.nchunk_max);
   dim3 tg((g.n_pad_max + 31) / 32, (g.ncols_pad_max + 31) / 32, g.np);
   int eb = (int)std::max<int64_t>(1, std::min<int64_t>((g.nc_max / 2 + 255) / 256, 128));
   tcg_resid_to_state<<<tg, 256, 0, s>>>(D);
   tcg_epilogue<<<dim3(eb, g.np), 256, 0, s>>>(D, 0);
   LAUNCH_NOTE(2);
   for (int j = 1; j < g.steps; ++j) {
-    cheb_tcg_kernel<<<g.units, 128, smem, s>>>(D, g.np, j, err);
+    cheb_tcg_kernel<<<2 * g.units, 128, TC_SMEM, s>>>(D, g.np, j, nst, err);
     tcg_epilogue<<<dim3(eb, g.np), 256, 0, s>>>(D, j);
     LAUNCH_NOTE(2);
   }

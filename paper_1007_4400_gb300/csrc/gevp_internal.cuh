@@ -327,12 +327,11 @@ void cluster_jacobi_batched(const BDesc* D, int np, int zsel, double rel, int ma
 
 // grouped tensor-core filter (residual-corrected recurrence) over the problems of a batch
 void tcg_geometry(int64_t n, int m, int* n_pad, int* ncols_pad, int* nchunk, int* nchunks);
-size_t tcg_smem_bytes(int nchunk_max);
 size_t tcg_map_bytes();                                  // bytes of one problem's tensor maps
 bool tcg_encode_maps(const BDesc& d, void* maps_host);   // host copy of d's maps (Cp, Yp set)
 void tcg_set_matrix(const BDesc* D, int np, int64_t npad2_max, cudaStream_t s);
 struct TcgShape { int np, units, n_pad_max, ncols_pad_max, nchunk_max, steps; int64_t nc_max; };
-cudaError_t tcg_prepare(int nchunk_max);
+cudaError_t tcg_prepare();
 cudaError_t tcg_filter(const BDesc* D, const TcgShape& g, int* err, cudaStream_t s);
 
 // ---------------------------------------------------------------- matrix variation

@@ -208,34 +208,6 @@ struct OzParams {
   float p[OZ_NMOD], ip[OZ_NMOD];
 };
 
-__device__ __forceinline__ uint32_t oz_mapa(uint32_t addr, uint32_t rank) {
-  uint32_t r;
-  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
-  return r;
-}
-__device__ __forceinline__ void oz_cluster_sync() {
-  asm volatile("barrier.cluster.arrive.release;" ::: "memory");
-  asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
-}
-__device__ __forceinline__ void oz_arrive_cluster(uint32_t remote) {
-  asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(remote) : "memory");
-}
-// mbar_wait for a barrier that the other CTA of the pair arrives on
-__device__ __forceinline__ bool oz_wait_cluster(uint64_t* bar, uint32_t parity, int* err, int code) {
-  const uint32_t addr = su32(bar);
-  for (uint32_t it = 0; it < (1u << 24); ++it) {
-    uint32_t ok;
-    asm volatile(
-        "{\n .reg .pred p;\n mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, "
-        "p;\n}\n"
-        : "=r"(ok)
-        : "r"(addr), "r"(parity)
-        : "memory");
-    if (ok) return true;
-  }
-  atomicCAS(err, 0, code);
-  return false;
-}
 // TMA load whose bytes count on the pair leader's barrier (a shared::cluster address)
 __device__ __forceinline__ void oz_tma(void* dst, const CUtensorMap* map, int x, int y, int z, uint32_t bar) {
   asm volatile(
@@ -244,21 +216,6 @@ __device__ __forceinline__ void oz_tma(void* dst, const CUtensorMap* map, int x,
       "l"((uint64_t)map), "r"(x), "r"(y), "r"(z), "r"(bar)
       : "memory");
 }
-__device__ __forceinline__ void oz_umma(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc, uint32_t acc) {
-  asm volatile(
-      "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(d),
-      "l"(a), "l"(b), "r"(idesc), "r"(acc)
-      : "memory");
-}
-// arrives on the barrier at this offset in both CTAs of the pair
-__device__ __forceinline__ void oz_commit(uint64_t* bar) {
-  asm volatile(
-      "tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(
-          su32(bar)),
-      "h"((uint16_t)3)
-      : "memory");
-}
-
 struct OzUnit {
   int slice, mod, m0, n0, klo, khi;   // klo, khi in 64-blocks
   bool skip;
@@ -340,7 +297,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) __cluster_dims__(2, 1, 1)
   }
   fence_before();
   __syncthreads();
-  oz_cluster_sync();   // both CTAs' barriers are initialised before any remote arrival
+  pair_sync();   // both CTAs' barriers are initialised before any remote arrival
   fence_after();
   const uint32_t tmem = tmem_sh;
 
@@ -352,13 +309,13 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) __cluster_dims__(2, 1, 1)
       const int z = t.mod - p.mod0;
       for (int kb = t.klo; kb < t.khi; ++kb, ++it) {
         const int st = it % p.nst;
-        if (it >= p.nst && !oz_wait_cluster(&empty[st], ((uint32_t)(it / p.nst) & 1u) ^ 1u, p.err, 21)) {
+        if (it >= p.nst && !pair_wait(&empty[st], ((uint32_t)(it / p.nst) & 1u) ^ 1u, p.err, 21)) {
           ok = false;
           break;
         }
         uint8_t* dst = smem + (size_t)st * stage;
         if (rank == 0) mbar_expect_tx(&full[st], 2 * stage);
-        const uint32_t bar = oz_mapa(su32(&full[st]), 0);
+        const uint32_t bar = pair_mapa(su32(&full[st]), 0);
         const int x = kb * OZ_TK, ya = t.m0 + 128 * rank, yb = t.n0 + (p.tn / 2) * rank;
         oz_tma(dst, &maps.a, x, ya, p.za + z, bar);
         oz_tma(dst + 2 * OZ_A_BYTES, &maps.b, x, yb, p.zb + z, bar);
@@ -392,7 +349,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) __cluster_dims__(2, 1, 1)
 #pragma unroll
           for (int part = 0; part < 2; ++part) {
             // a chunk's first MMAs wait until the previous chunk's sums have been read
-            if (k == kb && chunk > 0 && !oz_wait_cluster(&tempty[part], (chunk - 1) & 1u, p.err, 22)) {
+            if (k == kb && chunk > 0 && !pair_wait(&tempty[part], (chunk - 1) & 1u, p.err, 22)) {
               ok = false;
               break;
             }
@@ -401,17 +358,17 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) __cluster_dims__(2, 1, 1)
 #pragma unroll
             for (int kk = 0; kk < OZ_TK / 16; ++kk) {
               const uint64_t o = (uint64_t)(kk * 32) >> 4;
-              oz_umma(d, ar + o, (part ? bi : br) + o, part ? p.id_ri : p.id_rr, kk > 0 ? 1u : first);
+              pair_umma(d, ar + o, (part ? bi : br) + o, part ? p.id_ri : p.id_rr, kk > 0 ? 1u : first);
             }
 #pragma unroll
             for (int kk = 0; kk < OZ_TK / 16; ++kk) {
               const uint64_t o = (uint64_t)(kk * 32) >> 4;
-              oz_umma(d, ai + o, (part ? br : bi) + o, part ? p.id_ir : p.id_ii, 1u);
+              pair_umma(d, ai + o, (part ? br : bi) + o, part ? p.id_ir : p.id_ii, 1u);
             }
-            if (k == ke - 1) oz_commit(&tfull[part]);
+            if (k == ke - 1) pair_commit(&tfull[part]);
           }
           if (!ok) break;
-          oz_commit(&empty[st]);
+          pair_commit(&empty[st]);
         }
       }
     }
@@ -419,7 +376,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) __cluster_dims__(2, 1, 1)
     const int q = warp & 3;
     const uint32_t tq = tmem + ((uint32_t)(q * 32) << 16);
     const int ng = p.tn / 16;   // 16-column groups; this warp's: warp / 4, warp / 4 + 4, ...
-    const uint32_t te[2] = {oz_mapa(su32(&tempty[0]), 0), oz_mapa(su32(&tempty[1]), 0)};
+    const uint32_t te[2] = {pair_mapa(su32(&tempty[0]), 0), pair_mapa(su32(&tempty[1]), 0)};
     uint32_t chunk = 0;
     bool ok = true;
     for (int u = u0; u < units && ok; u += ustep) {
@@ -439,7 +396,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) __cluster_dims__(2, 1, 1)
       for (int kb = t.klo; kb < t.khi && ok; kb += OZ_CHUNK, ++chunk) {
         const bool last = kb + OZ_CHUNK >= t.khi;
         for (int part = 0; part < 2; ++part) {
-          ok = ok && __all_sync(0xffffffffu, oz_wait_cluster(&tfull[part], chunk & 1u, p.err, 24) ? 1 : 0) != 0;
+          ok = ok && __all_sync(0xffffffffu, pair_wait(&tfull[part], chunk & 1u, p.err, 24) ? 1 : 0) != 0;
           if (!ok) break;
           fence_after();
           for (int g = warp >> 2; g < ng; g += 4) {
@@ -468,18 +425,18 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) __cluster_dims__(2, 1, 1)
           if (!last) tmem_wait_st();
           fence_before();
           __syncwarp();
-          if (lane == 0) oz_arrive_cluster(te[part]);
+          if (lane == 0) pair_arrive(te[part]);
         }
       }
     }
   }
   fence_before();
   __syncthreads();
-  oz_cluster_sync();   // neither CTA leaves while the other's MMAs or arrivals may touch it
+  pair_sync();   // neither CTA leaves while the other's MMAs or arrivals may touch it
   fence_after();
   if (warp == 0)
     asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512) : "memory");
-  oz_cluster_sync();
+  pair_sync();
 }
 
 // ---------------------------------------------------------------- reconstruction
