@@ -619,7 +619,8 @@ void zgram(int64_t n, int mx, int my, const double2* X, int64_t ldx, const doubl
                        (ZS_M * ZS_N * (double)n + kZsOverhead);
   const double large = std::ceil((double)(active * slices) / kSMs) * (GT * GT * (double)per) +
                        (slices > 1 ? 2.0 * kZsOverhead : 0.0);
-  if (n > 0 && small < large && tm <= 65535)
+  // (a long column needs several CTAs an SM to hide its loads: n = 2048, m = 88 took 135 us)
+  if (n > 0 && n <= 512 && small < large && tm <= 65535)
     zgram_small_kernel<<<dim3((unsigned)tn, (unsigned)tm), ZS_THREADS, 0, s>>>((int)n, mx, my, X, ldx, Y, ldy, G, ldg, herm);
   else zgram_kernel<<<grid, GT * GT, 0, s>>>(n, mx, my, X, ldx, Y, ldy, G, ldg, herm, ntj, (int)slices, per, part, cnt);
   LAUNCH_NOTE(1);
