@@ -451,11 +451,17 @@ __global__ void __launch_bounds__(HT, 1) heev32_tri_kernel(Src src, int may_skip
       int64_t cap;
       __device__ bool room(int) {
         if (pos + m > cap || ns + 1 >= m * m) return false;
-        uint32_t spin = 0;
-        while ((pos + m - pub[3] > kRing || ns + 1 - *sc > kSweepRing) && ++spin < kSpin) __nanosleep(64);
-        if (spin >= kSpin && lane == 0) *failed = 1;
+        int ok = 0;   // lane 0's decision holds for the warp
+        if (lane == 0) {
+          uint32_t spin = 0;
+          while ((pos + m - pub[3] > kRing || ns + 1 - *sc > kSweepRing) && ++spin < kSpin) __nanosleep(64);
+          ok = spin < kSpin;
+          if (!ok) *failed = 1;
+        }
         pos0 = pos;
-        return spin < kSpin;
+        ok = __shfl_sync(0xffffffffu, ok, 0);
+        __syncwarp();
+        return ok != 0;
       }
       __device__ void start(int) {}
       __device__ void rotation(int, float c, float s) {
@@ -479,10 +485,18 @@ __global__ void __launch_bounds__(HT, 1) heev32_tri_kernel(Src src, int may_skip
     int done = 0, sc_ = 0, off_ = 0;
     uint32_t spin = 0;
     while (spin < kSpin) {
-      const int fin = ring_pub[2];
-      __threadfence_block();
-      const int ns = ring_pub[1];
-      __threadfence_block();
+      // one reading for the whole warp: lanes that saw different counts would publish a sweep that
+      // others have not copied
+      int fin = 0, ns = 0;
+      if (lane == 0) {
+        fin = ring_pub[2];
+        __threadfence_block();
+        ns = ring_pub[1];
+        __threadfence_block();
+      }
+      fin = __shfl_sync(0xffffffffu, fin, 0);
+      ns = __shfl_sync(0xffffffffu, ns, 0);
+      __syncwarp();   // the other lanes' reads of the ring come after lane 0's of the count
       if (ns > sc_) {
         spin = 0;
         for (int q = sc_ + lane; q < ns; q += 32) {
@@ -535,6 +549,7 @@ __global__ void __launch_bounds__(HT, 1) heev32_tri_kernel(Src src, int may_skip
         }
         n = __shfl_sync(0xffffffffu, n, 0);
         fin = __shfl_sync(0xffffffffu, fin, 0);
+        __syncwarp();   // (a shuffle alone orders no memory: the sweeps are read behind lane 0's acquire)
         if (mine >= n) {
           if (fin) break;
           __nanosleep(128);
