@@ -406,7 +406,8 @@ __global__ void __launch_bounds__(1024) b_sort_pairs(const BDesc* D, int zsel) {
   for (int i = threadIdx.x; i < m; i += blockDim.x) {
     double li = d.hlam[i];
     int r = 0;
-    for (int j = 0; j < m; ++j) r += (d.hlam[j] < li) || (d.hlam[j] == li && j < i);
+    const long long ki = rank_key(li);
+    for (int j = 0; j < m; ++j) r += rank_before(rank_key(d.hlam[j]), j, ki, i);
     rk[i] = r;
     d.theta[r] = li;
   }

@@ -33,6 +33,25 @@ __device__ __forceinline__ void cfma(float2& acc, float2 a, float2 b) {
   acc.y = fmaf(a.y, b.x, acc.y);
 }
 
+// Sorting by rank: whole-number keys in ascending order, NaN last, so that with ties broken by the
+// index every index has a rank of its own whatever the values are (a comparison with NaN is false
+// both ways: the ranks would collide and leave entries of the permutation unwritten). An FP64
+// comparison also costs as much as an FMA here, an integer one nothing.
+__device__ __forceinline__ long long rank_key(double x) {
+  const long long b = __double_as_longlong(x);
+  if ((b & 0x7fffffffffffffffll) > 0x7ff0000000000000ll) return 0x7fffffffffffffffll;
+  return b < 0 ? (long long)(0x8000000000000000ull - (unsigned long long)b) : b;
+}
+__device__ __forceinline__ int rank_key(float x) {
+  const int b = __float_as_int(x);
+  if ((b & 0x7fffffff) > 0x7f800000) return 0x7fffffff;
+  return b < 0 ? (int)(0x80000000u - (unsigned)b) : b;
+}
+template <class T>
+__device__ __forceinline__ bool rank_before(T a, int i, T b, int j) {
+  return a < b || (a == b && i < j);
+}
+
 // ---------------------------------------------------------------- FP64 complex GEMM
 // D = alpha * op(A) op(B) + beta * Cin + gamma * Ein   (real alpha, beta, gamma)
 // op(X) = X (op = 0) or X^H (op = 1). op(A) is M x K, op(B) is K x N, D is M x N.

@@ -230,8 +230,7 @@ __device__ void jacobi32_body(int m, float2* Gg, float2* Z, float* w, int* perm,
     float wi = G[i * m + i].x;
     int r = 0;
     for (int j = 0; j < m; ++j) {
-      float wj = G[j * m + j].x;
-      r += (wj < wi) || (wj == wi && j < i);
+      r += rank_before(rank_key(G[j * m + j].x), j, rank_key(wi), i);
     }
     perm[r] = i;
     w[r] = wi;
@@ -298,8 +297,7 @@ __global__ void __launch_bounds__(JT) jacobi32_coop_kernel(int m, float2* G, flo
     float wi = __ldcg(Gc + i * m + i).x;
     int r = 0;
     for (int j = 0; j < m; ++j) {
-      float wj = __ldcg(Gc + j * m + j).x;
-      r += (wj < wi) || (wj == wi && j < i);
+      r += rank_before(rank_key(__ldcg(Gc + j * m + j).x), j, rank_key(wi), i);
     }
     perm[r] = i;
     w[r] = wi;
@@ -584,7 +582,8 @@ __global__ void sort_pairs_kernel(int m, const double* lam, const double2* Zin, 
   for (int i = threadIdx.x; i < m; i += blockDim.x) {
     double li = lam[i];
     int r = 0;
-    for (int j = 0; j < m; ++j) r += (lam[j] < li) || (lam[j] == li && j < i);
+    const long long ki = rank_key(li);
+    for (int j = 0; j < m; ++j) r += rank_before(rank_key(lam[j]), j, ki, i);
     rk[i] = r;
     theta[r] = li;
   }

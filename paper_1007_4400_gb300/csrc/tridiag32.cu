@@ -603,12 +603,9 @@ __global__ void __launch_bounds__(256) heev32_back_kernel(Src src) {
   if (j0 >= m) return;
   const int j = min(m - 1, j0 + warp);
   const bool skip = p.ctl[2] != 0, bad = p.ctl[3] != 0;
-  const float wj = p.w[j];
+  const int kj = rank_key(p.w[j]);
   int rk = 0;
-  for (int i = lane; i < m; i += 32) {
-    const float wi = p.w[i];
-    rk += (wi < wj || (wi == wj && i < j)) ? 1 : 0;
-  }
+  for (int i = lane; i < m; i += 32) rk += rank_before(rank_key(p.w[i]), i, kj, j) ? 1 : 0;
   for (int o = 16; o > 0; o >>= 1) rk += __shfl_xor_sync(0xffffffffu, rk, o);
   float2 y[NT];
 #pragma unroll
@@ -651,7 +648,7 @@ __global__ void __launch_bounds__(256) heev32_back_kernel(Src src) {
 #pragma unroll
   for (int t = 0; t < NT; ++t) {
     const int r = 32 * t + lane;
-    if (r < m) p.Z[(int64_t)r * p.ldz + min(rk, m - 1)] = bad ? make_double2(nan, nan) : make_double2(y[t].x, y[t].y);
+    if (r < m) p.Z[(int64_t)r * p.ldz + rk] = bad ? make_double2(nan, nan) : make_double2(y[t].x, y[t].y);
   }
 }
 
@@ -702,7 +699,7 @@ __device__ void lanczos_tail(int k, int64_t n, int count, const float* ab, int k
   __syncwarp();
   for (int i = lane; i < kk; i += 32) {
     int r = 0;
-    for (int j = 0; j < kk; ++j) r += (d[j] < d[i] || (d[j] == d[i] && j < i)) ? 1 : 0;
+    for (int j = 0; j < kk; ++j) r += rank_before(rank_key(d[j]), j, rank_key(d[i]), i) ? 1 : 0;
     ws[r] = d[i];
     zs[r] = z[i];
   }
