@@ -178,6 +178,14 @@ namespace {
 
 // ---------------------------------------------------------------- plan
 
+// upload the items of one call (pointer fields may have changed)
+cudaError_t upload_call(BatchPlan* P, GCall& c, cudaStream_t s) {
+  if (c.items.empty()) return cudaSuccess;
+  c.total = zgemm_group_layout(c.items.data(), (int)c.items.size(), c.tile);
+  return cudaMemcpyAsync(P->pool + c.off, c.items.data(), c.items.size() * sizeof(ZgemmItem),
+                         cudaMemcpyHostToDevice, s);
+}
+
 gevp_status build_plan(gevp_ctx* h, BatchPlan* P, std::string& err) {
   const int np = P->np;
   const bool tc = P->tc;
@@ -449,22 +457,17 @@ gevp_status build_plan(gevp_ctx* h, BatchPlan* P, std::string& err) {
   e = cudaMalloc(&P->pool, (P->pool_items + P->tune_items) * sizeof(ZgemmItem));
   if (e != cudaSuccess) { err = "item pool cudaMalloc failed"; return GEVP_ERR_OOM; }
   P->tune_pool = P->pool + P->pool_items;
+  // every call's list is there from the start: a call may first run after the plan counts as tuned (a
+  // step that ends without its final check leaves that one's to a later step)
   for (auto& c : P->calls) {
     c.tile = zgemm_group_tile(c.items.data(), (int)c.items.size());
-    c.total = zgemm_group_layout(c.items.data(), (int)c.items.size(), c.tile);
+    e = upload_call(P, c, s);
+    if (e != cudaSuccess) { err = "item upload failed"; return GEVP_ERR_CUDA; }
   }
   P->bucket.resize(np);
   for (int p = 0; p < np; ++p) P->bucket[p] = (int)std::min<int64_t>(kBuckets - 1, P->n[p] / 512);
   for (int b = 0; b < kBuckets; ++b) P->cap_bucket[b] = P->deg_steps;
   return GEVP_OK;
-}
-
-// upload the items of one call (pointer fields may have changed)
-cudaError_t upload_call(BatchPlan* P, GCall& c, cudaStream_t s) {
-  if (c.items.empty()) return cudaSuccess;
-  c.total = zgemm_group_layout(c.items.data(), (int)c.items.size(), c.tile);
-  return cudaMemcpyAsync(P->pool + c.off, c.items.data(), c.items.size() * sizeof(ZgemmItem),
-                         cudaMemcpyHostToDevice, s);
 }
 
 cudaEvent_t evt(BatchPlan* P, size_t i) {
