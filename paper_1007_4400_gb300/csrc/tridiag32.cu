@@ -340,7 +340,11 @@ __global__ void __launch_bounds__(HT, 1) heev32_tri_kernel(Src src, int may_skip
     xn = wsum(xn);
     float beta = al.x;
     float2 tau = make_float2(0.f, 0.f), inv = make_float2(0.f, 0.f);
-    if (xn > 0.f || al.y != 0.f) {
+    // A column below 1e-15 of the matrix's largest entry (which is about 1 here) counts as reduced: QL
+    // drops such couplings, FP32 rounding is 1e-7, and its squares would leave the FP32 range (1 / |x|^2
+    // infinite, the reflector NaN). Matrices of low rank and graded ones come here: their rounding
+    // residue shrinks by 1e-8 a step.
+    if ((xn > 0.f || al.y != 0.f) && al.x * al.x + al.y * al.y + xn > 1e-30f) {
       beta = -copysignf(sqrtf(al.x * al.x + al.y * al.y + xn), al.x);
       const float ib = 1.f / beta;
       tau = make_float2((beta - al.x) * ib, -al.y * ib);
