@@ -257,7 +257,9 @@ gevp_status gevp_cholqr2(gevp_handle h, int64_t n, int m, void* Y, int64_t ldy, 
 gevp_status gevp_rayleigh_ritz(gevp_handle h, int64_t n, int m, const void* C, int64_t ldc, void* Q, int64_t ldq,
                                void* W, int64_t ldw, double* theta, double* res);
 
-/* Small dense Hermitian eigensolver: G (m x m) = Z diag(theta) Z^H, theta ascending. */
+/* Small dense Hermitian eigensolver: G (m x m) = Z diag(theta) Z^H, theta ascending (NaN last).
+ * GEVP_ERR_NO_CONVERGENCE or GEVP_ERR_TIMEOUT if its FP32 stage ran out of sweeps or of a bounded
+ * wait (theta and Z are NaN then; gevp_rayleigh_ritz likewise). */
 gevp_status gevp_heev_small(gevp_handle h, int m, const void* G, int64_t ldg, double* theta, void* Z, int64_t ldz);
 
 /* Lanczos spectral bounds of Hermitian C: out (host, 5 doubles) = {lowest Ritz value,
@@ -368,6 +370,12 @@ gevp_status gevp_zgemm_emulated(gevp_handle h, int opA, int opB, int M, int N, i
  * non-positive pivot met. */
 gevp_status gevp_reduce_emulated(gevp_handle h, int64_t n, const void* A, int64_t lda, const void* B, int64_t ldb,
                                  void* L, int64_t ldl, void* C, int64_t ldc, int64_t* info, int slices);
+
+/* Failure injection on the host, for tests of error handling: the next call on this handle that could
+ * report the failure `what` finds its device word set as if it had happened (nothing fails on the
+ * device). 1: a bounded wait of the small eigensolver ran out (gevp_heev_small,
+ * gevp_rayleigh_ritz). 0: take an injection back. */
+gevp_status gevp_inject_failure(gevp_handle h, int what);
 
 /* Measured FP64 FMA, FP64 DMMA and FP32 FMA rates of this device in TFLOP/s (host out[3]). */
 gevp_status gevp_probe_peaks(gevp_handle h, double* out);

@@ -94,9 +94,9 @@ struct gevp_ctx {
   int* ozflags = nullptr;                   // device: [0] kernel error code, [1] non-finite entry; [2], [3]
                                             // the same for the products of the per-step entry points
   bool em = false;                          // a per-step entry point whose large products are emulated
-  // pinned host mirror
-  double* hbuf = nullptr;
-  size_t hbuf_elems = 0;
+  const int* heev_word = nullptr;           // device word of the last small eigensolver's failure (null: none)
+  int inject = 0;                           // gevp_inject_failure: the next failure to report
+  double* hbuf = nullptr;                   // pinned host words, for the entry points' status reads
   // device staging of the host-buffer entry point (grown on demand)
   void* stage = nullptr;
   size_t stage_bytes = 0;
@@ -236,14 +236,13 @@ gevp_status ensure(gevp_ctx* h, int64_t n, int m) {
     cudaFree(h->arena);
     h->arena = nullptr;
   }
+  h->cap_n = 0;
+  h->cap_m = 0;
+  if (!h->hbuf) CK(cudaMallocHost(&h->hbuf, 64 * sizeof(double)));
   size_t bytes = layout(h, nullptr, nn, mm);
   void* p = nullptr;
   cudaError_t e = cudaMalloc(&p, bytes);
-  if (e != cudaSuccess) {
-    h->cap_n = 0;
-    h->cap_m = 0;
-    return cuda_fail(h, e, "workspace cudaMalloc");
-  }
+  if (e != cudaSuccess) return cuda_fail(h, e, "workspace cudaMalloc");
   h->arena = (char*)p;
   h->arena_bytes = bytes;
   layout(h, h->arena, nn, mm);
@@ -251,12 +250,6 @@ gevp_status ensure(gevp_ctx* h, int64_t n, int m) {
   h->cap_n = nn;
   h->cap_m = mm;
   h->chol_valid = false;
-  size_t hel = 8 * (size_t)mm + 64;
-  if (hel > h->hbuf_elems) {
-    if (h->hbuf) cudaFreeHost(h->hbuf);
-    CK(cudaMallocHost(&h->hbuf, hel * sizeof(double)));
-    h->hbuf_elems = hel;
-  }
   return GEVP_OK;
 }
 
@@ -658,21 +651,40 @@ bool gram(gevp_ctx* h, int64_t n, int mx, int my, const double2* X, int64_t ldx,
   return false;
 }
 
+// gevp_inject_failure: the device word reads as after the given failure
+void inject(gevp_ctx* h, int what, const int* word, int code) {
+  if (h->inject != what || !word) return;
+  h->inject = 0;
+  cudaMemsetAsync((void*)word, code, 1, h->stream);
+}
+
+// the status that the small eigensolver's failure word stands for
+gevp_status heev_status(gevp_ctx* h, int word) {
+  if (word == 0) return GEVP_OK;
+  h->err = word == 1 ? "a bounded wait of the small eigensolver ran out" : "the small eigensolver's QL iteration did not converge";
+  return word == 1 ? GEVP_ERR_TIMEOUT : GEVP_ERR_NO_CONVERGENCE;
+}
+
 // For the duration of a per-step entry point: its large products emulated where the device can,
 // and the kernels' error code read at the end
 struct EmScope {
   gevp_ctx* h;
   explicit EmScope(gevp_ctx* hh) : h(hh) { h->em = h->oz_slices == 0 && gevp::oz_supported(); }
   ~EmScope() { h->em = false; }
-  gevp_status check() {   // after the stream has been synchronised
-    if (!h->ozflags) return GEVP_OK;
-    int f = 0;
-    CK(cudaMemcpyAsync(&f, h->ozflags + 2, sizeof f, cudaMemcpyDeviceToHost, h->stream));
+  // waits for the call's work, then its error words
+  gevp_status finish(const int* heev_word = nullptr) {
+    int* f = (int*)h->hbuf;   // pinned
+    f[0] = f[1] = 0;
+    if (h->ozflags) CK(cudaMemcpyAsync(f, h->ozflags + 2, sizeof(int), cudaMemcpyDeviceToHost, h->stream));
+    if (heev_word) CK(cudaMemcpyAsync(f + 1, heev_word, sizeof(int), cudaMemcpyDeviceToHost, h->stream));
     CK(cudaStreamSynchronize(h->stream));
-    if (f == 0) return GEVP_OK;
-    CK(cudaMemsetAsync(h->ozflags + 2, 0, sizeof(int), h->stream));
-    h->err = "a bounded wait of the emulated FP64 product ran out";
-    return GEVP_ERR_TIMEOUT;
+    CK(cudaGetLastError());
+    if (f[0] != 0) {
+      CK(cudaMemsetAsync(h->ozflags + 2, 0, sizeof(int), h->stream));
+      h->err = "a bounded wait of the emulated FP64 product ran out";
+      return GEVP_ERR_TIMEOUT;
+    }
+    return heev_status(h, f[1]);
   }
 };
 
@@ -878,7 +890,8 @@ gevp_status rayleigh_ritz(gevp_ctx* h, int64_t n, int nlock, int ma, const doubl
   TRY(times_C(h, n, ma, C, ldc, Qa, h->Wt));
   // G = Q^H C Q is Hermitian: its lower tiles only, both triangles written
   gram(h, n, ma, ma, Qa, ld, h->Wt, ld, h->G, ma, 1);
-  heev_small(ma, h->G, ma, h->theta + nlock, h->Zs, ma, h->hw, refine, h->stream);
+  h->heev_word = heev_small(ma, h->G, ma, h->theta + nlock, h->Zs, ma, h->hw, refine, h->stream);
+  inject(h, 1, h->heev_word, 1);
   // [Q W] <- [Q Wt] Z. Emulated (when C's products are): the two blocks stacked into the
   // free n x n scratch T as one 2n x ma operand, so that one product fills the SMs; else one
   // FP64 launch (a batch of two products sharing Z). Q's result goes through T or Xf (free
@@ -1802,9 +1815,7 @@ gevp_status gevp_cholqr2(gevp_handle h, int64_t n, int m, void* Y, int64_t ldy, 
     gram(h, n, m, m, h->Y1, ld, h->Wt, ld, (double2*)R, ldr, 0);
     zero_lower(m, (double2*)R, ldr, h->stream);
   }
-  CK(cudaStreamSynchronize(h->stream));
-  CK(cudaGetLastError());
-  return em.check();
+  return em.finish();
 }
 
 gevp_status gevp_rayleigh_ritz(gevp_handle h, int64_t n, int m, const void* C, int64_t ldc, void* Q, int64_t ldq,
@@ -1824,9 +1835,7 @@ gevp_status gevp_rayleigh_ritz(gevp_handle h, int64_t n, int m, const void* C, i
   zcopy2d(n, m, h->W, ld, (double2*)W, ldw, h->stream);
   CK(cudaMemcpyAsync(theta, h->theta, m * sizeof(double), cudaMemcpyDeviceToDevice, h->stream));
   CK(cudaMemcpyAsync(res, h->res, m * sizeof(double), cudaMemcpyDeviceToDevice, h->stream));
-  CK(cudaStreamSynchronize(h->stream));
-  CK(cudaGetLastError());
-  return em.check();
+  return em.finish(h->heev_word);
 }
 
 gevp_status gevp_heev_small(gevp_handle h, int m, const void* G, int64_t ldg, double* theta, void* Z, int64_t ldz) {
@@ -1835,10 +1844,14 @@ gevp_status gevp_heev_small(gevp_handle h, int m, const void* G, int64_t ldg, do
   if (!G || !theta || !Z || bad_ld(ldg, m) || bad_ld(ldz, m)) return GEVP_ERR_INVALID_ARG;
   cudaSetDevice(h->device);
   TRY(ensure(h, std::max<int64_t>(m, h->cap_n), m));
-  heev_small(m, (const double2*)G, ldg, theta, (double2*)Z, ldz, h->hw, 3, h->stream);
+  const int* word = heev_small(m, (const double2*)G, ldg, theta, (double2*)Z, ldz, h->hw, 3, h->stream);
+  inject(h, 1, word, 1);
+  int* failed = (int*)h->hbuf;   // pinned
+  *failed = 0;
+  if (word) CK(cudaMemcpyAsync(failed, word, sizeof(int), cudaMemcpyDeviceToHost, h->stream));
   CK(cudaStreamSynchronize(h->stream));
   CK(cudaGetLastError());
-  return GEVP_OK;
+  return heev_status(h, *failed);
 }
 
 gevp_status gevp_spectral_bounds(gevp_handle h, int64_t n, const void* C, int64_t ldc, int k, int count,
@@ -2095,6 +2108,12 @@ gevp_status gevp_reduce_emulated(gevp_handle h, int64_t n, const void* A, int64_
   if (st == GEVP_OK) st = oz_check(h);
   h->oz_slices = keep;
   return st;
+}
+
+gevp_status gevp_inject_failure(gevp_handle h, int what) {
+  if (!h || what < 0 || what > 1) return GEVP_ERR_INVALID_ARG;
+  h->inject = what;
+  return GEVP_OK;
 }
 
 gevp_status gevp_probe_peaks(gevp_handle h, double* out) {

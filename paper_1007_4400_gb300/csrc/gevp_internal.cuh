@@ -158,8 +158,10 @@ struct HeevWork {
   unsigned* gcnt;               // zgram arrival counters (zgram_counters() words, zero)
 };
 size_t heev_ws_bytes(int m, size_t split_elems);
-void heev_small(int m, const double2* G, int64_t ldg, double* theta, double2* Z, int64_t ldz,
-                const HeevWork& w, int refine_iters, cudaStream_t s);
+// Returns the device word (in w) that says after the call whether the FP32 stage failed (0 no, 1 a
+// bounded wait ran out, 2 QL did not converge: theta and Z are NaN then), or null if it has none.
+const int* heev_small(int m, const double2* G, int64_t ldg, double* theta, double2* Z, int64_t ldz,
+                      const HeevWork& w, int refine_iters, cudaStream_t s);
 // FP32 eigenvectors of G (m x m FP32 Hermitian; not modified) in ascending order into the columns
 // of Z (FP64, ld ldz), by tridiagonalisation and QL (tridiag32.cu). Scratch: w (m floats), ctl (4
 // ints), tau (m), sV, sR, sS, sZ (m x m each). may_skip: a nearly diagonal G may give the unit

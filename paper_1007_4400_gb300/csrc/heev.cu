@@ -645,9 +645,10 @@ void cluster_jacobi_batched(const BDesc* D, int np, int zsel, double rel, int ma
   LAUNCH_NOTE(1);
 }
 
-void heev_small(int m, const double2* G, int64_t ldg, double* theta, double2* Zout, int64_t ldz,
-                const HeevWork& w, int refine_iters, cudaStream_t s) {
-  if (m <= 0) return;
+const int* heev_small(int m, const double2* G, int64_t ldg, double* theta, double2* Zout, int64_t ldz,
+                      const HeevWork& w, int refine_iters, cudaStream_t s) {
+  if (m <= 0) return nullptr;
+  const int* failed = (const int*)(w.scal + 16) + 3;
   int64_t mm = (int64_t)m * m;
   int blocks = (int)std::min<int64_t>((mm + 255) / 256, 152 * 4);
   g_to_c_kernel<<<blocks, 256, 0, s>>>(m, G, ldg, w.G32);
@@ -657,6 +658,7 @@ void heev_small(int m, const double2* G, int64_t ldg, double* theta, double2* Zo
   // its limit: Jacobi on all SMs (cooperative launch; E holds its second FP32 buffer), or, when
   // that cannot be launched, in one CTA.
   if (!heev32(m, w.G32, w.Z, m, w.w32, (int*)(w.scal + 16), w.Z32, w.T, w.R, w.S, w.E, refine_iters >= 3 ? 1 : 0, s)) {
+    failed = nullptr;
     bool done = false;
     if (m > kJacobiSmemMax)
       done = jacobi32_coop(m, w.G32, (float2*)w.E, w.Z32, w.w32, w.perm, 40, (float*)(w.scal + 16), s);
@@ -716,6 +718,7 @@ void heev_small(int m, const double2* G, int64_t ldg, double* theta, double2* Zo
   LAUNCH_NOTE(1);
   sort_pairs_kernel<<<1, 1024, 0, s>>>(m, w.lam, Z, theta, Zout, ldz);
   LAUNCH_NOTE(1);
+  return failed;
 }
 
 }  // namespace gevp

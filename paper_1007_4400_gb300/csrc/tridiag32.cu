@@ -35,8 +35,9 @@
 // quadratically, reaches FP64 accuracy in its last step as it would from computed vectors; the
 // clusters go to the exact rotations after it.
 //
-// Every wait on another warp's or CTA's progress is bounded; if one runs out the eigenvectors are
-// written as NaN (the solver then reports that it did not converge).
+// Every wait on another warp's or CTA's progress is bounded, and so are QL's sweeps and their memory;
+// if one runs out the eigenvectors are written as NaN (the solver then reports that it did not
+// converge, the per-step entry points the error).
 #include "gevp_internal.cuh"
 #include <cooperative_groups.h>
 #include <algorithm>
@@ -62,7 +63,7 @@ struct Heev32 {
   int4* sweeps;     // (first column, rotations, offset), m^2
   float* ZT;        // m x m: row j = the tridiagonal's eigenvector j
   float* w;         // eigenvalues (scaled), unsorted
-  int* ctl;         // [0] published sweeps, [1] 1 + all sweeps when done, [2] skipped, [3] failed
+  int* ctl;         // [0] published sweeps, [1] 1 + all sweeps when done, [2] skipped, [3] failed (1 a wait, 2 QL)
   double2* Z;       // result, ld ldz
   int64_t ldz;
 };
@@ -156,7 +157,7 @@ __host__ __device__ inline size_t h_smem(int m, int P) { return h_big(m, P) + (s
 template <class Sink>
 __device__ __forceinline__ void ql_warp(int m, float* d, float* e, int lane, Sink& sink) {
   for (int l = 0; l < m; ++l) {
-    for (int it = 0; it < 60; ++it) {
+    for (int it = 0;; ++it) {
       // the first negligible coupling at or after l
       int mm = m - 1;
       for (int b = l; b < m - 1; b += 32) {
@@ -169,6 +170,10 @@ __device__ __forceinline__ void ql_warp(int m, float* d, float* e, int lane, Sin
         }
       }
       if (mm == l) break;
+      if (it == 60) {   // (two sweeps an eigenvalue are usual)
+        sink.gave_up(fabsf(e[l]));
+        break;
+      }
       if (!sink.room(mm - l)) return;
       const float el = e[l];
       float g = (d[l + 1] - d[l]) / (2.f * el);
@@ -453,8 +458,14 @@ __global__ void __launch_bounds__(HT, 1) heev32_tri_kernel(Src src, int may_skip
       int* failed;
       int m, lane, pos, ns, pos0;
       int64_t cap;
+      __device__ void gave_up(float) {
+        if (lane == 0) *failed = 2;
+      }
       __device__ bool room(int) {
-        if (pos + m > cap || ns + 1 >= m * m) return false;
+        if (pos + m > cap || ns + 1 >= m * m) {
+          gave_up(0.f);
+          return false;
+        }
         int ok = 0;   // lane 0's decision holds for the warp
         if (lane == 0) {
           uint32_t spin = 0;
@@ -685,6 +696,7 @@ __device__ void lanczos_tail(int k, int64_t n, int count, const float* ab, int k
     float* z;
     int lane;
     float f;
+    __device__ void gave_up(float el) { left = fmaxf(left, el); }
     __device__ bool room(int) { return true; }
     __device__ void start(int mm) { f = z[mm]; }
     __device__ void rotation(int i, float c, float s) {
@@ -698,7 +710,8 @@ __device__ void lanczos_tail(int k, int64_t n, int count, const float* ab, int k
       last = -1;
     }
     int last;
-  } sink{z, lane, 0.f, -1};
+    float left;   // the largest coupling that an eigenvalue was left with
+  } sink{z, lane, 0.f, -1, 0.f};
   ql_warp(kk, d, e, lane, sink);
   __syncwarp();
   for (int i = lane; i < kk; i += 32) {
@@ -714,7 +727,7 @@ __device__ void lanczos_tail(int k, int64_t n, int count, const float* ab, int k
   const double beta = ke < 0 ? 0.0 : fabs((double)ab[2 * (kk - 1) + 1]);
   out[0] = tmin;
   out[1] = tmax;
-  out[2] = tmax + beta + 1e-5 * fmax(fabs(tmin), fabs(tmax));
+  out[2] = tmax + beta + 1e-5 * fmax(fabs(tmin), fabs(tmax)) + sink.left * up;
   out[4] = beta;
   double aest = tmax, cum = 0.0;
   if (count > 0)

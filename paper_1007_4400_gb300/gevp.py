@@ -124,6 +124,7 @@ def load(build_if_missing: bool = True):
         L.gevp_assign_min_cost.argtypes = [i32, i32, C.POINTER(f64), C.POINTER(i64)]
         L.gevp_zgemm_emulated.argtypes = [vp, i32, i32, i32, i32, i32, vp, i64, vp, i64, vp, i64, i32]
         L.gevp_reduce_emulated.argtypes = [vp, i64, vp, i64, vp, i64, vp, i64, vp, i64, C.POINTER(i64), i32]
+        L.gevp_inject_failure.argtypes = [vp, i32]
         L.gevp_kernel_timing.argtypes = [i32]
         L.gevp_kernel_timing_read.argtypes = [C.POINTER(f64)]
         L.gevp_kernel_launches.argtypes = [vp]
@@ -133,7 +134,7 @@ def load(build_if_missing: bool = True):
                      "gevp_heev_small", "gevp_spectral_bounds", "gevp_energy_backward", "gevp_band_energy", "gevp_reduce_update",
                      "gevp_probe_peaks",
                      "gevp_matrix_variation", "gevp_deviation_angles", "gevp_assign_min_cost",
-                     "gevp_zgemm_emulated", "gevp_reduce_emulated", "gevp_kernel_timing",
+                     "gevp_zgemm_emulated", "gevp_reduce_emulated", "gevp_inject_failure", "gevp_kernel_timing",
                      "gevp_kernel_timing_read"):
             getattr(L, name).restype = i32
         _LIB = L
@@ -395,6 +396,12 @@ def rayleigh_ritz(Cm: torch.Tensor, Q: torch.Tensor):
                                    _ptr(rs))
     _check(st, h)
     return th, Q, W, rs
+
+
+def inject_failure(what: int, device=None) -> None:
+    """gevp_inject_failure on the device's handle (for tests of error handling)."""
+    h = _handle(torch.device("cuda", torch.cuda.current_device() if device is None else device))
+    _check(load().gevp_inject_failure(h, int(what)), h)
 
 
 def heev_small(G: torch.Tensor):
