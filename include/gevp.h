@@ -279,7 +279,9 @@ gevp_status gevp_band_energy(gevp_handle h, int nprob, int nev, const double* La
  *   GA = gE * X X^H = dE/dA * gE,   GB = -gE * X diag(Lambda) X^H = dE/dB * gE,
  * X n x nev B-orthonormal eigenvectors (ld ldx), Lambda device (nev), gE a DEVICE scalar
  * (the incoming gradient, read on the device: no host synchronisation); GA, GB n x n (ld
- * ldg). Enqueued on the handle's stream; returns without waiting. */
+ * ldg). Enqueued on the handle's stream; returns without waiting, except that a call larger
+ * than any before it on the handle first waits for the device and grows the workspace. If a
+ * bounded wait of an emulated product runs out, GA and GB are NaN. */
 gevp_status gevp_energy_backward(gevp_handle h, int64_t n, int nev, const void* X, int64_t ldx,
                                  const double* Lambda, const double* gE, void* GA, void* GB, int64_t ldg);
 
@@ -374,7 +376,9 @@ gevp_status gevp_reduce_emulated(gevp_handle h, int64_t n, const void* A, int64_
 /* Failure injection on the host, for tests of error handling: the next call on this handle that could
  * report the failure `what` finds its device word set as if it had happened (nothing fails on the
  * device). 1: a bounded wait of the small eigensolver ran out (gevp_heev_small,
- * gevp_rayleigh_ritz). 0: take an injection back. */
+ * gevp_rayleigh_ritz). 2: a bounded wait of an emulated product ran out (gevp_zgemm_emulated,
+ * gevp_cholqr2, gevp_rayleigh_ritz and gevp_energy_backward, where their products are emulated).
+ * 0: take an injection back. */
 gevp_status gevp_inject_failure(gevp_handle h, int what);
 
 /* Measured FP64 FMA, FP64 DMMA and FP32 FMA rates of this device in TFLOP/s (host out[3]). */

@@ -543,6 +543,13 @@ gevp_status oz_check(gevp_ctx* h) {
   return GEVP_ERR_INVALID_VALUE;
 }
 
+// gevp_inject_failure: the device word reads as after the given failure
+void inject(gevp_ctx* h, int what, const int* word, int code) {
+  if (h->inject != what || !word) return;
+  h->inject = 0;
+  cudaMemsetAsync((void*)word, code, 1, h->stream);
+}
+
 // D (M x N) = op(A) op(B) with `slices` digits, operands and residues in the second scratch (the
 // side stream's, free outside a solve): all moduli's residues of both operands, or groups of four
 // where that would take more than a third of the device's memory or cannot be had. A Gram
@@ -588,7 +595,9 @@ cudaError_t em_enqueue(gevp_ctx* h, int opA, int opB, int M, int N, int K, const
     GEVP_CUDA_TRY(gevp::oz_split(b, mem + opb(M, group), N, K, B, ldb, opB, 0, slices, flags + 1, h->stream, opB == 0,
                                  nullptr, group, ks, 1));
   }
-  return gevp::oz_gemm(a, b, 0, triB, D, ldd, flags, h->stream, nullptr, h->ozmem[1], work, triD);
+  const cudaError_t e = gevp::oz_gemm(a, b, 0, triB, D, ldd, flags, h->stream, nullptr, h->ozmem[1], work, triD);
+  inject(h, 2, flags, 24);
+  return e;
 }
 
 // Per-step entry points (h->em): the FP64 pipe's rate (1.05 TFLOP/s) against the emulated product's
@@ -649,13 +658,6 @@ bool gram(gevp_ctx* h, int64_t n, int mx, int my, const double2* X, int64_t ldx,
   }
   zgram(n, mx, my, X, ldx, Y, ldy, G, ldg, herm, h->split, h->split_elems, h->gcnt, s);
   return false;
-}
-
-// gevp_inject_failure: the device word reads as after the given failure
-void inject(gevp_ctx* h, int what, const int* word, int code) {
-  if (h->inject != what || !word) return;
-  h->inject = 0;
-  cudaMemsetAsync((void*)word, code, 1, h->stream);
 }
 
 // the status that the small eigensolver's failure word stands for
@@ -1885,13 +1887,16 @@ gevp_status gevp_energy_backward(gevp_handle h, int64_t n, int nev, const void* 
   EmScope em(h);
   const double2* Xd = (const double2*)X;
   if (em_product(h, 0, 1, n, n, nev, Xd, ldx, Xd, ldx, 0, 1, (double2*)GA, ldg)) {
-    hermitize_scale_lower(n, (double2*)GA, ldg, gE, 1.0, h->stream);
+    // the call does not wait, so the products' error word is read on the device: it turns the gradients
+    // into NaN and is cleared behind them
+    const int* error = h->ozflags + 2;
+    hermitize_scale_lower(n, (double2*)GA, ldg, gE, 1.0, h->stream, error);
     scale_by_lam(n, nev, Xd, ldx, Lambda, h->T, h->stream);
-    if (em_product(h, 0, 1, n, n, nev, h->T, nev, Xd, ldx, 0, 1, (double2*)GB, ldg)) {
-      hermitize_scale_lower(n, (double2*)GB, ldg, gE, -1.0, h->stream);
-      CK(cudaGetLastError());
-      return GEVP_OK;
-    }
+    const bool both = em_product(h, 0, 1, n, n, nev, h->T, nev, Xd, ldx, 0, 1, (double2*)GB, ldg);
+    if (both) hermitize_scale_lower(n, (double2*)GB, ldg, gE, -1.0, h->stream, error);
+    CK(cudaMemsetAsync(h->ozflags + 2, 0, sizeof(int), h->stream));
+    CK(cudaGetLastError());
+    if (both) return GEVP_OK;
   }
   gevp::energy_backward_ws(n, nev, Xd, ldx, Lambda, gE, (double2*)GA, (double2*)GB, ldg, h->T, h->split,
                            h->split_elems, h->stream);
@@ -2111,7 +2116,7 @@ gevp_status gevp_reduce_emulated(gevp_handle h, int64_t n, const void* A, int64_
 }
 
 gevp_status gevp_inject_failure(gevp_handle h, int what) {
-  if (!h || what < 0 || what > 1) return GEVP_ERR_INVALID_ARG;
+  if (!h || what < 0 || what > 2) return GEVP_ERR_INVALID_ARG;
   h->inject = what;
   return GEVP_OK;
 }

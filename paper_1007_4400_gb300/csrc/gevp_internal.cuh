@@ -115,7 +115,8 @@ void zero_lower(int64_t n, double2* A, int64_t lda, cudaStream_t s);        // s
 void hermitize_lower(int64_t n, double2* C, int64_t ldc, cudaStream_t s);   // upper <- conj(lower), real diag
 void hermitize_avg(int64_t n, double2* C, int64_t ldc, cudaStream_t s);     // C <- (C + C^H)/2
 // lower triangle scaled by sign * (*scale) (device scalar), then upper <- conj(lower)
-void hermitize_scale_lower(int64_t n, double2* C, int64_t ldc, const double* scale, double sign, cudaStream_t s);
+void hermitize_scale_lower(int64_t n, double2* C, int64_t ldc, const double* scale, double sign, cudaStream_t s,
+                           const int* error = nullptr);
 // C <- C + D on the lower triangle, then upper <- conj(lower), real diagonal
 void add_lower_herm(int64_t n, double2* C, int64_t ldc, const double2* D, int64_t ldd, cudaStream_t s);
 // Out[i][t] = X[i][idx[t]] (rows x k) and Out[t][j] = X[idx[t]][j] (k x cols); idx device

@@ -52,9 +52,11 @@ __global__ void hermitize_lower_kernel(int64_t n, double2* C, int64_t ldc) {
   }
 }
 
-// lower triangle scaled by sign * (*scale) (a device scalar), upper <- conj(lower), real diagonal
-__global__ void hermitize_scale_lower_kernel(int64_t n, double2* C, int64_t ldc, const double* scale, double sign) {
-  const double f = sign * scale[0];
+// lower triangle scaled by sign * (*scale) (a device scalar), upper <- conj(lower), real diagonal; NaN
+// where the error word of the product that wrote the triangle is set (nullable)
+__global__ void hermitize_scale_lower_kernel(int64_t n, double2* C, int64_t ldc, const double* scale, double sign,
+                                             const int* error) {
+  const double f = error && *error != 0 ? __longlong_as_double(0x7ff8000000000000ll) : sign * scale[0];
   int64_t total = n * n;
   for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < total; e += (int64_t)gridDim.x * blockDim.x) {
     int64_t i = e / n, j = e % n;
@@ -267,8 +269,9 @@ void hermitize_lower(int64_t n, double2* C, int64_t ldc, cudaStream_t s) {
   hermitize_lower_kernel<<<grid_for(n * n), kThreads, 0, s>>>(n, C, ldc);
   LAUNCH_NOTE(1);
 }
-void hermitize_scale_lower(int64_t n, double2* C, int64_t ldc, const double* scale, double sign, cudaStream_t s) {
-  hermitize_scale_lower_kernel<<<grid_for(n * n), kThreads, 0, s>>>(n, C, ldc, scale, sign);
+void hermitize_scale_lower(int64_t n, double2* C, int64_t ldc, const double* scale, double sign, cudaStream_t s,
+                           const int* error) {
+  hermitize_scale_lower_kernel<<<grid_for(n * n), kThreads, 0, s>>>(n, C, ldc, scale, sign, error);
   LAUNCH_NOTE(1);
 }
 void add_lower_herm(int64_t n, double2* C, int64_t ldc, const double2* D, int64_t ldd, cudaStream_t s) {

@@ -32,3 +32,30 @@ def test_rayleigh_ritz(cuda, n, m):
         gevp.rayleigh_ritz(C, Q.clone())
     assert e.value.name == "GEVP_ERR_TIMEOUT"
     gevp.rayleigh_ritz(C, Q.clone())
+
+
+def test_gradient_products(cuda):
+    """The gradient's call does not wait: its own results are NaN, and the failure is not reported by
+    the next call that waits."""
+    from paper_1007_4400_gb300 import gevp
+    n, nev = 1024, 64
+    X = torch.randn(n, nev, dtype=torch.complex128, device=cuda)
+    lam = torch.linspace(-1, 1, nev, dtype=torch.float64, device=cuda)
+    ref = gevp.energy_backward(X, lam)
+    gevp.inject_failure(2)
+    for G in gevp.energy_backward(X, lam):
+        assert torch.isnan(G.real).all()
+    gevp.cholqr2(X.clone())
+    for G, R in zip(gevp.energy_backward(X, lam), ref):
+        assert torch.equal(torch.view_as_real(G), torch.view_as_real(R))
+
+
+def test_products_that_wait(cuda):
+    from paper_1007_4400_gb300 import gevp
+    X = torch.randn(1024, 96, dtype=torch.complex128, device=cuda)
+    for call in (lambda: gevp.cholqr2(X.clone()), lambda: gevp.zgemm_emulated(X, X, opA="C", opB="N")):
+        gevp.inject_failure(2)
+        with pytest.raises(gevp.GevpError) as e:
+            call()
+        assert e.value.name == "GEVP_ERR_TIMEOUT"
+        call()
