@@ -1110,9 +1110,9 @@ extern "C" gevp_status gevp_solve_batched(gevp_handle h, int nk, int nsteps, con
     BCK(cudaEventRecord(evt(P, EV_RED), s));
     // ---- bounds of C (and ||A||_2)
     bk_to_c32(P->dD, np, P->nmax, 0, s);
-    bk_lanczos(P->dD, np, P->nmax, kl, 1, 0, o.seed + 7919ull * l, s);
+    BCK(bk_lanczos(P->dD, np, P->nmax, kl, 1, 0, o.seed + 7919ull * l, s));
     bk_to_c32(P->dD, np, P->nmax, 1, s);
-    bk_lanczos(P->dD, np, P->nmax, kl, 0, 12, o.seed + 104729ull * l + 1, s);
+    BCK(bk_lanczos(P->dD, np, P->nmax, kl, 0, 12, o.seed + 104729ull * l + 1, s));
     bk_post_bounds(P->dD, np, s);
     if (tc) tcg_set_matrix(P->dD, np, (int64_t)P->tg.n_pad_max * P->tg.n_pad_max, s);
     // ---- start block

@@ -837,19 +837,25 @@ void bk_post_bounds(const BDesc* D, int np, cudaStream_t s) {
   b_post_bounds<<<(np + 63) / 64, 64, 0, s>>>(D, np);
   LAUNCH_NOTE(1);
 }
-void bk_lanczos(const BDesc* D, int np, int64_t nmax, int k, int use_count, int out_off, uint64_t seed,
+cudaError_t bk_lanczos(const BDesc* D, int np, int64_t nmax, int k, int use_count, int out_off, uint64_t seed,
                 cudaStream_t s) {
   b_lanczos_init<<<np, 1024, 0, s>>>(D, seed);
   LAUNCH_NOTE(1);
   const int rows_per_block = 8;
   const int blocks = (int)std::max<int64_t>(1, std::min<int64_t>((nmax + rows_per_block - 1) / rows_per_block, 256));
-  if (!lanczos_batched(D, np, nmax, 0, k, 1, s))
+  if (lanczos_whole(nmax)) {
+    const cudaError_t e = lanczos_batched(D, np, nmax, 0, k, 1, s);
+    if (e != cudaSuccess) return e;
+  } else {
     for (int j = 0; j < k; ++j) {
       b_matvec32<<<dim3(blocks, np), 32 * rows_per_block, 0, s>>>(D, j);
       LAUNCH_NOTE(1);
-      lanczos_batched(D, np, nmax, j, j + 1, 0, s);
+      const cudaError_t e = lanczos_batched(D, np, nmax, j, j + 1, 0, s);
+      if (e != cudaSuccess) return e;
     }
+  }
   lanczos_tail_batched(D, np, k, use_count, KMAX, out_off, s);
+  return cudaGetLastError();
 }
 void bk_heev_prep(const BDesc* D, int np, int mmax, cudaStream_t s) {
   b_g_to_c<<<g2((int64_t)mmax * mmax, np), 256, 0, s>>>(D);

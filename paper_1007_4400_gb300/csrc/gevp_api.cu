@@ -936,7 +936,7 @@ double2* filter_fp64(gevp_ctx* h, int64_t n, const double2* C, int64_t ldc, cons
 gevp_status lanczos(gevp_ctx* h, int64_t n, const double2* M, int64_t ldm, int k, int count, uint64_t seed,
                     double* host_out) {
   z_to_c(n, n, M, ldm, h->M32, n, h->stream);
-  lanczos_bounds(n, h->M32, n, k, count, seed, h->lw, h->bounds, h->stream);
+  CK(lanczos_bounds(n, h->M32, n, k, count, seed, h->lw, h->bounds, h->stream));
   return sync_read(h, h->bounds, host_out, 5 * sizeof(double));
 }
 
@@ -1255,9 +1255,9 @@ gevp_status prefetch_problem(gevp_ctx* h, int64_t n, int m, const double2* A, in
   else
     reduce_into_ws(n, h->Linv, A, lda, h->C2, n, h->T2, h->split2, h->split2_elems, h->side);
   z_to_c(n, n, h->C2, n, h->M32b, n, h->side);
-  lanczos_bounds(n, h->M32b, n, o.lanczos_steps, m, o.seed + 7919ull * idx, h->lw2, h->bounds2, h->side);
+  CK(lanczos_bounds(n, h->M32b, n, o.lanczos_steps, m, o.seed + 7919ull * idx, h->lw2, h->bounds2, h->side));
   z_to_c(n, n, A, lda, h->M32b, n, h->side);
-  lanczos_bounds(n, h->M32b, n, o.lanczos_steps, 0, o.seed + 104729ull * idx + 1, h->lw2, h->bounds2 + 8, h->side);
+  CK(lanczos_bounds(n, h->M32b, n, o.lanczos_steps, 0, o.seed + 104729ull * idx + 1, h->lw2, h->bounds2 + 8, h->side));
   CK(cudaMemcpyAsync(h->hb2, h->bounds2, 16 * sizeof(double), cudaMemcpyDeviceToHost, h->side));
   if (o.filter_prec != GEVP_PREC_FP64) {
     CK(filter_tc_reserve(&h->tc2, n, m, h->side));

@@ -180,7 +180,7 @@ size_t lanczos_ws_bytes(int64_t n, int k);
 // k-step Lanczos with full re-orthogonalisation on the FP32 copy of a Hermitian matrix.
 // Writes to dev_out[0..4] = {theta_min, theta_max, upper bound, estimate of the count-th
 // eigenvalue from the Ritz-weight density, |beta_k|}. count <= 0 skips the estimate.
-void lanczos_bounds(int64_t n, const float2* M32, int64_t ldm, int k, int count, uint64_t seed,
+cudaError_t lanczos_bounds(int64_t n, const float2* M32, int64_t ldm, int k, int count, uint64_t seed,
                     const LanczosWork& w, double* dev_out, cudaStream_t s);
 
 struct BDesc;
@@ -320,7 +320,7 @@ void bk_copy_nm(const BDesc* D, int np, int64_t nm_max, int from, int to, cudaSt
 void bk_potrf_small(const BDesc* D, int np, cudaStream_t s);
 void bk_trtri_small(const BDesc* D, int np, cudaStream_t s);
 void bk_step_reset(const BDesc* D, int np, double tol, int filter64, cudaStream_t s);
-void bk_lanczos(const BDesc* D, int np, int64_t nmax, int k, int use_count, int out_off, uint64_t seed,
+cudaError_t bk_lanczos(const BDesc* D, int np, int64_t nmax, int k, int use_count, int out_off, uint64_t seed,
                 cudaStream_t s);
 void bk_post_bounds(const BDesc* D, int np, cudaStream_t s);
 void bk_heev_prep(const BDesc* D, int np, int mmax, cudaStream_t s);
@@ -343,7 +343,8 @@ size_t bk_partial_elems(int m);
 // where that cannot be launched (mmax > 600), Jacobi into Z32 / w32 / perm; the Lanczos ends
 bool heev32_batched(const BDesc* D, int np, int mmax, cudaStream_t s);
 void jacobi32_batched(const BDesc* D, int np, int mmax, int max_sweeps, cudaStream_t s);
-bool lanczos_batched(const BDesc* D, int np, int64_t nmax, int j0, int k, int full, cudaStream_t s);
+bool lanczos_whole(int64_t nmax);   // whole runs in one launch (full), not a launch a step
+cudaError_t lanczos_batched(const BDesc* D, int np, int64_t nmax, int j0, int k, int full, cudaStream_t s);
 void lanczos_tail_batched(const BDesc* D, int np, int k, int use_count, int k_max, int out_off, cudaStream_t s);
 void cluster_jacobi_batched(const BDesc* D, int np, int zsel, double rel, int max_sweeps, cudaStream_t s);
 

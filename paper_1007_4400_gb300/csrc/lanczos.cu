@@ -240,32 +240,47 @@ __global__ void __launch_bounds__(LT, 1) lanczos_cluster_kernel(Src src, int j0,
 }
 
 template <class Src>
-void run_cluster(const Src& src, int np, int64_t nmax, int j0, int k, int full, cudaStream_t s) {
+cudaError_t run_cluster(const Src& src, int np, int64_t nmax, int j0, int k, int full, cudaStream_t s) {
   static std::atomic<int> most[64];   // CTAs of a cluster that a device takes (0: not asked yet)
   int dev = 0;
   cudaGetDevice(&dev);
+  cudaLaunchConfig_t cfg{};
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeClusterDimension;
+  at.val.clusterDim.y = at.val.clusterDim.z = 1;
+  cfg.blockDim = dim3(LT);
+  cfg.stream = s;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
   int top = dev < 64 ? most[dev].load(std::memory_order_relaxed) : 0;
   if (top == 0) {
-    cudaFuncSetAttribute(lanczos_cluster_kernel<Src>, cudaFuncAttributeMaxDynamicSharedMemorySize, kLanczosSmem);
-    top = cudaFuncSetAttribute(lanczos_cluster_kernel<Src>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) ==
-                  cudaSuccess ? kLanczosCta : 8;
+    cudaError_t e = cudaFuncSetAttribute(lanczos_cluster_kernel<Src>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         kLanczosSmem);
+    if (e != cudaSuccess) return e;
+    // sixteen, or the largest power of two below it that the device schedules
+    top = kLanczosCta;
+    if (cudaFuncSetAttribute(lanczos_cluster_kernel<Src>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) !=
+        cudaSuccess)
+      top = 8;
+    cfg.dynamicSmemBytes = kLanczosSmem;
+    for (; top > 1; top /= 2) {
+      int clusters = 0;
+      at.val.clusterDim.x = top;
+      cfg.gridDim = dim3((unsigned)top);
+      if (cudaOccupancyMaxActiveClusters(&clusters, lanczos_cluster_kernel<Src>, &cfg) == cudaSuccess && clusters > 0)
+        break;
+    }
+    cudaGetLastError();
     if (dev < 64) most[dev].store(top, std::memory_order_relaxed);
   }
   int C = 1;   // 64 rows a CTA
   while (C < top && (int64_t)C * 64 < nmax) C *= 2;
-  cudaLaunchConfig_t cfg{};
-  cudaLaunchAttribute at{};
-  at.id = cudaLaunchAttributeClusterDimension;
   at.val.clusterDim.x = C;
-  at.val.clusterDim.y = at.val.clusterDim.z = 1;
   cfg.gridDim = dim3((unsigned)(np * C));
-  cfg.blockDim = dim3(LT);
   cfg.dynamicSmemBytes = (size_t)((nmax + C - 1) / C + (full ? nmax : 0)) * sizeof(float2);
-  cfg.stream = s;
-  cfg.attrs = &at;
-  cfg.numAttrs = 1;
-  cudaLaunchKernelEx(&cfg, lanczos_cluster_kernel<Src>, src, j0, k, full);
-  LAUNCH_NOTE(1);
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, lanczos_cluster_kernel<Src>, src, j0, k, full);
+  if (e == cudaSuccess) LAUNCH_NOTE(1);
+  return e;
 }
 
 }  // namespace
@@ -287,30 +302,31 @@ size_t lanczos_ws_bytes(int64_t n, int k) {
 bool lanczos_whole(int64_t nmax) { return nmax <= 2304; }
 
 // the steps of a batch's problems (V[0] is there)
-bool lanczos_batched(const BDesc* D, int np, int64_t nmax, int j0, int k, int full, cudaStream_t s) {
-  if (full && !lanczos_whole(nmax)) return false;
-  run_cluster(LanczosSrcBatch{D}, np, nmax, j0, k, full, s);
-  return true;
+cudaError_t lanczos_batched(const BDesc* D, int np, int64_t nmax, int j0, int k, int full, cudaStream_t s) {
+  return run_cluster(LanczosSrcBatch{D}, np, nmax, j0, k, full, s);
 }
 
-void lanczos_bounds(int64_t n, const float2* M32, int64_t ldm, int k, int count, uint64_t seed,
+cudaError_t lanczos_bounds(int64_t n, const float2* M32, int64_t ldm, int k, int count, uint64_t seed,
                     const LanczosWork& w, double* dev_out, cudaStream_t s) {
   k = std::max(1, std::min<int>(k, (int)std::min<int64_t>(n, KMAX)));
   lanczos_init_kernel<<<1, 1024, 0, s>>>(n, w.V, seed, w.ab);
   LAUNCH_NOTE(1);
   const LanczosSrcOne src{{n, M32, ldm, w.V, w.w, w.ab}};
   if (lanczos_whole(n)) {
-    run_cluster(src, 1, n, 0, k, 1, s);
+    const cudaError_t e = run_cluster(src, 1, n, 0, k, 1, s);
+    if (e != cudaSuccess) return e;
   } else {
     const int rows_per_block = 8;
     const int blocks = (int)((n + rows_per_block - 1) / rows_per_block);
     for (int j = 0; j < k; ++j) {
       matvec32_kernel<<<blocks, 32 * rows_per_block, 0, s>>>(n, M32, ldm, w.V + (int64_t)j * n, w.w);
       LAUNCH_NOTE(1);
-      run_cluster(src, 1, n, j, j + 1, 0, s);
+      const cudaError_t e = run_cluster(src, 1, n, j, j + 1, 0, s);
+      if (e != cudaSuccess) return e;
     }
   }
   lanczos_tail(k, n, count, w.ab, KMAX, dev_out, s);
+  return cudaGetLastError();
 }
 
 }  // namespace gevp
