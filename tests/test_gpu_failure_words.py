@@ -52,7 +52,7 @@ def test_gradient_products(cuda):
 
 def test_products_that_wait(cuda):
     from paper_1007_4400_gb300 import gevp
-    X = torch.randn(1024, 96, dtype=torch.complex128, device=cuda)
+    X = torch.randn(2048, 128, dtype=torch.complex128, device=cuda)   # Gram matrix emulated
     for call in (lambda: gevp.cholqr2(X.clone()), lambda: gevp.zgemm_emulated(X, X, opA="C", opB="N")):
         gevp.inject_failure(2)
         with pytest.raises(gevp.GevpError) as e:
