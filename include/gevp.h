@@ -378,6 +378,8 @@ gevp_status gevp_reduce_emulated(gevp_handle h, int64_t n, const void* A, int64_
  * device). 1: a bounded wait of the small eigensolver ran out (gevp_heev_small,
  * gevp_rayleigh_ritz). 2: a bounded wait of an emulated product ran out (gevp_zgemm_emulated,
  * gevp_cholqr2, gevp_rayleigh_ritz and gevp_energy_backward, where their products are emulated).
+ * 3, 4: the emulated products' scratch of the main stream, of the second stream cannot be had for
+ * all moduli at once (their operands are then kept for groups of four; no call fails).
  * 0: take an injection back. */
 gevp_status gevp_inject_failure(gevp_handle h, int what);
 

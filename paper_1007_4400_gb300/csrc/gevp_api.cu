@@ -71,7 +71,7 @@ struct gevp_ctx {
   int oz_group[2] = {0, 0};                 // moduli per group the operands are kept in (0: all of them)
   int64_t oz_n[2] = {0, 0};                 // order the scratch was last prepared for
   int oz_S[2] = {0, 0};
-  int64_t oz_full_max = INT64_MAX;          // order from which on only a group's planes are kept
+  bool oz_lean[2] = {false, false};         // this call keeps only a group's planes on that side
   gevp::OzOperand ozLA, ozLB, ozAB[2], ozTA[2];
   // solver products on the main stream: C (rows, per problem), A (rows, per final check),
   // B (rows, kept while the factorisation is), the block (columns, per product)
@@ -253,6 +253,18 @@ gevp_status ensure(gevp_ctx* h, int64_t n, int m) {
   return GEVP_OK;
 }
 
+// ---------------------------------------------------------------- injected failures
+// whether gevp_inject_failure asked for this one (once)
+bool injected(gevp_ctx* h, int what) {
+  if (h->inject != what) return false;
+  h->inject = 0;
+  return true;
+}
+// the device word reads as after the given failure
+void inject(gevp_ctx* h, int what, const int* word, int code) {
+  if (word && injected(h, what)) cudaMemsetAsync((void*)word, code, 1, h->stream);
+}
+
 // ---------------------------------------------------------------- phase timing
 enum Phase { PH_CHOL, PH_REDUCE, PH_BOUNDS, PH_FILTER, PH_ORTH, PH_RR, PH_RESID, PH_FINAL, PH_N };
 
@@ -388,10 +400,37 @@ gevp_status oz_flags_ready(gevp_ctx* h) {
 // stream); side stream: 0 tril(A), 1 T.
 // A region holds the residues of all moduli (64 bytes per entry at 8 digits), unless that
 // would take more than a third of the device's memory or cannot be had: then those of a group
-// of four (16 bytes per entry), rewritten from the matrix for every product.
+// of four (16 bytes per entry), rewritten from the matrix for every product. Each side decides for
+// itself and for one call of an entry point: the next call tries again, and the operands of one
+// side stay where they are when the other cannot grow.
 size_t oz_result_bytes(int64_t n, int S) {
   const size_t panel = gevp::oz_work_bytes(256, (int)n, (int)n, S);
   return al(std::max(panel, std::min<size_t>(gevp::oz_work_bytes((int)n, (int)n, (int)n, S), (size_t)1 << 30)));
+}
+// at least `bytes` of scratch on a side (its contents are lost); optional: not at the cost of what
+// is there, when that much memory is not to be had (cudaErrorMemoryAllocation, nothing changed)
+cudaError_t oz_grow(gevp_ctx* h, int side, size_t bytes, bool optional) {
+  if (optional && injected(h, 3 + side)) return cudaErrorMemoryAllocation;
+  if (optional && h->ozmem[side]) {
+    size_t avail = 0, total = 0;
+    GEVP_CUDA_TRY(cudaMemGetInfo(&avail, &total));
+    if (avail + h->ozmem_bytes[side] < bytes) return cudaErrorMemoryAllocation;
+  }
+  // the other stream may still read this side's (or, for side 0, the shared) operands
+  cudaDeviceSynchronize();
+  if (h->ozmem[side]) cudaFree(h->ozmem[side]);
+  h->ozmem[side] = nullptr;
+  h->ozmem_bytes[side] = 0;
+  h->oz_n[side] = 0;
+  void* p = nullptr;
+  const cudaError_t e = cudaMalloc(&p, bytes);
+  if (e != cudaSuccess) {
+    cudaGetLastError();
+    return e;
+  }
+  h->ozmem[side] = (char*)p;
+  h->ozmem_bytes[side] = bytes;
+  return cudaSuccess;
 }
 size_t oz_region_bytes(const gevp_ctx* h, int side, int64_t n) {
   return al(gevp::oz_operand_bytes((int)n, (int)n, h->oz_slices, h->oz_group[side]));
@@ -399,30 +438,17 @@ size_t oz_region_bytes(const gevp_ctx* h, int side, int64_t n) {
 gevp_status oz_prepare(gevp_ctx* h, int side, int64_t n) {
   TRY(oz_flags_ready(h));
   const int S = h->oz_slices, regions = side == 0 ? h->oz_regions : 2;
-  if (n < h->oz_full_max) {
-    const size_t full = regions * al(gevp::oz_operand_bytes((int)n, (int)n, S, 0));
-    if (full > h->total_mem / 3) h->oz_full_max = n;
-  }
-  for (int pass = 0; pass < 2; ++pass) {
-    const int group = (pass == 0 && n < h->oz_full_max) ? 0 : 4;
+  if (h->oz_regions * al(gevp::oz_operand_bytes((int)n, (int)n, S, 0)) > h->total_mem / 3) h->oz_lean[side] = true;
+  for (;;) {
+    const int group = h->oz_lean[side] ? 4 : 0;
     const size_t need = oz_result_bytes(n, S) + regions * al(gevp::oz_operand_bytes((int)n, (int)n, S, group));
     if (need > h->ozmem_bytes[side]) {
-      // the other stream may still read this side's (or, for side 0, the shared) operands
-      cudaDeviceSynchronize();
-      if (h->ozmem[side]) cudaFree(h->ozmem[side]);
-      h->ozmem[side] = nullptr;
-      h->ozmem_bytes[side] = 0;
-      h->oz_n[side] = 0;
-      void* p = nullptr;
-      const cudaError_t e = cudaMalloc(&p, need);
+      const cudaError_t e = oz_grow(h, side, need, group == 0);
       if (e == cudaErrorMemoryAllocation && group == 0) {
-        cudaGetLastError();
-        h->oz_full_max = n;
+        h->oz_lean[side] = true;
         continue;
       }
       CK(e);
-      h->ozmem[side] = (char*)p;
-      h->ozmem_bytes[side] = need;
     }
     if (h->oz_n[side] != n || h->oz_S[side] != S || h->oz_group[side] != group) {
       if (side == 0) {
@@ -437,7 +463,6 @@ gevp_status oz_prepare(gevp_ctx* h, int side, int64_t n) {
     }
     return GEVP_OK;
   }
-  return GEVP_ERR_OOM;
 }
 char* oz_region(gevp_ctx* h, int64_t n, int which, int side = 0) {
   return h->ozmem[side] + oz_result_bytes(n, h->oz_slices) + which * oz_region_bytes(h, side, n);
@@ -543,13 +568,6 @@ gevp_status oz_check(gevp_ctx* h) {
   return GEVP_ERR_INVALID_VALUE;
 }
 
-// gevp_inject_failure: the device word reads as after the given failure
-void inject(gevp_ctx* h, int what, const int* word, int code) {
-  if (h->inject != what || !word) return;
-  h->inject = 0;
-  cudaMemsetAsync((void*)word, code, 1, h->stream);
-}
-
 // D (M x N) = op(A) op(B) with `slices` digits, operands and residues in the second scratch (the
 // side stream's, free outside a solve): all moduli's residues of both operands, or groups of four
 // where that would take more than a third of the device's memory or cannot be had. A Gram
@@ -565,20 +583,9 @@ cudaError_t em_enqueue(gevp_ctx* h, int opA, int opB, int M, int N, int K, const
   const size_t work = al(std::max(panel, std::min<size_t>(gevp::oz_work_bytes(M, N, K, slices), (size_t)1 << 30)));
   int group = need(0) > h->total_mem / 3 ? 4 : 0;
   for (; work + need(group) > h->ozmem_bytes[1]; group = 4) {
-    cudaDeviceSynchronize();
-    if (h->ozmem[1]) cudaFree(h->ozmem[1]);
-    h->ozmem[1] = nullptr;
-    h->ozmem_bytes[1] = 0;
-    void* p = nullptr;
-    const cudaError_t e = cudaMalloc(&p, work + need(group));
-    if (e == cudaErrorMemoryAllocation && group == 0) {
-      cudaGetLastError();
-      continue;
-    }
-    if (e != cudaSuccess) return e;
-    h->ozmem[1] = (char*)p;
-    h->ozmem_bytes[1] = work + need(group);
-    break;
+    const cudaError_t e = oz_grow(h, 1, work + need(group), group == 0);
+    if (e == cudaSuccess) break;
+    if (e != cudaErrorMemoryAllocation || group != 0) return e;
   }
   h->oz_n[1] = 0;   // the side stream's regions are laid out anew
   char* mem = h->ozmem[1] + work;
@@ -1432,6 +1439,7 @@ gevp_status gevp_reduce_update(gevp_handle h, int64_t n, const void* B, int64_t 
     return GEVP_ERR_UNSUPPORTED;
   }
   TRY(ensure(h, n, k));
+  h->oz_lean[0] = h->oz_lean[1] = false;
   if (!(reuse_factor && h->chol_valid && h->upd_B == B && h->upd_n == n && h->upd_gen == h->chol_gen)) {
     h->upd_B = nullptr;
     TRY(factor_B(h, n, (const double2*)B, ldb, info));
@@ -1564,6 +1572,7 @@ gevp_status gevp_solve_sequence(gevp_handle h, int nprob, int64_t n, const void*
     ~OzScope() { h->oz_slices = 0; }
   } oz_scope{h};
   h->oz_slices = o.reduce_slices;
+  h->oz_lean[0] = h->oz_lean[1] = false;
   TRY(ensure(h, n, m));
   TRY(ensure_pipeline(h));
   PipelineScope pipe(h);
@@ -2108,6 +2117,7 @@ gevp_status gevp_reduce_emulated(gevp_handle h, int64_t n, const void* A, int64_
   const int keep = h->oz_slices;
   h->oz_slices = slices;
   h->oz_regions = 3;
+  h->oz_lean[0] = h->oz_lean[1] = false;
   gevp_status st = gevp_reduce(h, n, A, lda, B, ldb, L, ldl, C, ldc, info);
   h->oz_regions = 6;
   if (st == GEVP_OK) st = oz_check(h);
@@ -2116,7 +2126,7 @@ gevp_status gevp_reduce_emulated(gevp_handle h, int64_t n, const void* A, int64_
 }
 
 gevp_status gevp_inject_failure(gevp_handle h, int what) {
-  if (!h || what < 0 || what > 2) return GEVP_ERR_INVALID_ARG;
+  if (!h || what < 0 || what > 4) return GEVP_ERR_INVALID_ARG;
   h->inject = what;
   return GEVP_OK;
 }
