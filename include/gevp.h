@@ -27,7 +27,12 @@
  *    a one-line message for the last failure on a handle.
  *  - A handle is not thread-safe; use one handle per host thread.
  *  - Workspace belongs to the handle, is sized lazily, grows and is released by
- *    gevp_destroy.
+ *    gevp_destroy. With emulated products it is large: gevp_solve_sequence keeps about
+ *    690 n^2 bytes (100 GB at n = 12000; 180 n^2 without), gevp_solve_batched about 350 n^2 for
+ *    every k-point and four lanes of up to 140 n^2 + 1 GiB for the largest. When the device has no
+ *    memory left, the one that grows gives the other up (its next call makes it again), then keeps
+ *    the operands of the emulated products for groups of moduli (a quarter of their memory,
+ *    slower), then returns GEVP_ERR_OOM.
  */
 #ifndef GEVP_H
 #define GEVP_H
@@ -379,7 +384,8 @@ gevp_status gevp_reduce_emulated(gevp_handle h, int64_t n, const void* A, int64_
  * gevp_rayleigh_ritz). 2: a bounded wait of an emulated product ran out (gevp_zgemm_emulated,
  * gevp_cholqr2, gevp_rayleigh_ritz and gevp_energy_backward, where their products are emulated).
  * 3, 4: the emulated products' scratch of the main stream, of the second stream cannot be had for
- * all moduli at once (their operands are then kept for groups of four; no call fails).
+ * all moduli at once (their operands are then kept for groups of four; no call fails). 5: the
+ * next growth of a workspace finds no memory at its first attempt.
  * 0: take an injection back. */
 gevp_status gevp_inject_failure(gevp_handle h, int what);
 

@@ -287,7 +287,7 @@ gevp_status build_plan(gevp_ctx* h, BatchPlan* P, std::string& err) {
   };
   size_t bytes = layout(nullptr);
   void* mem = nullptr;
-  cudaError_t e = cudaMalloc(&mem, bytes);
+  cudaError_t e = ctx_plan_malloc(h, &mem, bytes);
   if (e != cudaSuccess) {
     err = "batched workspace cudaMalloc failed";
     return e == cudaErrorMemoryAllocation ? GEVP_ERR_OOM : GEVP_ERR_CUDA;
@@ -454,7 +454,7 @@ gevp_status build_plan(gevp_ctx* h, BatchPlan* P, std::string& err) {
   }
   P->pool_items = total + np;
   P->tune_items = largest;
-  e = cudaMalloc(&P->pool, (P->pool_items + P->tune_items) * sizeof(ZgemmItem));
+  e = ctx_plan_malloc(h, (void**)&P->pool, (P->pool_items + P->tune_items) * sizeof(ZgemmItem));
   if (e != cudaSuccess) { err = "item pool cudaMalloc failed"; return GEVP_ERR_OOM; }
   P->tune_pool = P->pool + P->pool_items;
   // every call's list is there from the start: a call may first run after the plan counts as tuned (a
@@ -901,10 +901,10 @@ extern "C" gevp_status gevp_solve_batched(gevp_handle h, int nk, int nsteps, con
       }
       ws = al256(ws);
       const size_t lane = 2 * big + tall + small + ws;
-      e = cudaMalloc(&P->oz_mem, mem);
-      if (e == cudaSuccess) e = cudaMalloc(&P->oz_cq, cq);
-      if (e == cudaSuccess) e = cudaMalloc(&P->oz_fin, fb);
-      if (e == cudaSuccess) e = cudaMalloc(&P->oz_lane, lanes * lane);
+      e = ctx_plan_malloc(h, (void**)&P->oz_mem, mem);
+      if (e == cudaSuccess) e = ctx_plan_malloc(h, (void**)&P->oz_cq, cq);
+      if (e == cudaSuccess) e = ctx_plan_malloc(h, (void**)&P->oz_fin, fb);
+      if (e == cudaSuccess) e = ctx_plan_malloc(h, (void**)&P->oz_lane, lanes * lane);
       if (e == cudaSuccess) {
         P->oz_group = group;
         P->lanes = lanes;

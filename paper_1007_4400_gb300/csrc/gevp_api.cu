@@ -132,6 +132,38 @@ cudaStream_t ctx_stream(gevp_ctx* h) { return h->stream; }
 int ctx_device(gevp_ctx* h) { return h->device; }
 void ctx_set_error(gevp_ctx* h, const char* msg) { h->err = msg; }
 BatchPlan*& ctx_batch(gevp_ctx* h) { return h->batch; }
+cudaError_t ctx_plan_malloc(gevp_ctx* h, void** p, size_t bytes) {
+  *p = nullptr;
+  cudaError_t e = cudaErrorMemoryAllocation;
+  if (h->inject == 5) h->inject = 0;
+  else e = cudaMalloc(p, bytes);
+  if (e != cudaErrorMemoryAllocation) return e;
+  cudaGetLastError();
+  cudaDeviceSynchronize();
+  for (int side = 0; side < 2; ++side) {
+    if (h->ozmem[side]) cudaFree(h->ozmem[side]);
+    h->ozmem[side] = nullptr;
+    h->ozmem_bytes[side] = 0;
+    h->oz_n[side] = 0;   // (no operand is taken from here before it is split again)
+  }
+  if (h->parena) cudaFree(h->parena);
+  h->parena = nullptr;
+  h->parena_bytes = 0;
+  for (FilterTC** f : {&h->tc, &h->tc2}) {
+    if (*f) filter_tc_release(*f);
+    *f = nullptr;
+  }
+  if (h->stage) cudaFree(h->stage);
+  if (h->vd2) cudaFree(h->vd2);
+  if (h->dvbuf) cudaFree(h->dvbuf);
+  h->stage = nullptr;
+  h->vd2 = nullptr;
+  h->dvbuf = nullptr;
+  h->stage_bytes = h->vd2_bytes = h->dvbuf_bytes = 0;
+  e = cudaMalloc(p, bytes);
+  if (e != cudaSuccess) cudaGetLastError();
+  return e;
+}
 }  // namespace gevp
 
 namespace {
@@ -144,6 +176,7 @@ gevp_status cuda_fail(gevp_ctx* h, cudaError_t e, const char* where) {
   char buf[256];
   snprintf(buf, sizeof buf, "%s: %s", where, cudaGetErrorString(e));
   h->err = buf;
+  if (e == cudaErrorMemoryAllocation) cudaGetLastError();   // reported here; the next call starts clean
   return e == cudaErrorMemoryAllocation ? GEVP_ERR_OOM : GEVP_ERR_CUDA;
 }
 
@@ -160,6 +193,46 @@ gevp_status cuda_fail(gevp_ctx* h, cudaError_t e, const char* where) {
   } while (0)
 
 inline size_t al(size_t b) { return (b + 255) & ~(size_t)255; }
+
+// ---------------------------------------------------------------- injected failures
+// whether gevp_inject_failure asked for this one (once)
+bool injected(gevp_ctx* h, int what) {
+  if (h->inject != what) return false;
+  h->inject = 0;
+  return true;
+}
+// the device word reads as after the given failure
+void inject(gevp_ctx* h, int what, const int* word, int code) {
+  if (word && injected(h, what)) cudaMemsetAsync((void*)word, code, 1, h->stream);
+}
+
+// ---------------------------------------------------------------- device memory
+// The solver's scratch and the batch's plan are each sized for the largest call so far and kept, and
+// with emulated products each may take a third of the device. When one of them cannot grow, the other
+// is given up: its next call makes it again.
+bool give_up_batch(gevp_ctx* h) {
+  if (!h->batch) return false;
+  cudaDeviceSynchronize();
+  gevp::batch_release(h->batch);
+  h->batch = nullptr;
+  return true;
+}
+cudaError_t handle_malloc(gevp_ctx* h, void** p, size_t bytes) {
+  *p = nullptr;
+  cudaError_t e = injected(h, 5) ? cudaErrorMemoryAllocation : cudaMalloc(p, bytes);
+  if (e != cudaErrorMemoryAllocation) return e;
+  cudaGetLastError();
+  if (!give_up_batch(h)) return e;
+  e = cudaMalloc(p, bytes);
+  if (e != cudaSuccess) cudaGetLastError();
+  return e;
+}
+cudaError_t reserve_filter(gevp_ctx* h, gevp::FilterTC** f, int64_t n, int m, cudaStream_t s) {
+  cudaError_t e = gevp::filter_tc_reserve(f, n, m, s);
+  if (e != cudaErrorMemoryAllocation) return e;
+  cudaGetLastError();
+  return give_up_batch(h) ? gevp::filter_tc_reserve(f, n, m, s) : e;
+}
 
 // Lay out (or only measure, when base == nullptr) every buffer for sizes (n, m).
 size_t layout(gevp_ctx* h, char* base, int64_t n, int m) {
@@ -241,7 +314,7 @@ gevp_status ensure(gevp_ctx* h, int64_t n, int m) {
   if (!h->hbuf) CK(cudaMallocHost(&h->hbuf, 64 * sizeof(double)));
   size_t bytes = layout(h, nullptr, nn, mm);
   void* p = nullptr;
-  cudaError_t e = cudaMalloc(&p, bytes);
+  const cudaError_t e = handle_malloc(h, &p, bytes);
   if (e != cudaSuccess) return cuda_fail(h, e, "workspace cudaMalloc");
   h->arena = (char*)p;
   h->arena_bytes = bytes;
@@ -251,18 +324,6 @@ gevp_status ensure(gevp_ctx* h, int64_t n, int m) {
   h->cap_m = mm;
   h->chol_valid = false;
   return GEVP_OK;
-}
-
-// ---------------------------------------------------------------- injected failures
-// whether gevp_inject_failure asked for this one (once)
-bool injected(gevp_ctx* h, int what) {
-  if (h->inject != what) return false;
-  h->inject = 0;
-  return true;
-}
-// the device word reads as after the given failure
-void inject(gevp_ctx* h, int what, const int* word, int code) {
-  if (word && injected(h, what)) cudaMemsetAsync((void*)word, code, 1, h->stream);
 }
 
 // ---------------------------------------------------------------- phase timing
@@ -414,6 +475,7 @@ cudaError_t oz_grow(gevp_ctx* h, int side, size_t bytes, bool optional) {
   if (optional && h->ozmem[side]) {
     size_t avail = 0, total = 0;
     GEVP_CUDA_TRY(cudaMemGetInfo(&avail, &total));
+    if (avail + h->ozmem_bytes[side] < bytes && give_up_batch(h)) GEVP_CUDA_TRY(cudaMemGetInfo(&avail, &total));
     if (avail + h->ozmem_bytes[side] < bytes) return cudaErrorMemoryAllocation;
   }
   // the other stream may still read this side's (or, for side 0, the shared) operands
@@ -423,11 +485,7 @@ cudaError_t oz_grow(gevp_ctx* h, int side, size_t bytes, bool optional) {
   h->ozmem_bytes[side] = 0;
   h->oz_n[side] = 0;
   void* p = nullptr;
-  const cudaError_t e = cudaMalloc(&p, bytes);
-  if (e != cudaSuccess) {
-    cudaGetLastError();
-    return e;
-  }
+  GEVP_CUDA_TRY(handle_malloc(h, &p, bytes));
   h->ozmem[side] = (char*)p;
   h->ozmem_bytes[side] = bytes;
   return cudaSuccess;
@@ -735,7 +793,7 @@ gevp_status ensure_pipeline(gevp_ctx* h) {
       h->parena = nullptr;
     }
     void* p = nullptr;
-    CK(cudaMalloc(&p, need));
+    CK(handle_malloc(h, &p, need));
     h->parena = (char*)p;
     h->parena_bytes = need;
   }
@@ -1046,7 +1104,7 @@ gevp_status solve_one(gevp_ctx* h, int64_t n, const double2* A, int64_t lda, con
   int prec = o.filter_prec;
   const int nsplit = (prec == GEVP_PREC_FP32) ? 3 : 1;
   if (prec != GEVP_PREC_FP64 && !tc_ready) {
-    CK(filter_tc_reserve(&h->tc, n, m, h->stream));
+    CK(reserve_filter(h, &h->tc, n, m, h->stream));
     CK(filter_tc_set_matrix(h->tc, n, h->C, n, nsplit, h->stream));
   }
   // emulated products: the residues of C for every W = C Q of this problem
@@ -1267,7 +1325,7 @@ gevp_status prefetch_problem(gevp_ctx* h, int64_t n, int m, const double2* A, in
   CK(lanczos_bounds(n, h->M32b, n, o.lanczos_steps, 0, o.seed + 104729ull * idx + 1, h->lw2, h->bounds2 + 8, h->side));
   CK(cudaMemcpyAsync(h->hb2, h->bounds2, 16 * sizeof(double), cudaMemcpyDeviceToHost, h->side));
   if (o.filter_prec != GEVP_PREC_FP64) {
-    CK(filter_tc_reserve(&h->tc2, n, m, h->side));
+    CK(reserve_filter(h, &h->tc2, n, m, h->side));
     CK(filter_tc_set_matrix(h->tc2, n, h->C2, n, o.filter_prec == GEVP_PREC_FP32 ? 3 : 1, h->side));
   }
   CK(cudaEventRecord(h->ev_side, h->side));
@@ -1721,7 +1779,8 @@ gevp_status gevp_solve_sequence_host(gevp_handle h, int nprob, int64_t n, const 
   const size_t need = (size_t)(nprob + nb) * mat + 2 * (size_t)nprob * nev * sizeof(double) + out_x + 4096;
   if (need > h->stage_bytes) {
     if (h->stage) { cudaStreamSynchronize(h->stream); cudaFree(h->stage); h->stage = nullptr; }
-    CK(cudaMalloc(&h->stage, need));
+    h->stage_bytes = 0;
+    CK(handle_malloc(h, &h->stage, need));
     h->stage_bytes = need;
   }
   char* p = (char*)h->stage;
@@ -1774,7 +1833,7 @@ gevp_status gevp_chebyshev_filter(gevp_handle h, int64_t n, const void* C, int64
   if (prec != GEVP_PREC_FP64) {
     if (!tc_filter_supported()) return GEVP_ERR_UNSUPPORTED;
     const int nsplit = (prec == GEVP_PREC_FP32) ? 3 : 1;
-    CK(filter_tc_reserve(&h->tc, n, m, h->stream));
+    CK(reserve_filter(h, &h->tc, n, m, h->stream));
     CK(filter_tc_set_matrix(h->tc, n, (const double2*)C, ldc, nsplit, h->stream));
     int err = 0;
     CK(filter_tc_apply(h->tc, n, m, (const double2*)Y, ldy, (double2*)Y, ldy, degree, lo, hi, s, nsplit, &err,
@@ -1798,7 +1857,7 @@ gevp_status gevp_matmul_tc(gevp_handle h, int64_t n, int m, const void* C, int64
   if (!C || !Y || !D || bad_ld(ldc, n) || bad_ld(ldy, m) || bad_ld(ldd, m)) return GEVP_ERR_INVALID_ARG;
   cudaSetDevice(h->device);
   if (!tc_filter_supported()) return GEVP_ERR_UNSUPPORTED;
-  CK(filter_tc_reserve(&h->tc, n, m, h->stream));
+  CK(reserve_filter(h, &h->tc, n, m, h->stream));
   CK(filter_tc_set_matrix(h->tc, n, (const double2*)C, ldc, 1, h->stream));
   int err = 0;
   CK(filter_tc_product(h->tc, n, m, (const double2*)Y, ldy, (double2*)D, ldd, 1, &err, h->stream));
@@ -1935,7 +1994,7 @@ gevp_status gevp_matrix_variation(gevp_handle h, int64_t n, const void* A_new, i
       h->vd2_bytes = 0;
     }
     void* p = nullptr;
-    CK(cudaMalloc(&p, need));
+    CK(handle_malloc(h, &p, need));
     h->vd2 = (unsigned long long*)p;
     h->vd2_bytes = need;
   }
@@ -1987,7 +2046,7 @@ gevp_status gevp_deviation_angles(gevp_handle h, int64_t n, int k_old, int k_new
       h->dvbuf_bytes = 0;
     }
     void* p = nullptr;
-    CK(cudaMalloc(&p, need));
+    CK(handle_malloc(h, &p, need));
     h->dvbuf = (char*)p;
     h->dvbuf_bytes = need;
   }
@@ -2126,7 +2185,7 @@ gevp_status gevp_reduce_emulated(gevp_handle h, int64_t n, const void* A, int64_
 }
 
 gevp_status gevp_inject_failure(gevp_handle h, int what) {
-  if (!h || what < 0 || what > 4) return GEVP_ERR_INVALID_ARG;
+  if (!h || what < 0 || what > 5) return GEVP_ERR_INVALID_ARG;
   h->inject = what;
   return GEVP_OK;
 }

@@ -427,6 +427,9 @@ cudaStream_t ctx_stream(gevp_ctx* h);
 int ctx_device(gevp_ctx* h);
 void ctx_set_error(gevp_ctx* h, const char* msg);
 BatchPlan*& ctx_batch(gevp_ctx* h);
+// device memory for the plan; when there is none left, the handle's scratch for sequences and single
+// steps is given up first
+cudaError_t ctx_plan_malloc(gevp_ctx* h, void** p, size_t bytes);
 
 // ---------------------------------------------------------------- probes
 void probe_peaks(double* fp64_fma_tflops, double* fp64_dmma_tflops, double* fp32_fma_tflops, cudaStream_t s);
