@@ -82,12 +82,16 @@ typedef struct {
                         /* needed at least as many filter matvecs as the latest cold one, */
                         /* the next problem starts cold (the paper's refresh when progress */
                         /* flattens out, Sec. "A new computational philosophy")           */
-  int reduce_slices;    /* 0: the products with an n x n operand (the reduction to standard */
-                        /* form, W = C Q, X = L^-H Q, A X, B X) run on the FP64 pipe. 1..8: */
-                        /* they are emulated on the tensor cores with entries of that many 7-bit */
-                        /* digits (exact integer products by residues; 8 digits keep        */
-                        /* FP64-class accuracy), see gevp_zgemm_emulated; the batched form  */
-                        /* emulates them one k-point at a time. Requires n <= 30720.        */
+  int reduce_slices;    /* 0: every product outside the filter runs on the FP64 pipe. 1..8: */
+                        /* the products with an n x n operand (the reduction to standard    */
+                        /* form, W = C Q, X = L^-H Q, A X, B X), CholQR's Y Li^H and the     */
+                        /* rotation [Q W] Z are emulated on the tensor cores with entries   */
+                        /* of that many 7-bit digits (exact integer products by residues;   */
+                        /* 8 digits keep FP64-class accuracy in terms of the rows' and      */
+                        /* columns' largest entries), see gevp_zgemm_emulated; with 8, Gram  */
+                        /* matrices too where that is faster (in a batch: all of a round's  */
+                        /* n m^2 products). The batched form takes the k-points over up to  */
+                        /* four streams. Requires n <= 30720.                               */
 } gevp_opts;
 
 /* Per-problem counters and CUDA-event phase times (milliseconds). */
@@ -237,6 +241,16 @@ gevp_status gevp_solve_batched(gevp_handle h, int nk, int nsteps, const int64_t*
                                void* const* X, const int64_t* ldx, gevp_batch_stats* stats);
 
 /* ---- individual steps of the solver (same kernels as the solver uses) ---------------- */
+
+/* How the large products (above about 80 us on the FP64 pipe, K <= 30720) of gevp_cholqr2,
+ * gevp_rayleigh_ritz and gevp_energy_backward are formed in later calls on the handle. 8 (the
+ * default): emulated with 8 digits as in gevp_zgemm_emulated, where the device can: errors as on
+ * the FP64 pipe in terms of the norms of the operands' rows and columns, not of single entries many
+ * decades below them. CholQR's columns may differ in length by any factor (their scales are taken
+ * out); gevp_energy_backward takes the FP64 pipe by itself where the entries of a row of X (or X
+ * diag(Lambda)) are not of one size. 0: all on the FP64 pipe. GEVP_ERR_INVALID_ARG for any other
+ * value. */
+gevp_status gevp_set_step_slices(gevp_handle h, int slices);
 
 /* Scaled Chebyshev filter (Zhou, Saad, Tiago & Chelikowsky 2006), in place:
  *   Y <- p(C) Y,  p(t) = T_d((t-c)/e) / T_d((s-c)/e),  c = (lo+hi)/2, e = (hi-lo)/2,

@@ -92,7 +92,9 @@ struct gevp_ctx {
   int oz_l_S = 0;
   int64_t chol_gen = 0;                     // incremented by every factorisation of B
   int* ozflags = nullptr;                   // device: [0] kernel error code, [1] non-finite entry; [2], [3]
-                                            // the same for the products of the per-step entry points
+                                            // the same for the products of the per-step entry points; [4]
+                                            // not 0: the rows of the product at hand are even
+  int step_slices = 8;                      // gevp_set_step_slices
   bool em = false;                          // a per-step entry point whose large products are emulated
   const int* heev_word = nullptr;           // device word of the last small eigensolver's failure (null: none)
   int inject = 0;                           // gevp_inject_failure: the next failure to report
@@ -447,8 +449,8 @@ void reduce_into_ws(int64_t n, const double2* Linv, const double2* A, int64_t ld
 gevp_status oz_flags_ready(gevp_ctx* h) {
   if (h->ozflags) return GEVP_OK;
   void* p = nullptr;
-  CK(cudaMalloc(&p, 4 * sizeof(int)));
-  CK(cudaMemsetAsync(p, 0, 4 * sizeof(int), h->stream));
+  CK(cudaMalloc(&p, 8 * sizeof(int)));
+  CK(cudaMemsetAsync(p, 0, 8 * sizeof(int), h->stream));
   h->ozflags = (int*)p;
   return GEVP_OK;
 }
@@ -630,10 +632,11 @@ gevp_status oz_check(gevp_ctx* h) {
 // side stream's, free outside a solve): all moduli's residues of both operands, or groups of four
 // where that would take more than a third of the device's memory or cannot be had. A Gram
 // product (op(A) = A^H, B = A) splits its block once. flags: error code and non-finite word. ks
-// (rows of A and of B^H only): column exponents moved from A to B; ex_out: op(A)'s exponents.
+// (rows of A and of B^H only): column exponents moved from A to B; ex_out: op(A)'s exponents. even
+// (nullable, A B^H only): cleared where a row of A or B spreads over decades; D is then not written.
 cudaError_t em_enqueue(gevp_ctx* h, int opA, int opB, int M, int N, int K, const double2* A, int64_t lda,
                        const double2* B, int64_t ldb, int triB, int triD, double2* D, int64_t ldd, int slices,
-                       int* flags, const int* ks = nullptr, int* ex_out = nullptr) {
+                       int* flags, const int* ks = nullptr, int* ex_out = nullptr, int* even = nullptr) {
   const bool gram = A == B && lda == ldb && opA == 1 && opB == 0 && M == N;
   const auto opb = [&](int rows, int group) { return al(gevp::oz_operand_bytes(rows, K, slices, group)); };
   const auto need = [&](int group) { return opb(M, group) + (gram ? 0 : opb(N, group)); };
@@ -651,16 +654,16 @@ cudaError_t em_enqueue(gevp_ctx* h, int opA, int opB, int M, int N, int K, const
   // rows of op(A): rows of A, or conjugated columns; columns of op(B): columns of B, or
   // conjugated rows
   GEVP_CUDA_TRY(gevp::oz_split(a, mem, M, K, A, lda, opA, 0, slices, flags + 1, h->stream, opA == 1, nullptr, group, ks,
-                               -1));
+                               -1, even));
   if (ex_out) GEVP_CUDA_TRY(cudaMemcpyAsync(ex_out, a.ex, (size_t)M * sizeof(int), cudaMemcpyDeviceToDevice, h->stream));
   if (gram) {
     b = a;
     b.conj = 0;
   } else {
     GEVP_CUDA_TRY(gevp::oz_split(b, mem + opb(M, group), N, K, B, ldb, opB, 0, slices, flags + 1, h->stream, opB == 0,
-                                 nullptr, group, ks, 1));
+                                 nullptr, group, ks, 1, even));
   }
-  const cudaError_t e = gevp::oz_gemm(a, b, 0, triB, D, ldd, flags, h->stream, nullptr, h->ozmem[1], work, triD);
+  const cudaError_t e = gevp::oz_gemm(a, b, 0, triB, D, ldd, flags, h->stream, even, h->ozmem[1], work, triD);
   inject(h, 2, flags, 24);
   return e;
 }
@@ -674,11 +677,11 @@ bool em_worth(double macs) { return 8.0 * macs > 80e-6 * 1.05e12; }
 // (too small, or no memory for the operands)
 bool em_product(gevp_ctx* h, int opA, int opB, int64_t M, int64_t N, int64_t K, const double2* A, int64_t lda,
                 const double2* B, int64_t ldb, int triB, int triD, double2* D, int64_t ldd,
-                const int* ks = nullptr, int* ex_out = nullptr) {
+                const int* ks = nullptr, int* ex_out = nullptr, int* even = nullptr) {
   if (!h->em || K > 30720 || !em_worth((double)M * N * K * (triB || triD ? 0.5 : 1.0))) return false;
   if (oz_flags_ready(h) != GEVP_OK) return false;
   if (em_enqueue(h, opA, opB, (int)M, (int)N, (int)K, A, lda, B, ldb, triB, triD, D, ldd, 8, h->ozflags + 2, ks,
-                 ex_out) == cudaSuccess)
+                 ex_out, even) == cudaSuccess)
     return true;
   cudaGetLastError();
   return false;
@@ -736,7 +739,9 @@ gevp_status heev_status(gevp_ctx* h, int word) {
 // and the kernels' error code read at the end
 struct EmScope {
   gevp_ctx* h;
-  explicit EmScope(gevp_ctx* hh) : h(hh) { h->em = h->oz_slices == 0 && gevp::oz_supported(); }
+  explicit EmScope(gevp_ctx* hh) : h(hh) {
+    h->em = h->step_slices > 0 && h->oz_slices == 0 && gevp::oz_supported();
+  }
   ~EmScope() { h->em = false; }
   // waits for the call's work, then its error words
   gevp_status finish(const int* heev_word = nullptr) {
@@ -1954,17 +1959,35 @@ gevp_status gevp_energy_backward(gevp_handle h, int64_t n, int nev, const void* 
   // 24), then the Hermitian completion with the incoming gradient; on the FP64 pipe where small
   EmScope em(h);
   const double2* Xd = (const double2*)X;
-  if (em_product(h, 0, 1, n, n, nev, Xd, ldx, Xd, ldx, 0, 1, (double2*)GA, ldg)) {
-    // the call does not wait, so the products' error word is read on the device: it turns the gradients
-    // into NaN and is cleared behind them
-    const int* error = h->ozflags + 2;
-    hermitize_scale_lower(n, (double2*)GA, ldg, gE, 1.0, h->stream, error);
-    scale_by_lam(n, nev, Xd, ldx, Lambda, h->T, h->stream);
-    const bool both = em_product(h, 0, 1, n, n, nev, h->T, nev, Xd, ldx, 0, 1, (double2*)GB, ldg);
-    if (both) hermitize_scale_lower(n, (double2*)GB, ldg, gE, -1.0, h->stream, error);
-    CK(cudaMemsetAsync(h->ozflags + 2, 0, sizeof(int), h->stream));
+  if (h->em) {
+    TRY(oz_flags_ready(h));
+    // The emulated product rounds a row's entries to 2^-57 of the largest one, the FP64 pipe each to its
+    // own last bit: an entry of the gradient that is small only because two rows have their large
+    // entries in different columns (x_i = [1, 1e-9], x_j = [1e-12, 1]) would lose what the FP64 sum
+    // keeps. So the splitter looks at the rows: where three quarters of the entries of each are within
+    // 2^-6 of its largest, half of the columns are in common, sum_k |x_ik||x_jk| is at least K 2^-15 of the
+    // product of the largest entries, and the product is emulated; else the FP64 pipe forms it. The word
+    // is read on the device, the launches of the form not taken return at once.
+    int* even = h->ozflags + 4;
+    const int* error = h->ozflags + 2;   // (also read on the device: NaN; cleared behind the products)
+    const auto product = [&](const double2* L, int64_t ldl, double2* G, double sign) {
+      cudaMemsetAsync(even, 1, sizeof(int), h->stream);
+      if (!em_product(h, 0, 1, n, n, nev, L, ldl, Xd, ldx, 0, 1, G, ldg, nullptr, nullptr, even)) return false;
+      ZgemmArgs f = zg((int)n, (int)n, nev, L, ldl, 0, Xd, ldx, 1, G, ldg);
+      f.triD = 1;
+      f.unless = even;
+      zgemm(f, h->split, h->split_elems, h->stream);
+      hermitize_scale_lower(n, G, ldg, gE, sign, h->stream, error);
+      return true;
+    };
+    bool done = product(Xd, ldx, (double2*)GA, 1.0);
+    if (done) {
+      scale_by_lam(n, nev, Xd, ldx, Lambda, h->T, h->stream);
+      done = product(h->T, nev, (double2*)GB, -1.0);
+      CK(cudaMemsetAsync(h->ozflags + 2, 0, sizeof(int), h->stream));
+    }
     CK(cudaGetLastError());
-    if (both) return GEVP_OK;
+    if (done) return GEVP_OK;
   }
   gevp::energy_backward_ws(n, nev, Xd, ldx, Lambda, gE, (double2*)GA, (double2*)GB, ldg, h->T, h->split,
                            h->split_elems, h->stream);
@@ -2182,6 +2205,12 @@ gevp_status gevp_reduce_emulated(gevp_handle h, int64_t n, const void* A, int64_
   if (st == GEVP_OK) st = oz_check(h);
   h->oz_slices = keep;
   return st;
+}
+
+gevp_status gevp_set_step_slices(gevp_handle h, int slices) {
+  if (!h || (slices != 0 && slices != 8)) return GEVP_ERR_INVALID_ARG;
+  h->step_slices = slices;
+  return GEVP_OK;
 }
 
 gevp_status gevp_inject_failure(gevp_handle h, int what) {

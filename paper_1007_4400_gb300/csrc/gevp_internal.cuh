@@ -75,6 +75,7 @@ struct ZgemmArgs {
   int ksplit;
   int batch;
   int64_t sA, sB, sD, sC, sE;   // batch strides in elements
+  const int* unless;            // nullable device word: nothing is done where it is not 0
 };
 
 void zgemm(const ZgemmArgs& a, double2* split_ws, size_t split_ws_elems, cudaStream_t s);
@@ -384,17 +385,20 @@ struct OzOperand {
   int* bad = nullptr;
   const int* ks = nullptr;   // rows only: entry k scaled by 2^(ks_sign ks[k]) (exponents of another operand)
   int ks_sign = 0;
+  int* even = nullptr;       // rows only: cleared by a row whose entries are spread over decades
 };
 // group 0: all moduli at once
 size_t oz_operand_bytes(int rows, int K, int S, int group = 0);
 bool oz_supported();
 // rows of X (cols = false; X is rows x K) or its columns (cols = true; X is K x rows) as
 // operand rows, conjugated if conj, mask 1: k >= r with the diagonal halved, 2: k <= r,
-// 3: k >= r; into residue form in `mem` (oz_operand_bytes); *bad = 1 on a non-finite entry
+// 3: k >= r; into residue form in `mem` (oz_operand_bytes); *bad = 1 on a non-finite entry;
+// *even = 0 (nullable; rows of X only) where fewer than three quarters of a row's entries are within
+// 2^-6 of its largest (each by its larger part), or one is not finite
 // active: nullable device flag, 0 = the launch does nothing (a converged batch problem)
 cudaError_t oz_split(OzOperand& op, void* mem, int rows, int K, const double2* X, int64_t ldx, int conj, int mask,
                      int S, int* bad, cudaStream_t s, bool cols = false, const int* active = nullptr, int group = 0,
-                     const int* ks = nullptr, int ks_sign = 0);
+                     const int* ks = nullptr, int ks_sign = 0, int* even = nullptr);
 // D (A.rows x B.rows) = op(A) op(B); triA 1: op(A) lower, 2: upper; triB 1: op(B) lower, 2:
 // upper. ws: room for the result's residues; oz_work_bytes(M, N, K, S) holds the whole
 // result, less makes the product run in panels of rows (at least one of min(M, 256) rows).

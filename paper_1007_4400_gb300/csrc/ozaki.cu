@@ -692,7 +692,7 @@ __device__ __forceinline__ void oz_write_pair(double2 v0, double2 v1, int shift,
 __global__ void __launch_bounds__(256) oz_split_rows_kernel(int rows, int K, const double2* X, int64_t ldx, int mask,
                                                             const int* ks, int sg, int S, int mod0, int cnt, int nmod,
                                                             int k_pad, __nv_bfloat16* planes, int* ex, int need_ex,
-                                                            int* bad,
+                                                            int* bad, int* even,
                                                             const __grid_constant__ OzModTab tab, const int* active) {
   if (active && *active == 0) return;
   __shared__ unsigned long long red[8];
@@ -717,6 +717,23 @@ __global__ void __launch_bounds__(256) oz_split_rows_kernel(int rows, int K, con
     // 2^e > 2 max|entry|: the scaled row lies below 1/2
     e = mx > 0 ? oz_key_ilogb(mx) + 2 : 0;
     if (threadIdx.x == 0) ex[r] = nonfinite ? kExpBad : e;
+    if (even) {
+      int small = 0;
+      for (int k = threadIdx.x; k < K; k += 256) {
+        const double2 v = oz_entry(X, ldx, r, k, K, mask, ks, sg);
+        const unsigned long long key = max(oz_abs_key(v.x), oz_abs_key(v.y));
+        small += key == 0 || oz_key_ilogb(key) < e - 8 ? 1 : 0;
+      }
+      for (int o = 16; o > 0; o >>= 1) small += __shfl_xor_sync(0xffffffffu, small, o);
+      __syncthreads();
+      if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = (unsigned)small;
+      __syncthreads();
+      if (threadIdx.x == 0) {
+        unsigned long long all = 0;
+        for (int w = 0; w < 8; ++w) all += red[w];
+        if (nonfinite || (mx > 0 && 4 * all > (unsigned)K)) *even = 0;   // (a zero row's products are exact)
+      }
+    }
   } else {
     e = ex[r] == kExpBad ? 0 : ex[r];
   }
@@ -832,7 +849,8 @@ cudaError_t oz_split_group(const OzOperand& op, int mod0, int cnt, bool need_ex,
   const OzModTab& tab = oz_mod_tab();
   if (!op.cols) {
     oz_split_rows_kernel<<<op.rows, 256, 0, s>>>(op.rows, op.K, op.X, op.ldx, op.mask, op.ks, op.ks_sign, op.S, mod0,
-                                                 cnt, op.nmod, op.k_pad, op.planes, op.ex, need_ex ? 1 : 0, bad, tab, active);
+                                                 cnt, op.nmod, op.k_pad, op.planes, op.ex, need_ex ? 1 : 0, bad, op.even, tab,
+                                                 active);
     LAUNCH_NOTE(1);
     return cudaGetLastError();
   }
@@ -874,7 +892,7 @@ bool oz_supported() {
 
 cudaError_t oz_split(OzOperand& op, void* mem, int rows, int K, const double2* X, int64_t ldx, int conj, int mask,
                      int S, int* bad, cudaStream_t s, bool cols, const int* active, int group, const int* ks,
-                     int ks_sign) {
+                     int ks_sign, int* even) {
   const int nm = oz_moduli(K, S);
   if (S < 1 || S > kOzSlicesMax || nm > OZ_NMOD) return cudaErrorInvalidValue;
   op.rows = rows;
@@ -892,6 +910,7 @@ cudaError_t oz_split(OzOperand& op, void* mem, int rows, int K, const double2* X
   op.bad = bad;
   op.ks = cols ? nullptr : ks;
   op.ks_sign = ks_sign;
+  op.even = cols ? nullptr : even;
   // in groups: the exponents only (oz_gemm writes each group's residues before it uses them)
   return oz_split_group(op, 0, op.nmod == nm ? nm : 0, true, bad, s, active);
 }

@@ -15,6 +15,7 @@ namespace {
 template <int BM, int BN, int BK, int TM, int TN>
 __global__ void __launch_bounds__((BM / TM) * (BN / TN))
 zgemm_kernel(ZgemmArgs p, double2* ws) {
+  if (p.unless && *p.unless != 0) return;
   constexpr int NT = (BM / TM) * (BN / TN);
   __shared__ double2 As[BK][BM];
   __shared__ double2 Bs[BK][BN];
@@ -140,6 +141,7 @@ zgemm_kernel(ZgemmArgs p, double2* ws) {
 
 // the same on 4 x 8 tiles (zsmall.cuh), without split-K
 __global__ void __launch_bounds__(ZS_THREADS) zgemm_small_kernel(ZgemmArgs p) {
+  if (p.unless && *p.unless != 0) return;
   __shared__ double part[ZS_WARPS][64];
   const int m0 = blockIdx.y * ZS_M, n0 = blockIdx.x * ZS_N, b = blockIdx.z;
   if (p.triD == 1 && n0 > m0 + ZS_M - 1) return;
@@ -161,6 +163,7 @@ __global__ void __launch_bounds__(ZS_THREADS) zgemm_small_kernel(ZgemmArgs p) {
 
 // Sum the k-slices in a fixed order (deterministic) and apply the epilogue.
 __global__ void zgemm_reduce_kernel(ZgemmArgs p, const double2* ws, int BM, int BN) {
+  if (p.unless && *p.unless != 0) return;
   int64_t total = (int64_t)p.M * p.N;
   int b = blockIdx.y;
   double2* D = p.D + (int64_t)b * p.sD;
@@ -261,7 +264,7 @@ void zgemm(const ZgemmArgs& in, double2* split_ws, size_t split_ws_elems, cudaSt
   int bm = best_b, bn = best_b;
   dim3 grid;
   if (bm > 0) grid = dim3((p.N + bn - 1) / bn, (p.M + bm - 1) / bm, p.batch * p.ksplit);
-  void* kt0 = kt_enabled() ? kt_begin(s) : nullptr;
+  void* kt0 = kt_enabled() && !p.unless ? kt_begin(s) : nullptr;
   if (bm == 0)
     zgemm_small_kernel<<<dim3((p.N + ZS_N - 1) / ZS_N, (p.M + ZS_M - 1) / ZS_M, p.batch), ZS_THREADS, 0, s>>>(p);
   else if (bm == 64) zgemm_kernel<64, 64, 8, 4, 4><<<grid, 256, 0, s>>>(p, split_ws);

@@ -125,6 +125,7 @@ def load(build_if_missing: bool = True):
         L.gevp_zgemm_emulated.argtypes = [vp, i32, i32, i32, i32, i32, vp, i64, vp, i64, vp, i64, i32]
         L.gevp_reduce_emulated.argtypes = [vp, i64, vp, i64, vp, i64, vp, i64, vp, i64, C.POINTER(i64), i32]
         L.gevp_inject_failure.argtypes = [vp, i32]
+        L.gevp_set_step_slices.argtypes = [vp, i32]
         L.gevp_kernel_timing.argtypes = [i32]
         L.gevp_kernel_timing_read.argtypes = [C.POINTER(f64)]
         L.gevp_kernel_launches.argtypes = [vp]
@@ -134,7 +135,7 @@ def load(build_if_missing: bool = True):
                      "gevp_heev_small", "gevp_spectral_bounds", "gevp_energy_backward", "gevp_band_energy", "gevp_reduce_update",
                      "gevp_probe_peaks",
                      "gevp_matrix_variation", "gevp_deviation_angles", "gevp_assign_min_cost",
-                     "gevp_zgemm_emulated", "gevp_reduce_emulated", "gevp_inject_failure", "gevp_kernel_timing",
+                     "gevp_zgemm_emulated", "gevp_reduce_emulated", "gevp_inject_failure", "gevp_set_step_slices", "gevp_kernel_timing",
                      "gevp_kernel_timing_read"):
             getattr(L, name).restype = i32
         _LIB = L
@@ -373,10 +374,17 @@ def chebyshev_filter(Cm: torch.Tensor, Y: torch.Tensor, degree: int, lo: float, 
     return Y
 
 
-def cholqr2(Y: torch.Tensor, want_R: bool = False):
-    """Q (in place in Y) and optionally R with Y_in = Q R."""
+def _step_handle(device: torch.device, slices: int):
+    h = _handle(device)
+    _check(load().gevp_set_step_slices(h, int(slices)), h)
+    return h
+
+
+def cholqr2(Y: torch.Tensor, want_R: bool = False, slices: int = 8):
+    """Q (in place in Y) and optionally R with Y_in = Q R. slices: 8 (large products emulated)
+    or 0 (FP64 pipe), see gevp_set_step_slices; so for rayleigh_ritz and energy_backward."""
     _mat(Y, "Y")
-    h = _handle(Y.device)
+    h = _step_handle(Y.device, slices)
     m = Y.shape[1]
     R = torch.zeros((m, m), dtype=torch.complex128, device=Y.device) if want_R else None
     st = load().gevp_cholqr2(h, Y.shape[0], m, _ptr(Y), Y.stride(0), _ptr(R), m if want_R else 0)
@@ -384,10 +392,10 @@ def cholqr2(Y: torch.Tensor, want_R: bool = False):
     return (Y, R) if want_R else Y
 
 
-def rayleigh_ritz(Cm: torch.Tensor, Q: torch.Tensor):
+def rayleigh_ritz(Cm: torch.Tensor, Q: torch.Tensor, slices: int = 8):
     """(theta, Q <- Q Z in place, W = C Q, res)."""
     _mat(Cm, "C"); _mat(Q, "Q")
-    h = _handle(Q.device)
+    h = _step_handle(Q.device, slices)
     n, m = Q.shape
     W = torch.empty_like(Q)
     th = torch.empty(m, dtype=torch.float64, device=Q.device)
@@ -440,12 +448,12 @@ def reduce_update(Cm: torch.Tensor, B: torch.Tensor, dA: torch.Tensor, rows, sli
     return Cm
 
 
-def energy_backward(X: torch.Tensor, Lambda: torch.Tensor, gE=1.0):
+def energy_backward(X: torch.Tensor, Lambda: torch.Tensor, gE=1.0, slices: int = 8):
     """(GA, GB) = (gE X X^H, -gE X diag(Lambda) X^H). gE: a number or a one-element float64
     tensor on X's device (read there by the library, no host synchronisation)."""
     _mat(X, "X")
     _mat(Lambda, "Lambda", torch.float64)
-    h = _handle(X.device)
+    h = _step_handle(X.device, slices)
     n, nev = X.shape
     if isinstance(gE, torch.Tensor):
         g = gE.detach().to(device=X.device, dtype=torch.float64).reshape(1).contiguous()
@@ -578,12 +586,14 @@ class GevpEnergy(torch.autograd.Function):
         r = solve_sequence([A], B, nev, **(opts or {}))
         ctx.save_for_backward(r.X, r.Lambda[0])
         ctx.result = r
+        # a caller that keeps the solve's products on the FP64 pipe keeps the gradient's there
+        ctx.slices = 0 if (opts or {}).get("reduce_slices") == 0 else 8
         return band_energy_of(r.Lambda[:1])[0]
 
     @staticmethod
     def backward(ctx, gE):
         X, lam = ctx.saved_tensors
-        GA, GB = energy_backward(X, lam, gE)
+        GA, GB = energy_backward(X, lam, gE, slices=ctx.slices)
         return GA, GB, None, None
 
 
