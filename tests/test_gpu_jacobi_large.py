@@ -12,7 +12,7 @@ def test_eigenpairs(cuda, m, multiple):
     g = torch.Generator(device=cuda).manual_seed(m)
     V = torch.linalg.qr(torch.randn(m, m, dtype=torch.complex128, device=cuda, generator=g))[0]
     lam = torch.linspace(-2, 5, m, dtype=torch.float64, device=cuda)
-    lam[:multiple] = lam[0]
+    lam[:multiple] = lam[0].item()
     G = (V * lam) @ V.conj().T
     G = 0.5 * (G + G.conj().T)
     th, Z = gevp.heev_small(G)
