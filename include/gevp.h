@@ -403,6 +403,10 @@ gevp_status gevp_reduce_emulated(gevp_handle h, int64_t n, const void* A, int64_
  * 0: take an injection back. */
 gevp_status gevp_inject_failure(gevp_handle h, int what);
 
+/* r[i] = 1 / v[i] (device, n) as the Cholesky-inverse kernels form a pivot's reciprocal, for the test of
+ * its error (below 2^-52 relative). */
+gevp_status gevp_probe_recip(gevp_handle h, int64_t n, const double* v, double* r);
+
 /* Measured FP64 FMA, FP64 DMMA and FP32 FMA rates of this device in TFLOP/s (host out[3]). */
 gevp_status gevp_probe_peaks(gevp_handle h, double* out);
 

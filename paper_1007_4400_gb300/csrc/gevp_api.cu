@@ -2219,6 +2219,15 @@ gevp_status gevp_inject_failure(gevp_handle h, int what) {
   return GEVP_OK;
 }
 
+gevp_status gevp_probe_recip(gevp_handle h, int64_t n, const double* v, double* r) {
+  if (!h || n < 0 || (n > 0 && (!v || !r))) return GEVP_ERR_INVALID_ARG;
+  cudaSetDevice(h->device);
+  gevp::pivot_recips(n, v, r, h->stream);
+  CK(cudaStreamSynchronize(h->stream));
+  CK(cudaGetLastError());
+  return GEVP_OK;
+}
+
 gevp_status gevp_probe_peaks(gevp_handle h, double* out) {
   if (!h || !out) return GEVP_ERR_INVALID_ARG;
   cudaSetDevice(h->device);

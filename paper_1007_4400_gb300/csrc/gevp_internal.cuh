@@ -104,7 +104,7 @@ struct ZgemmItem {
   const int* active;
 };
 struct ZgemmGroupFlags { int opA, opB, triA, triB, triD, maskB; };
-int zgemm_group_tile(const ZgemmItem* items_host, int nitems);
+int zgemm_group_tile(const ZgemmItem* items_host, int nitems);    // 32 or 64
 int zgemm_group_layout(ZgemmItem* items_host, int nitems, int tile);   // returns total tiles
 void zgemm_grouped(const ZgemmItem* items_dev, int nitems, int total_tiles, int tile, const ZgemmGroupFlags& f,
                    cudaStream_t s);
@@ -212,6 +212,7 @@ void zgram(int64_t n, int mx, int my, const double2* X, int64_t ldx, const doubl
 // outputs are incomplete then). false: not launchable (m > cholinv_max_order() or no
 // cluster): nothing was enqueued.
 int cholinv_max_order();
+void pivot_recips(int64_t n, const double* v, double* r, cudaStream_t s);   // its reciprocals, for the test
 bool cholinv_small(int m, const double2* W, int64_t ldw, double shift, double2* Li, int64_t ldi, double2* Lf,
                    int64_t ldl, int* info, cudaStream_t s, int info_base = 0);
 // the same for every Gw of a batch (Li into Gwi, the pivot into flags[2]); the shift is

@@ -116,6 +116,7 @@ def load(build_if_missing: bool = True):
         L.gevp_reduce_update.argtypes = [vp, i64, vp, i64, i32, vp, i64, i32, C.POINTER(i64), vp, i64, i32,
                                          C.POINTER(i64)]
         L.gevp_probe_peaks.argtypes = [vp, C.POINTER(f64)]
+        L.gevp_probe_recip.argtypes = [vp, i64, vp, vp]
         L.gevp_matrix_variation.argtypes = [vp, i64, vp, i64, vp, i64, i32, C.POINTER(f64), C.POINTER(f64),
                                             C.POINTER(i64), vp]
         L.gevp_deviation_angles.argtypes = [vp, i64, i32, i32, vp, i64, vp, i64, vp, i64, C.POINTER(f64),
@@ -133,7 +134,7 @@ def load(build_if_missing: bool = True):
         for name in ("gevp_create", "gevp_destroy", "gevp_set_stream", "gevp_reduce", "gevp_solve_sequence",
                      "gevp_solve_sequence_host", "gevp_solve_batched", "gevp_chebyshev_filter", "gevp_cholqr2", "gevp_rayleigh_ritz",
                      "gevp_heev_small", "gevp_spectral_bounds", "gevp_energy_backward", "gevp_band_energy", "gevp_reduce_update",
-                     "gevp_probe_peaks",
+                     "gevp_probe_peaks", "gevp_probe_recip",
                      "gevp_matrix_variation", "gevp_deviation_angles", "gevp_assign_min_cost",
                      "gevp_zgemm_emulated", "gevp_reduce_emulated", "gevp_inject_failure", "gevp_set_step_slices", "gevp_kernel_timing",
                      "gevp_kernel_timing_read"):
@@ -538,6 +539,15 @@ def assign_min_cost(cost) -> np.ndarray:
     if st != 0:
         raise ValueError(f"gevp_assign_min_cost: status {st}")
     return perm[:ko]
+
+
+def probe_recip(v: torch.Tensor) -> torch.Tensor:
+    """gevp_probe_recip: 1 / v as the Cholesky-inverse kernels form it."""
+    _mat(v, "v", torch.float64)
+    h = _handle(v.device)
+    r = torch.empty_like(v)
+    _check(load().gevp_probe_recip(h, v.numel(), _ptr(v), _ptr(r)), h)
+    return r
 
 
 def probe_peaks(device=None) -> dict:
