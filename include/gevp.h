@@ -214,7 +214,8 @@ typedef struct {
  * GEMMs over a global tile list, one CTA per problem for the small dense work, one
  * grouped tcgen05 launch per filter step), converged k-points are skipped by device
  * flags, and a round is captured once as a CUDA graph and replayed. An autotuner picks
- * the grouped GEMM tile per call class (timed on the first round of a new batch shape)
+ * the larger grouped GEMM tiles per call class (timed on the first round of a new batch
+ * shape; both add up in the same order, the small ones are chosen by the sizes alone)
  * and the filter degree cap per size bucket (a cost model fed by measured times and the
  * Chebyshev convergence factors of the previous step).
  *   n, nev, nex: host arrays of nk (nex nullable: opts->nex for all, at least 2 used);

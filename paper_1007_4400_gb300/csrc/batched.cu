@@ -20,8 +20,9 @@
 // final residuals in the original space (re-opening a problem with a tighter tolerance
 // and the FP64 filter if they miss tol).
 //
-// Autotuner: (1) every grouped GEMM call of a new batch shape is timed with 4 x 8,
-// 32 x 32 and 64 x 64 tiles on its first execution and keeps the fastest; (2) after each step the
+// Autotuner: (1) every grouped GEMM call of a new batch shape that takes the larger tiles
+// (zgemm_group_small says which) is timed with 32 x 32 and 64 x 64 ones on its first execution and keeps the
+// faster; (2) after each step the
 // filter degree cap of every size bucket is set by minimising the modelled time of the
 // next step, R (T_rest + sum_b d_b T_step share_b), over the number of rounds R, where
 // d_b(R) is the degree at which the Chebyshev factor rho_b of the bucket's slowest wanted
@@ -460,7 +461,11 @@ gevp_status build_plan(gevp_ctx* h, BatchPlan* P, std::string& err) {
   // every call's list is there from the start: a call may first run after the plan counts as tuned (a
   // step that ends without its final check leaves that one's to a later step)
   for (auto& c : P->calls) {
-    c.tile = zgemm_group_tile(c.items.data(), (int)c.items.size());
+    // (the FP64 filter's steps beside the tensor cores' are lists of inactive tiles as a rule: few of them)
+    const bool idle = c.cls == CC_FILTER && tc;
+    c.tile = !idle && zgemm_group_small(c.items.data(), (int)c.items.size())
+                 ? 0
+                 : zgemm_group_tile(c.items.data(), (int)c.items.size());
     e = upload_call(P, c, s);
     if (e != cudaSuccess) { err = "item upload failed"; return GEVP_ERR_CUDA; }
   }
@@ -479,15 +484,16 @@ cudaEvent_t evt(BatchPlan* P, size_t i) {
   return P->ev[i];
 }
 
-// one grouped GEMM call; on its first run for a new shape the tiles are timed
+// one grouped GEMM call; on its first run for a new shape the larger tiles are timed (both add up an
+// output in the same order; the 4 x 8 ones do not, so they are chosen by the sizes alone)
 void launch(BatchPlan* P, int ci, cudaStream_t s, bool tune) {
   GCall& c = P->calls[ci];
   const int ni = (int)c.items.size();
   if (ni == 0) return;
-  if (tune && !c.tuned) {
+  if (tune && !c.tuned && c.tile != 0) {
     float best = 1e30f;
     int best_tile = c.tile;
-    for (int t : {0, 32, 64}) {
+    for (int t : {32, 64}) {
       std::vector<ZgemmItem> tmp = c.items;
       int tot = zgemm_group_layout(tmp.data(), ni, t);
       cudaMemcpyAsync(P->tune_pool, tmp.data(), ni * sizeof(ZgemmItem), cudaMemcpyHostToDevice, s);

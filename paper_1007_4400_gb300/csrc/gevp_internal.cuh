@@ -105,6 +105,7 @@ struct ZgemmItem {
 };
 struct ZgemmGroupFlags { int opA, opB, triA, triB, triD, maskB; };
 int zgemm_group_tile(const ZgemmItem* items_host, int nitems);    // 32 or 64
+bool zgemm_group_small(const ZgemmItem* items_host, int nitems);  // whether tiles of 4 x 8 (tile 0) are better
 int zgemm_group_layout(ZgemmItem* items_host, int nitems, int tile);   // returns total tiles
 void zgemm_grouped(const ZgemmItem* items_dev, int nitems, int total_tiles, int tile, const ZgemmGroupFlags& f,
                    cudaStream_t s);

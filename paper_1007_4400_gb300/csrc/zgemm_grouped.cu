@@ -165,6 +165,25 @@ int zgemm_group_tile(const ZgemmItem* items_host, int nitems) {
   return t64 >= 4 * 152 ? 64 : 32;
 }
 
+// The rule of the single products (zgemm.cu) over the list: the share of the busiest SM, in outputs'
+// K steps, or the longest tile if that is more. An SM's tiles of 4 x 8 add up eight partial sums, so
+// this is not left to a timing: the rounding of a batch would depend on it.
+bool zgemm_group_small(const ZgemmItem* items_host, int nitems) {
+  double small = 0.0, large = 0.0;
+  int64_t tiles = 0, kmax = 0;
+  for (int i = 0; i < nitems; ++i) {
+    const ZgemmItem& it = items_host[i];
+    const int64_t ts = (int64_t)((it.M + ZS_M - 1) / ZS_M) * ((it.N + ZS_N - 1) / ZS_N);
+    tiles += ts;
+    small += (double)ts * (ZS_M * ZS_N * (double)it.K + kZsOverhead);
+    large += (double)((it.M + 31) / 32) * ((it.N + 31) / 32) * 1024.0 * it.K;
+    kmax = std::max<int64_t>(kmax, it.K);
+  }
+  small = std::max(small / 152, ZS_M * ZS_N * (double)kmax + kZsOverhead);
+  large = std::max(large / 152, 1024.0 * (double)kmax);
+  return 1.08 * small < large && (kmax <= 512 || tiles >= 4 * 152);
+}
+
 int zgemm_group_layout(ZgemmItem* items_host, int nitems, int tile) {
   int total = 0;
   for (int i = 0; i < nitems; ++i) {
