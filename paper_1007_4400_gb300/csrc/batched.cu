@@ -158,6 +158,7 @@ void batch_release(BatchPlan* P) {
   if (P->gexec) cudaGraphExecDestroy(P->gexec);
   if (P->graph) cudaGraphDestroy(P->graph);
   if (P->arena) cudaFree(P->arena);
+  if (P->pool) cudaFree(P->pool);
   if (P->oz_mem) cudaFree(P->oz_mem);
   if (P->oz_cq) cudaFree(P->oz_cq);
   if (P->oz_fin) cudaFree(P->oz_fin);
