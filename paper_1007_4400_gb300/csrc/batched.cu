@@ -662,7 +662,7 @@ cudaError_t enqueue_rr(BatchPlan* P, cudaStream_t s, bool tune) {
   launch(P, P->c_Ef[zsel], s, tune);
   launch(P, P->c_Sf[zsel], s, tune);
   bk_hermitize_avg_S(P->dD, np, mmax, s);
-  cluster_jacobi_batched(P->dD, np, zsel, 1e-15, 12, s);
+  cluster_jacobi_batched(P->dD, np, zsel, 1e-15, 20, s);
   bk_sort_pairs(P->dD, np, zsel, s);
   if (P->oz_round) {
     // Q <- Q Z, W = W' Z
