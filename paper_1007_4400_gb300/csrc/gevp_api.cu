@@ -663,7 +663,22 @@ cudaError_t em_enqueue(gevp_ctx* h, int opA, int opB, int M, int N, int K, const
     GEVP_CUDA_TRY(gevp::oz_split(b, mem + opb(M, group), N, K, B, ldb, opB, 0, slices, flags + 1, h->stream, opB == 0,
                                  nullptr, group, ks, 1, even));
   }
-  const cudaError_t e = gevp::oz_gemm(a, b, 0, triB, D, ldd, flags, h->stream, even, h->ozmem[1], work, triD);
+  // In groups of moduli the operands are read again for every panel of rows, so a result over an
+  // operand's memory (fine where all residues are made first) is formed beside it
+  const auto overlap = [&](const double2* X, int64_t rows, int64_t ld, int64_t cols) {
+    return X < D + ((int64_t)(M - 1) * ldd + N) && D < X + ((rows - 1) * ld + cols);
+  };
+  void* tmp = nullptr;
+  if (group != 0 && M > 0 && (overlap(A, opA ? K : M, lda, opA ? M : K) || overlap(B, opB ? N : K, ldb, opB ? K : N)))
+    GEVP_CUDA_TRY(handle_malloc(h, &tmp, (size_t)M * N * sizeof(double2)));
+  cudaError_t e = gevp::oz_gemm(a, b, 0, triB, tmp ? (double2*)tmp : D, tmp ? N : ldd, flags, h->stream, even,
+                                h->ozmem[1], work, triD);
+  if (tmp) {
+    if (e == cudaSuccess) zcopy2d(M, N, (const double2*)tmp, N, D, ldd, h->stream);
+    const cudaError_t f = cudaStreamSynchronize(h->stream);
+    if (e == cudaSuccess) e = f;
+    cudaFree(tmp);
+  }
   inject(h, 2, flags, 24);
   return e;
 }
