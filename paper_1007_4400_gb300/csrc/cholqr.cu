@@ -457,8 +457,6 @@ bool cholinv_launch(const Src& src, int np, int m, cudaStream_t s) {
   constexpr int kMaxSmem = 203 * 1024;   // with the static arrays below the SM's 227 KB
   const size_t smem = cholinv_smem<P>(m);
   if (smem > kMaxSmem) return false;
-  static int ready = 0;   // 0 unknown, 1 usable, -1 not launchable on this device
-  if (ready < 0) return false;
   auto* kern = cholinv_cluster_kernel<P, Src>;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(P * np, 1, 1);
@@ -472,26 +470,20 @@ bool cholinv_launch(const Src& src, int np, int m, cudaStream_t s) {
   at[0].val.clusterDim.z = 1;
   cfg.attrs = at;
   cfg.numAttrs = 1;
-  if (ready == 0) {
-    ready = -1;
-    if (P > 8 && cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) {
-      cudaGetLastError();
-      return false;
-    }
-    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem) != cudaSuccess) {
-      cudaGetLastError();
-      return false;
-    }
+  // whether the device can run it, asked once (other threads wait for the answer)
+  static const bool usable = [&] {
     cudaLaunchConfig_t probe = cfg;
     probe.gridDim = dim3(P, 1, 1);
     probe.dynamicSmemBytes = kMaxSmem;
     int nclusters = 0;
-    if (cudaOccupancyMaxActiveClusters(&nclusters, kern, &probe) != cudaSuccess || nclusters < 1) {
-      cudaGetLastError();
-      return false;
-    }
-    ready = 1;
-  }
+    const bool ok =
+        (P <= 8 || cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess) &&
+        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem) == cudaSuccess &&
+        cudaOccupancyMaxActiveClusters(&nclusters, kern, &probe) == cudaSuccess && nclusters > 0;
+    if (!ok) cudaGetLastError();
+    return ok;
+  }();
+  if (!usable) return false;
   if (cudaLaunchKernelEx(&cfg, kern, src) != cudaSuccess) {
     cudaGetLastError();
     return false;

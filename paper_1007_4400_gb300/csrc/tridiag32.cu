@@ -753,8 +753,6 @@ __global__ void __launch_bounds__(32) lanczos_tail_batched_kernel(const BDesc* D
 
 template <int P, int NT, class Src>
 bool tri_launch(const Src& src, int np, int mmax, int may_skip, cudaStream_t s) {
-  static int ready = 0;   // 0 unknown, 1 usable, -1 not launchable on this device
-  if (ready < 0) return false;
   auto* kern = heev32_tri_kernel<P, NT, Src>;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(P * np, 1, 1);
@@ -768,27 +766,21 @@ bool tri_launch(const Src& src, int np, int mmax, int may_skip, cudaStream_t s) 
   at[0].val.clusterDim.z = 1;
   cfg.attrs = at;
   cfg.numAttrs = 1;
-  if (ready == 0) {
-    ready = -1;
+  // whether the device can run it, asked once (other threads wait for the answer)
+  static const bool usable = [&] {
     constexpr int kSmem = 220 * 1024;
-    if (P > 8 && cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) {
-      cudaGetLastError();
-      return false;
-    }
-    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem) != cudaSuccess) {
-      cudaGetLastError();
-      return false;
-    }
     cudaLaunchConfig_t probe = cfg;
     probe.gridDim = dim3(P, 1, 1);
     probe.dynamicSmemBytes = kSmem;
     int n = 0;
-    if (cudaOccupancyMaxActiveClusters(&n, kern, &probe) != cudaSuccess || n < 1) {
-      cudaGetLastError();
-      return false;
-    }
-    ready = 1;
-  }
+    const bool ok =
+        (P <= 8 || cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess) &&
+        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem) == cudaSuccess &&
+        cudaOccupancyMaxActiveClusters(&n, kern, &probe) == cudaSuccess && n > 0;
+    if (!ok) cudaGetLastError();
+    return ok;
+  }();
+  if (!usable) return false;
   if (cfg.dynamicSmemBytes > 220 * 1024) return false;
   if (cudaLaunchKernelEx(&cfg, kern, src, may_skip) != cudaSuccess) {
     cudaGetLastError();
