@@ -156,8 +156,9 @@ __host__ __device__ inline size_t h_smem(int m, int P) { return h_big(m, P) + (s
 // dependent multiply-adds).
 template <class Sink>
 __device__ __forceinline__ void ql_warp(int m, float* d, float* e, int lane, Sink& sink) {
+  int sweeps = 0;
   for (int l = 0; l < m; ++l) {
-    for (int it = 0;; ++it) {
+    for (;;) {
       // the first negligible coupling at or after l
       int mm = m - 1;
       for (int b = l; b < m - 1; b += 32) {
@@ -170,9 +171,11 @@ __device__ __forceinline__ void ql_warp(int m, float* d, float* e, int lane, Sin
         }
       }
       if (mm == l) break;
-      if (it == 60) {   // (two sweeps an eigenvalue are usual)
+      // Two sweeps an eigenvalue are usual, thirty the limit: of all of them together, as the sweeps from
+      // one l also split what lies above (three values of 416: 124 at one l, 760 in all)
+      if (sweeps++ == 30 * m) {
         sink.gave_up(fabsf(e[l]));
-        break;
+        return;
       }
       if (!sink.room(mm - l)) return;
       const float el = e[l];
