@@ -133,6 +133,10 @@ __device__ __forceinline__ void tc_tile(const CUtensorMap* amaps, const CUtensor
     if (rank == 0)
       for (int i = max(0, issued - p.nst); i < issued; ++i)
         mbar_wait(&full[i % NFULL], (uint32_t)(i / NFULL) & 1u, p.err, 4);
+    // and so has every release of a stage (an arrival after this CTA has left would count on a barrier of
+    // the next one)
+    for (int i = max(0, issued - p.nst); i < issued; ++i)
+      if (!pair_wait(&empty[i % p.nst], (uint32_t)(i / p.nst) & 1u, p.err, 5)) break;
   } else if (warp > 0 && lane == 0 && rank == 0) {
     // Warp 1 + part issues that part's MMAs, so that three threads share the issue: one alone takes
     // 80 clocks an MMA, more than the 72 of a 144-wide tile. The order within an accumulator is one

@@ -324,10 +324,14 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) __cluster_dims__(2, 1, 1)
       }
     }
     // every copy issued has landed before the CTAs leave (normally they were all consumed;
-    // after a wait elsewhere gave up they may still be in flight)
+    // after a wait elsewhere gave up they may still be in flight), ...
     if (rank == 0)
       for (int i = max(0, it - p.nst); i < it; ++i)
         mbar_wait(&full[i % p.nst], (uint32_t)(i / p.nst) & 1u, p.err, 25);
+    // ... and so has every release of a stage: the last commits come behind the one that the epilogue
+    // goes on from, and an arrival after this CTA has left would count on a barrier of the next one
+    for (int i = max(0, it - p.nst); i < it; ++i)
+      if (!pair_wait(&empty[i % p.nst], (uint32_t)(i / p.nst) & 1u, p.err, 26)) break;
   } else if (warp == OZ_EPI_WARPS + 1 && lane == 0 && rank == 0) {
     int it = 0;
     uint32_t chunk = 0;
