@@ -956,6 +956,7 @@ extern "C" gevp_status gevp_solve_batched(gevp_handle h, int nk, int nsteps, con
   // ---- Cholesky of every B_k (sequence-invariant): recursive with emulated off-diagonal
   // products when the products are emulated, else blocked on the FP64 pipe
   BCK(cudaMemsetAsync(P->dInfo, 0, np * sizeof(int), s));
+  BCK(cudaMemsetAsync(P->dErr, 0, sizeof(int), s));   // (an expired wait ended an earlier call)
   std::vector<char> factored(np, 0);
   if (P->oz_S > 0) {
     // the chain of leaves of one matrix leaves most SMs idle: 8 orders of 800 to 1900 take 17 ms
@@ -1261,7 +1262,9 @@ extern "C" gevp_status gevp_solve_batched(gevp_handle h, int nk, int nsteps, con
       if (P->tc) {
         BCK(cudaMemcpy(P->hErr, P->dErr, sizeof(int), cudaMemcpyDeviceToHost));
         if (P->hErr[0]) {
-          ctx_set_error(h, "batched tensor-core filter: a bounded wait expired");
+          char buf[96];
+          snprintf(buf, sizeof buf, "a bounded wait of the batched tensor-core filter ran out (code %d)", P->hErr[0]);
+          ctx_set_error(h, buf);
           return GEVP_ERR_TIMEOUT;
         }
       }
@@ -1295,7 +1298,9 @@ extern "C" gevp_status gevp_solve_batched(gevp_handle h, int nk, int nsteps, con
     int f[2] = {0, 0};
     BCK(cudaMemcpy(f, P->oz_flags, sizeof f, cudaMemcpyDeviceToHost));
     if (f[0]) {
-      ctx_set_error(h, "a bounded wait of the emulated FP64 product ran out");
+      char buf[96];
+      snprintf(buf, sizeof buf, "a bounded wait of the emulated FP64 product ran out (code %d)", f[0]);
+      ctx_set_error(h, buf);
       return GEVP_ERR_TIMEOUT;
     }
   }

@@ -575,6 +575,8 @@ cudaError_t filter_tc_reserve(FilterTC** pf, int64_t n, int m, cudaStream_t s) {
   return cudaSuccess;
 }
 
+const int* filter_tc_error(const FilterTC* f) { return f->err; }
+
 void filter_tc_release(FilterTC* f) {
   if (!f) return;
   if (f->h_pcoef) cudaFreeHost(f->h_pcoef);

@@ -611,6 +611,13 @@ gevp_status reduce_into(gevp_ctx* h, int64_t n, const double2* A, int64_t lda, d
   return GEVP_OK;
 }
 
+gevp_status wait_expired(gevp_ctx* h, const char* where, int code) {
+  char buf[96];
+  snprintf(buf, sizeof buf, "a bounded wait of %s ran out (code %d)", where, code);
+  h->err = buf;
+  return GEVP_ERR_TIMEOUT;
+}
+
 // error code of an emulated-product kernel since the last check (0: none), then cleared
 gevp_status oz_check(gevp_ctx* h) {
   if (!h->ozflags) return GEVP_OK;
@@ -620,10 +627,7 @@ gevp_status oz_check(gevp_ctx* h) {
   if (f[0] == 0 && f[1] == 0) return GEVP_OK;
   CK(cudaMemsetAsync(h->ozflags, 0, 2 * sizeof(int), h->stream));
   CK(cudaStreamSynchronize(h->stream));
-  if (f[0] != 0) {
-    h->err = "a bounded wait of the emulated FP64 product ran out";
-    return GEVP_ERR_TIMEOUT;
-  }
+  if (f[0] != 0) return wait_expired(h, "the emulated FP64 product", f[0]);
   h->err = "NaN or Inf in an operand of the emulated FP64 product";
   return GEVP_ERR_INVALID_VALUE;
 }
@@ -768,8 +772,7 @@ struct EmScope {
     CK(cudaGetLastError());
     if (f[0] != 0) {
       CK(cudaMemsetAsync(h->ozflags + 2, 0, sizeof(int), h->stream));
-      h->err = "a bounded wait of the emulated FP64 product ran out";
-      return GEVP_ERR_TIMEOUT;
+      return wait_expired(h, "the emulated FP64 product", f[0]);
     }
     return heev_status(h, f[1]);
   }
@@ -1228,6 +1231,7 @@ gevp_status solve_one(gevp_ctx* h, int64_t n, const double2* A, int64_t lda, con
     if (it >= o.max_outer) break;
     orth_val = -1.0;   // Q changes in this round
     // ---- filter the active columns
+    const bool lowp = prec != GEVP_PREC_FP64;
     int ma = m - S.nlock;
     double hi = S.upper;
     double lo = S.have_theta ? S.theta[m - 1] : S.a_est;
@@ -1266,10 +1270,12 @@ gevp_status solve_one(gevp_ctx* h, int64_t n, const double2* A, int64_t lda, con
     tm.mark(PH_ORTH);
     TRY(rayleigh_ritz(h, n, S.nlock, ma, h->C, n, o.refine_iters, st));
     // one status read per round: the Ritz values, residuals and the CholQR passes' pivots
-    int orth_info[2] = {0, 0};
-    TRY(sync_reads(h, {{h->theta + S.nlock, S.theta.data() + S.nlock, ma * sizeof(double)},
+    int orth_info[2] = {0, 0}, filter_err = 0;
+    TRY(sync_reads(h, {{lowp ? filter_tc_error(h->tc) : nullptr, &filter_err, lowp ? sizeof filter_err : 0},
+                       {h->theta + S.nlock, S.theta.data() + S.nlock, ma * sizeof(double)},
                        {h->res + S.nlock, S.res.data() + S.nlock, ma * sizeof(double)},
                        {h->info, orth_info, pend ? sizeof orth_info : 0}}));
+    if (filter_err != 0) return wait_expired(h, "the tensor-core filter", filter_err);
     if (pend && (orth_info[0] != 0 || orth_info[1] != 0)) {
       // a CholQR pass met a non-positive pivot: the projection above used a bad basis.
       // Orthonormalise the (intact) filtered block again with the shifted fallback and
@@ -1859,7 +1865,7 @@ gevp_status gevp_chebyshev_filter(gevp_handle h, int64_t n, const void* C, int64
     CK(filter_tc_apply(h->tc, n, m, (const double2*)Y, ldy, (double2*)Y, ldy, degree, lo, hi, s, nsplit, &err,
                        h->stream));
     CK(cudaStreamSynchronize(h->stream));
-    if (err) { h->err = "tensor-core filter: a bounded wait expired"; return GEVP_ERR_TIMEOUT; }
+    if (err) return wait_expired(h, "the tensor-core filter", err);
     return GEVP_OK;
   }
   double2* out = filter_fp64(h, n, (const double2*)C, ldc, (const double2*)Y, ldy, m, degree, lo, hi, s, h->Y1,
@@ -1883,7 +1889,7 @@ gevp_status gevp_matmul_tc(gevp_handle h, int64_t n, int m, const void* C, int64
   CK(filter_tc_product(h->tc, n, m, (const double2*)Y, ldy, (double2*)D, ldd, 1, &err, h->stream));
   CK(cudaStreamSynchronize(h->stream));
   CK(cudaGetLastError());
-  if (err) { h->err = "tensor-core product: a bounded wait expired"; return GEVP_ERR_TIMEOUT; }
+  if (err) return wait_expired(h, "the tensor-core product", err);
   return GEVP_OK;
 }
 

@@ -262,6 +262,7 @@ void energy_backward_ws(int64_t n, int nev, const double2* X, int64_t ldx, const
 struct FilterTC;   // opaque, owned by the handle
 bool tc_filter_supported();
 cudaError_t filter_tc_reserve(FilterTC** f, int64_t n, int m, cudaStream_t s);
+const int* filter_tc_error(const FilterTC* f);   // device: the code of an expired wait of the last application
 void filter_tc_release(FilterTC* f);
 // nsplit: BF16 pieces per operand (1 = BF16 filter, 3 = FP32-class, see filter_tc.cu)
 cudaError_t filter_tc_set_matrix(FilterTC* f, int64_t n, const double2* C, int64_t ldc, int nsplit, cudaStream_t s);

@@ -19,10 +19,24 @@ __device__ __forceinline__ void mbar_expect_tx(uint64_t* bar, uint32_t bytes) {
 __device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
   asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(su32(bar)) : "memory");
 }
+// Waits are bounded in time (about two seconds of SM clocks): the hardware may suspend a try_wait for
+// as long as it likes, so a number of tries is no bound.
+constexpr long long kWaitClocks = 1ll << 32;
+struct WaitLimit {
+  long long from = 0;
+  uint32_t tries = 0;
+  __device__ __forceinline__ bool over() {
+    if (++tries & 63u) return false;
+    const long long now = clock64();
+    if (from == 0) from = now;
+    return now - from > kWaitClocks;
+  }
+};
 // bounded wait on the phase with the given parity; false (and an error code) on expiry
 __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, int* err, int code) {
   uint32_t addr = su32(bar);
-  for (uint32_t it = 0; it < (1u << 24); ++it) {
+  WaitLimit limit;
+  do {
     uint32_t ok;
     asm volatile(
         "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}\n"
@@ -30,7 +44,7 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, int* e
         : "r"(addr), "r"(parity)
         : "memory");
     if (ok) return true;
-  }
+  } while (!limit.over());
   atomicCAS(err, 0, code);
   return false;
 }
@@ -92,7 +106,8 @@ __device__ __forceinline__ void pair_arrive(uint32_t remote) {
 // mbar_wait for a barrier that the other CTA of the pair arrives on
 __device__ __forceinline__ bool pair_wait(uint64_t* bar, uint32_t parity, int* err, int code) {
   const uint32_t addr = su32(bar);
-  for (uint32_t it = 0; it < (1u << 24); ++it) {
+  WaitLimit limit;
+  do {
     uint32_t ok;
     asm volatile(
         "{\n .reg .pred p;\n mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, "
@@ -101,7 +116,7 @@ __device__ __forceinline__ bool pair_wait(uint64_t* bar, uint32_t parity, int* e
         : "r"(addr), "r"(parity)
         : "memory");
     if (ok) return true;
-  }
+  } while (!limit.over());
   atomicCAS(err, 0, code);
   return false;
 }
