@@ -153,6 +153,7 @@ __global__ void __launch_bounds__(LT, 1) lanczos_cluster_kernel(Src src, int j0,
   };
   float bprev = j0 > 0 ? p.ab[2 * j0 - 1] : 0.f;
   int made = 0;
+  if (C > 1) cl.sync();   // every CTA has started before another writes to its slots
   for (int j = j0; j < k; ++j) {
     if (full) {
       const float2* vj = p.V + (int64_t)j * n;
