@@ -100,6 +100,8 @@ __device__ __forceinline__ void tc_tile(const CUtensorMap* amaps, const CUtensor
     mbar_init(&done, 3);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
+  __syncwarp();
+  pair_sync();   // both CTAs run (the allocation takes both), their barriers are initialised
   if (warp == 0) {
     asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(su32(&tmem_sh)),
                  "r"(p.tmem_cols)
@@ -108,7 +110,6 @@ __device__ __forceinline__ void tc_tile(const CUtensorMap* amaps, const CUtensor
   }
   fence_before();
   __syncthreads();
-  pair_sync();   // both CTAs' barriers are initialised before any remote arrival
   fence_after();
   const uint32_t tmem = tmem_sh;
   const int row0 = m0 + TM * rank;

@@ -290,6 +290,8 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) __cluster_dims__(2, 1, 1)
     }
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
+  __syncwarp();
+  pair_sync();   // both CTAs run (the allocation takes both), their barriers are initialised
   if (warp == 0) {
     asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(su32(&tmem_sh)), "r"(512)
                  : "memory");
@@ -297,7 +299,6 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) __cluster_dims__(2, 1, 1)
   }
   fence_before();
   __syncthreads();
-  pair_sync();   // both CTAs' barriers are initialised before any remote arrival
   fence_after();
   const uint32_t tmem = tmem_sh;
 

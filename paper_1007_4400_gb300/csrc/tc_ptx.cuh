@@ -24,9 +24,7 @@ __device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
 constexpr long long kWaitClocks = 1ll << 32;
 struct WaitLimit {
   long long from = 0;
-  uint32_t tries = 0;
   __device__ __forceinline__ bool over() {
-    if (++tries & 63u) return false;
     const long long now = clock64();
     if (from == 0) from = now;
     return now - from > kWaitClocks;
