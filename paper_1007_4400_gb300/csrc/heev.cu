@@ -4,7 +4,7 @@
 // CTA would take milliseconds. Instead:
 //   1. FP32 eigenvectors accurate to about 1e-6 (FP32 runs at 128 FMA per clock per SM):
 //      Householder tridiagonalisation and QL in a thread-block cluster (tridiag32.cu); orders
-//      above its limit by parallel-ordered two-sided Jacobi on all SMs, a launch a round;
+//      above its limit by parallel-ordered two-sided Jacobi on all SMs (cooperative launch);
 //   2. Ogita & Aishima's iterative refinement for symmetric/Hermitian eigenvector
 //      matrices (Japan J. Ind. Appl. Math. 35, 2018), which converges quadratically and
 //      consists of four FP64 GEMMs per step spread over all SMs. Pairs closer than the
@@ -18,6 +18,7 @@
 // make the phase, hence the rotation, non-unitary) and skips couplings below FP32
 // significance relative to the diagonal.
 #include "gevp_internal.cuh"
+#include <cooperative_groups.h>
 #include <algorithm>
 
 namespace gevp {
@@ -52,17 +53,34 @@ __device__ float block_sum(float v, float* red) {
   return s;
 }
 
-// Element access to G for the Jacobi rounds (shared or global memory).
-struct GMat {
+// L2 = true: load through L2 only (the multi-CTA variant; other CTAs wrote these
+// elements in the previous round and L1 is not coherent across SMs)
+template <bool L2>
+__device__ __forceinline__ float2 ld2(const float2* p) {
+  if constexpr (L2) return __ldcg(p);
+  else return *p;
+}
+
+// Element access to G for the Jacobi rounds: a plain matrix (shared or global memory, the
+// one-CTA forms), or a global matrix read through L2 (the cooperative form: other CTAs wrote
+// it and L1 is not coherent across SMs).
+struct GPlain {
   float2* g;
   int m;
   __device__ __forceinline__ float2 ld(int i, int j) const { return g[i * m + j]; }
   __device__ __forceinline__ void st(int i, int j, float2 v) const { g[i * m + j] = v; }
 };
+struct GL2 {
+  float2* g;
+  int m;
+  __device__ __forceinline__ float2 ld(int i, int j) const { return __ldcg(g + i * m + j); }
+  __device__ __forceinline__ void st(int i, int j, float2 v) const { g[i * m + j] = v; }
+};
 // Rotation of pair k of round `step`: U = [[c, s], [-s conj(ph), c conj(ph)]] acting on
 // columns (p, q), stored as (c, s, Re ph, Im ph); identity for the dummy index q = m of
 // odd orders and for couplings below FP32 significance relative to the diagonal.
-__device__ __forceinline__ void jacobi_pair_params(const GMat& G, int m, int np, int step, int k, float4* U,
+template <class Acc>
+__device__ __forceinline__ void jacobi_pair_params(const Acc& G, int m, int np, int step, int k, float4* U,
                                                    int (*PQ)[2]) {
   int p, q;
   block_pair(step, k, np, &p, &q);
@@ -94,7 +112,8 @@ __device__ __forceinline__ float2 cmulf(float2 a, float2 b) {
 // e < npairs^2, a = row pair, b = column pair), and Z <- Z U into independent row pieces
 // (tasks after those). Every element of G is read from G and written to Gout once per
 // step (Gout = G in place, or the other buffer of a ping-pong pair).
-__device__ __forceinline__ void jacobi_apply(const GMat& G, const GMat& Gout, float2* Z, int m, int npairs, int e,
+template <class Acc, bool ZL2>
+__device__ __forceinline__ void jacobi_apply(const Acc& G, const Acc& Gout, float2* Z, int m, int npairs, int e,
                                              const float4* U, const int (*PQ)[2]) {
   if (e < npairs * npairs) {
     const int a = e / npairs, b = e % npairs;
@@ -154,7 +173,7 @@ __device__ __forceinline__ void jacobi_apply(const GMat& G, const GMat& Gout, fl
     const float4 u = U[b];
     const float c = u.x, sn = u.y;
     const float2 phc = make_float2(u.z, -u.w);
-    const float2 zr = Z[i * m + r], zs = cmulf(Z[i * m + s], phc);
+    const float2 zr = ld2<ZL2>(Z + i * m + r), zs = cmulf(ld2<ZL2>(Z + i * m + s), phc);
     Z[i * m + r] = make_float2(c * zr.x - sn * zs.x, c * zr.y - sn * zs.y);
     Z[i * m + s] = make_float2(sn * zr.x + c * zs.x, sn * zr.y + c * zs.y);
   }
@@ -198,11 +217,11 @@ __device__ void jacobi32_body(int m, float2* Gg, float2* Z, float* w, int* perm,
     if (off <= tol2 || (off > 0.9f * off_prev && off <= 1e-12f * fro2)) break;
     off_prev = off;
     for (int step = 0; step < np - 1; ++step) {
-      const GMat Ga{G, m};
+      const GPlain Ga{G, m};
       for (int k = tid; k < npairs; k += JT) jacobi_pair_params(Ga, m, np, step, k, U, PQ);
       __syncthreads();
       for (int e = tid; e < npairs * npairs + m * npairs; e += JT)
-        jacobi_apply(Ga, Ga, Z, m, npairs, e, U, PQ);
+        jacobi_apply<GPlain, false>(Ga, Ga, Z, m, npairs, e, U, PQ);
       __syncthreads();
     }
   }
@@ -220,48 +239,66 @@ __device__ void jacobi32_body(int m, float2* Gg, float2* Z, float* w, int* perm,
 
 constexpr int kJacobiSmemMax = 160;   // largest m whose G (m * m FP32 complex) is kept in shared memory
 
-// The same for orders above the one-CTA shared-memory size, on all SMs: a launch a rotation round, so
-// that no CTA ever waits for another one to be placed. (One launch with a grid barrier a round needs
-// every SM at a time; a thread-block cluster of another stream needs its SMs at a time too, and the two
-// have been seen to wait for each other without end.) Every CTA computes the round's rotations from G
-// and applies its share of the 2 x 2 block and Z tasks; the rounds alternate between G and Gb (m x m
-// each): a round reads one and writes the other, so the rotations are never computed from entries that
-// another CTA has already rotated. red[0] += ||G||_F^2, red[1] += the off-diagonal's.
-__global__ void __launch_bounds__(JT) jacobi32_norms_kernel(int m, const float2* G, float* red_g) {
-  __shared__ float red[32];
-  float all = 0.f, off = 0.f;
-  for (int e = blockIdx.x * JT + threadIdx.x; e < m * m; e += gridDim.x * JT) {
-    const float2 g = G[e];
-    const float a = g.x * g.x + g.y * g.y;
-    all += a;
-    if (e / m != e % m) off += a;
-  }
-  all = block_sum(all, red);
-  off = block_sum(off, red);
-  if (threadIdx.x == 0) {
-    atomicAdd(&red_g[0], all);
-    atomicAdd(&red_g[1], off);
-  }
-}
-__global__ void __launch_bounds__(JT) jacobi32_unit_kernel(int m, float2* Z) {
-  for (int e = blockIdx.x * JT + threadIdx.x; e < m * m; e += gridDim.x * JT)
-    Z[e] = make_float2((e / m) == (e % m) ? 1.f : 0.f, 0.f);
-}
-__global__ void __launch_bounds__(JT) jacobi32_round_kernel(int m, float2* G, float2* Gb, float2* Z, int step) {
+// Multi-CTA variant for orders above the one-CTA shared-memory size: the same rounds, each
+// CTA computing every rotation of a round (redundantly, from G in global memory) and
+// applying its share of the 2 x 2 block and Z tasks, with one grid barrier per round
+// (cooperative launch: all CTAs are resident). The rounds alternate between G and Gb
+// (m x m each): a round reads one and writes the other, so a CTA still computing the
+// round's rotations never sees entries another CTA has already rotated. red: 2 +
+// max_sweeps floats, zero on entry. G and Gb are both destroyed.
+__global__ void __launch_bounds__(JT) jacobi32_coop_kernel(int m, float2* G, float2* Gb, float2* Z, float* w,
+                                                           int* perm, int max_sweeps, float* red_g) {
+  namespace cg = cooperative_groups;
+  cg::grid_group grid = cg::this_grid();
   __shared__ float4 U[512];
   __shared__ int PQ[512][2];
-  const int np = (m % 2) ? m + 1 : m, npairs = np / 2;
-  const GMat A{G, m}, B{Gb, m};
-  for (int k = threadIdx.x; k < npairs; k += JT) jacobi_pair_params(A, m, np, step, k, U, PQ);
-  __syncthreads();
-  for (int e = blockIdx.x * JT + threadIdx.x; e < npairs * npairs + m * npairs; e += gridDim.x * JT)
-    jacobi_apply(A, B, Z, m, npairs, e, U, PQ);
-}
-__global__ void __launch_bounds__(JT) jacobi32_sort_kernel(int m, const float2* G, float* w, int* perm) {
-  for (int i = threadIdx.x; i < m; i += JT) {
-    const float wi = G[i * m + i].x;
+  __shared__ float red[32];
+  const int tid = threadIdx.x;
+  const int gtid = blockIdx.x * JT + tid, gsz = gridDim.x * JT;
+  for (int e = gtid; e < m * m; e += gsz) Z[e] = make_float2((e / m) == (e % m) ? 1.f : 0.f, 0.f);
+  const int np = (m % 2) ? m + 1 : m;
+  const int npairs = np / 2;
+  float f = 0.f;
+  for (int e = gtid; e < m * m; e += gsz) { float2 g = G[e]; f += g.x * g.x + g.y * g.y; }
+  f = block_sum(f, red);
+  if (tid == 0) atomicAdd(&red_g[0], f);
+  grid.sync();
+  const float fro2 = __ldcg(&red_g[0]);
+  const float tol2 = 1e-16f * fro2;
+  float off_prev = 3.0e38f;
+  float2* Gc = G;    // the current matrix; rounds write the other buffer
+  float2* Gn = Gb;
+  for (int sweep = 0; sweep < max_sweeps && m > 1; ++sweep) {
+    float off = 0.f;
+    for (int e = gtid; e < m * m; e += gsz) {
+      int i = e / m, j = e % m;
+      if (i != j) { float2 g = __ldcg(Gc + e); off += g.x * g.x + g.y * g.y; }
+    }
+    off = block_sum(off, red);
+    if (tid == 0) atomicAdd(&red_g[1 + sweep], off);
+    grid.sync();
+    off = __ldcg(&red_g[1 + sweep]);   // the same value in every CTA: a uniform decision
+    if (off <= tol2 || (off > 0.9f * off_prev && off <= 1e-12f * fro2)) break;
+    off_prev = off;
+    for (int step = 0; step < np - 1; ++step) {
+      const GL2 Ac{Gc, m}, An{Gn, m};
+      for (int k = tid; k < npairs; k += JT) jacobi_pair_params(Ac, m, np, step, k, U, PQ);
+      __syncthreads();
+      for (int e = gtid; e < npairs * npairs + m * npairs; e += gsz)
+        jacobi_apply<GL2, true>(Ac, An, Z, m, npairs, e, U, PQ);
+      grid.sync();
+      float2* t = Gc;
+      Gc = Gn;
+      Gn = t;
+    }
+  }
+  if (blockIdx.x != 0) return;
+  for (int i = tid; i < m; i += JT) {
+    float wi = __ldcg(Gc + i * m + i).x;
     int r = 0;
-    for (int j = 0; j < m; ++j) r += rank_before(rank_key(G[j * m + j].x), j, rank_key(wi), i);
+    for (int j = 0; j < m; ++j) {
+      r += rank_before(rank_key(__ldcg(Gc + j * m + j).x), j, rank_key(wi), i);
+    }
     perm[r] = i;
     w[r] = wi;
   }
@@ -568,36 +605,30 @@ size_t heev_ws_bytes(int m, size_t split_elems) {
   return b + 16 * 256;
 }
 
-// Jacobi on all SMs for large m (G and Gb are destroyed, red: 2 floats). The host reads the norms before
-// every sweep; false if a CUDA call failed.
-bool jacobi32_large(int m, float2* G, float2* Gb, float2* Z, float* w, int* perm, int max_sweeps, float* red,
-                    cudaStream_t s) {
+// Cooperative multi-CTA Jacobi for large m; false if it cannot be launched (then the
+// caller runs the one-CTA kernel).
+bool jacobi32_coop(int m, float2* G, float2* Gb, float2* Z, float* w, int* perm, int max_sweeps, float* red,
+                   cudaStream_t s) {
+  int dev = 0, sms = 0, coop = 0, per_sm = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) return false;
+  cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  if (!coop || cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, jacobi32_coop_kernel, JT, 0) != cudaSuccess ||
+      per_sm < 1)
+    return false;
   const int np = (m % 2) ? m + 1 : m, npairs = np / 2;
   const int64_t tasks = (int64_t)npairs * npairs + (int64_t)m * npairs;
-  const int grid = (int)std::min<int64_t>(2 * 152, (tasks + JT - 1) / JT);
-  jacobi32_unit_kernel<<<152, JT, 0, s>>>(m, Z);
-  LAUNCH_NOTE(1);
-  float off_prev = 3.0e38f;
-  for (int sweep = 0; sweep < max_sweeps; ++sweep) {
-    float h[2] = {0.f, 0.f};
-    if (cudaMemsetAsync(red, 0, 2 * sizeof(float), s) != cudaSuccess) return false;
-    jacobi32_norms_kernel<<<152, JT, 0, s>>>(m, G, red);
-    LAUNCH_NOTE(1);
-    if (cudaMemcpyAsync(h, red, sizeof h, cudaMemcpyDeviceToHost, s) != cudaSuccess ||
-        cudaStreamSynchronize(s) != cudaSuccess)
-      return false;
-    // converged to FP32 noise (1e-8 ||G||_F), stagnated near it, or not finite
-    if (!(h[1] > 1e-16f * h[0]) || (h[1] > 0.9f * off_prev && h[1] <= 1e-12f * h[0])) break;
-    off_prev = h[1];
-    for (int step = 0; step < np - 1; ++step) {
-      jacobi32_round_kernel<<<grid, JT, 0, s>>>(m, G, Gb, Z, step);
-      std::swap(G, Gb);
-    }
-    LAUNCH_NOTE(np - 1);
+  int grid = (int)std::min<int64_t>((int64_t)per_sm * sms, (tasks + JT - 1) / JT);
+  grid = std::max(grid, 1);
+  if (max_sweeps > 62) max_sweeps = 62;
+  if (cudaMemsetAsync(red, 0, 64 * sizeof(float), s) != cudaSuccess) return false;
+  void* args[] = {&m, &G, &Gb, &Z, &w, &perm, &max_sweeps, &red};
+  if (cudaLaunchCooperativeKernel((const void*)jacobi32_coop_kernel, grid, JT, args, 0, s) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
   }
-  jacobi32_sort_kernel<<<1, JT, 0, s>>>(m, G, w, perm);
   LAUNCH_NOTE(1);
-  return cudaGetLastError() == cudaSuccess;
+  return true;
 }
 
 // mmax: the largest matrix order among the problems
@@ -624,13 +655,13 @@ const int* heev_small(int m, const double2* G, int64_t ldg, double* theta, doubl
   LAUNCH_NOTE(1);
   // FP32 eigenvectors by tridiagonalisation (a nearly diagonal G may start from Z = I when the
   // refinement has the three steps that needs; the FP64 scratch is free until then). Orders above
-  // its limit: Jacobi on all SMs (E holds its second FP32 buffer), below it (no cluster to be had) in
-  // one CTA.
+  // its limit: Jacobi on all SMs (cooperative launch; E holds its second FP32 buffer), or, when
+  // that cannot be launched, in one CTA.
   if (!heev32(m, w.G32, w.Z, m, w.w32, (int*)(w.scal + 16), w.Z32, w.T, w.R, w.S, w.E, refine_iters >= 3 ? 1 : 0, s)) {
     failed = nullptr;
     bool done = false;
     if (m > kJacobiSmemMax)
-      done = jacobi32_large(m, w.G32, (float2*)w.E, w.Z32, w.w32, w.perm, 40, (float*)(w.scal + 16), s);
+      done = jacobi32_coop(m, w.G32, (float2*)w.E, w.Z32, w.w32, w.perm, 40, (float*)(w.scal + 16), s);
     if (!done) {
       jacobi32_kernel<<<1, JT, jacobi_smem(m), s>>>(m, w.G32, w.Z32, w.w32, w.perm, 40);
       LAUNCH_NOTE(1);

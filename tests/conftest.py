@@ -14,6 +14,11 @@ def pytest_configure(config):
     config.addinivalue_line("markers", "slow: full-size parity case")
 
 
+def pytest_collection_modifyitems(items):
+    # the full-size cases last: a run that a time limit ends has seen the others
+    items.sort(key=lambda item: item.get_closest_marker("slow") is not None)
+
+
 @pytest.fixture(scope="session")
 def orc():
     import oracle

@@ -1,5 +1,5 @@
-"""The small eigensolver above the order of its tridiagonal start (600), where FP32 Jacobi runs as one
-launch a round: even and odd orders up to the largest, well separated values and a multiple one."""
+"""The small eigensolver above the order of its tridiagonal start (600), where FP32 Jacobi runs on all
+SMs: even and odd orders up to the largest, well separated values and a multiple one."""
 import pytest
 import torch
 
