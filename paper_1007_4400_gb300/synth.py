@@ -23,6 +23,8 @@ torch on the requested device (CPU or CUDA); the draws do not depend on the devi
 from __future__ import annotations
 
 import math
+from collections import deque
+from concurrent.futures import ThreadPoolExecutor
 from dataclasses import dataclass, field
 
 import numpy as np
@@ -121,8 +123,12 @@ def _norm2_lanczos(P: torch.Tensor, k: int = 60) -> float:
 def hermitian_unit_norm(rng: np.random.Generator, n: int, device="cpu") -> torch.Tensor:
     """P = (G + G^H)/2 with complex standard normal G, divided by its spectral norm (for
     n > 8192 by a Lanczos estimate of it)."""
-    G = torch.from_numpy(_cnormal(rng, (n, n))).to(device)
-    P = hermitian_part(G)
+    return _unit_norm(_cnormal(rng, (n, n)), device)
+
+
+def _unit_norm(G: np.ndarray, device) -> torch.Tensor:
+    n = G.shape[0]
+    P = hermitian_part(torch.from_numpy(G).to(device))
     del G
     if n > 8192:
         return (P / _norm2_lanczos(P)).contiguous()
@@ -178,13 +184,21 @@ def make_sequence(config_id: int, n: int, nprob: int, nev: int, nex: int, device
     A0, B = known_spectrum_pencil(L, Q, torch.from_numpy(lam).to(device))
     As = [A0]
     eps = []
-    for l in range(nprob - 1):
-        prng = rng_for(config_id, seed_index, offset=100 + l)
-        P = hermitian_unit_norm(prng, n, device)
-        e = eps0 * decay ** l
-        eps.append(e)
-        As.append(hermitian_part(As[-1] + e * P).contiguous())
-        del P
+    # every P_l has a generator of its own: the draws of the next three run beside the device's work
+    with ThreadPoolExecutor(max_workers=3) as pool:
+        def draw(l):
+            return pool.submit(lambda: _cnormal(rng_for(config_id, seed_index, offset=100 + l), (n, n)))
+
+        ahead = deque(draw(l) for l in range(min(3, nprob - 1)))
+        for l in range(nprob - 1):
+            G = ahead.popleft().result()
+            if l + 3 < nprob - 1:
+                ahead.append(draw(l + 3))
+            P = _unit_norm(G, device)
+            e = eps0 * decay ** l
+            eps.append(e)
+            As.append(hermitian_part(As[-1] + e * P).contiguous())
+            del P, G
     return Sequence(n=n, nev=nev, nex=nex, A=As, B=B, lam0=lam, L_true=L, Q_true=Q,
                     eps=eps, config_id=config_id)
 
