@@ -144,9 +144,9 @@ def kernel_case(args):
         Y = Y * torch.logspace(0, 3, m, dtype=torch.float64, device=dev)[None, :]
         G = torch.randn((n, n), dtype=torch.complex128, device=dev, generator=g)
         C = (0.5 * (G + G.conj().T) * (25.0 / n ** 0.5)).contiguous()
-        Q = gevp.cholqr2(Y)
-        Q = gevp.cholqr2(Q)
-        gevp.rayleigh_ritz(C, Q)
+        Q = gevp.cholqr2(Y, slices=0)   # (by default its Gram matrix is emulated)
+        Q = gevp.cholqr2(Q, slices=0)
+        gevp.rayleigh_ritz(C, Q, slices=0)
         torch.cuda.synchronize()
         print(f"kernel case cholqr done: n={n} m={m}")
         return 0
@@ -350,7 +350,7 @@ def roofline_entries(gevp, dev, live, ms_total, steps, sm_mhz):
     the next problem's reduction runs concurrently on a side stream, so these include
     contention). isolated: one launch shape timed alone, the shape of the committed ncu
     capture whose DRAM traffic is quoted: the emulated product on the reduction's shape (the
-    largest share of its time), the Gram kernel on a Gram matrix below the emulated ones, the FP64 GEMM on
+    largest share of its time), the Gram kernel on the bench's Gram matrix (FP64 pipe), the FP64 GEMM on
     an FP64 filter step (its largest single shape; in the default step it runs the n m^2
     and m^3 products of the projections, CholQR and the small eigensolver).
     Peaks: FP64 from the unit count (152 SMs x 2 FMA/clk x 2 flop x the max SM clock); BF16
@@ -399,18 +399,18 @@ def roofline_entries(gevp, dev, live, ms_total, steps, sm_mhz):
             "traffic": _profile_traffic("oz_gemm_n2048"), "alg_bytes_per_launch": 3 * 16.0 * 2048 ** 2,
             "fp64_equiv_tflops": rec["alg_flop"] / (rec["ms"] * 1e-3) / 1e12}
         del Ai, Bi
-    # Gram kernel, Y^H Y of a block whose Gram matrix is not emulated (n 2048, m 88): 8 n m (m + 1) / 2 flop
+    # Gram kernel, Y^H Y of the bench's block (n 2048, m 140) on the FP64 pipe: 8 n m (m + 1) / 2 flop
     if "zgram_kernel" in per:
-        n, m = 2048, 88
+        n, m = 2048, 140
         Y0 = torch.randn((n, m), dtype=torch.complex128, device=dev, generator=g)
         Y0 = Y0 * torch.logspace(0, 3, m, dtype=torch.float64, device=dev)[None, :]
-        rec = _timed_class(gevp, "zgram_kernel", lambda: gevp.cholqr2(Y0.clone()), 5)
+        rec = _timed_class(gevp, "zgram_kernel", lambda: gevp.cholqr2(Y0.clone(), slices=0), 5)
         ms = rec["ms"] / max(1, rec["launches"])
         ach = 8.0 * n * m * (m + 1) / 2 / (ms * 1e-3) / 1e12
         per["zgram_kernel"]["isolated"] = {
-            "shape": "Gram matrix Y^H Y, n 2048, m 88 (lower triangle, 8 n m (m+1)/2 flop)", "ms_per_launch": ms,
-            "achieved": ach, "peak": fp64_peak, "frac": ach / fp64_peak, "traffic": None,
-            "alg_bytes_per_launch": 16.0 * n * m}
+            "shape": "Gram matrix Y^H Y, n 2048, m 140 (lower triangle, 8 n m (m+1)/2 flop)", "ms_per_launch": ms,
+            "achieved": ach, "peak": fp64_peak, "frac": ach / fp64_peak,
+            "traffic": _profile_traffic("zgram_n2048_m140"), "alg_bytes_per_launch": 16.0 * n * m}
         del Y0
     # FP64 GEMM: one FP64 filter step C Y, n 2048 x m 140 (8 n^2 m flop), C read once
     if "zgemm_kernel" in per:

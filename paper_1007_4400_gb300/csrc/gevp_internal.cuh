@@ -151,7 +151,8 @@ size_t trtri_ws_elems(int64_t n);
 
 // ---------------------------------------------------------------- small Hermitian eigensolver
 // G (m x m Hermitian, FP64) -> theta ascending (m), Z (m x m, columns = eigenvectors).
-// FP32 parallel Jacobi followed by FP64 Ogita-Aishima refinement built from FP64 GEMMs.
+// FP32 eigenvectors (tridiag32.cu; Jacobi above order 600), then FP64 Ogita-Aishima refinement built
+// from FP64 GEMMs and exact rotations.
 struct HeevWork {
   float2* G32; float2* Z32; float* w32; int* perm;
   double2 *Z, *R, *S, *T, *E;   // m x m each

@@ -1,6 +1,6 @@
-// Inline-PTX wrappers shared by the tcgen05 kernels: mbarriers (bounded waits), TMA tile
-// loads, UMMA shared-memory and instruction descriptors, MMA issue/commit and TMEM
-// loads/stores. Everything is in an anonymous namespace: each kernel file gets its own copy.
+// Inline-PTX wrappers shared by the tcgen05 kernels: mbarriers (bounded waits), UMMA
+// shared-memory and instruction descriptors, TMA tile loads and MMA issue/commit of a pair of
+// CTAs, TMEM loads/stores. Everything is in an anonymous namespace: each kernel file gets its own copy.
 #pragma once
 #include <cuda.h>
 #include <cstdint>
@@ -15,9 +15,6 @@ __device__ __forceinline__ void mbar_init(uint64_t* bar, uint32_t count) {
 }
 __device__ __forceinline__ void mbar_expect_tx(uint64_t* bar, uint32_t bytes) {
   asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(su32(bar)), "r"(bytes) : "memory");
-}
-__device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
-  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(su32(bar)) : "memory");
 }
 // Waits are bounded in time (about two seconds of SM clocks): the hardware may suspend a try_wait for
 // as long as it likes, so a number of tries is no bound.
@@ -46,20 +43,6 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, int* e
   atomicCAS(err, 0, code);
   return false;
 }
-__device__ __forceinline__ void tma_load_2d(void* dst, const CUtensorMap* map, int x, int y, uint64_t* bar) {
-  asm volatile(
-      "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];" ::"r"(
-          su32(dst)),
-      "l"((uint64_t)map), "r"(x), "r"(y), "r"(su32(bar))
-      : "memory");
-}
-__device__ __forceinline__ void tma_load_3d(void* dst, const CUtensorMap* map, int x, int y, int z, uint64_t* bar) {
-  asm volatile(
-      "cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], [%5];" ::
-          "r"(su32(dst)),
-      "l"((uint64_t)map), "r"(x), "r"(y), "r"(z), "r"(su32(bar))
-      : "memory");
-}
 __device__ __forceinline__ void fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 
@@ -77,17 +60,6 @@ __device__ __forceinline__ uint64_t sdesc(uint32_t saddr) {
 __host__ __device__ constexpr uint32_t idesc_bf16(int M, int N) {
   return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
 }
-__device__ __forceinline__ void umma(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc, uint32_t acc) {
-  asm volatile(
-      "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(d),
-      "l"(a), "l"(b), "r"(idesc), "r"(acc)
-      : "memory");
-}
-__device__ __forceinline__ void umma_commit(uint64_t* bar) {
-  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(su32(bar))
-               : "memory");
-}
-
 // ---- pairs of CTAs (cta_group::2, a cluster of two)
 __device__ __forceinline__ uint32_t pair_mapa(uint32_t addr, uint32_t rank) {
   uint32_t r;

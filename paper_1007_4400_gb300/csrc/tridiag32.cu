@@ -16,7 +16,7 @@
 //      sweep's rotations in a shared-memory ring; warp 1 copies them to global memory and
 //      publishes the number of finished sweeps; the remaining warps of all CTAs hold the rows of
 //      the tridiagonal's eigenvector matrix, 32 to a warp, in shared memory and apply the
-//      sweeps as they come. The recurrence is the critical path (about 60 clocks a rotation).
+//      sweeps as they come. The recurrence is the critical path (about 100 clocks a rotation).
 // heev32_back_kernel: one warp per eigenvector applies the reflectors, H_0 .. H_{m-2}, and writes
 // the column to its place in ascending order in FP64.
 //
@@ -147,7 +147,8 @@ __host__ __device__ inline size_t h_big(int m, int P) {
 }
 __host__ __device__ inline size_t h_smem(int m, int P) { return h_big(m, P) + (size_t)6 * m * 8 + (size_t)2 * m * 4; }
 
-// Implicit QL iteration (Wilkinson shifts, chased from the bottom up) on the symmetric
+// Implicit QL iteration (Wilkinson shifts, chased from the bottom up; the procedure imtql2 of Martin
+// and Wilkinson, Handbook for Automatic Computation II, published in EISPACK) on the symmetric
 // tridiagonal matrix d[0..m-1], e[0..m-2] (shared memory, entries about 1 or less; d receives the
 // eigenvalues), by one warp with all lanes alike. Rotation i mixes columns i and i + 1 of the
 // eigenvector matrix: z_{i+1} <- s z_i + c z_{i+1}, z_i <- c z_i - s z_{i+1}; a sweep's come in

@@ -1,5 +1,5 @@
 """The stream of rotations from the QL recurrence to the warps that apply them: eigenproblems whose
-rotations fill the ring several times over, again and again and from two streams at once. A count
+rotations fill the ring several times over, again and again, with other work on the SMs. A count
 that some lanes of the copying warp saw and others did not would leave a sweep uncopied."""
 import numpy as np
 import pytest
